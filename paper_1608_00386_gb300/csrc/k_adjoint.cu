@@ -1,24 +1,19 @@
-// Adjoint of the noise-free wavefront sensing: exact derivatives of the slopes with respect to
-// the residual phase and to the DM commands ("The calibration of the interaction matrices":
-// the interaction matrix is the slopes' response to each command; here it is the Jacobian at
-// the current state rather than a finite poke).
+// Adjoint of the DM and layer projections: what the derivatives of the slopes with respect to the
+// residual phase (k_lag.cu) say about the DM commands, the pupil phase and the screens ("The
+// calibration of the interaction matrices": the interaction matrix is the slopes' response to each
+// command; here it is the Jacobian at the current state rather than a finite poke).
 //
-// Forward model of one subaperture (the sensing step of "The closed loop"):
-//   E(x) = A(x) exp(i (s phi(x) - pi (x + y) / N)) on the n_px^2 pupil samples, zero-padded to N,
-//   F = FFT2(E), I = |F|^2, I' = M I with M = IFFT2 . diag(O_s) . FFT2 (sodium elongation; O_s the
-//   OTF made even, (O(u) + O(-u)) / 2, which equals the forward's Re IFFT2(FFT2(I) O) for real
-//   I), shift by N/2, bin b x b into det, CoG (sx, sy) = sum (m - c) det / sum det.
-// Reverse pass for one slope (sx shown): g_det(m) = (m_x - c - sx) / T; unbin and unshift to g;
-//   g <- M g (M is symmetric); H = sum_k g(k) F(k) exp(+2 pi i k.x / N) (unnormalized inverse DFT);
-//   d sx / d phi(x) = -2 s Im(E(x) conj(H(x))).
-// The x and y slopes of a subaperture share the forward pass; their adjoint images travel as the
-// real and imaginary parts of one complex image through the (real) elongation operator.
-//
-// Projection on the DMs: phi(p) = ... - bilinear(S_m, p) and S_m = Gy C Gx^T, so
+// phi(p) = ... - bilinear(S_m, p) and S_m = Gy C Gx^T, so
 //   d phi(p) / d C[b][a] = -((1 - t_x) Gx[i0][a] + t_x Gx[i1][a]) ((1 - t_y) Gy[j0][b] + t_y Gy[j1][b]),
 // the same fixed-point sample positions and clamped bilinear weights as the forward; actuators
 // outside the union of the forward's per-tile bands (weights below 1e-10) are left out.  A
 // rotated DM has no separable tables: its weights are evaluated at each bilinear corner.
+//
+// The interaction matrix is written row by row, zeros included, by one pass (dm_rows_kernel); the
+// product of its transpose with given vectors never forms a row: the pupil-phase gradient of each
+// sensor goes through the two separable weight tables (dm_project_x / dm_project_y).
+#include <algorithm>
+
 #include "device_common.cuh"
 #include "mcao_internal.h"
 
@@ -27,250 +22,47 @@ namespace mcao {
 namespace {
 
 constexpr int kAdjThreads = 256;
-constexpr float kPi = 3.14159265358979323846f;
 constexpr int kAdjMaxBand = 128;   // actuators per axis acting on one subaperture footprint
 
-__device__ __forceinline__ float2* fft2_smem(float2* a, float2* b, int N, const int* rad, int nr, const float2* W,
-                                             int tid, int nthr) {
-    float2* r = stockham_fft(a, b, N, rad, nr, N, N, 1, W, tid, nthr);          // rows
-    return stockham_fft(r, r == a ? b : a, N, rad, nr, N, 1, N, W, tid, nthr);  // columns
+// d slope / d phase on the slope's n_px^2 samples (axis 0: x slope, 1: y slope)
+__device__ __forceinline__ const float* sens_row(const float* sens, const WfsDev& w, int axis, int rank) {
+    return sens + w.sens0 + ((long long)axis * w.n_valid + rank) * (w.n_px * w.n_px);
 }
 
-// even elongation OTF at frequency index (kx, ky): (O(u) + O(-u)) / 2, O(u) = exp(-a (u . d)^2),
-// u the signed frequency of the index
-__device__ __forceinline__ float otf_even(int kx, int ky, int N, float a, float dx, float dy) {
-    const int ux = kx < N / 2 ? kx : kx - N, uy = ky < N / 2 ? ky : ky - N;
-    const int mx = (N - kx) % N, my = (N - ky) % N;
-    const int vx = mx < N / 2 ? mx : mx - N, vy = my < N / 2 ? my : my - N;
-    const float d1 = (float)ux * dx + (float)uy * dy, d2 = (float)vx * dx + (float)vy * dy;
-    return 0.5f * (expf(-a * d1 * d1) + expf(-a * d2 * d2));
+// 1 - t and t of a pupil column / row's two table rows, combined for actuator a
+__device__ __forceinline__ float axis_weight(const float* G, int na, AxisEnt e, int a) {
+    return (1.0f - e.t) * G[(long long)(e.idx & 0xffff) * na + a] + e.t * G[(long long)(e.idx >> 16) * na + a];
 }
 
-// x <- M x = IFFT2(O_s FFT2(x)) for the image in a; returns the buffer holding the result
-__device__ float2* elongate(float2* a, float2* b, int N, const int* rad, int nr, const float2* W, float ea, float dx,
-                            float dy, int tid, int nthr) {
-    float2* r = fft2_smem(a, b, N, rad, nr, W, tid, nthr);
-    for (int q = tid; q < N * N; q += nthr) {
-        const float o = otf_even(q % N, q / N, N, ea, dx, dy);
-        r[q] = make_float2(r[q].x * o, -r[q].y * o);   // conj for the inverse by a forward FFT
-    }
-    __syncthreads();
-    float2* r2 = fft2_smem(r, r == a ? b : a, N, rad, nr, W, tid, nthr);
-    const float inv = 1.0f / (float)(N * N);
-    for (int q = tid; q < N * N; q += nthr) r2[q] = make_float2(r2[q].x * inv, -r2[q].y * inv);
-    __syncthreads();
-    return r2;
-}
-
-__device__ __forceinline__ float block_sum(float v, float* red, int tid, int nthr) {
-    v = warp_sum(v);
-    if ((tid & 31) == 0) red[tid >> 5] = v;
-    __syncthreads();
-    float s = 0.0f;
-    for (int q = 0; q < nthr / 32; ++q) s += red[q];
-    __syncthreads();
-    return s;
-}
-
-// One block per valid subaperture of one sensor: d s / d phi on its n_px^2 pupil samples for
-// both of its slopes, rows slope0 + rank (x) and slope0 + n_valid + rank (y) of sens.
-__global__ void __launch_bounds__(kAdjThreads) wfs_sens_kernel(SensLaunch L) {
-    extern __shared__ float4 smem_raw[];
-    const SubapDev sd = L.subaps[blockIdx.x];
-    const WfsDev& w = L.ctx.wfs[sd.wfs];
-    const int N = w.n_fft, npx = w.n_px, nb = w.n_bin, nd = w.n_det, NN = N * N;
-    float2* E = reinterpret_cast<float2*>(smem_raw);
-    float2* F = E + NN;
-    float2* G = F + NN;
-    float2* A = G + NN;
-    float2* B = A + NN;
-    float2* W = B + NN;
-    float* red = reinterpret_cast<float*>(W + N);
-    const int tid = threadIdx.x, nthr = blockDim.x;
-
-    int rad[8];
-    int nr = 0;
-    for (int n = N; n > 1 && nr < 8;) {
-        const int r = (n % 4 == 0) ? 4 : 2;
-        rad[nr++] = r;
-        n /= r;
-    }
-    for (int q = tid; q < N; q += nthr) {
-        float s, c;
-        sincospif(-2.0f * (float)q / (float)N, &s, &c);
-        W[q] = make_float2(c, s);
-    }
-    for (int q = tid; q < NN; q += nthr) E[q] = make_float2(0.0f, 0.0f);
-    __syncthreads();
-
-    // forward: residual phase, field, spectrum
-    const GridView* V = L.ctx.views + L.real * L.ctx.view_stride + (long long)sd.wfs * L.ctx.n_grids;
-    const long long k = L.ctx.st->k;
-    const int i0 = sd.sx * npx, j0 = sd.sy * npx;
-    const float scale = w.scale;
-    for (int q = tid; q < npx * npx; q += nthr) {
-        const int x = q % npx, y = q / npx;
-        float phi = 0.0f;
-        for (int g = 0; g < L.ctx.n_grids; ++g) {
-            const GridView& v = V[g];
-            const AxisEnt ex = axis_entry(v.ax + (long long)(i0 + x) * v.bp + k * v.vx, v.n, v.periodic, v.inv_n);
-            const AxisEnt ey = axis_entry(v.ay + (long long)(j0 + y) * v.bp + k * v.vy, v.n, v.periodic, v.inv_n);
-            phi = fmaf(v.sign, bilinear(v.data, v.n, ex, ey), phi);
-        }
-        const float a = __ldg(w.amp + (long long)(j0 + y) * w.N + i0 + x);
-        const float arg = scale * phi - kPi * (float)(x + y) / (float)N;
-        float sn, cs;
-        sincosf(arg, &sn, &cs);
-        E[y * N + x] = make_float2(a * cs, a * sn);
-    }
-    __syncthreads();
-    for (int q = tid; q < NN; q += nthr) A[q] = E[q];
-    __syncthreads();
-    {
-        const float2* r = fft2_smem(A, B, N, rad, nr, W, tid, nthr);
-        for (int q = tid; q < NN; q += nthr) F[q] = r[q];
-    }
-    __syncthreads();
-    for (int q = tid; q < NN; q += nthr) A[q] = make_float2(F[q].x * F[q].x + F[q].y * F[q].y, 0.0f);
-    __syncthreads();
-    const bool elong = sd.elong_a > 0.0f;
-    const float2* img = elong ? elongate(A, B, N, rad, nr, W, sd.elong_a, sd.dir_x, sd.dir_y, tid, nthr) : A;
-
-    // binned detector image and its centre of gravity
-    const float c0 = 0.5f * (float)(nd - 1);
-    float tv = 0.0f, tx = 0.0f, ty = 0.0f;
-    for (int m = tid; m < nd * nd; m += nthr) {
-        const int my = m / nd, mx = m % nd;
-        float b = 0.0f;
-        for (int yy = 0; yy < nb; ++yy)
-            for (int xx = 0; xx < nb; ++xx) {
-                const int r = (my * nb + yy + N / 2) % N, c = (mx * nb + xx + N / 2) % N;
-                b += img[r * N + c].x;
-            }
-        tv += b;
-        tx += ((float)mx - c0) * b;
-        ty += ((float)my - c0) * b;
-    }
-    tv = block_sum(tv, red, tid, nthr);
-    tx = block_sum(tx, red, tid, nthr);
-    ty = block_sum(ty, red, tid, nthr);
-    const bool live = tv > 0.0f;
-    const float inv_t = live ? 1.0f / tv : 0.0f;
-    const float sx = tx * inv_t, sy = ty * inv_t;
-
-    // adjoint image of the two slopes (x in the real part, y in the imaginary part), unbinned and
-    // unshifted back to the spectrum's index order
-    float2* g = (img == A) ? B : A;
-    for (int q = tid; q < NN; q += nthr) {
-        const int r = q / N, c = q % N;
-        const int my = ((r + N / 2) % N) / nb, mx = ((c + N / 2) % N) / nb;
-        g[q] = live ? make_float2(((float)mx - c0 - sx) * inv_t, ((float)my - c0 - sy) * inv_t) : make_float2(0.0f, 0.0f);
-    }
-    __syncthreads();
-    if (elong) {
-        const float2* r = elongate(g, g == A ? B : A, N, rad, nr, W, sd.elong_a, sd.dir_x, sd.dir_y, tid, nthr);
-        for (int q = tid; q < NN; q += nthr) G[q] = r[q];
-    } else {
-        for (int q = tid; q < NN; q += nthr) G[q] = g[q];
-    }
-    __syncthreads();
-
-    // per slope: H = unnormalized inverse DFT of g F = conj(FFT2(conj(g F))); d s / d phi
-    const long long row_x = (long long)(w.slope0 + sd.rank) * L.P;
-    const long long row_y = (long long)(w.slope0 + w.n_valid + sd.rank) * L.P;
-    for (int part = 0; part < 2; ++part) {
-        for (int q = tid; q < NN; q += nthr) {
-            const float gv = part == 0 ? G[q].x : G[q].y;
-            A[q] = make_float2(gv * F[q].x, -gv * F[q].y);
-        }
-        __syncthreads();
-        const float2* h = fft2_smem(A, B, N, rad, nr, W, tid, nthr);   // conj(H)
-        float* out = L.sens + (part == 0 ? row_x : row_y);
-        for (int q = tid; q < npx * npx; q += nthr) {
-            const int x = q % npx, y = q / npx;
-            const float2 e = E[y * N + x], hc = h[y * N + x];
-            // -2 s Im(E conj(H)), with hc = conj(H)
-            out[q] = -2.0f * scale * (e.x * hc.y + e.y * hc.x);
-        }
-        __syncthreads();
-    }
-}
-
-// Rotated DM: the weight of actuator (a, b) on surface sample (i, j) is the influence function
-// at q(i, j) = R(-rot)((x_i, y_j) - shift) / mag; the slope's row entry sums the subaperture
-// derivative over the four bilinear corners of every pupil sample.
-__device__ void dm_adjoint_general(const ProjLaunch& L, const GridView& v, const DmDesc& dd, int row, int npx,
-                                   const float* s_L, const AxisEnt* s_ex, const AxisEnt* s_ey, int* s_rng) {
-    const int tid = threadIdx.x, nthr = blockDim.x;
-    const float c0 = 0.5f * (float)(dd.surf_n - 1), ca = 0.5f * (float)(dd.nx - 1), cb = 0.5f * (float)(dd.ny - 1);
-    auto to_act = [&](int i, int j, float& ua, float& ub) {
-        const float x = ((float)i - c0) * dd.dx - dd.shx, y = ((float)j - c0) * dd.dx - dd.shy;
-        ua = (dd.cr * x + dd.sr * y) * dd.inv_mag / dd.pitch + ca;
-        ub = (-dd.sr * x + dd.cr * y) * dd.inv_mag / dd.pitch + cb;
-    };
-    if (tid == 0) {
-        int cx0 = v.n, cx1 = 0, cy0 = v.n, cy1 = 0;
-        for (int q = 0; q < npx; ++q) {
-            cx0 = min(cx0, s_ex[q].idx & 0xffff);
-            cx1 = max(cx1, s_ex[q].idx >> 16);
-            cy0 = min(cy0, s_ey[q].idx & 0xffff);
-            cy1 = max(cy1, s_ey[q].idx >> 16);
-        }
+// Actuators [a0, a1) x [b0, b1) of a DM that act on surface samples [cx0, cx1] x [cy0, cy1]: for a
+// separable DM the union of the forward's per-tile bands over the tiles the footprint touches, for a
+// rotated one the actuators within rc pitches of the footprint's corners.
+__device__ void actuator_range(const DmDesc& dd, const int2* band, int cx0, int cx1, int cy0, int cy1, int (&rng)[4]) {
+    int a0 = dd.nx, a1 = 0, b0 = dd.ny, b1 = 0;
+    if (dd.general) {
+        const float c0 = 0.5f * (float)(dd.surf_n - 1), ca = 0.5f * (float)(dd.nx - 1), cb = 0.5f * (float)(dd.ny - 1);
         float lo_a = 1e30f, hi_a = -1e30f, lo_b = 1e30f, hi_b = -1e30f;
         for (int c = 0; c < 4; ++c) {
-            float ua, ub;
-            to_act((c & 1) ? cx1 : cx0, (c & 2) ? cy1 : cy0, ua, ub);
+            const float x = ((float)((c & 1) ? cx1 : cx0) - c0) * dd.dx - dd.shx;
+            const float y = ((float)((c & 2) ? cy1 : cy0) - c0) * dd.dx - dd.shy;
+            const float ua = (dd.cr * x + dd.sr * y) * dd.inv_mag / dd.pitch + ca;
+            const float ub = (-dd.sr * x + dd.cr * y) * dd.inv_mag / dd.pitch + cb;
             lo_a = fminf(lo_a, ua); hi_a = fmaxf(hi_a, ua);
             lo_b = fminf(lo_b, ub); hi_b = fmaxf(hi_b, ub);
         }
-        int a0 = max(0, (int)ceilf(lo_a - dd.rc)), a1 = min(dd.nx - 1, (int)floorf(hi_a + dd.rc)) + 1;
-        int b0 = max(0, (int)ceilf(lo_b - dd.rc)), b1 = min(dd.ny - 1, (int)floorf(hi_b + dd.rc)) + 1;
-        if (a1 < a0) a1 = a0;
-        if (b1 < b0) b1 = b0;
-        if (a1 - a0 > kAdjMaxBand || b1 - b0 > kAdjMaxBand) {
-            atomicExch(L.err, 1);
-            a1 = a0;
-            b1 = b0;
+        a0 = max(0, (int)ceilf(lo_a - dd.rc)); a1 = min(dd.nx - 1, (int)floorf(hi_a + dd.rc)) + 1;
+        b0 = max(0, (int)ceilf(lo_b - dd.rc)); b1 = min(dd.ny - 1, (int)floorf(hi_b + dd.rc)) + 1;
+    } else {
+        for (int t = cx0 / kDmTile; t <= cx1 / kDmTile; ++t) {
+            const int2 bt = band[dd.tband_x + t];
+            if (bt.y > bt.x) { a0 = min(a0, bt.x); a1 = max(a1, bt.y); }
         }
-        s_rng[0] = a0; s_rng[1] = a1; s_rng[2] = b0; s_rng[3] = b1;
-    }
-    __syncthreads();
-    const int a0 = s_rng[0], na = s_rng[1] - s_rng[0], b0 = s_rng[2], nbd = s_rng[3] - s_rng[2];
-    for (int idx = tid; idx < na * nbd; idx += nthr) {
-        const int b = idx / na, a = idx - b * na;
-        const float fa = (float)(a0 + a), fb = (float)(b0 + b);
-        float acc = 0.0f;
-        for (int y = 0; y < npx; ++y) {
-            const AxisEnt ey = s_ey[y];
-            const int r0 = ey.idx & 0xffff, r1 = ey.idx >> 16;
-            for (int x = 0; x < npx; ++x) {
-                const float lv = s_L[y * npx + x];
-                if (lv == 0.0f) continue;
-                const AxisEnt ex = s_ex[x];
-                const int q0 = ex.idx & 0xffff, q1 = ex.idx >> 16;
-                float w = 0.0f;
-                for (int c = 0; c < 4; ++c) {
-                    const int i = (c & 1) ? q1 : q0, j = (c & 2) ? r1 : r0;
-                    const float wc = ((c & 1) ? ex.t : 1.0f - ex.t) * ((c & 2) ? ey.t : 1.0f - ey.t);
-                    float ua, ub;
-                    to_act(i, j, ua, ub);
-                    const float da = (ua - fa) * dd.pitch, db = (ub - fb) * dd.pitch;
-                    w = fmaf(wc, expf(-(da * da + db * db) * dd.inv2s2), w);
-                }
-                acc = fmaf(lv, w, acc);
-            }
+        for (int t = cy0 / kDmTile; t <= cy1 / kDmTile; ++t) {
+            const int2 bt = band[dd.tband_y + t];
+            if (bt.y > bt.x) { b0 = min(b0, bt.x); b1 = max(b1, bt.y); }
         }
-        const float val = v.sign * acc;
-        const int cmd = L.act_map[dd.map_off + (long long)(b0 + b) * dd.nx + a0 + a];
-        if (cmd < 0) continue;
-        if (L.D) L.D[(long long)row * L.ld + cmd] = val;
-        if (L.gc)
-            for (int vv = 0; vv < L.n_vec; ++vv) {
-                const float gv = L.gvec[(long long)vv * L.n_slopes + row];
-                if (gv != 0.0f) atomicAdd(L.gc + (long long)vv * L.n_cmd + cmd, gv * val);
-            }
     }
-    __syncthreads();
+    rng[0] = a0; rng[1] = max(a0, a1); rng[2] = b0; rng[3] = max(b0, b1);
 }
 
 // Gauss-Newton terms of a DM misregistration fit, one block per slope row of one sensor, for DM m
@@ -299,7 +91,8 @@ __global__ void __launch_bounds__(256) misreg_gn_kernel(ProjLaunch L, int m, con
     const int i0 = sd.sx * npx, j0 = sd.sy * npx;
     const GridView* V = L.ctx.views + L.real * L.ctx.view_stride + (long long)sd.wfs * L.ctx.n_grids;
     const long long k = L.ctx.st->k;
-    for (int q = tid; q < npx * npx; q += nthr) s_L[q] = L.sens[(long long)row * L.P + q];
+    const float* sens = sens_row(L.sens, w, axis, sd.rank);
+    for (int q = tid; q < npx * npx; q += nthr) s_L[q] = sens[q];
     const GridView& v = V[L.n_layers + m];
     const DmDesc dd = L.desc[m];
     if (tid < npx)
@@ -421,154 +214,292 @@ __global__ void misreg_sum_kernel(const double* __restrict__ rec, int n_rows, do
     }
 }
 
-// One block per slope of one sensor: the slope's row of d s / d c from its pupil-sample
-// derivatives, written to D (interaction matrix) and/or accumulated as g_v[row] * row into the
-// command gradients of every vector v.
-__global__ void __launch_bounds__(256) dm_adjoint_kernel(ProjLaunch L) {
-    __shared__ float s_L[kMaxNpx * kMaxNpx];
-    __shared__ float s_T[kAdjMaxBand * kMaxNpx];
-    __shared__ float s_gy[kAdjMaxBand * kMaxNpx];
+// Interaction-matrix rows of both slopes of one subaperture (block x) over a part of one DM's
+// commands (block y = DM, block z = part).  Every command of the part is written once, zero
+// outside the actuators that reach the subaperture, so the matrix needs no clearing and its lines
+// are written whole: the pass is bound by the matrix's own bytes (39 m: 1.79 GB).  Before, the
+// matrix was cleared and one block per slope scattered its band into it: 160 us per laser star
+// (9264 blocks waiting at 15 barriers each) and 131 us per natural star (8 blocks) on top of the
+// clearing; x and y slopes now share the axis entries, bands and row weights, and a sensor of a few
+// subapertures is cut into enough parts to fill the GPU.
+// With gvec set (rotated DMs only) the rows are not stored: sum over both slopes of g row is added
+// to the command gradients of every vector.
+__global__ void __launch_bounds__(kAdjThreads) dm_rows_kernel(ProjLaunch L) {
+    extern __shared__ float rows_sm[];
     __shared__ AxisEnt s_ex[kMaxNpx], s_ey[kMaxNpx];
     __shared__ int s_rng[4];
     const int tid = threadIdx.x, nthr = blockDim.x;
-    const int axis = blockIdx.x / L.n_valid, rank = blockIdx.x - axis * L.n_valid;
-    const SubapDev sd = L.subaps[rank];
+    const SubapDev sd = L.subaps[blockIdx.x];
     const WfsDev& w = L.ctx.wfs[sd.wfs];
-    const int npx = w.n_px;
-    const int row = w.slope0 + axis * w.n_valid + sd.rank;
-    const int i0 = sd.sx * npx, j0 = sd.sy * npx;
-    const GridView* V = L.ctx.views + L.real * L.ctx.view_stride + (long long)sd.wfs * L.ctx.n_grids;
-    const long long k = L.ctx.st->k;
-    for (int q = tid; q < npx * npx; q += nthr) s_L[q] = L.sens[(long long)row * L.P + q];
-    for (int m = 0; m < L.n_dms; ++m) {
-        const GridView& v = V[L.n_layers + m];
-        const DmDesc dd = L.desc[m];
-        if (tid < npx)
-            s_ex[tid] = axis_entry(v.ax + (long long)(i0 + tid) * v.bp + k * v.vx, v.n, v.periodic, v.inv_n);
-        else if (tid < 2 * npx)
-            s_ey[tid - npx] = axis_entry(v.ay + (long long)(j0 + tid - npx) * v.bp + k * v.vy, v.n, v.periodic, v.inv_n);
-        __syncthreads();
-        if (dd.general) {
-            dm_adjoint_general(L, v, dd, row, npx, s_L, s_ex, s_ey, s_rng);
-            continue;
+    const DmDesc dd = L.desc[blockIdx.y];
+    if (L.gvec && !dd.general) return;
+    const int npx = w.n_px, i0 = sd.sx * npx, j0 = sd.sy * npx;
+    const GridView& v = L.ctx.views[L.real * L.ctx.view_stride + (long long)sd.wfs * L.ctx.n_grids + L.n_layers + blockIdx.y];
+    float* s_L = rows_sm;                                  // [2][npx][npx]
+    float* s_T = s_L + 2 * npx * npx;                      // [2][npx][kAdjMaxBand]
+    float* s_gy = s_T + 2 * npx * kAdjMaxBand;             // [kAdjMaxBand][npx]
+    const float *lx = sens_row(L.sens, w, 0, sd.rank), *ly = sens_row(L.sens, w, 1, sd.rank);
+    for (int q = tid; q < npx * npx; q += nthr) {
+        s_L[q] = lx[q];
+        s_L[npx * npx + q] = ly[q];
+    }
+    if (tid < npx)
+        s_ex[tid] = axis_entry(v.ax + (long long)(i0 + tid) * v.bp, v.n, v.periodic, v.inv_n);
+    else if (tid < 2 * npx)
+        s_ey[tid - npx] = axis_entry(v.ay + (long long)(j0 + tid - npx) * v.bp, v.n, v.periodic, v.inv_n);
+    __syncthreads();
+    if (tid == 0) {
+        // the axis entries ascend (a DM grid does not wrap): the footprint is the first and last
+        int rng[4];
+        actuator_range(dd, L.band, s_ex[0].idx & 0xffff, s_ex[npx - 1].idx >> 16, s_ey[0].idx & 0xffff,
+                       s_ey[npx - 1].idx >> 16, rng);
+        if (rng[1] - rng[0] > kAdjMaxBand || rng[3] - rng[2] > kAdjMaxBand) {
+            atomicExch(L.err, 1);
+            rng[1] = rng[0];
+            rng[3] = rng[2];
         }
-        if (tid == 0) {
-            int cx0 = v.n, cx1 = 0, cy0 = v.n, cy1 = 0;
-            for (int q = 0; q < npx; ++q) {
-                cx0 = min(cx0, s_ex[q].idx & 0xffff);
-                cx1 = max(cx1, s_ex[q].idx >> 16);
-                cy0 = min(cy0, s_ey[q].idx & 0xffff);
-                cy1 = max(cy1, s_ey[q].idx >> 16);
-            }
-            // union of the forward's per-tile actuator bands over the tiles the footprint touches
-            int a0 = dd.nx, a1 = 0, b0 = dd.ny, b1 = 0;
-            for (int t = cx0 / kDmTile; t <= cx1 / kDmTile; ++t) {
-                const int2 bt = L.band[dd.tband_x + t];
-                if (bt.y > bt.x) { a0 = min(a0, bt.x); a1 = max(a1, bt.y); }
-            }
-            for (int t = cy0 / kDmTile; t <= cy1 / kDmTile; ++t) {
-                const int2 bt = L.band[dd.tband_y + t];
-                if (bt.y > bt.x) { b0 = min(b0, bt.x); b1 = max(b1, bt.y); }
-            }
-            if (a1 < a0) a1 = a0;
-            if (b1 < b0) b1 = b0;
-            if (a1 - a0 > kAdjMaxBand || b1 - b0 > kAdjMaxBand) {
-                atomicExch(L.err, 1);
-                a1 = a0;
-                b1 = b0;
-            }
-            s_rng[0] = a0; s_rng[1] = a1; s_rng[2] = b0; s_rng[3] = b1;
-        }
-        __syncthreads();
-        const int a0 = s_rng[0], na = s_rng[1] - s_rng[0], b0 = s_rng[2], nbd = s_rng[3] - s_rng[2];
-        const float* Gx = L.g + dd.gx_off;
-        const float* Gy = L.g + dd.gy_off;
-        // T[a][y] = sum_x L[y][x] gx_a(x)
+        for (int q = 0; q < 4; ++q) s_rng[q] = rng[q];
+    }
+    __syncthreads();
+    const int a0 = s_rng[0], na = s_rng[1] - s_rng[0], b0 = s_rng[2], nbd = s_rng[3] - s_rng[2];
+    if (!dd.general) {
+        // T[axis][y][a] = sum_x L[axis][y][x] gx_a(x)
+        const float *Gx = L.g + dd.gx_off + a0, *Gy = L.g + dd.gy_off + b0;
         for (int idx = tid; idx < na * npx; idx += nthr) {
-            const int a = idx / npx, y = idx - a * npx;
-            float acc = 0.0f;
+            const int y = idx / na, a = idx - y * na;
+            float ax = 0.0f, ay = 0.0f;
             for (int x = 0; x < npx; ++x) {
-                const AxisEnt e = s_ex[x];
-                const int c0 = e.idx & 0xffff, c1 = e.idx >> 16;
-                const float gxa = (1.0f - e.t) * Gx[(long long)c0 * dd.nx + a0 + a] + e.t * Gx[(long long)c1 * dd.nx + a0 + a];
-                acc = fmaf(s_L[y * npx + x], gxa, acc);
+                const float g = axis_weight(Gx, dd.nx, s_ex[x], a);
+                ax = fmaf(s_L[y * npx + x], g, ax);
+                ay = fmaf(s_L[(npx + y) * npx + x], g, ay);
             }
-            s_T[a * npx + y] = acc;
+            s_T[y * kAdjMaxBand + a] = ax;
+            s_T[(npx + y) * kAdjMaxBand + a] = ay;
         }
         for (int idx = tid; idx < nbd * npx; idx += nthr) {
-            const int b = idx / npx, y = idx - b * npx;
-            const AxisEnt e = s_ey[y];
-            const int r0 = e.idx & 0xffff, r1 = e.idx >> 16;
-            s_gy[b * npx + y] = (1.0f - e.t) * Gy[(long long)r0 * dd.ny + b0 + b] + e.t * Gy[(long long)r1 * dd.ny + b0 + b];
+            const int y = idx / nbd, b = idx - y * nbd;
+            s_gy[b * npx + y] = axis_weight(Gy, dd.ny, s_ey[y], b);
         }
         __syncthreads();
-        for (int idx = tid; idx < na * nbd; idx += nthr) {
-            const int b = idx / na, a = idx - b * na;
-            float acc = 0.0f;
-            for (int y = 0; y < npx; ++y) acc = fmaf(s_gy[b * npx + y], s_T[a * npx + y], acc);
-            const float val = v.sign * acc;
-            const int cmd = L.act_map[dd.map_off + (long long)(b0 + b) * dd.nx + a0 + a];
-            if (cmd < 0) continue;
-            if (L.D) L.D[(long long)row * L.ld + cmd] = val;
-            if (L.gc)
+    }
+    const float c0 = 0.5f * (float)(dd.surf_n - 1), ca = 0.5f * (float)(dd.nx - 1), cb = 0.5f * (float)(dd.ny - 1);
+    const int len = (dd.n_cmd + gridDim.z - 1) / gridDim.z, first = blockIdx.z * len;
+    const int last = min(dd.n_cmd, first + len);
+    const int row_x = w.slope0 + sd.rank, row_y = row_x + w.n_valid;
+    float* out_x = L.D ? L.D + (long long)row_x * L.ld + dd.cmd0 : nullptr;
+    float* out_y = L.D ? L.D + (long long)row_y * L.ld + dd.cmd0 : nullptr;
+    for (int j = first + tid; j < last; j += nthr) {
+        const int ab = __ldg(L.cmd_act + dd.cmd0 + j), a = (ab & 0xffff) - a0, b = (int)((unsigned)ab >> 16) - b0;
+        float vx = 0.0f, vy = 0.0f;
+        if ((unsigned)a < (unsigned)na && (unsigned)b < (unsigned)nbd) {
+            if (!dd.general) {
+                for (int y = 0; y < npx; ++y) {
+                    const float g = s_gy[b * npx + y];
+                    vx = fmaf(g, s_T[y * kAdjMaxBand + a], vx);
+                    vy = fmaf(g, s_T[(npx + y) * kAdjMaxBand + a], vy);
+                }
+            } else {
+                // influence function of actuator (a, b) at q(i, j) = R(-rot)((x_i, y_j) - shift) / mag,
+                // at the four bilinear corners of every sample
+                const float fa = (float)(a0 + a), fb = (float)(b0 + b);
+                for (int q = 0; q < npx * npx; ++q) {
+                    const float l0 = s_L[q], l1 = s_L[npx * npx + q];
+                    if (l0 == 0.0f && l1 == 0.0f) continue;
+                    const AxisEnt ex = s_ex[q % npx], ey = s_ey[q / npx];
+                    float wt = 0.0f;
+                    for (int c = 0; c < 4; ++c) {
+                        const int i = (c & 1) ? ex.idx >> 16 : ex.idx & 0xffff, k = (c & 2) ? ey.idx >> 16 : ey.idx & 0xffff;
+                        const float wc = ((c & 1) ? ex.t : 1.0f - ex.t) * ((c & 2) ? ey.t : 1.0f - ey.t);
+                        const float x = ((float)i - c0) * dd.dx - dd.shx, y = ((float)k - c0) * dd.dx - dd.shy;
+                        const float ua = (dd.cr * x + dd.sr * y) * dd.inv_mag / dd.pitch + ca;
+                        const float ub = (-dd.sr * x + dd.cr * y) * dd.inv_mag / dd.pitch + cb;
+                        const float da = (ua - fa) * dd.pitch, db = (ub - fb) * dd.pitch;
+                        wt = fmaf(wc, expf(-(da * da + db * db) * dd.inv2s2), wt);
+                    }
+                    vx = fmaf(l0, wt, vx);
+                    vy = fmaf(l1, wt, vy);
+                }
+            }
+            vx *= v.sign;
+            vy *= v.sign;
+            if (L.gvec)
                 for (int vv = 0; vv < L.n_vec; ++vv) {
-                    const float gv = L.gvec[(long long)vv * L.n_slopes + row];
-                    if (gv != 0.0f) atomicAdd(L.gc + (long long)vv * L.n_cmd + cmd, gv * val);
+                    const float* g = L.gvec + (long long)vv * L.n_slopes;
+                    const float add = fmaf(g[row_x], vx, g[row_y] * vy);
+                    if (add != 0.0f) atomicAdd(L.gc + (long long)vv * L.n_cmd + dd.cmd0 + j, add);
                 }
         }
-        __syncthreads();
+        if (out_x) {
+            __stcs(out_x + j, vx);
+            __stcs(out_y + j, vy);
+        }
+    }
+    // padding columns past the last command
+    if (L.D && blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1)
+        for (long long j = L.n_cmd + tid; j < L.ld; j += nthr) L.D[(long long)row_x * L.ld + j] = L.D[(long long)row_y * L.ld + j] = 0.0f;
+}
+
+// Flags a subaperture whose footprint on a DM meets more actuators than the rows kernel takes (one
+// thread per subaperture and DM), so that the products refuse what the matrix refuses.
+__global__ void dm_range_kernel(ProjLaunch L) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= L.n_valid * L.n_dms) return;
+    const int m = i / L.n_valid;
+    const SubapDev sd = L.subaps[i - m * L.n_valid];
+    const WfsDev& w = L.ctx.wfs[sd.wfs];
+    const GridView& v = L.ctx.views[L.real * L.ctx.view_stride + (long long)sd.wfs * L.ctx.n_grids + L.n_layers + m];
+    auto at = [&](long long a, int i0, int q) { return axis_entry(a + (long long)(i0 + q) * v.bp, v.n, v.periodic, v.inv_n).idx; };
+    const int i0 = sd.sx * w.n_px, j0 = sd.sy * w.n_px;
+    int rng[4];
+    actuator_range(L.desc[m], L.band, at(v.ax, i0, 0) & 0xffff, at(v.ax, i0, w.n_px - 1) >> 16, at(v.ay, j0, 0) & 0xffff,
+                   at(v.ay, j0, w.n_px - 1) >> 16, rng);
+    if (rng[1] - rng[0] > kAdjMaxBand || rng[3] - rng[2] > kAdjMaxBand) atomicExch(L.err, 1);
+}
+
+// D^T g of the separable DMs from the sensors' pupil-phase gradients, in two passes over the
+// separable weights: U[y][a] = sum_x g(y, x) gx_a(x), then C[b][a] -= sum_y gy_b(y) U[y][a] over
+// every sensor, in a fixed order.  The products are N^2 n_x + N n_x n_y per sensor and DM, whatever
+// the number of subapertures (before: each slope's row, added into the gradient by atomics).
+// Block: 8 pupil rows (one per warp) x 32 actuators per pass; x in tiles of 32 whose band of
+// actuators with a weight meets the 32.
+__global__ void __launch_bounds__(256) dm_project_x(ProjLaunch L, const float* __restrict__ g_phase, long long phase_stride,
+                                                    float* __restrict__ U, int u_rows, int u_cols) {
+    __shared__ float s_w[32][33];
+    __shared__ float s_g[8][32];
+    const int wi = blockIdx.y / L.n_dms, m = blockIdx.y - wi * L.n_dms, vec = blockIdx.z;
+    const WfsDev& w = L.ctx.wfs[wi];
+    const DmDesc dd = L.desc[m];
+    const int N = w.N, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int y = blockIdx.x * 8 + warp;
+    if (dd.general || (int)blockIdx.x * 8 >= N) return;
+    long long off = vec * phase_stride;
+    for (int q = 0; q < wi; ++q) off += (long long)L.ctx.wfs[q].N * L.ctx.wfs[q].N;
+    const GridView& v = L.ctx.views[L.real * L.ctx.view_stride + (long long)wi * L.ctx.n_grids + L.n_layers + m];
+    float* u = U + (((long long)vec * gridDim.y + blockIdx.y) * u_rows + y) * u_cols;
+    for (int a0 = 0; a0 < dd.nx; a0 += 32) {
+        float acc = 0.0f;
+        for (int x0 = 0; x0 < N; x0 += 32) {
+            const int xe = min(x0 + 32, N) - 1;
+            const AxisEnt e0 = axis_entry(v.ax + (long long)x0 * v.bp, v.n, v.periodic, v.inv_n);
+            const AxisEnt e1 = axis_entry(v.ax + (long long)xe * v.bp, v.n, v.periodic, v.inv_n);
+            int lo = dd.nx, hi = 0;
+            for (int t = (e0.idx & 0xffff) / kDmTile; t <= (e1.idx >> 16) / kDmTile; ++t) {
+                const int2 bt = L.band[dd.tband_x + t];
+                if (bt.y > bt.x) { lo = min(lo, bt.x); hi = max(hi, bt.y); }
+            }
+            if (hi <= a0 || lo >= a0 + 32) continue;   // the same for the whole block
+            __syncthreads();
+            for (int q = threadIdx.x; q < 32 * 32; q += 256) {
+                const int x = x0 + (q >> 5), a = a0 + (q & 31);
+                float wt = 0.0f;
+                if (x < N && a >= lo && a < hi)
+                    wt = axis_weight(L.g + dd.gx_off, dd.nx, axis_entry(v.ax + (long long)x * v.bp, v.n, v.periodic, v.inv_n), a);
+                s_w[q >> 5][q & 31] = wt;
+            }
+            s_g[warp][lane] = (y < N && x0 + lane < N) ? g_phase[off + (long long)y * N + x0 + lane] : 0.0f;
+            __syncthreads();
+#pragma unroll 8
+            for (int x = 0; x < 32; ++x) acc = fmaf(s_g[warp][x], s_w[x][lane], acc);
+        }
+        if (y < N && a0 + lane < dd.nx) u[a0 + lane] = acc;
+    }
+}
+
+// one block per (DM row b, 32 actuator columns): 8 warps take the pupil rows in turn
+__global__ void __launch_bounds__(256) dm_project_y(ProjLaunch L, int n_wfs, const float* __restrict__ U, int u_rows,
+                                                    int u_cols) {
+    __shared__ float s_sum[8][32];
+    const int m = blockIdx.z % L.n_dms, vec = blockIdx.z / L.n_dms;
+    const DmDesc dd = L.desc[m];
+    const int b = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, a = blockIdx.x * 32 + lane;
+    if (dd.general || b >= dd.ny || (int)blockIdx.x * 32 >= dd.nx) return;
+    float acc = 0.0f;
+    for (int wi = 0; wi < n_wfs; ++wi) {
+        const WfsDev& w = L.ctx.wfs[wi];
+        const GridView& v = L.ctx.views[L.real * L.ctx.view_stride + (long long)wi * L.ctx.n_grids + L.n_layers + m];
+        const float* u = U + ((long long)vec * n_wfs + wi) * L.n_dms * u_rows * u_cols + (long long)m * u_rows * u_cols;
+        for (int y = warp; y < w.N; y += 8) {
+            const AxisEnt e = axis_entry(v.ay + (long long)y * v.bp, v.n, v.periodic, v.inv_n);
+            const int2 b0 = L.band[dd.tband_y + (e.idx & 0xffff) / kDmTile], b1 = L.band[dd.tband_y + (e.idx >> 16) / kDmTile];
+            if (!((b >= b0.x && b < b0.y) || (b >= b1.x && b < b1.y))) continue;
+            const float gy = axis_weight(L.g + dd.gy_off, dd.ny, e, b);
+            if (a < dd.nx) acc = fmaf(v.sign * gy, u[(long long)y * u_cols + a], acc);
+        }
+    }
+    s_sum[warp][lane] = acc;
+    __syncthreads();
+    if (warp == 0 && a < dd.nx) {
+        float s = 0.0f;
+        for (int q = 0; q < 8; ++q) s += s_sum[q][lane];
+        const int cmd = L.act_map[dd.map_off + (long long)b * dd.nx + a];
+        if (cmd >= 0) L.gc[(long long)vec * L.n_cmd + cmd] = s;
     }
 }
 
 // Per subaperture and vector: g_phi = g_v[x slope] L_x + g_v[y slope] L_y on its pupil samples,
-// stored in g_phase[v][off + (j0 + y) N + i0 + x] and/or scattered onto the layers (the adjoint of
-// the periodic bilinear sampling at the frozen-flow position of the step) in g_layers[v][...].
-__global__ void phase_adjoint_kernel(ProjLaunch L, float* g_phase, long long phase_stride, long long phase_off,
-                                     float* g_layers, long long layer_stride, const long long* layer_off) {
+// stored in g_phase[v][sensor's offset + (j0 + y) N + i0 + x] and/or scattered onto the layers (the
+// adjoint of the periodic bilinear sampling at the frozen-flow position of the step) in
+// g_layers[v][...].  The subapertures of every sensor in one launch, block y = vector.
+__global__ void __launch_bounds__(128) phase_adjoint_kernel(ProjLaunch L, float* g_phase, long long phase_stride,
+                                                            float* g_layers, long long layer_stride,
+                                                            const long long* layer_off) {
     const SubapDev sd = L.subaps[blockIdx.x];
     const WfsDev& w = L.ctx.wfs[sd.wfs];
-    const int npx = w.n_px;
-    const int rx = w.slope0 + sd.rank, ry = w.slope0 + w.n_valid + sd.rank;
+    const int npx = w.n_px, vv = blockIdx.y;
     const int i0 = sd.sx * npx, j0 = sd.sy * npx;
     const GridView* V = L.ctx.views + L.real * L.ctx.view_stride + (long long)sd.wfs * L.ctx.n_grids;
     const long long k = L.ctx.st->k;
-    for (int vv = 0; vv < L.n_vec; ++vv) {
-        const float gx = L.gvec[(long long)vv * L.n_slopes + rx], gy = L.gvec[(long long)vv * L.n_slopes + ry];
-        for (int q = threadIdx.x; q < npx * npx; q += blockDim.x) {
-            const int x = q % npx, y = q / npx;
-            const float gp = gx * L.sens[(long long)rx * L.P + q] + gy * L.sens[(long long)ry * L.P + q];
-            if (g_phase) g_phase[vv * phase_stride + phase_off + (long long)(j0 + y) * w.N + i0 + x] = gp;
-            if (!g_layers || gp == 0.0f) continue;
-            for (int l = 0; l < L.n_layers; ++l) {
-                const GridView& v = V[l];
-                const AxisEnt ex = axis_entry(v.ax + (long long)(i0 + x) * v.bp + k * v.vx, v.n, v.periodic, v.inv_n);
-                const AxisEnt ey = axis_entry(v.ay + (long long)(j0 + y) * v.bp + k * v.vy, v.n, v.periodic, v.inv_n);
-                float* gl = g_layers + vv * layer_stride + layer_off[l];
-                const int c0 = ex.idx & 0xffff, c1 = ex.idx >> 16, r0 = ey.idx & 0xffff, r1 = ey.idx >> 16;
-                const float s = v.sign * gp;
-                atomicAdd(gl + (long long)r0 * v.n + c0, s * (1.0f - ex.t) * (1.0f - ey.t));
-                atomicAdd(gl + (long long)r0 * v.n + c1, s * ex.t * (1.0f - ey.t));
-                atomicAdd(gl + (long long)r1 * v.n + c0, s * (1.0f - ex.t) * ey.t);
-                atomicAdd(gl + (long long)r1 * v.n + c1, s * ex.t * ey.t);
-            }
+    const float *lx = sens_row(L.sens, w, 0, sd.rank), *ly = sens_row(L.sens, w, 1, sd.rank);
+    const float* g = L.gvec + (long long)vv * L.n_slopes + w.slope0 + sd.rank;
+    const float gx = g[0], gy = g[w.n_valid];
+    long long off = vv * phase_stride;
+    for (int q = 0; q < sd.wfs; ++q) off += (long long)L.ctx.wfs[q].N * L.ctx.wfs[q].N;
+    for (int q = threadIdx.x; q < npx * npx; q += blockDim.x) {
+        const int x = q % npx, y = q / npx;
+        const float gp = gx * lx[q] + gy * ly[q];
+        if (g_phase) g_phase[off + (long long)(j0 + y) * w.N + i0 + x] = gp;
+        if (!g_layers || gp == 0.0f) continue;
+        for (int l = 0; l < L.n_layers; ++l) {
+            const GridView& v = V[l];
+            const AxisEnt ex = axis_entry(v.ax + (long long)(i0 + x) * v.bp + k * v.vx, v.n, v.periodic, v.inv_n);
+            const AxisEnt ey = axis_entry(v.ay + (long long)(j0 + y) * v.bp + k * v.vy, v.n, v.periodic, v.inv_n);
+            float* gl = g_layers + vv * layer_stride + layer_off[l];
+            const int c0 = ex.idx & 0xffff, c1 = ex.idx >> 16, r0 = ey.idx & 0xffff, r1 = ey.idx >> 16;
+            const float s = v.sign * gp;
+            atomicAdd(gl + (long long)r0 * v.n + c0, s * (1.0f - ex.t) * (1.0f - ey.t));
+            atomicAdd(gl + (long long)r0 * v.n + c1, s * ex.t * (1.0f - ey.t));
+            atomicAdd(gl + (long long)r1 * v.n + c0, s * (1.0f - ex.t) * ey.t);
+            atomicAdd(gl + (long long)r1 * v.n + c1, s * ex.t * ey.t);
         }
     }
 }
 
 }  // namespace
 
-size_t sens_smem(int n_fft) { return sizeof(float2) * (5 * (size_t)n_fft * n_fft + n_fft) + sizeof(float) * 32; }
-
-cudaError_t launch_sens(const SensLaunch& L, int n_fft, cudaStream_t s) {
-    const size_t bytes = sens_smem(n_fft);
-    cudaError_t e = cudaFuncSetAttribute(wfs_sens_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+cudaError_t launch_dm_rows(const ProjLaunch& L, int n_px, int sm_count, cudaStream_t s) {
+    if (!L.n_valid || !L.n_dms) return cudaSuccess;
+    const size_t bytes = sizeof(float) * (2 * n_px * n_px + 3 * n_px * kAdjMaxBand);   // at most 57344
+    cudaError_t e = cudaFuncSetAttribute(dm_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
-    if (L.n_subaps) wfs_sens_kernel<<<(unsigned)L.n_subaps, kAdjThreads, bytes, s>>>(L);
+    // parts of a DM's commands: two blocks per SM where the subapertures alone do not give them
+    const int parts = std::max(1, std::min(16, 2 * sm_count / std::max(1, L.n_valid * L.n_dms)));
+    dm_rows_kernel<<<dim3((unsigned)L.n_valid, (unsigned)L.n_dms, (unsigned)parts), kAdjThreads, bytes, s>>>(L);
     return cudaGetLastError();
 }
 
-cudaError_t launch_dm_adjoint(const ProjLaunch& L, cudaStream_t s) {
-    if (L.n_valid && L.n_dms) dm_adjoint_kernel<<<(unsigned)(2 * L.n_valid), 256, 0, s>>>(L);
+cudaError_t launch_dm_range(const ProjLaunch& L, cudaStream_t s) {
+    const int n = L.n_valid * L.n_dms;
+    if (n) dm_range_kernel<<<(n + 127) / 128, 128, 0, s>>>(L);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_dm_project(const ProjLaunch& L, int n_wfs, int max_n, int max_nx, int max_ny, const float* g_phase,
+                              long long phase_stride, float* U, cudaStream_t s) {
+    if (!L.n_dms || !n_wfs) return cudaSuccess;
+    dm_project_x<<<dim3((unsigned)((max_n + 7) / 8), (unsigned)(n_wfs * L.n_dms), (unsigned)L.n_vec), 256, 0, s>>>(
+        L, g_phase, phase_stride, U, max_n, max_nx);
+    dm_project_y<<<dim3((unsigned)((max_nx + 31) / 32), (unsigned)max_ny, (unsigned)(L.n_dms * L.n_vec)), 256, 0, s>>>(
+        L, n_wfs, U, max_n, max_nx);
     return cudaGetLastError();
 }
 
@@ -583,11 +514,11 @@ cudaError_t launch_misreg_sum(const double* rec, int n_rows, double* out, cudaSt
     return cudaGetLastError();
 }
 
-cudaError_t launch_phase_adjoint(const ProjLaunch& L, float* g_phase, long long phase_stride, long long phase_off,
-                                 float* g_layers, long long layer_stride, const long long* layer_off, cudaStream_t s) {
+cudaError_t launch_phase_adjoint(const ProjLaunch& L, float* g_phase, long long phase_stride, float* g_layers,
+                                 long long layer_stride, const long long* layer_off, cudaStream_t s) {
     if (L.n_valid)
-        phase_adjoint_kernel<<<(unsigned)L.n_valid, 128, 0, s>>>(L, g_phase, phase_stride, phase_off, g_layers,
-                                                                 layer_stride, layer_off);
+        phase_adjoint_kernel<<<dim3((unsigned)L.n_valid, (unsigned)L.n_vec), 128, 0, s>>>(L, g_phase, phase_stride, g_layers,
+                                                                                         layer_stride, layer_off);
     return cudaGetLastError();
 }
 

@@ -52,7 +52,12 @@ struct WfsHost {
     std::vector<int> valid;        // subaperture index sy*n_sub+sx
     std::vector<double> frac;
     std::vector<SubapDev> subaps;
-    SubapDev* d_subaps = nullptr;
+    SubapDev* d_subaps = nullptr;  // this sensor's part of mcao_sim::d_subaps_all
+};
+
+struct WfsRun {                    // consecutive sensors with the same n_px: one launch of the noise-free kernels
+    int n_px, n_subaps;
+    const SubapDev* d_subaps;
 };
 
 struct FftGroup {                  // block-per-subaperture sensors sharing one kernel variant
@@ -103,6 +108,13 @@ struct mcao_sim {
 
     // wfs
     WfsDev* d_wfs = nullptr;
+    SubapDev* d_subaps_all = nullptr;     // every sensor's valid subapertures, in sensor order
+    std::vector<WfsRun> runs;
+    long long sens_total = 0;             // floats of every slope's derivatives
+    float* d_sens = nullptr;              // calibration workspace: allocated by the first call that needs it
+    int* d_adj_err = nullptr;             // band overflow flag of the calibration kernels
+    float* d_vjp = nullptr;               // command-gradient workspace: pupil gradients, then U
+    size_t vjp_floats = 0;
     float* d_amp_all = nullptr;
     float* d_slopes = nullptr;
     float* d_slopes_pad = nullptr;        // slopes in R's padded column layout
@@ -130,6 +142,7 @@ struct mcao_sim {
     int dm_nb = 1;                        // largest actuator band of a 64 x 64 DM block (either axis)
     int2* d_dm_band = nullptr;
     int* d_dm_map = nullptr;
+    int* d_cmd_act = nullptr;             // [n_cmd] actuator of each command
     float* d_dm_surf = nullptr;
     int dm_tile_start[kMaxDms + 1] = {0};
     int n_cmd = 0;
@@ -714,7 +727,7 @@ void destroy_all(mcao_sim* S) {
     for (cudaStream_t st : {S->s0, S->s1, S->s2, S->s3})
         if (st) cudaStreamSynchronize(st);
     release_graph(S);
-    for (auto& w : S->wfs) dfree(w.d_subaps);
+    dfree(S->d_subaps_all); dfree(S->d_sens); dfree(S->d_adj_err); dfree(S->d_vjp); dfree(S->d_cmd_act);
     for (auto& g : S->fft_groups) dfree(g.d_subaps);
     for (auto& c : S->sci) {
         dfree(c.d_amp); dfree(c.d_field); dfree(c.d_ft); dfree(c.d_psf_t); dfree(c.d_sr_part); dfree(c.d_w);
@@ -905,9 +918,6 @@ mcao_status mcao_sim_create(const mcao_config* cfg, mcao_sim** out) {
             if (el) set_elongation(H, d);
             H.subaps.push_back(d);
         }
-        CKC(dalloc(&H.d_subaps, H.subaps.size()));
-        if (!H.subaps.empty())
-            CKC(cudaMemcpyAsync(H.d_subaps, H.subaps.data(), sizeof(SubapDev) * H.subaps.size(), cudaMemcpyHostToDevice, S->s0));
         WfsDev D{};
         D.type = H.p.type;
         D.n_sub = H.p.n_sub; D.n_px = npx; D.n_fft = H.p.n_fft; D.n_bin = H.p.n_bin; D.n_det = H.n_det;
@@ -930,10 +940,43 @@ mcao_status mcao_sim_create(const mcao_config* cfg, mcao_sim** out) {
             double a = 2.0 * M_PI * (double)k / (double)H.n_det;
             D.tw[k] = make_float2((float)std::cos(a), (float)std::sin(a));
         }
+        // lag weights of the centre of gravity: h(u) sum_m (m - c) exp(2 pi i u m / n_det) / (n_bin n_det)
+        for (int u = -(npx - 1); u <= npx - 1 && npx <= kMaxNpx; ++u) {
+            double hr = 0, hi = 0, dr = 0, di = 0;
+            for (int t = 0; t < H.p.n_bin; ++t) {
+                const double a = 2.0 * M_PI * (double)((long long)u * t % H.p.n_fft) / (double)H.p.n_fft;
+                hr += std::cos(a);
+                hi += std::sin(a);
+            }
+            for (int m = 0; m < H.n_det; ++m) {
+                const double a = 2.0 * M_PI * (double)((long long)u * m % H.n_det) / (double)H.n_det;
+                dr += ((double)m - 0.5 * (H.n_det - 1)) * std::cos(a);
+                di += ((double)m - 0.5 * (H.n_det - 1)) * std::sin(a);
+            }
+            const double f = ((u % 2) ? -1.0 : 1.0) / ((double)H.p.n_bin * H.n_det);
+            D.kap[u + npx - 1] = u % H.n_det ? make_float2((float)(f * (hr * dr - hi * di)), (float)(f * (hr * di + hi * dr)))
+                                             : make_float2(0.0f, 0.0f);
+        }
+        D.sens0 = S->sens_total;
+        S->sens_total += 2LL * H.n_valid * npx * npx;
         amp_off.push_back(amp_all.size());
         amp_all.insert(amp_all.end(), H.amp.begin(), H.amp.end());
         wdev.push_back(D);
         S->wfs.push_back(std::move(H));
+    }
+    // every sensor's subapertures in one array; runs of sensors with the same samples per subaperture
+    std::vector<SubapDev> all_subaps;
+    for (auto& H : S->wfs) all_subaps.insert(all_subaps.end(), H.subaps.begin(), H.subaps.end());
+    CKC(dalloc(&S->d_subaps_all, all_subaps.size()));
+    if (!all_subaps.empty())
+        CKC(cudaMemcpyAsync(S->d_subaps_all, all_subaps.data(), sizeof(SubapDev) * all_subaps.size(), cudaMemcpyHostToDevice,
+                            S->s0));
+    SubapDev* sub_at = S->d_subaps_all;
+    for (auto& H : S->wfs) {
+        H.d_subaps = sub_at;
+        sub_at += H.n_valid;
+        if (S->runs.empty() || S->runs.back().n_px != H.p.n_px) S->runs.push_back(WfsRun{H.p.n_px, 0, H.d_subaps});
+        S->runs.back().n_subaps += H.n_valid;
     }
     S->n_slopes = ns;
     S->n_frame_px = nframe;
@@ -1243,7 +1286,7 @@ mcao_status mcao_load_dms(mcao_sim* S, int n_dms, const mcao_dm* dms) {
     S->dm_cmd0.assign(n_dms + 1, 0);
     std::vector<float> g;
     std::vector<int2> band;
-    std::vector<int> map;
+    std::vector<int> map, cmd_act;
     long long surf_total = 0;
     int ncmd = 0, tiles = 0;
     for (int m = 0; m < n_dms; ++m) {
@@ -1254,9 +1297,14 @@ mcao_status mcao_load_dms(mcao_sim* S, int n_dms, const mcao_dm* dms) {
         D.map_off = (long long)map.size();
         int cnt = 0;
         for (int a = 0; a < d.nx * d.ny; ++a) {
-            if (d.valid[a]) { map.push_back(ncmd + cnt); ++cnt; }
-            else map.push_back(-1);
+            if (d.valid[a]) {
+                map.push_back(ncmd + cnt);
+                cmd_act.push_back((int)((unsigned)(a % d.nx) | (unsigned)(a / d.nx) << 16));
+                ++cnt;
+            } else map.push_back(-1);
         }
+        D.cmd0 = ncmd;
+        D.n_cmd = cnt;
         ncmd += cnt;
         S->dm_cmd0[m + 1] = ncmd;
         D.surf_off = surf_total;
@@ -1278,6 +1326,10 @@ mcao_status mcao_load_dms(mcao_sim* S, int n_dms, const mcao_dm* dms) {
     if (!band.empty()) CK(cudaMemcpyAsync(S->d_dm_band, band.data(), sizeof(int2) * band.size(), cudaMemcpyHostToDevice, S->s0));
     CK(dalloc(&S->d_dm_map, map.size()));
     if (!map.empty()) CK(cudaMemcpyAsync(S->d_dm_map, map.data(), sizeof(int) * map.size(), cudaMemcpyHostToDevice, S->s0));
+    dfree(S->d_cmd_act);
+    CK(dalloc(&S->d_cmd_act, cmd_act.size()));
+    if (!cmd_act.empty())
+        CK(cudaMemcpyAsync(S->d_cmd_act, cmd_act.data(), sizeof(int) * cmd_act.size(), cudaMemcpyHostToDevice, S->s0));
     S->surf_total = surf_total;
     CK(dalloc(&S->d_dm_surf, (size_t)S->n_real * std::max<long long>(surf_total, 1)));
     CK(cudaMemsetAsync(S->d_dm_surf, 0, sizeof(float) * (size_t)S->n_real * std::max<long long>(surf_total, 1), S->s0));
@@ -1664,6 +1716,13 @@ mcao_status mcao_get_wfs_phase(mcao_sim* S, int wfs, float* out, size_t n) {
 static cudaError_t enqueue_sensing(mcao_sim* S, int noise) {
     cudaError_t e = launch_dm_surfaces(make_dm_launch(S), S->s0);
     if (e != cudaSuccess) return e;
+    // nobody keeps the images of a noise-free measurement: slopes straight from the field's lags.  The
+    // loop stays on the image route, noise or not: its Strehl ratios are doubles of the commands.
+    if (!noise && !S->cfg.keep_frames) {
+        for (const auto& r : S->runs)
+            if ((e = launch_wfs_lag(make_wfs_launch(S, r.d_subaps, r.n_subaps), r.n_px, S->s0)) != cudaSuccess) return e;
+        return cudaSuccess;
+    }
     auto run = [&](const SubapDev* sub, int n, unsigned int* work, int npx, int nfft, int nbin) {
         WfsLaunch L = make_wfs_launch(S, sub, n, work);
         L.ctx.noise = noise;
@@ -1712,23 +1771,100 @@ mcao_status mcao_reconstruct_batch(mcao_sim* S, const float* slopes, int n_rhs, 
     return sync_all(S);
 }
 
-// d slope / d phase of every slope on its subaperture's samples (current realization), then the
-// command rows (D) or the command gradients (gvec -> gc) and the phase gradients
-static mcao_status run_adjoint(mcao_sim* S, float* D, long long ld, const float* gvec, int n_vec, float* gc,
-                               float* g_phase, float* g_layers) {
-    int P = 1;
-    for (const auto& W : S->wfs) P = std::max(P, W.p.n_px * W.p.n_px);
+// DM surfaces, then d slope / d phase of every slope on its subaperture's samples (current
+// realization), into the simulation's workspace
+static cudaError_t enqueue_sens(mcao_sim* S) {
+    cudaError_t e = cudaSuccess;
+    if (!S->d_sens) e = dalloc(&S->d_sens, (size_t)S->sens_total);
+    if (e == cudaSuccess && !S->d_adj_err) {
+        e = dalloc(&S->d_adj_err, 1);
+        if (e == cudaSuccess) e = cudaMemsetAsync(S->d_adj_err, 0, sizeof(int), S->s0);
+    }
+    if (e == cudaSuccess) e = launch_dm_surfaces(make_dm_launch(S), S->s0);
+    for (const auto& r : S->runs)
+        if (e == cudaSuccess) e = launch_sens(make_wfs_launch(S, r.d_subaps, r.n_subaps), r.n_px, S->cur, S->d_sens, S->s0);
+    return e;
+}
+
+static ProjLaunch make_proj_launch(mcao_sim* S, const SubapDev* subaps, int n) {
+    ProjLaunch J{};
+    J.ctx = make_ctx(S);
+    J.real = S->cur;
+    J.n_layers = S->n_layers;
+    J.n_dms = S->n_dms;
+    J.desc = S->d_dm_desc;
+    J.g = S->d_dm_g;
+    J.band = S->d_dm_band;
+    J.act_map = S->d_dm_map;
+    J.cmd_act = S->d_cmd_act;
+    J.subaps = subaps;
+    J.n_valid = n;
+    J.sens = S->d_sens;
+    J.n_slopes = S->n_slopes;
+    J.n_cmd = S->n_cmd;
+    J.err = S->d_adj_err;
+    return J;
+}
+
+// waits for the queued calibration work; a band overflow becomes MCAO_E_UNSUPPORTED
+static mcao_status finish_adjoint(mcao_sim* S, cudaError_t e) {
+    int h_err = 0;
+    if (e == cudaSuccess) e = cudaStreamSynchronize(S->s0);
+    if (e == cudaSuccess) e = cudaMemcpy(&h_err, S->d_adj_err, sizeof(int), cudaMemcpyDeviceToHost);
+    CK(e);
+    if (h_err) {
+        CK(cudaMemset(S->d_adj_err, 0, sizeof(int)));
+        return fail(S, MCAO_E_UNSUPPORTED, "a subaperture footprint meets more than 128 actuators per axis");
+    }
+    return MCAO_OK;
+}
+
+// interaction matrix (current realization)
+static mcao_status run_matrix(mcao_sim* S, float* D, long long ld) {
+    CK(cudaDeviceSynchronize());   // D may still be in use on any stream
+    { mcao_status r_ = sync_all(S); if (r_ != MCAO_OK) return r_; }
+    cudaError_t e = enqueue_sens(S);
+    if (e == cudaSuccess && S->n_dms == 0) e = cudaMemsetAsync(D, 0, sizeof(float) * (size_t)S->n_slopes * ld, S->s0);
+    for (const auto& r : S->runs) {
+        ProjLaunch J = make_proj_launch(S, r.d_subaps, r.n_subaps);
+        J.D = D;
+        J.ld = ld;
+        if (e == cudaSuccess) e = launch_dm_rows(J, r.n_px, S->sm_count, S->s0);
+    }
+    return finish_adjoint(S, e);
+}
+
+// vector-Jacobian products: pupil-phase gradients of every vector, from them the command and layer
+// gradients.  Vectors go in groups, which bounds the workspace.
+static mcao_status run_vjp(mcao_sim* S, const float* gvec, int n_vec, float* gc, float* g_phase, float* g_layers) {
+    constexpr int kGroup = 8;
     CK(cudaDeviceSynchronize());   // inputs produced on any stream are complete
     { mcao_status r_ = sync_all(S); if (r_ != MCAO_OK) return r_; }
-    float* sens = nullptr;
-    int* d_err = nullptr;
-    cudaError_t e = dalloc(&sens, (size_t)S->n_slopes * P);
-    if (e == cudaSuccess) e = dalloc(&d_err, 1);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d_err, 0, sizeof(int), S->s0);
-    if (e == cudaSuccess) e = launch_dm_surfaces(make_dm_launch(S), S->s0);
     long long phase_total = 0;
-    for (const auto& W : S->wfs) phase_total += (long long)W.N * W.N;
-    if (e == cudaSuccess && D) e = cudaMemsetAsync(D, 0, sizeof(float) * (size_t)S->n_slopes * ld, S->s0);
+    int max_n = 1, max_nx = 1, max_ny = 1, n_all = 0;
+    bool rotated = false;
+    for (const auto& W : S->wfs) {
+        phase_total += (long long)W.N * W.N;
+        max_n = std::max(max_n, W.N);
+        n_all += W.n_valid;
+    }
+    for (const auto& d : S->dm_desc) {
+        max_nx = std::max(max_nx, d.nx);
+        max_ny = std::max(max_ny, d.ny);
+        rotated = rotated || d.general;
+    }
+    const int group = std::min(n_vec, kGroup), n_wfs = (int)S->wfs.size();
+    // workspace of a group: the pupil gradients (unless the caller takes them), then U
+    const size_t need_phase = (gc && !g_phase) ? (size_t)group * phase_total : 0;
+    const size_t need = need_phase + (gc ? (size_t)group * n_wfs * S->n_dms * max_n * max_nx : 0);
+    cudaError_t e = cudaSuccess;
+    if (need > S->vjp_floats) {
+        dfree(S->d_vjp);
+        S->vjp_floats = 0;
+        e = dalloc(&S->d_vjp, need);
+        if (e == cudaSuccess) S->vjp_floats = need;
+    }
+    if (e == cudaSuccess) e = enqueue_sens(S);
     if (e == cudaSuccess && gc) e = cudaMemsetAsync(gc, 0, sizeof(float) * (size_t)n_vec * S->n_cmd, S->s0);
     if (e == cudaSuccess && g_phase) e = cudaMemsetAsync(g_phase, 0, sizeof(float) * (size_t)n_vec * phase_total, S->s0);
     // layers concatenated: offsets and total length
@@ -1741,54 +1877,30 @@ static mcao_status run_adjoint(mcao_sim* S, float* D, long long ld, const float*
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(d_loff, loff.data(), sizeof(long long) * loff.size(), cudaMemcpyHostToDevice, S->s0);
     }
-    long long phase_off = 0;
-    for (size_t w = 0; w < S->wfs.size() && e == cudaSuccess; ++w) {
-        const WfsHost& W = S->wfs[w];
-        if (W.n_valid > 0) {
-            SensLaunch L{};
-            L.ctx = make_ctx(S);
-            L.real = S->cur;
-            L.subaps = W.d_subaps;
-            L.n_subaps = W.n_valid;
-            L.sens = sens;
-            L.P = P;
-            e = launch_sens(L, W.p.n_fft, S->s0);
-            ProjLaunch J{};
-            J.ctx = L.ctx;
-            J.real = S->cur;
-            J.n_layers = S->n_layers;
-            J.n_dms = S->n_dms;
-            J.desc = S->d_dm_desc;
-            J.g = S->d_dm_g;
-            J.band = S->d_dm_band;
-            J.act_map = S->d_dm_map;
-            J.subaps = W.d_subaps;
-            J.n_valid = W.n_valid;
-            J.sens = sens;
-            J.P = P;
-            J.D = D;
-            J.ld = ld;
-            J.gvec = gvec;
-            J.n_vec = n_vec;
-            J.n_slopes = S->n_slopes;
-            J.gc = gc;
-            J.n_cmd = S->n_cmd;
-            J.err = d_err;
-            if (e == cudaSuccess && (D || gc)) e = launch_dm_adjoint(J, S->s0);
-            if (e == cudaSuccess && (g_phase || g_layers))
-                e = launch_phase_adjoint(J, g_phase, phase_total, phase_off, g_layers, loff[S->n_layers], d_loff, S->s0);
+    for (int v0 = 0; v0 < n_vec && e == cudaSuccess; v0 += group) {
+        ProjLaunch J = make_proj_launch(S, S->d_subaps_all, n_all);
+        J.gvec = gvec + (size_t)v0 * S->n_slopes;
+        J.n_vec = std::min(group, n_vec - v0);
+        J.gc = gc ? gc + (size_t)v0 * S->n_cmd : nullptr;
+        float* gp = g_phase ? g_phase + (size_t)v0 * phase_total : gc ? S->d_vjp : nullptr;
+        if (gp && !g_phase) e = cudaMemsetAsync(gp, 0, sizeof(float) * (size_t)J.n_vec * phase_total, S->s0);
+        if (e == cudaSuccess)
+            e = launch_phase_adjoint(J, gp, phase_total, g_layers ? g_layers + (size_t)v0 * loff[S->n_layers] : nullptr,
+                                     loff[S->n_layers], d_loff, S->s0);
+        if (e == cudaSuccess && gc && v0 == 0) e = launch_dm_range(J, S->s0);
+        if (e == cudaSuccess && gc) {
+            e = launch_dm_project(J, n_wfs, max_n, max_nx, max_ny, gp, phase_total, S->d_vjp + need_phase, S->s0);
+            for (const auto& r : S->runs) {
+                ProjLaunch K = J;
+                K.subaps = r.d_subaps;
+                K.n_valid = r.n_subaps;
+                if (e == cudaSuccess && rotated) e = launch_dm_rows(K, r.n_px, S->sm_count, S->s0);
+            }
         }
-        phase_off += (long long)W.N * W.N;
     }
-    int h_err = 0;
-    if (e == cudaSuccess) e = cudaStreamSynchronize(S->s0);
-    if (e == cudaSuccess) e = cudaMemcpy(&h_err, d_err, sizeof(int), cudaMemcpyDeviceToHost);
-    cudaFree(sens);
-    cudaFree(d_err);
+    const mcao_status r = finish_adjoint(S, e);
     cudaFree(d_loff);
-    CK(e);
-    if (h_err) return fail(S, MCAO_E_UNSUPPORTED, "a subaperture footprint meets more than 128 actuators per axis");
-    return MCAO_OK;
+    return r;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1939,50 +2051,21 @@ mcao_status mcao_misreg_normal_equations(mcao_sim* S, int dm, const float* D_mea
     const int cmd0 = S->dm_cmd0[dm], n_cols = S->dm_cmd0[dm + 1] - cmd0;
     if (ld < (size_t)n_cols) return fail(S, MCAO_E_SHAPE, "ld must be >= %d (the DM's commands)", n_cols);
     CK(cudaSetDevice(S->device));
-    int P = 1;
-    for (const auto& W : S->wfs) P = std::max(P, W.p.n_px * W.p.n_px);
     CK(cudaDeviceSynchronize());   // D_meas may come from any stream
     { mcao_status r_ = sync_all(S); if (r_ != MCAO_OK) return r_; }
-    float* sens = nullptr;
     double* rec = nullptr;
-    cudaError_t e = dalloc(&sens, (size_t)S->n_slopes * P);
-    if (e == cudaSuccess) e = cudaMalloc(&rec, sizeof(double) * ((size_t)S->n_slopes * 16 + 16));
+    cudaError_t e = cudaMalloc(&rec, sizeof(double) * ((size_t)S->n_slopes * 16 + 16));
     if (e == cudaSuccess) e = cudaMemsetAsync(rec, 0, sizeof(double) * (size_t)S->n_slopes * 16, S->s0);
-    if (e == cudaSuccess) e = launch_dm_surfaces(make_dm_launch(S), S->s0);
-    for (size_t w = 0; w < S->wfs.size() && e == cudaSuccess; ++w) {
-        const WfsHost& W = S->wfs[w];
-        if (W.n_valid == 0) continue;
-        SensLaunch L{};
-        L.ctx = make_ctx(S);
-        L.real = S->cur;
-        L.subaps = W.d_subaps;
-        L.n_subaps = W.n_valid;
-        L.sens = sens;
-        L.P = P;
-        e = launch_sens(L, W.p.n_fft, S->s0);
-        ProjLaunch J{};
-        J.ctx = L.ctx;
-        J.real = S->cur;
-        J.n_layers = S->n_layers;
-        J.n_dms = S->n_dms;
-        J.desc = S->d_dm_desc;
-        J.g = S->d_dm_g;
-        J.band = S->d_dm_band;
-        J.act_map = S->d_dm_map;
-        J.subaps = W.d_subaps;
-        J.n_valid = W.n_valid;
-        J.sens = sens;
-        J.P = P;
-        J.n_slopes = S->n_slopes;
-        J.n_cmd = S->n_cmd;
-        if (e == cudaSuccess) e = launch_misreg_gn(J, dm, D_meas, (long long)ld, cmd0, rec, S->s0);
-    }
+    if (e == cudaSuccess) e = enqueue_sens(S);
+    for (size_t w = 0; w < S->wfs.size() && e == cudaSuccess; ++w)
+        if (S->wfs[w].n_valid > 0)
+            e = launch_misreg_gn(make_proj_launch(S, S->wfs[w].d_subaps, S->wfs[w].n_valid), dm, D_meas, (long long)ld, cmd0,
+                                 rec, S->s0);
     double* out = rec + (size_t)S->n_slopes * 16;
     double h[16] = {0};
     if (e == cudaSuccess) e = launch_misreg_sum(rec, S->n_slopes, out, S->s0);
     if (e == cudaSuccess) e = cudaStreamSynchronize(S->s0);
     if (e == cudaSuccess) e = cudaMemcpy(h, out, sizeof(h), cudaMemcpyDeviceToHost);
-    cudaFree(sens);
     cudaFree(rec);
     CK(e);
     // records: cost, Jte[4], upper triangle of JtJ row by row, sum D_meas^2
@@ -2003,7 +2086,7 @@ mcao_status mcao_interaction_matrix(mcao_sim* S, float* D, size_t ld) {
     if (!S->atm_loaded || !S->dms_loaded) return fail(S, MCAO_E_STATE, "atmosphere and DMs must be loaded");
     if (ld < (size_t)S->n_cmd) return fail(S, MCAO_E_SHAPE, "ld must be >= %d", S->n_cmd);
     CK(cudaSetDevice(S->device));
-    return run_adjoint(S, D, (long long)ld, nullptr, 0, nullptr, nullptr, nullptr);
+    return run_matrix(S, D, (long long)ld);
 }
 
 mcao_status mcao_slopes_vjp(mcao_sim* S, const float* g_slopes, int n_vec, float* g_commands, float* g_phase,
@@ -2011,7 +2094,7 @@ mcao_status mcao_slopes_vjp(mcao_sim* S, const float* g_slopes, int n_vec, float
     if (!S || !g_slopes || n_vec < 1 || (!g_commands && !g_phase && !g_layers)) return MCAO_E_INVALID_ARG;
     if (!S->atm_loaded || !S->dms_loaded) return fail(S, MCAO_E_STATE, "atmosphere and DMs must be loaded");
     CK(cudaSetDevice(S->device));
-    return run_adjoint(S, nullptr, 0, g_slopes, n_vec, g_commands, g_phase, g_layers);
+    return run_vjp(S, g_slopes, n_vec, g_commands, g_phase, g_layers);
 }
 
 mcao_status mcao_get_dm_surface(mcao_sim* S, int dm, float* out, size_t n) {

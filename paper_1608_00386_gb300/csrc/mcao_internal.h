@@ -56,6 +56,8 @@ struct WfsDev {
     const float* amp;    // [N][N] pupil amplitude
     float2 h[2 * kMaxNpx - 1];  // (-1)^u sum_{t<n_bin} exp(2 pi i u t / n_fft), u = -(n_px-1)..n_px-1
     float2 tw[kMaxNd];          // exp(2 pi i k / n_det)
+    float2 kap[2 * kMaxNpx - 1];   // lag weights of the centre of gravity without elongation (k_lag.cu), u = -(n_px-1)..n_px-1
+    long long sens0;            // first float of this sensor's block of slope derivatives: [2 n_valid][n_px^2]
 };
 
 // One valid subaperture.
@@ -123,6 +125,7 @@ struct DmDesc {
     float dx, pitch;     // surface sample pitch, actuator pitch (m)
     float inv2s2;        // 1 / (2 sigma^2) of the influence function (DM coordinates)
     float rc;            // window radius in actuator pitches (weights below 1e-10 left out)
+    int cmd0, n_cmd;     // this DM's block of the command vector
 };
 constexpr int kDmTile = 32;
 constexpr int kDmMaxBand = 64;   // actuators per tile and axis (checked on the host)
@@ -296,14 +299,6 @@ cudaError_t launch_screen(int n, double pixel, double r0, double L0, unsigned lo
 // ---------------------------------------------------------------------------------------------
 // adjoint of the noise-free sensing (interaction matrix, vector-Jacobian products)
 // ---------------------------------------------------------------------------------------------
-struct SensLaunch {
-    Ctx ctx;
-    int real;
-    const SubapDev* subaps;  // one sensor's valid subapertures
-    int n_subaps;
-    float* sens;             // [n_slopes][P]: d slope / d phase on the slope's subaperture samples
-    int P;                   // row length (largest n_px^2)
-};
 struct ProjLaunch {
     Ctx ctx;
     int real, n_layers, n_dms;
@@ -311,10 +306,10 @@ struct ProjLaunch {
     const float* g;
     const int2* band;
     const int* act_map;
-    const SubapDev* subaps;  // one sensor's valid subapertures
+    const int* cmd_act;      // [n_cmd] actuator of each command: column | row << 16
+    const SubapDev* subaps;  // valid subapertures (of one or several sensors)
     int n_valid;
-    const float* sens;
-    int P;
+    const float* sens;       // d slope / d phase (WfsDev::sens0)
     float* D;                // interaction matrix rows (or null)
     long long ld;
     const float* gvec;       // [n_vec][n_slopes] (or null)
@@ -323,16 +318,26 @@ struct ProjLaunch {
     int n_cmd;
     int* err;                // set when a footprint meets more actuators than a block holds
 };
-size_t sens_smem(int n_fft);
-cudaError_t launch_sens(const SensLaunch& L, int n_fft, cudaStream_t s);
-cudaError_t launch_dm_adjoint(const ProjLaunch& L, cudaStream_t s);
+// noise-free slopes of L.subaps (sensors of n_px samples per subaperture) without forming an image,
+// and their derivatives with respect to the phase (realization `real`) into sens
+cudaError_t launch_wfs_lag(const WfsLaunch& L, int n_px, cudaStream_t s);
+cudaError_t launch_sens(const WfsLaunch& L, int n_px, int real, float* sens, cudaStream_t s);
+// interaction-matrix rows of L.subaps (all of n_px samples), or with L.gvec the rotated DMs' share of
+// the command gradients
+cudaError_t launch_dm_rows(const ProjLaunch& L, int n_px, int sm_count, cudaStream_t s);
+// sets *L.err where launch_dm_rows would (too many actuators on a footprint)
+cudaError_t launch_dm_range(const ProjLaunch& L, cudaStream_t s);
+// the separable DMs' command gradients of L.n_vec pupil-phase gradients; U: [n_vec][n_wfs][n_dms]
+// [max_n][max_nx] scratch
+cudaError_t launch_dm_project(const ProjLaunch& L, int n_wfs, int max_n, int max_nx, int max_ny, const float* g_phase,
+                              long long phase_stride, float* U, cudaStream_t s);
 // Gauss-Newton records (16 doubles per slope row) of DM m's misregistration fit against D_meas
 // (columns = DM m's commands, from cmd0), then their fixed-order sum
 cudaError_t launch_misreg_gn(const ProjLaunch& L, int m, const float* D_meas, long long ld_meas, int cmd0, double* rec,
                              cudaStream_t s);
 cudaError_t launch_misreg_sum(const double* rec, int n_rows, double* out, cudaStream_t s);
-cudaError_t launch_phase_adjoint(const ProjLaunch& L, float* g_phase, long long phase_stride, long long phase_off,
-                                 float* g_layers, long long layer_stride, const long long* layer_off, cudaStream_t s);
+cudaError_t launch_phase_adjoint(const ProjLaunch& L, float* g_phase, long long phase_stride, float* g_layers,
+                                 long long layer_stride, const long long* layer_off, cudaStream_t s);
 
 // per science direction: (long-exposure, instantaneous) Strehl ratio into out[2 q], out[2 q + 1]
 cudaError_t launch_strehl_out(const SciAcc* acc, int n_sci, double* out, cudaStream_t s);
