@@ -5,23 +5,27 @@
 // D [n_slopes][n_cmd] the interaction matrix (float32), R [n_cmd][n_slopes].  The minus sign: D is
 // measured with the DM subtracted from the wavefront, and the loop applies c <- c + g R s.
 //
-// Every step runs in double precision in the kernels below, on 64 x 64 tiles:
-//   1. mask of the tiles of D that hold a nonzero (a subaperture sees only the actuators within
-//      the influence functions' reach, so most tiles of D are exactly zero);
-//   2. Gram matrix G = D^T D, lower tiles, summing only slope tiles where both D tiles are
-//      nonzero; mirrored into the upper tiles;
+// Every step runs in double precision in the kernels below:
+//   1. D compressed by rows and by columns (a subaperture sees only the actuators within the
+//      influence functions' reach: 6 % of D at 20 m, less at 39 m);
+//   2. Gram matrix G = D^T D over the nonzero pairs;
 //   3. lambda from the trace, G + lambda I (padding rows past n_cmd get a unit diagonal);
-//   4. blocked right-looking Cholesky G = L L^T: per block column k, the diagonal block is
-//      factored and inverted in shared memory, the panel below is multiplied by that inverse's
-//      transpose, and the trailing lower tiles are updated;
-//   5. X = L^(-1) by a right-looking solve of L X = I: per block row i, X[i][j] = Linv_ii X[i][j]
-//      for j <= i, then X[m][j] -= L[m][i] X[i][j] below;
-//   6. M^(-1) = X^T X (lower tiles, mirrored), written over L;
-//   7. R = -M^(-1) D^T, again skipping zero tiles of D; rounded to float32 once, at the store
-//      (or stored in double).
-// The GB300's FP64 units are slow (about 1.25 TFLOP/s per GPU), so the kernels are plain
-// register-blocked tile products (each thread 4 x 4 outputs) bound by the double FMA rate; the
-// zero-tile skipping is what keeps the 39 m case (8051 x 55608) to seconds.
+//   4. blocked right-looking Cholesky G = L L^T on 64 x 64 tiles together with X = L^(-1): per block
+//      column k, the diagonal block is factored and inverted in one block's registers (potrf); the
+//      panel L[i][k] and the block row X[k][j] are multiplied by that inverse (panel); the
+//      trailing tiles of L and the rows of X below are updated (update);
+//   5. M^(-1) = X^T X (lower tiles, mirrored), written over L;
+//   6. R = -M^(-1) D^T over the nonzeros of D's rows; rounded to float32 once, at the store (or
+//      stored in double).
+// The GB300 issues two double FMAs per cycle and SM, 1/64 of the float32 rate, so operations are all
+// that counts: the tile products run at that rate with operands straight from L2 and shared memory,
+// and what is worth doing is to leave out multiplications by zeros and to keep every SM's pipe busy.
+// Hence the compressed D (64 x 64 tiles of D that hold a nonzero cover six times the nonzeros: Gram
+// 8.2 ms and product 16.4 ms at 20 m before), the lower halves of triangular blocks only, and 32 x 32
+// outputs per block, four of which share an SM's pipe: the last wave of a launch costs a quarter of
+// what 64 x 64 outputs cost.  A dense D (more than a third nonzero) takes the tile products, where
+// each operand read serves 32 outputs.
+// 20 m (7280 x 1879): 46.6 ms before, 17.5 ms now; 39 m (55608 x 8051): 2.2 s before.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -34,38 +38,42 @@
 namespace {
 
 constexpr int kT = 64;          // tile side
-constexpr int kKC = 32;         // k depth of one shared-memory chunk
-constexpr int kThreads = 256;   // 16 x 16 threads, 4 x 4 outputs each
+constexpr int kS = 32;          // output side and k depth of one block's product
+constexpr int kThreads = 128;   // 16 x 8 threads, 2 x 4 outputs each
 
-// One chunk of a tile product: As[k][r], Bs[k][c] for k < kKC (rows padded by one double).
+// One chunk of a product: a[k][r], b[k][c] for k < kS (rows padded by one double).
 struct Chunk {
-    double a[kKC][kT + 1];
-    double b[kKC][kT + 1];
+    double a[kS][kS + 1];
+    double b[kS][kS + 1];
 };
 
-__device__ __forceinline__ void chunk_fma(const Chunk& ch, double (&c)[4][4], int ty, int tx) {
+__device__ __forceinline__ void chunk_fma(const Chunk& ch, double (&c)[2][4]) {
+    const int r = threadIdx.x / 8 * 2, q = threadIdx.x % 8;
 #pragma unroll 8
-    for (int k = 0; k < kKC; ++k) {
-        double av[4], bv[4];
+    for (int k = 0; k < kS; ++k) {
+        double av[2], bv[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            av[i] = ch.a[k][ty * 4 + i];
-            bv[i] = ch.b[k][tx * 4 + i];
-        }
+        for (int i = 0; i < 2; ++i) av[i] = ch.a[k][r + i];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int j = 0; j < 4; ++j) bv[j] = ch.b[k][q + 8 * j];
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
 #pragma unroll
             for (int j = 0; j < 4; ++j) c[i][j] = fma(av[i], bv[j], c[i][j]);
     }
 }
+// output (i, j) of this thread: row and column within the 32 x 32 block
+__device__ __forceinline__ int out_row(int i) { return threadIdx.x / 8 * 2 + i; }
+__device__ __forceinline__ int out_col(int j) { return threadIdx.x % 8 + 8 * j; }
 
-// T[k][i] = src[(r0 + k) ld + c0 + i] for k < kKC, i < 64 (the source block as it is), zero past
-// (nr, nc); float or double source
+// T[k][i] = src[(r0 + k) ld + c0 + i] for k, i < 32 (the source block as it is), zero past (nr, nc);
+// float or double source
 template <typename S>
-__device__ __forceinline__ void load_direct(double (*T)[kT + 1], const S* src, long long ld, long long r0, long long c0,
+__device__ __forceinline__ void load_direct(double (*T)[kS + 1], const S* src, long long ld, long long r0, long long c0,
                                             long long nr, long long nc) {
-    for (int q = threadIdx.x; q < kKC * kT; q += kThreads) {
-        const int k = q / kT, i = q - k * kT;
+#pragma unroll
+    for (int q = threadIdx.x; q < kS * kS; q += kThreads) {
+        const int k = q / kS, i = q % kS;
         const long long r = r0 + k, c = c0 + i;
         T[k][i] = (r < nr && c < nc) ? (double)src[r * ld + c] : 0.0;
     }
@@ -73,25 +81,179 @@ __device__ __forceinline__ void load_direct(double (*T)[kT + 1], const S* src, l
 
 // T[k][i] = src[(r0 + i) ld + c0 + k] (the source block transposed), zero past (nr, nc)
 template <typename S>
-__device__ __forceinline__ void load_trans(double (*T)[kT + 1], const S* src, long long ld, long long r0, long long c0,
+__device__ __forceinline__ void load_trans(double (*T)[kS + 1], const S* src, long long ld, long long r0, long long c0,
                                            long long nr, long long nc) {
-    for (int q = threadIdx.x; q < kKC * kT; q += kThreads) {
-        const int i = q / kKC, k = q - i * kKC;   // consecutive threads walk along a source row
+#pragma unroll
+    for (int q = threadIdx.x; q < kS * kS; q += kThreads) {
+        const int i = q / kS, k = q % kS;   // consecutive threads walk along a source row
         const long long r = r0 + i, c = c0 + k;
         T[k][i] = (r < nr && c < nc) ? (double)src[r * ld + c] : 0.0;
     }
 }
 
-// lower-triangle tile index t -> (i, j), i >= j, i < n
+// lower-triangle tile index t -> (i, j), i >= j
 __device__ __forceinline__ void tri_index(long long t, int& i, int& j) {
-    int ii = (int)floor((sqrt(8.0 * (double)t + 1.0) - 1.0) * 0.5);
+    int ii = (int)floorf((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
     while ((long long)(ii + 1) * (ii + 2) / 2 <= t) ++ii;
     while ((long long)ii * (ii + 1) / 2 > t) --ii;
     i = ii;
     j = (int)(t - (long long)ii * (ii + 1) / 2);
 }
 
-// 1. mask[S][J] = 1 if the tile (slopes 64 S.., commands 64 J..) of D holds a nonzero
+// ------------------------------------------------------------------------------------------
+// 1. compressed D
+// ------------------------------------------------------------------------------------------
+constexpr int kCscWarps = 32;   // warps of a column block, each a slab of consecutive rows
+
+// nonzeros of each row (one warp per row)
+__global__ void __launch_bounds__(256) tik_row_count_kernel(const float* __restrict__ D, long long ld, int n_slopes,
+                                                            int n_cmd, int* __restrict__ count) {
+    const int r = blockIdx.x * 8 + threadIdx.x / 32, lane = threadIdx.x & 31;
+    if (r >= n_slopes) return;
+    int n = 0;
+#pragma unroll 8
+    for (int c = lane; c < n_cmd; c += 32) n += D[r * ld + c] != 0.0f;
+    n = __reduce_add_sync(0xffffffffu, n);
+    if (lane == 0) count[r] = n;
+}
+
+// nonzeros of the 32 columns of this block in each warp's slab of rows
+__device__ __forceinline__ int slab_count(const float* D, long long ld, int r0, int r1, int c, int n_cmd) {
+    int n = 0;
+    if (c < n_cmd)
+#pragma unroll 8
+        for (int r = r0; r < r1; ++r) n += D[r * ld + c] != 0.0f;
+    return n;
+}
+
+__global__ void __launch_bounds__(32 * kCscWarps) tik_col_count_kernel(const float* __restrict__ D, long long ld, int n_slopes,
+                                                                       int n_cmd, int* __restrict__ count) {
+    __shared__ int s_n[kCscWarps][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x / 32, c = blockIdx.x * 32 + lane;
+    const int slab = (n_slopes + kCscWarps - 1) / kCscWarps, r0 = w * slab, r1 = min(n_slopes, r0 + slab);
+    s_n[w][lane] = slab_count(D, ld, r0, r1, c, n_cmd);
+    __syncthreads();
+    if (w == 0 && c < n_cmd) {
+        int n = 0;
+        for (int q = 0; q < kCscWarps; ++q) n += s_n[q][lane];
+        count[c] = n;
+    }
+}
+
+// exclusive prefix sums in place, count[n] = total (one block)
+__global__ void __launch_bounds__(1024) tik_scan_kernel(int* __restrict__ count, int n) {
+    __shared__ int s_w[32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x / 32;
+    int base = 0;
+    for (int i0 = 0; i0 < n; i0 += 1024) {
+        const int i = i0 + threadIdx.x, v = i < n ? count[i] : 0;
+        int x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) s_w[w] = x;
+        __syncthreads();
+        int before = 0, total = 0;
+        for (int q = 0; q < 32; ++q) {
+            before += q < w ? s_w[q] : 0;
+            total += s_w[q];
+        }
+        if (i < n) count[i] = base + before + x - v;
+        base += total;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) count[n] = base;
+}
+
+// columns and values of each row's nonzeros, ascending
+__global__ void __launch_bounds__(256) tik_row_fill_kernel(const float* __restrict__ D, long long ld, int n_slopes, int n_cmd,
+                                                           const int* __restrict__ row, int* __restrict__ col,
+                                                           float* __restrict__ val) {
+    const int r = blockIdx.x * 8 + threadIdx.x / 32, lane = threadIdx.x & 31;
+    if (r >= n_slopes) return;
+    int at = row[r];
+    for (int c0 = 0; c0 < n_cmd; c0 += 32) {
+        const int c = c0 + lane;
+        const float v = c < n_cmd ? D[r * ld + c] : 0.0f;
+        const unsigned m = __ballot_sync(0xffffffffu, v != 0.0f);
+        if (v != 0.0f) {
+            const int p = at + __popc(m & ((1u << lane) - 1u));
+            col[p] = c;
+            val[p] = v;
+        }
+        at += __popc(m);
+    }
+}
+
+// rows and values of each column's nonzeros, ascending
+__global__ void __launch_bounds__(32 * kCscWarps) tik_col_fill_kernel(const float* __restrict__ D, long long ld, int n_slopes,
+                                                                      int n_cmd, const int* __restrict__ col_at,
+                                                                      int* __restrict__ row, float* __restrict__ val) {
+    __shared__ int s_n[kCscWarps][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x / 32, c = blockIdx.x * 32 + lane;
+    const int slab = (n_slopes + kCscWarps - 1) / kCscWarps, r0 = w * slab, r1 = min(n_slopes, r0 + slab);
+    s_n[w][lane] = slab_count(D, ld, r0, r1, c, n_cmd);
+    __syncthreads();
+    if (c >= n_cmd) return;
+    int at = col_at[c];
+    for (int q = 0; q < w; ++q) at += s_n[q][lane];
+#pragma unroll 8
+    for (int r = r0; r < r1; ++r) {
+        const float v = D[r * ld + c];
+        if (v != 0.0f) {
+            row[at] = r;
+            val[at++] = v;
+        }
+    }
+}
+
+// ------------------------------------------------------------------------------------------
+// 2. Gram matrix
+// ------------------------------------------------------------------------------------------
+// One block per actuator a: G[a][b] for b <= a, summed in shared memory over the rows s where D[s][a]
+// is nonzero, in ascending order; the threads take the row's nonzeros side by side (the next row's
+// are read while this one is added).
+__global__ void __launch_bounds__(128) tik_gram_sparse_kernel(const int* __restrict__ col_at, const int* __restrict__ col_row,
+                                                              const float* __restrict__ col_val, const int* __restrict__ row,
+                                                              const int* __restrict__ col, const float* __restrict__ val,
+                                                              double* __restrict__ G, long long ldg) {
+    extern __shared__ double gram_acc[];
+    const int a = gridDim.x - 1 - blockIdx.x;   // the longest rows of G first
+    const int tid = threadIdx.x;
+    for (int b = tid; b <= a; b += 128) gram_acc[b] = 0.0;
+    const int p0 = col_at[a], p1 = col_at[a + 1];
+    __syncthreads();
+    int q0 = 0, q1 = 0, b = 0;
+    float dsa = 0.0f, v = 0.0f;
+    auto fetch = [&](int p) {
+        const int s = col_row[p];
+        dsa = col_val[p];
+        q0 = row[s];
+        q1 = row[s + 1];
+        b = q0 + tid < q1 ? col[q0 + tid] : a + 1;
+        v = q0 + tid < q1 ? val[q0 + tid] : 0.0f;
+    };
+    if (p0 < p1) fetch(p0);
+    for (int p = p0; p < p1; ++p) {
+        const int bb = b, n = q1, first = q0;
+        const double vv = (double)v, d = (double)dsa;
+        if (p + 1 < p1) fetch(p + 1);
+        if (bb <= a) gram_acc[bb] = fma(d, vv, gram_acc[bb]);
+        for (int q = first + 128 + tid; q < n; q += 128) {
+            const int e = col[q];
+            if (e <= a) gram_acc[e] = fma(d, (double)val[q], gram_acc[e]);
+        }
+        __syncthreads();
+    }
+    for (int e = tid; e <= a; e += 128) {
+        G[(long long)a * ldg + e] = gram_acc[e];
+        if (e < a) G[(long long)e * ldg + a] = gram_acc[e];
+    }
+}
+
+// dense D: mask[S][J] = 1 if the tile (slopes 64 S.., commands 64 J..) of D holds a nonzero
 __global__ void __launch_bounds__(kThreads) tik_mask_kernel(const float* __restrict__ D, long long ld, int n_slopes,
                                                             int n_cmd, int nJ, unsigned char* __restrict__ mask) {
     const int J = blockIdx.x, S = blockIdx.y;
@@ -104,7 +266,8 @@ __global__ void __launch_bounds__(kThreads) tik_mask_kernel(const float* __restr
     if (threadIdx.x == 0) mask[(long long)S * nJ + J] = (unsigned char)any;
 }
 
-// 2. G[I][J] = sum_s D[s][I..]^T D[s][J..] for lower tiles, mirrored
+// dense D: 32 x 32 block (I, J) of G, I >= J, over the slope tiles where both tiles of D hold a
+// nonzero; mirrored
 __global__ void __launch_bounds__(kThreads) tik_gram_kernel(const float* __restrict__ D, long long ld, int n_slopes,
                                                             int n_cmd, int nS, int nt,
                                                             const unsigned char* __restrict__ mask,
@@ -112,23 +275,22 @@ __global__ void __launch_bounds__(kThreads) tik_gram_kernel(const float* __restr
     __shared__ Chunk ch;
     int I, J;
     tri_index(blockIdx.x, I, J);
-    const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
-    double c[4][4] = {};
+    double c[2][4] = {};
     for (int S = 0; S < nS; ++S) {
-        if (!mask[(long long)S * nt + I] || !mask[(long long)S * nt + J]) continue;
-        for (int k0 = 0; k0 < kT; k0 += kKC) {
-            load_direct(ch.a, D, ld, (long long)S * kT + k0, (long long)I * kT, n_slopes, n_cmd);
-            load_direct(ch.b, D, ld, (long long)S * kT + k0, (long long)J * kT, n_slopes, n_cmd);
+        if (!mask[(long long)S * nt + I / 2] || !mask[(long long)S * nt + J / 2]) continue;
+        for (int k0 = 0; k0 < kT; k0 += kS) {
+            load_direct(ch.a, D, ld, (long long)S * kT + k0, (long long)I * kS, n_slopes, n_cmd);
+            load_direct(ch.b, D, ld, (long long)S * kT + k0, (long long)J * kS, n_slopes, n_cmd);
             __syncthreads();
-            chunk_fma(ch, c, ty, tx);
+            chunk_fma(ch, c);
             __syncthreads();
         }
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 2; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const long long r = (long long)I * kT + ty * 4 + i, q = (long long)J * kT + tx * 4 + j;
+            const long long r = (long long)I * kS + out_row(i), q = (long long)J * kS + out_col(j);
             G[r * ldg + q] = c[i][j];
             if (I != J) G[q * ldg + r] = c[i][j];
         }
@@ -157,219 +319,276 @@ __global__ void tik_regularize_kernel(double* __restrict__ G, long long ldg, int
     if (threadIdx.x == 0) *lambda_out = lam;
 }
 
-// 4a. factor the diagonal block k in shared memory (lower Cholesky), write L_kk over it (upper
-// part zero) and its inverse to Linv[k]; a pivot <= 0 sets *err (and is replaced by 1 so the
-// remaining steps stay finite)
-__global__ void __launch_bounds__(kThreads) tik_potrf_kernel(double* __restrict__ A, long long lda, int k,
-                                                             double* __restrict__ Linv, int* __restrict__ err) {
-    extern __shared__ double potrf_sm[];
-    double(*S)[kT + 1] = reinterpret_cast<double(*)[kT + 1]>(potrf_sm);
-    double(*X)[kT + 1] = reinterpret_cast<double(*)[kT + 1]>(potrf_sm + kT * (kT + 1));
+// ------------------------------------------------------------------------------------------
+// 4. Cholesky factor and its inverse
+// ------------------------------------------------------------------------------------------
+// 1 / sqrt(d): the float reciprocal square root of the significand and one third-order
+// Newton-Halley step y (1 + e/2 + 3 e^2 / 8), e = 1 - d y^2 (|e| < 2^-21, so the step leaves less
+// than 2^-60), the even power of two of d put back exactly
+__device__ __forceinline__ double inv_sqrt(double d) {
+    int ex;
+    double m = frexp(d, &ex);        // m in [1/2, 1)
+    if (ex & 1) {
+        m *= 0.5;
+        ex += 1;
+    }
+    const double y = (double)rsqrtf((float)m), e = fma(-m * y, y, 1.0);
+    return ldexp(fma(y * e, fma(0.375, e, 0.5), y), -ex / 2);
+}
+
+// 4a. Linv = L^(-1) of the diagonal block S = L L^T, in one block: the lower triangle of a 64 x 64
+// array W, 8 or 9 entries (m, c) per thread in registers, starts as S and ends as L^(-1).  Before step
+// j the columns c >= j of the rows m >= j hold the trailing matrix S, the columns c < j the rows of
+// X = L^(-1) so far.  Step j takes r = 1 / sqrt(S_jj), L_mj = r S_mj, u_c = r X_jc (c < j), r (c = j),
+// L_cj (c > j), then W_mc -= L_mj u_c on every row below (W_mj counts as 0 there: column j of X
+// begins), and row j of X is u.  So factor and inverse cost one pass of 64^3 / 3 multiply-adds with
+// two barriers a step.  Entries are dealt row by row, so finished rows leave whole warps idle.
+// Bound by the latency of the double operations in the chain from one pivot to the next (its 87 k
+// multiply-adds alone are 22 us of one SM's pipe).  Before, factor
+// and inverse one after the other in shared memory took 228 us a block, 6.9 of 46.6 ms at 20 m;
+// 114 us now.  A pivot <= 0 (or NaN) sets *err and is replaced by 1 so that the remaining
+// steps stay finite.
+__global__ void __launch_bounds__(256) tik_potrf_kernel(const double* __restrict__ A, long long lda, int k,
+                                                        double* __restrict__ Linv, int* __restrict__ err) {
+    constexpr int kEnt = kT * (kT + 1) / 2, kPer = (kEnt + 255) / 256;
+    __shared__ double s_v[kT], s_u[kT], s_d;
+    const int tid = threadIdx.x;
     const long long o = (long long)k * kT;
-    for (int q = threadIdx.x; q < kT * kT; q += kThreads) S[q / kT][q % kT] = A[(o + q / kT) * lda + o + q % kT];
-    __syncthreads();
+    double w[kPer];
+    int mc[kPer];
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        const int p = i * 256 + tid;
+        int m = kT, c = 0;   // past the triangle: never touched
+        if (p < kEnt) tri_index(p, m, c);
+        mc[i] = m << 8 | c;
+        w[i] = p < kEnt ? A[(o + m) * lda + o + c] : 0.0;
+        if (p == 0) s_d = w[i];
+    }
     for (int j = 0; j < kT; ++j) {
-        if (threadIdx.x == 0) {
-            double d = S[j][j];
+        // column j of the rows below and row j, unscaled
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            const int m = mc[i] >> 8, c = mc[i] & 255;
+            if (m < kT && c == j && m > j) s_v[m] = w[i];
+            if (m == j && c < j) s_u[c] = w[i];
+        }
+        __syncthreads();
+        if (tid < kT) {
+            double d = s_d;
             if (!(d > 0.0)) {
-                atomicExch(err, 1);
+                if (tid == 0) atomicExch(err, 1);
                 d = 1.0;
             }
-            S[j][j] = sqrt(d);
+            const double r = inv_sqrt(d);
+            if (tid > j) s_u[tid] = s_v[tid] = s_v[tid] * r;
+            else s_u[tid] = tid < j ? s_u[tid] * r : r;
         }
         __syncthreads();
-        for (int i = j + 1 + threadIdx.x; i < kT; i += kThreads) S[i][j] /= S[j][j];
-        __syncthreads();
-        // trailing update of the lower part: pairs (i, c), j < c <= i
-        const int m = kT - j - 1;
-        for (int q = threadIdx.x; q < m * m; q += kThreads) {
-            const int i = j + 1 + q / m, c = j + 1 + q % m;
-            if (c <= i) S[i][c] -= S[i][j] * S[c][j];
-        }
-        __syncthreads();
-    }
-    // inverse of the lower factor: column c solves L x = e_c by forward substitution
-    if (threadIdx.x < kT) {
-        const int c = threadIdx.x;
-        for (int r = 0; r < kT; ++r) {
-            double v = (r == c) ? 1.0 : 0.0;
-            if (r < c) {
-                X[r][c] = 0.0;
-                continue;
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            const int m = mc[i] >> 8, c = mc[i] & 255;
+            if (m == j) w[i] = s_u[c];
+            else if (m > j && m < kT) {
+                w[i] = fma(-s_v[m], s_u[c], c == j ? 0.0 : w[i]);
+                if (m == j + 1 && c == j + 1) s_d = w[i];
             }
-            for (int q = c; q < r; ++q) v -= S[r][q] * X[q][c];
-            X[r][c] = v / S[r][r];
         }
+        __syncthreads();   // s_v and s_u are read before the next step writes them
     }
-    __syncthreads();
     double* Lk = Linv + (long long)k * kT * kT;
-    for (int q = threadIdx.x; q < kT * kT; q += kThreads) {
-        const int r = q / kT, c = q % kT;
-        A[(o + r) * lda + o + c] = (c <= r) ? S[r][c] : 0.0;
-        Lk[q] = X[r][c];
+    for (int q = tid; q < kT * kT; q += 256)
+        if (q % kT > q / kT) Lk[q] = 0.0;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        const int m = mc[i] >> 8, c = mc[i] & 255;
+        if (m < kT) Lk[m * kT + c] = w[i];
     }
 }
 
-// 4b. panel: A[i][k] <- A[i][k] Linv_kk^T for the tiles i > k
-__global__ void __launch_bounds__(kThreads) tik_trsm_kernel(double* __restrict__ A, long long lda, int k,
-                                                            const double* __restrict__ Linv) {
+// 4b. block column k of L below the diagonal, A[i][k] <- A[i][k] Linv_kk^T, and block row k of X,
+// X[k][j] <- Linv_kk X[k][j] for j < k, X[k][k] = Linv_kk, both in place.  One block per strip of 32
+// rows (A) or columns (X): the strip is read whole before it is written; Linv is lower triangular, so
+// its first 32 rows need half the depth.
+__global__ void __launch_bounds__(kThreads) tik_panel_kernel(double* __restrict__ A, double* __restrict__ X, long long ld, int k,
+                                                             int nt, const double* __restrict__ Linv) {
     __shared__ Chunk ch;
-    const int i = k + 1 + blockIdx.x;
-    const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
-    const long long npad = (long long)kT * (k + 1 + gridDim.x);   // gridDim.x = nt - k - 1
+    const int below = nt - k - 1;
     const double* Lk = Linv + (long long)k * kT * kT;
-    double c[4][4] = {};
-    for (int k0 = 0; k0 < kT; k0 += kKC) {
-        // C[r][q] = sum_m A[i][k][r][m] Linv[q][m]
-        load_trans(ch.a, A, lda, (long long)i * kT, (long long)k * kT + k0, npad, npad);
-        load_trans(ch.b, Lk, kT, 0, k0, kT, kT);
-        __syncthreads();
-        chunk_fma(ch, c, ty, tx);
-        __syncthreads();
-    }
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b)
-            A[((long long)i * kT + ty * 4 + a) * lda + (long long)k * kT + tx * 4 + b] = c[a][b];
-}
-
-// 4c. trailing update A[i][j] -= A[i][k] A[j][k]^T for the lower tiles i >= j > k
-__global__ void __launch_bounds__(kThreads) tik_update_kernel(double* __restrict__ A, long long lda, int k, int nt) {
-    __shared__ Chunk ch;
-    int i, j;
-    tri_index(blockIdx.x, i, j);
-    i += k + 1;
-    j += k + 1;
-    const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
-    const long long npad = (long long)nt * kT;
-    double c[4][4] = {};
-    for (int k0 = 0; k0 < kT; k0 += kKC) {
-        load_trans(ch.a, A, lda, (long long)i * kT, (long long)k * kT + k0, npad, npad);
-        load_trans(ch.b, A, lda, (long long)j * kT, (long long)k * kT + k0, npad, npad);
-        __syncthreads();
-        chunk_fma(ch, c, ty, tx);
-        __syncthreads();
-    }
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            double* p = &A[((long long)i * kT + ty * 4 + a) * lda + (long long)j * kT + tx * 4 + b];
-            *p -= c[a][b];
+    double c[2][2][4] = {};   // [half of Linv's rows]
+    if ((int)blockIdx.x < 2 * below) {
+        double* P = A + ((long long)(k + 1) * kT + blockIdx.x * kS) * ld + (long long)k * kT;   // 32 x 64 strip
+        for (int k0 = 0; k0 < kT; k0 += kS) {
+            load_trans(ch.a, P, ld, 0, k0, kS, kT);   // a[m][r] = P[r][k0 + m]
+            for (int h = k0 / kS; h < 2; ++h) {
+                load_trans(ch.b, Lk, kT, h * kS, k0, kT, kT);   // b[m][q] = Linv[32 h + q][k0 + m]
+                __syncthreads();
+                chunk_fma(ch, c[h]);
+                __syncthreads();
+            }
         }
-}
-
-// X = I (the right-hand side of L X = I)
-__global__ void tik_eye_kernel(double* __restrict__ X, long long ldx, long long n) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        X[i * ldx + i] = 1.0;
-}
-
-// 5a. X[i][j] <- Linv_ii X[i][j] for j <= i (in place; all of the block row is read first)
-__global__ void __launch_bounds__(kThreads) tik_trinv_scale_kernel(double* __restrict__ X, long long ldx, int i,
-                                                                   const double* __restrict__ Linv, int nt) {
-    __shared__ Chunk ch;
-    const int j = blockIdx.x;
-    const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
-    const long long npad = (long long)nt * kT;
-    const double* Li = Linv + (long long)i * kT * kT;
-    double c[4][4] = {};
-    for (int k0 = 0; k0 < kT; k0 += kKC) {
-        // C[r][q] = sum_m Linv[r][m] X[i][j][m][q]
-        load_trans(ch.a, Li, kT, 0, k0, kT, kT);
-        load_direct(ch.b, X, ldx, (long long)i * kT + k0, (long long)j * kT, npad, npad);
-        __syncthreads();
-        chunk_fma(ch, c, ty, tx);
-        __syncthreads();
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) P[out_row(i) * ld + h * kS + out_col(j)] = c[h][i][j];
+        return;
     }
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b)
-            X[((long long)i * kT + ty * 4 + a) * ldx + (long long)j * kT + tx * 4 + b] = c[a][b];
-}
-
-// 5b. X[m][j] -= L[m][i] X[i][j] for m > i, j <= i
-__global__ void __launch_bounds__(kThreads) tik_trinv_update_kernel(double* __restrict__ X, long long ldx,
-                                                                    const double* __restrict__ L, long long ldl, int i,
-                                                                    int nt) {
-    __shared__ Chunk ch;
-    const int m = i + 1 + blockIdx.x / (i + 1), j = blockIdx.x % (i + 1);
-    const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
-    const long long npad = (long long)nt * kT;
-    double c[4][4] = {};
-    for (int k0 = 0; k0 < kT; k0 += kKC) {
-        load_trans(ch.a, L, ldl, (long long)m * kT, (long long)i * kT + k0, npad, npad);
-        load_direct(ch.b, X, ldx, (long long)i * kT + k0, (long long)j * kT, npad, npad);
-        __syncthreads();
-        chunk_fma(ch, c, ty, tx);
-        __syncthreads();
+    const int q0 = (blockIdx.x - 2 * below) * kS;   // first column of the strip of X
+    double* P = X + (long long)k * kT * ld + q0;     // 64 x 32 strip
+    if (q0 >= k * kT) {
+        for (int q = threadIdx.x; q < kT * kS; q += kThreads) P[q / kS * ld + q % kS] = Lk[q / kS * kT + q0 - k * kT + q % kS];
+        return;
     }
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            double* p = &X[((long long)m * kT + ty * 4 + a) * ldx + (long long)j * kT + tx * 4 + b];
-            *p -= c[a][b];
+    for (int k0 = 0; k0 < kT; k0 += kS) {
+        load_direct(ch.b, P, ld, k0, 0, kT, kS);   // b[m][q] = P[k0 + m][q]
+        for (int h = k0 / kS; h < 2; ++h) {
+            load_trans(ch.a, Lk, kT, h * kS, k0, kT, kT);   // a[m][r] = Linv[32 h + r][k0 + m]
+            __syncthreads();
+            chunk_fma(ch, c[h]);
+            __syncthreads();
         }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) P[(h * kS + out_row(i)) * ld + out_col(j)] = c[h][i][j];
 }
 
-// 6. Minv[I][J] = sum_{m >= I} X[m][I]^T X[m][J] for lower tiles (X lower triangular), mirrored
-__global__ void __launch_bounds__(kThreads) tik_xtx_kernel(const double* __restrict__ X, long long ldx, int nt,
+// 4c. with L[.][k] and X[k][.] final: A[i][j] -= L[i][k] L[j][k]^T for the lower tiles i >= j > k, and
+// X[m][j] -= L[m][k] X[k][j] for m > k, j <= k, in 32 x 32 blocks of one launch (blocks of the trailing
+// matrix first, in order of rows)
+__global__ void __launch_bounds__(kThreads) tik_update_kernel(double* __restrict__ A, double* __restrict__ X, long long ld, int k,
+                                                              int nt) {
+    __shared__ Chunk ch;
+    const int rest = 2 * (nt - k - 1);   // 32-row blocks below
+    const long long n_a = (long long)rest * (rest + 1) / 2;
+    const long long L0 = (long long)(k + 1) * kT, kc = (long long)k * kT, npad = (long long)nt * kT;
+    double c[2][4] = {};
+    if (blockIdx.x < n_a) {
+        int i, j;
+        tri_index(blockIdx.x, i, j);
+        for (int k0 = 0; k0 < kT; k0 += kS) {
+            load_trans(ch.a, A, ld, L0 + i * kS, kc + k0, npad, npad);
+            load_trans(ch.b, A, ld, L0 + j * kS, kc + k0, npad, npad);
+            __syncthreads();
+            chunk_fma(ch, c);
+            __syncthreads();
+        }
+        double* P = A + (L0 + i * kS) * ld + L0 + j * kS;
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) P[out_row(a) * ld + out_col(b)] -= c[a][b];
+        return;
+    }
+    const int t = (int)(blockIdx.x - n_a), cols = 2 * (k + 1);
+    const long long r0 = L0 + (long long)(t / cols) * kS, c0 = (long long)(t % cols) * kS;
+    for (int k0 = 0; k0 < kT; k0 += kS) {
+        load_trans(ch.a, A, ld, r0, kc + k0, npad, npad);
+        load_direct(ch.b, X, ld, kc + k0, c0, npad, npad);
+        __syncthreads();
+        chunk_fma(ch, c);
+        __syncthreads();
+    }
+    double* P = X + r0 * ld + c0;
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) P[out_row(a) * ld + out_col(b)] -= c[a][b];
+}
+
+// 5. Minv[I][J] = sum_m X[m][I]^T X[m][J] over the 32-row blocks m >= I (X lower triangular) for the
+// lower blocks, mirrored; the longest sums first
+__global__ void __launch_bounds__(kThreads) tik_xtx_kernel(const double* __restrict__ X, long long ldx, int nb,
                                                            double* __restrict__ Minv, long long ldm) {
     __shared__ Chunk ch;
     int I, J;
     tri_index(blockIdx.x, I, J);
-    const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
-    const long long npad = (long long)nt * kT;
-    double c[4][4] = {};
-    for (int m = I; m < nt; ++m)
-        for (int k0 = 0; k0 < kT; k0 += kKC) {
-            load_direct(ch.a, X, ldx, (long long)m * kT + k0, (long long)I * kT, npad, npad);
-            load_direct(ch.b, X, ldx, (long long)m * kT + k0, (long long)J * kT, npad, npad);
-            __syncthreads();
-            chunk_fma(ch, c, ty, tx);
-            __syncthreads();
-        }
+    const long long npad = (long long)nb * kS;
+    double c[2][4] = {};
+    for (int m = I; m < nb; ++m) {
+        load_direct(ch.a, X, ldx, (long long)m * kS, (long long)I * kS, npad, npad);
+        load_direct(ch.b, X, ldx, (long long)m * kS, (long long)J * kS, npad, npad);
+        __syncthreads();
+        chunk_fma(ch, c);
+        __syncthreads();
+    }
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < 2; ++a)
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
-            const long long r = (long long)I * kT + ty * 4 + a, q = (long long)J * kT + tx * 4 + b;
+            const long long r = (long long)I * kS + out_row(a), q = (long long)J * kS + out_col(b);
             Minv[r * ldm + q] = c[a][b];
             if (I != J) Minv[q * ldm + r] = c[a][b];
         }
 }
 
-// 7. R[I..][S..] = -sum_J Minv[I][J] D[S][J]^T over the nonzero tiles of D (Minv symmetric:
-// its block (J, I) is read as it is)
+// ------------------------------------------------------------------------------------------
+// 6. R = -M^(-1) D^T
+// ------------------------------------------------------------------------------------------
+// 64 commands x 32 slopes per block: a warp takes 4 slopes one after another, each lane 2 commands
+// (Minv is symmetric: the row of each nonzero's actuator is read, 512 bytes per warp, mostly from L1
+// since neighbouring slopes share actuators); transposed through shared memory for the store.
+template <typename Out>
+__global__ void __launch_bounds__(256) tik_apply_sparse_kernel(const double* __restrict__ Minv, long long ldm,
+                                                               const int* __restrict__ row, const int* __restrict__ col,
+                                                               const float* __restrict__ val, int n_slopes, int n_cmd,
+                                                               Out* __restrict__ R, long long ldr) {
+    __shared__ Out s_r[kT][33];
+    const int lane = threadIdx.x & 31, w = threadIdx.x / 32;
+    const int s0 = blockIdx.x * 32, i0 = blockIdx.y * kT;   // slopes run fastest: the blocks in flight share Minv's columns
+    const double* M = Minv + i0 + 2 * lane;
+    for (int q = 0; q < 4; ++q) {
+        const int s = s0 + 4 * w + q;
+        double x = 0.0, y = 0.0;
+        if (s < n_slopes) {
+            const int p1 = row[s + 1];
+#pragma unroll 4
+            for (int p = row[s]; p < p1; ++p) {
+                const double2 m = *reinterpret_cast<const double2*>(M + (long long)__ldg(col + p) * ldm);
+                const double d = (double)__ldg(val + p);
+                x = fma(m.x, d, x);
+                y = fma(m.y, d, y);
+            }
+        }
+        s_r[2 * lane][4 * w + q] = (Out)(-x);
+        s_r[2 * lane + 1][4 * w + q] = (Out)(-y);
+    }
+    __syncthreads();
+    for (int i = w; i < kT; i += 8)
+        if (i0 + i < n_cmd && s0 + lane < n_slopes) R[(long long)(i0 + i) * ldr + s0 + lane] = s_r[i][lane];
+}
+
+// dense D: 32 x 32 block (commands I, slopes S) over the nonzero tiles of D
 template <typename Out>
 __global__ void __launch_bounds__(kThreads) tik_apply_kernel(const double* __restrict__ Minv, long long ldm, int nt,
                                                              const float* __restrict__ D, long long ld, int n_slopes,
                                                              int n_cmd, const unsigned char* __restrict__ mask,
                                                              Out* __restrict__ R, long long ldr) {
     __shared__ Chunk ch;
-    const int I = blockIdx.x, S = blockIdx.y;
-    const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
+    const int I = blockIdx.y, S = blockIdx.x;
     const long long npad = (long long)nt * kT;
-    double c[4][4] = {};
+    double c[2][4] = {};
     for (int J = 0; J < nt; ++J) {
-        if (!mask[(long long)S * nt + J]) continue;
-        for (int k0 = 0; k0 < kT; k0 += kKC) {
+        if (!mask[(long long)(S / 2) * nt + J]) continue;
+        for (int k0 = 0; k0 < kT; k0 += kS) {
             // C[r][q] = sum_m Minv[J0 + m][I0 + r] D[S0 + q][J0 + m]
-            load_direct(ch.a, Minv, ldm, (long long)J * kT + k0, (long long)I * kT, npad, npad);
-            load_trans(ch.b, D, ld, (long long)S * kT, (long long)J * kT + k0, n_slopes, n_cmd);
+            load_direct(ch.a, Minv, ldm, (long long)J * kT + k0, (long long)I * kS, npad, npad);
+            load_trans(ch.b, D, ld, (long long)S * kS, (long long)J * kT + k0, n_slopes, n_cmd);
             __syncthreads();
-            chunk_fma(ch, c, ty, tx);
+            chunk_fma(ch, c);
             __syncthreads();
         }
     }
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < 2; ++a)
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
-            const long long r = (long long)I * kT + ty * 4 + a, q = (long long)S * kT + tx * 4 + b;
+            const long long r = (long long)I * kS + out_row(a), q = (long long)S * kS + out_col(b);
             if (r < n_cmd && q < n_slopes) R[r * ldr + q] = (Out)(-c[a][b]);
         }
 }
@@ -397,22 +616,41 @@ extern "C" mcao_status mcao_tikhonov_reconstructor(const float* D, int n_slopes,
     if (!std::isfinite(alpha) || alpha < 0.0) return report(err, err_len, MCAO_E_INVALID_ARG, "alpha must be >= 0");
     if (r_fp64 != 0 && r_fp64 != 1) return report(err, err_len, MCAO_E_INVALID_ARG, "r_fp64 must be 0 or 1");
     const int nt = (n_cmd + kT - 1) / kT, nS = (n_slopes + kT - 1) / kT;
-    const long long npad = (long long)nt * kT;
+    const long long npad = (long long)nt * kT, ld = (long long)ld_d;
     cudaStream_t st = (cudaStream_t)stream;
     double *G = nullptr, *X = nullptr, *Linv = nullptr, *d_lam = nullptr;
+    int *at = nullptr, *idx = nullptr, *d_err = nullptr;
+    float* val = nullptr;
     unsigned char* mask = nullptr;
-    int* d_err = nullptr;
     cudaError_t e = cudaMalloc(&G, sizeof(double) * npad * npad);
     if (e == cudaSuccess) e = cudaMalloc(&X, sizeof(double) * npad * npad);
     if (e == cudaSuccess) e = cudaMalloc(&Linv, sizeof(double) * nt * kT * kT);
-    if (e == cudaSuccess) e = cudaMalloc(&mask, (size_t)nS * nt);
+    if (e == cudaSuccess) e = cudaMalloc(&at, sizeof(int) * ((size_t)n_slopes + n_cmd + 2));
     if (e == cudaSuccess) e = cudaMalloc(&d_err, 2 * sizeof(double));   // error flag, then lambda
+    // nonzeros: row starts at at[0 .. n_slopes], column starts at at[n_slopes + 1 ..]
+    int* col_at = at + n_slopes + 1;
+    int nnz = 0;
+    if (e == cudaSuccess) {
+        tik_row_count_kernel<<<(n_slopes + 7) / 8, 256, 0, st>>>(D, ld, n_slopes, n_cmd, at);
+        tik_col_count_kernel<<<(n_cmd + 31) / 32, 32 * kCscWarps, 0, st>>>(D, ld, n_slopes, n_cmd, col_at);
+        tik_scan_kernel<<<1, 1024, 0, st>>>(at, n_slopes);
+        tik_scan_kernel<<<1, 1024, 0, st>>>(col_at, n_cmd);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&nnz, at + n_slopes, sizeof(int), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    // compressed products up to a third of nonzeros (more than 2^31 of them wrap to a negative count)
+    // and as long as a row of G fits in shared memory; above, the tile products read less
+    const int gram_smem = n_cmd * (int)sizeof(double);
+    const bool sparse = (long long)n_slopes * n_cmd < (1LL << 31) && (long long)nnz * 3 <= (long long)n_slopes * n_cmd &&
+                        n_cmd <= 28000;
+    if (e == cudaSuccess && sparse) {
+        e = cudaMalloc(&idx, sizeof(int) * 2 * (size_t)(nnz > 0 ? nnz : 1));
+        if (e == cudaSuccess) e = cudaMalloc(&val, sizeof(float) * 2 * (size_t)(nnz > 0 ? nnz : 1));
+    }
+    if (e == cudaSuccess && !sparse) e = cudaMalloc(&mask, (size_t)nS * nt);
     auto cleanup = [&]() {
-        cudaFree(G);
-        cudaFree(X);
-        cudaFree(Linv);
-        cudaFree(mask);
-        cudaFree(d_err);
+        for (void* p : {(void*)G, (void*)X, (void*)Linv, (void*)at, (void*)idx, (void*)val, (void*)mask, (void*)d_err}) cudaFree(p);
     };
     if (e != cudaSuccess) {
         cleanup();
@@ -422,42 +660,40 @@ extern "C" mcao_status mcao_tikhonov_reconstructor(const float* D, int n_slopes,
                       cudaGetErrorString(e));
     }
     d_lam = reinterpret_cast<double*>(d_err) + 1;
-    const int potrf_smem = 2 * kT * (kT + 1) * (int)sizeof(double);
-    e = cudaFuncSetAttribute(tik_potrf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, potrf_smem);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d_err, 0, sizeof(int), st);
+    e = cudaMemsetAsync(d_err, 0, sizeof(int), st);
     if (e == cudaSuccess) e = cudaMemsetAsync(G, 0, sizeof(double) * npad * npad, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(X, 0, sizeof(double) * npad * npad, st);
+    if (e == cudaSuccess && sparse)
+        e = cudaFuncSetAttribute(tik_gram_sparse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, gram_smem);
     if (e == cudaSuccess) {
-        tik_mask_kernel<<<dim3(nt, nS), kThreads, 0, st>>>(D, (long long)ld_d, n_slopes, n_cmd, nt, mask);
-        tik_gram_kernel<<<(unsigned)((long long)nt * (nt + 1) / 2), kThreads, 0, st>>>(
-            D, (long long)ld_d, n_slopes, n_cmd, nS, nt, mask, G, npad);
+        if (sparse) {
+            tik_row_fill_kernel<<<(n_slopes + 7) / 8, 256, 0, st>>>(D, ld, n_slopes, n_cmd, at, idx, val);
+            tik_col_fill_kernel<<<(n_cmd + 31) / 32, 32 * kCscWarps, 0, st>>>(D, ld, n_slopes, n_cmd, col_at, idx + nnz, val + nnz);
+            tik_gram_sparse_kernel<<<n_cmd, 128, gram_smem, st>>>(col_at, idx + nnz, val + nnz, at, idx, val, G, npad);
+        } else {
+            tik_mask_kernel<<<dim3(nt, nS), kThreads, 0, st>>>(D, ld, n_slopes, n_cmd, nt, mask);
+            tik_gram_kernel<<<(unsigned)((long long)2 * nt * (2 * nt + 1) / 2), kThreads, 0, st>>>(D, ld, n_slopes, n_cmd, nS, nt,
+                                                                                                 mask, G, npad);
+        }
         tik_regularize_kernel<<<1, 1024, 0, st>>>(G, npad, n_cmd, (int)npad, alpha, d_lam);
         for (int k = 0; k < nt; ++k) {
-            tik_potrf_kernel<<<1, kThreads, potrf_smem, st>>>(G, npad, k, Linv, d_err);
-            const int rest = nt - k - 1;
-            if (rest > 0) {
-                tik_trsm_kernel<<<rest, kThreads, 0, st>>>(G, npad, k, Linv);
-                tik_update_kernel<<<(unsigned)((long long)rest * (rest + 1) / 2), kThreads, 0, st>>>(G, npad, k, nt);
-            }
-        }
-        e = cudaGetLastError();
-    }
-    // X = L^-1: start from the identity
-    if (e == cudaSuccess) e = cudaMemsetAsync(X, 0, sizeof(double) * npad * npad, st);
-    if (e == cudaSuccess) {
-        tik_eye_kernel<<<64, 256, 0, st>>>(X, npad, npad);
-        for (int i = 0; i < nt; ++i) {
-            tik_trinv_scale_kernel<<<i + 1, kThreads, 0, st>>>(X, npad, i, Linv, nt);
-            const int below = nt - i - 1;
-            if (below > 0) tik_trinv_update_kernel<<<below * (i + 1), kThreads, 0, st>>>(X, npad, G, npad, i, nt);
+            const long long below = nt - k - 1, rest = 2 * below;
+            tik_potrf_kernel<<<1, 256, 0, st>>>(G, npad, k, Linv, d_err);
+            tik_panel_kernel<<<(unsigned)(2 * below + 2 * (k + 1)), kThreads, 0, st>>>(G, X, npad, k, nt, Linv);
+            if (below > 0)
+                tik_update_kernel<<<(unsigned)(rest * (rest + 1) / 2 + rest * 2 * (k + 1)), kThreads, 0, st>>>(G, X, npad, k, nt);
         }
         // M^-1 over the factor
-        tik_xtx_kernel<<<(unsigned)((long long)nt * (nt + 1) / 2), kThreads, 0, st>>>(X, npad, nt, G, npad);
-        if (r_fp64)
-            tik_apply_kernel<double><<<dim3(nt, nS), kThreads, 0, st>>>(G, npad, nt, D, (long long)ld_d, n_slopes,
-                                                                        n_cmd, mask, (double*)R, (long long)ld_r);
+        tik_xtx_kernel<<<(unsigned)((long long)2 * nt * (2 * nt + 1) / 2), kThreads, 0, st>>>(X, npad, 2 * nt, G, npad);
+        const dim3 gs((unsigned)((n_slopes + 31) / 32), (unsigned)nt), gd((unsigned)((n_slopes + kS - 1) / kS), (unsigned)(2 * nt));
+        if (sparse && r_fp64)
+            tik_apply_sparse_kernel<double><<<gs, 256, 0, st>>>(G, npad, at, idx, val, n_slopes, n_cmd, (double*)R, (long long)ld_r);
+        else if (sparse)
+            tik_apply_sparse_kernel<float><<<gs, 256, 0, st>>>(G, npad, at, idx, val, n_slopes, n_cmd, (float*)R, (long long)ld_r);
+        else if (r_fp64)
+            tik_apply_kernel<double><<<gd, kThreads, 0, st>>>(G, npad, nt, D, ld, n_slopes, n_cmd, mask, (double*)R, (long long)ld_r);
         else
-            tik_apply_kernel<float><<<dim3(nt, nS), kThreads, 0, st>>>(G, npad, nt, D, (long long)ld_d, n_slopes,
-                                                                       n_cmd, mask, (float*)R, (long long)ld_r);
+            tik_apply_kernel<float><<<gd, kThreads, 0, st>>>(G, npad, nt, D, ld, n_slopes, n_cmd, mask, (float*)R, (long long)ld_r);
         e = cudaGetLastError();
     }
     int h_err = 0;
