@@ -214,129 +214,178 @@ __global__ void misreg_sum_kernel(const double* __restrict__ rec, int n_rows, do
     }
 }
 
-// Interaction-matrix rows of both slopes of one subaperture (block x) over a part of one DM's
-// commands (block y = DM, block z = part).  Every command of the part is written once, zero
-// outside the actuators that reach the subaperture, so the matrix needs no clearing and its lines
-// are written whole: the pass is bound by the matrix's own bytes (39 m: 1.79 GB).  Before, the
-// matrix was cleared and one block per slope scattered its band into it: 160 us per laser star
-// (9264 blocks waiting at 15 barriers each) and 131 us per natural star (8 blocks) on top of the
-// clearing; x and y slopes now share the axis entries, bands and row weights, and a sensor of a few
-// subapertures is cut into enough parts to fill the GPU.
+// n floats from p set to zero by the block: whole 16-byte vectors between the unaligned ends
+__device__ __forceinline__ void zero_run(float* p, int n, int tid, int nthr) {
+    const int head = min(n, (int)((16 - (reinterpret_cast<uintptr_t>(p) & 15)) & 15) / 4), vecs = (n - head) / 4;
+    float4* v = reinterpret_cast<float4*>(p + head);
+    for (int q = tid; q < vecs; q += nthr) __stcs(v + q, make_float4(0.0f, 0.0f, 0.0f, 0.0f));
+    const int rest = n - 4 * vecs;   // at most 3 before and 3 after
+    if (tid < rest) __stcs(p + (tid < head ? tid : tid + 4 * vecs), 0.0f);
+}
+
+// Interaction-matrix rows of both slopes of one subaperture (block x) over a part of the commands
+// (block z).  Every command of the part is written once, zero outside the actuators that reach the
+// subaperture, so the matrix needs no clearing and its lines are written whole: the pass is bound by
+// the matrix's own bytes.  Commands run along DM rows, so on each DM they are a run of zeros, the
+// rows of the band (each command checked against the band's columns) and a run of zeros.  One block
+// does every DM, so that the three barriers of the setup are paid once per 2 n_cmd stored floats and
+// hide behind the other blocks' stores; a sensor of a few subapertures is cut into enough parts to
+// fill the GPU.  39 m (55608 x 8051, 1.79 GB), six laser stars: 484 us; with a block per DM and
+// a check of every command 789 us; before that the matrix was cleared and one block per slope
+// scattered its band: 6 x 160 us and 3 x 131 us (natural stars) on top of the clearing.
 // With gvec set (rotated DMs only) the rows are not stored: sum over both slopes of g row is added
 // to the command gradients of every vector.
-__global__ void __launch_bounds__(kAdjThreads) dm_rows_kernel(ProjLaunch L) {
+struct RowsDm {                // one DM's view from the block's subaperture
+    AxisEnt ex[kMaxNpx], ey[kMaxNpx];
+    int rng[4];                // actuators [a0, a1) x [b0, b1)
+    int c0, c1;                // commands of rows [b0, b1)
+};
+
+// nbw: most actuators per axis on a footprint, at most kAdjMaxBand (shared-memory row length)
+template <bool ROTATED>
+__global__ void __launch_bounds__(kAdjThreads, ROTATED ? 2 : 8) dm_rows_kernel(ProjLaunch L, int nbw) {
     extern __shared__ float rows_sm[];
-    __shared__ AxisEnt s_ex[kMaxNpx], s_ey[kMaxNpx];
-    __shared__ int s_rng[4];
+    __shared__ RowsDm s_dm[kMaxDms];
     const int tid = threadIdx.x, nthr = blockDim.x;
     const SubapDev sd = L.subaps[blockIdx.x];
     const WfsDev& w = L.ctx.wfs[sd.wfs];
-    const DmDesc dd = L.desc[blockIdx.y];
-    if (L.gvec && !dd.general) return;
     const int npx = w.n_px, i0 = sd.sx * npx, j0 = sd.sy * npx;
-    const GridView& v = L.ctx.views[L.real * L.ctx.view_stride + (long long)sd.wfs * L.ctx.n_grids + L.n_layers + blockIdx.y];
+    const GridView* V = L.ctx.views + L.real * L.ctx.view_stride + (long long)sd.wfs * L.ctx.n_grids + L.n_layers;
     float* s_L = rows_sm;                                  // [2][npx][npx]
-    float* s_T = s_L + 2 * npx * npx;                      // [2][npx][kAdjMaxBand]
-    float* s_gy = s_T + 2 * npx * kAdjMaxBand;             // [kAdjMaxBand][npx]
+    float* s_T = s_L + 2 * npx * npx;                      // [n_dms][2][npx][nbw]
+    float* s_gy = s_T + L.n_dms * 2 * npx * nbw;   // [n_dms][nbw][npx]
     const float *lx = sens_row(L.sens, w, 0, sd.rank), *ly = sens_row(L.sens, w, 1, sd.rank);
     for (int q = tid; q < npx * npx; q += nthr) {
         s_L[q] = lx[q];
         s_L[npx * npx + q] = ly[q];
     }
-    if (tid < npx)
-        s_ex[tid] = axis_entry(v.ax + (long long)(i0 + tid) * v.bp, v.n, v.periodic, v.inv_n);
-    else if (tid < 2 * npx)
-        s_ey[tid - npx] = axis_entry(v.ay + (long long)(j0 + tid - npx) * v.bp, v.n, v.periodic, v.inv_n);
+    for (int q = tid; q < L.n_dms * 2 * npx; q += nthr) {
+        const int m = q / (2 * npx), r = q - m * 2 * npx;
+        const GridView& v = V[m];
+        if (r < npx) s_dm[m].ex[r] = axis_entry(v.ax + (long long)(i0 + r) * v.bp, v.n, v.periodic, v.inv_n);
+        else s_dm[m].ey[r - npx] = axis_entry(v.ay + (long long)(j0 + r - npx) * v.bp, v.n, v.periodic, v.inv_n);
+    }
     __syncthreads();
-    if (tid == 0) {
+    if ((tid & 31) == 0 && tid / 32 < L.n_dms) {
         // the axis entries ascend (a DM grid does not wrap): the footprint is the first and last
+        RowsDm& d = s_dm[tid / 32];
+        const DmDesc& dd = L.desc[tid / 32];
         int rng[4];
-        actuator_range(dd, L.band, s_ex[0].idx & 0xffff, s_ex[npx - 1].idx >> 16, s_ey[0].idx & 0xffff,
-                       s_ey[npx - 1].idx >> 16, rng);
-        if (rng[1] - rng[0] > kAdjMaxBand || rng[3] - rng[2] > kAdjMaxBand) {
+        actuator_range(dd, L.band, d.ex[0].idx & 0xffff, d.ex[npx - 1].idx >> 16, d.ey[0].idx & 0xffff,
+                       d.ey[npx - 1].idx >> 16, rng);
+        if (rng[1] - rng[0] > nbw || rng[3] - rng[2] > nbw) {
             atomicExch(L.err, 1);
             rng[1] = rng[0];
             rng[3] = rng[2];
         }
-        for (int q = 0; q < 4; ++q) s_rng[q] = rng[q];
+        if (L.gvec && !dd.general) rng[3] = rng[2];
+        for (int q = 0; q < 4; ++q) d.rng[q] = rng[q];
+        const int* row0 = L.cmd_act + dd.row_off;          // first command of each DM row, and the total
+        d.c0 = row0[min(rng[2], dd.ny)];
+        d.c1 = row0[min(rng[3], dd.ny)];
     }
     __syncthreads();
-    const int a0 = s_rng[0], na = s_rng[1] - s_rng[0], b0 = s_rng[2], nbd = s_rng[3] - s_rng[2];
-    if (!dd.general) {
+    const int len = (L.n_cmd + gridDim.z - 1) / gridDim.z, first = blockIdx.z * len;
+    const int last = min(L.n_cmd, first + len);
+    for (int m = 0; m < L.n_dms; ++m) {
+        const DmDesc& dd = L.desc[m];
+        const RowsDm& d = s_dm[m];
+        const int a0 = d.rng[0], na = d.rng[1] - a0, b0 = d.rng[2], nbd = d.rng[3] - b0;
+        if (ROTATED && dd.general) continue;
+        if (dd.cmd0 >= last || dd.cmd0 + dd.n_cmd <= first) continue;   // not in this part
         // T[axis][y][a] = sum_x L[axis][y][x] gx_a(x)
         const float *Gx = L.g + dd.gx_off + a0, *Gy = L.g + dd.gy_off + b0;
+        float* T = s_T + m * 2 * npx * nbw;
+        float* gy = s_gy + m * npx * nbw;
         for (int idx = tid; idx < na * npx; idx += nthr) {
             const int y = idx / na, a = idx - y * na;
             float ax = 0.0f, ay = 0.0f;
+#pragma unroll 4
             for (int x = 0; x < npx; ++x) {
-                const float g = axis_weight(Gx, dd.nx, s_ex[x], a);
+                const float g = axis_weight(Gx, dd.nx, d.ex[x], a);
                 ax = fmaf(s_L[y * npx + x], g, ax);
                 ay = fmaf(s_L[(npx + y) * npx + x], g, ay);
             }
-            s_T[y * kAdjMaxBand + a] = ax;
-            s_T[(npx + y) * kAdjMaxBand + a] = ay;
+            T[y * nbw + a] = ax;
+            T[(npx + y) * nbw + a] = ay;
         }
         for (int idx = tid; idx < nbd * npx; idx += nthr) {
             const int y = idx / nbd, b = idx - y * nbd;
-            s_gy[b * npx + y] = axis_weight(Gy, dd.ny, s_ey[y], b);
+            gy[b * npx + y] = axis_weight(Gy, dd.ny, d.ey[y], b);
         }
-        __syncthreads();
     }
-    const float c0 = 0.5f * (float)(dd.surf_n - 1), ca = 0.5f * (float)(dd.nx - 1), cb = 0.5f * (float)(dd.ny - 1);
-    const int len = (dd.n_cmd + gridDim.z - 1) / gridDim.z, first = blockIdx.z * len;
-    const int last = min(dd.n_cmd, first + len);
+    __syncthreads();
     const int row_x = w.slope0 + sd.rank, row_y = row_x + w.n_valid;
-    float* out_x = L.D ? L.D + (long long)row_x * L.ld + dd.cmd0 : nullptr;
-    float* out_y = L.D ? L.D + (long long)row_y * L.ld + dd.cmd0 : nullptr;
-    for (int j = first + tid; j < last; j += nthr) {
-        const int ab = __ldg(L.cmd_act + dd.cmd0 + j), a = (ab & 0xffff) - a0, b = (int)((unsigned)ab >> 16) - b0;
-        float vx = 0.0f, vy = 0.0f;
-        if ((unsigned)a < (unsigned)na && (unsigned)b < (unsigned)nbd) {
-            if (!dd.general) {
-                for (int y = 0; y < npx; ++y) {
-                    const float g = s_gy[b * npx + y];
-                    vx = fmaf(g, s_T[y * kAdjMaxBand + a], vx);
-                    vy = fmaf(g, s_T[(npx + y) * kAdjMaxBand + a], vy);
-                }
-            } else {
-                // influence function of actuator (a, b) at q(i, j) = R(-rot)((x_i, y_j) - shift) / mag,
-                // at the four bilinear corners of every sample
-                const float fa = (float)(a0 + a), fb = (float)(b0 + b);
-                for (int q = 0; q < npx * npx; ++q) {
-                    const float l0 = s_L[q], l1 = s_L[npx * npx + q];
-                    if (l0 == 0.0f && l1 == 0.0f) continue;
-                    const AxisEnt ex = s_ex[q % npx], ey = s_ey[q / npx];
-                    float wt = 0.0f;
-                    for (int c = 0; c < 4; ++c) {
-                        const int i = (c & 1) ? ex.idx >> 16 : ex.idx & 0xffff, k = (c & 2) ? ey.idx >> 16 : ey.idx & 0xffff;
-                        const float wc = ((c & 1) ? ex.t : 1.0f - ex.t) * ((c & 2) ? ey.t : 1.0f - ey.t);
-                        const float x = ((float)i - c0) * dd.dx - dd.shx, y = ((float)k - c0) * dd.dx - dd.shy;
-                        const float ua = (dd.cr * x + dd.sr * y) * dd.inv_mag / dd.pitch + ca;
-                        const float ub = (-dd.sr * x + dd.cr * y) * dd.inv_mag / dd.pitch + cb;
-                        const float da = (ua - fa) * dd.pitch, db = (ub - fb) * dd.pitch;
-                        wt = fmaf(wc, expf(-(da * da + db * db) * dd.inv2s2), wt);
-                    }
-                    vx = fmaf(l0, wt, vx);
-                    vy = fmaf(l1, wt, vy);
-                }
-            }
-            vx *= v.sign;
-            vy *= v.sign;
-            if (L.gvec)
-                for (int vv = 0; vv < L.n_vec; ++vv) {
-                    const float* g = L.gvec + (long long)vv * L.n_slopes;
-                    const float add = fmaf(g[row_x], vx, g[row_y] * vy);
-                    if (add != 0.0f) atomicAdd(L.gc + (long long)vv * L.n_cmd + dd.cmd0 + j, add);
-                }
+    float* out_x = L.D ? L.D + (long long)row_x * L.ld : nullptr;
+    float* out_y = L.D ? L.D + (long long)row_y * L.ld : nullptr;
+    for (int m = 0; m < L.n_dms; ++m) {
+        const DmDesc& dd = L.desc[m];
+        const RowsDm& d = s_dm[m];
+        const int a0 = d.rng[0], na = d.rng[1] - a0, b0 = d.rng[2], nbd = d.rng[3] - b0;
+        const float sign = V[m].sign;
+        const float* T = s_T + m * 2 * npx * nbw;
+        const float* gy = s_gy + m * npx * nbw;
+        // this part's share of the DM's commands, split at the band's rows
+        const int lo = max(first, dd.cmd0), hi = max(lo, min(last, dd.cmd0 + dd.n_cmd));
+        const int c0 = min(max(dd.cmd0 + d.c0, lo), hi), c1 = min(max(dd.cmd0 + d.c1, c0), hi);
+        if (L.D) {
+            zero_run(out_x + lo, c0 - lo, tid, nthr);
+            zero_run(out_y + lo, c0 - lo, tid, nthr);
+            zero_run(out_x + c1, hi - c1, tid, nthr);
+            zero_run(out_y + c1, hi - c1, tid, nthr);
         }
-        if (out_x) {
-            __stcs(out_x + j, vx);
-            __stcs(out_y + j, vy);
+        for (int j = c0 + tid; j < c1; j += nthr) {
+            const int ab = __ldg(L.cmd_act + j), a = (ab & 0xffff) - a0, b = (int)((unsigned)ab >> 16) - b0;
+            float vx = 0.0f, vy = 0.0f;
+            if ((unsigned)a < (unsigned)na && (unsigned)b < (unsigned)nbd) {
+                if (!ROTATED || !dd.general) {
+#pragma unroll 8
+                    for (int y = 0; y < npx; ++y) {
+                        const float g = gy[b * npx + y];
+                        vx = fmaf(g, T[y * nbw + a], vx);
+                        vy = fmaf(g, T[(npx + y) * nbw + a], vy);
+                    }
+                } else {
+                    // influence function of actuator (a, b) at q(i, j) = R(-rot)((x_i, y_j) - shift) / mag,
+                    // at the four bilinear corners of every sample
+                    const float g0 = 0.5f * (float)(dd.surf_n - 1);
+                    const float fa = (float)(a0 + a) - 0.5f * (float)(dd.nx - 1), fb = (float)(b0 + b) - 0.5f * (float)(dd.ny - 1);
+                    for (int q = 0; q < npx * npx; ++q) {
+                        const float l0 = s_L[q], l1 = s_L[npx * npx + q];
+                        if (l0 == 0.0f && l1 == 0.0f) continue;
+                        const AxisEnt ex = d.ex[q % npx], ey = d.ey[q / npx];
+                        float wt = 0.0f;
+                        for (int c = 0; c < 4; ++c) {
+                            const int i = (c & 1) ? ex.idx >> 16 : ex.idx & 0xffff, k = (c & 2) ? ey.idx >> 16 : ey.idx & 0xffff;
+                            const float wc = ((c & 1) ? ex.t : 1.0f - ex.t) * ((c & 2) ? ey.t : 1.0f - ey.t);
+                            const float x = ((float)i - g0) * dd.dx - dd.shx, y = ((float)k - g0) * dd.dx - dd.shy;
+                            const float ua = (dd.cr * x + dd.sr * y) * dd.inv_mag / dd.pitch;
+                            const float ub = (-dd.sr * x + dd.cr * y) * dd.inv_mag / dd.pitch;
+                            const float da = (ua - fa) * dd.pitch, db = (ub - fb) * dd.pitch;
+                            wt = fmaf(wc, expf(-(da * da + db * db) * dd.inv2s2), wt);
+                        }
+                        vx = fmaf(l0, wt, vx);
+                        vy = fmaf(l1, wt, vy);
+                    }
+                }
+                vx *= sign;
+                vy *= sign;
+                if (L.gvec)
+                    for (int vv = 0; vv < L.n_vec; ++vv) {
+                        const float* g = L.gvec + (long long)vv * L.n_slopes;
+                        const float add = fmaf(g[row_x], vx, g[row_y] * vy);
+                        if (add != 0.0f) atomicAdd(L.gc + (long long)vv * L.n_cmd + j, add);
+                    }
+            }
+            if (L.D) {
+                __stcs(out_x + j, vx);
+                __stcs(out_y + j, vy);
+            }
         }
     }
     // padding columns past the last command
-    if (L.D && blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1)
-        for (long long j = L.n_cmd + tid; j < L.ld; j += nthr) L.D[(long long)row_x * L.ld + j] = L.D[(long long)row_y * L.ld + j] = 0.0f;
+    if (L.D && blockIdx.z == gridDim.z - 1)
+        for (long long j = L.n_cmd + tid; j < L.ld; j += nthr) out_x[j] = out_y[j] = 0.0f;
 }
 
 // Flags a subaperture whose footprint on a DM meets more actuators than the rows kernel takes (one
@@ -360,77 +409,93 @@ __global__ void dm_range_kernel(ProjLaunch L) {
 // separable weights: U[y][a] = sum_x g(y, x) gx_a(x), then C[b][a] -= sum_y gy_b(y) U[y][a] over
 // every sensor, in a fixed order.  The products are N^2 n_x + N n_x n_y per sensor and DM, whatever
 // the number of subapertures (before: each slope's row, added into the gradient by atomics).
-// Block: 8 pupil rows (one per warp) x 32 actuators per pass; x in tiles of 32 whose band of
-// actuators with a weight meets the 32.
+// Block: 8 pupil rows (one per warp) x 32 actuators; x in tiles of 32, and only the tiles whose band
+// of actuators with a weight meets the block's 32 (found for all tiles at once, one thread each: the
+// dependent reads of the band table one tile after another took most of the 39 us this pass took at
+// 320 x 320 samples and 3 sensors; 27 us now).
+constexpr int kProjMaxTiles = 512;   // pupil grids of at most 16384 samples per side
 __global__ void __launch_bounds__(256) dm_project_x(ProjLaunch L, const float* __restrict__ g_phase, long long phase_stride,
                                                     float* __restrict__ U, int u_rows, int u_cols) {
     __shared__ float s_w[32][33];
     __shared__ float s_g[8][32];
-    const int wi = blockIdx.y / L.n_dms, m = blockIdx.y - wi * L.n_dms, vec = blockIdx.z;
+    __shared__ int2 s_band[kProjMaxTiles];
+    const int wi = blockIdx.y / L.n_dms, m = blockIdx.y - wi * L.n_dms;
+    const int a_tiles = (u_cols + 31) / 32, vec = blockIdx.z / a_tiles, a0 = (blockIdx.z - vec * a_tiles) * 32;
     const WfsDev& w = L.ctx.wfs[wi];
     const DmDesc dd = L.desc[m];
     const int N = w.N, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int y = blockIdx.x * 8 + warp;
-    if (dd.general || (int)blockIdx.x * 8 >= N) return;
+    if (dd.general || a0 >= dd.nx || (int)blockIdx.x * 8 >= N) return;
     long long off = vec * phase_stride;
     for (int q = 0; q < wi; ++q) off += (long long)L.ctx.wfs[q].N * L.ctx.wfs[q].N;
     const GridView& v = L.ctx.views[L.real * L.ctx.view_stride + (long long)wi * L.ctx.n_grids + L.n_layers + m];
-    float* u = U + (((long long)vec * gridDim.y + blockIdx.y) * u_rows + y) * u_cols;
-    for (int a0 = 0; a0 < dd.nx; a0 += 32) {
-        float acc = 0.0f;
-        for (int x0 = 0; x0 < N; x0 += 32) {
-            const int xe = min(x0 + 32, N) - 1;
-            const AxisEnt e0 = axis_entry(v.ax + (long long)x0 * v.bp, v.n, v.periodic, v.inv_n);
-            const AxisEnt e1 = axis_entry(v.ax + (long long)xe * v.bp, v.n, v.periodic, v.inv_n);
-            int lo = dd.nx, hi = 0;
-            for (int t = (e0.idx & 0xffff) / kDmTile; t <= (e1.idx >> 16) / kDmTile; ++t) {
-                const int2 bt = L.band[dd.tband_x + t];
-                if (bt.y > bt.x) { lo = min(lo, bt.x); hi = max(hi, bt.y); }
-            }
-            if (hi <= a0 || lo >= a0 + 32) continue;   // the same for the whole block
-            __syncthreads();
-            for (int q = threadIdx.x; q < 32 * 32; q += 256) {
-                const int x = x0 + (q >> 5), a = a0 + (q & 31);
-                float wt = 0.0f;
-                if (x < N && a >= lo && a < hi)
-                    wt = axis_weight(L.g + dd.gx_off, dd.nx, axis_entry(v.ax + (long long)x * v.bp, v.n, v.periodic, v.inv_n), a);
-                s_w[q >> 5][q & 31] = wt;
-            }
-            s_g[warp][lane] = (y < N && x0 + lane < N) ? g_phase[off + (long long)y * N + x0 + lane] : 0.0f;
-            __syncthreads();
-#pragma unroll 8
-            for (int x = 0; x < 32; ++x) acc = fmaf(s_g[warp][x], s_w[x][lane], acc);
+    auto entry = [&](int x) { return axis_entry(v.ax + (long long)x * v.bp, v.n, v.periodic, v.inv_n); };
+    const int tiles = (N + 31) / 32;
+    for (int t = threadIdx.x; t < tiles; t += 256) {
+        int lo = dd.nx, hi = 0;
+        const int t1 = (entry(min(32 * t + 32, N) - 1).idx >> 16) / kDmTile;
+        for (int q = (entry(32 * t).idx & 0xffff) / kDmTile; q <= t1; ++q) {
+            const int2 bt = L.band[dd.tband_x + q];
+            if (bt.y > bt.x) { lo = min(lo, bt.x); hi = max(hi, bt.y); }
         }
-        if (y < N && a0 + lane < dd.nx) u[a0 + lane] = acc;
+        s_band[t] = make_int2(lo, hi);
     }
+    float acc = 0.0f;
+    __syncthreads();
+    for (int t = 0; t < tiles; ++t) {
+        const int2 bt = s_band[t];
+        if (bt.y <= a0 || bt.x >= a0 + 32) continue;   // the same for the whole block
+        const int x0 = 32 * t;
+        __syncthreads();
+        for (int q = threadIdx.x; q < 32 * 32; q += 256) {
+            const int x = x0 + (q >> 5), a = a0 + (q & 31);
+            s_w[q >> 5][q & 31] = (x < N && a >= bt.x && a < bt.y) ? axis_weight(L.g + dd.gx_off, dd.nx, entry(x), a) : 0.0f;
+        }
+        s_g[warp][lane] = (y < N && x0 + lane < N) ? g_phase[off + (long long)y * N + x0 + lane] : 0.0f;
+        __syncthreads();
+#pragma unroll 8
+        for (int x = 0; x < 32; ++x) acc = fmaf(s_g[warp][x], s_w[x][lane], acc);
+    }
+    if (y < N && a0 + lane < dd.nx) U[(((long long)vec * gridDim.y + blockIdx.y) * u_rows + y) * u_cols + a0 + lane] = acc;
 }
 
-// one block per (DM row b, 32 actuator columns): 8 warps take the pupil rows in turn
-__global__ void __launch_bounds__(256) dm_project_y(ProjLaunch L, int n_wfs, const float* __restrict__ U, int u_rows,
+// One block per (DM row b, 32 actuator columns).  The 32 warps take chunks of 32 pupil rows of each
+// sensor in turn: lane l forms the weight of row l, then the rows with one are added in order.
+// (A row at a time, each waiting for its band and table reads: 44 us; 23 us now.)
+__global__ void __launch_bounds__(1024) dm_project_y(ProjLaunch L, int n_wfs, const float* __restrict__ U, int u_rows,
                                                     int u_cols) {
-    __shared__ float s_sum[8][32];
+    __shared__ float s_sum[32][32];
     const int m = blockIdx.z % L.n_dms, vec = blockIdx.z / L.n_dms;
     const DmDesc dd = L.desc[m];
     const int b = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, a = blockIdx.x * 32 + lane;
     if (dd.general || b >= dd.ny || (int)blockIdx.x * 32 >= dd.nx) return;
     float acc = 0.0f;
+    int turn = 0;
     for (int wi = 0; wi < n_wfs; ++wi) {
         const WfsDev& w = L.ctx.wfs[wi];
         const GridView& v = L.ctx.views[L.real * L.ctx.view_stride + (long long)wi * L.ctx.n_grids + L.n_layers + m];
         const float* u = U + ((long long)vec * n_wfs + wi) * L.n_dms * u_rows * u_cols + (long long)m * u_rows * u_cols;
-        for (int y = warp; y < w.N; y += 8) {
-            const AxisEnt e = axis_entry(v.ay + (long long)y * v.bp, v.n, v.periodic, v.inv_n);
-            const int2 b0 = L.band[dd.tband_y + (e.idx & 0xffff) / kDmTile], b1 = L.band[dd.tband_y + (e.idx >> 16) / kDmTile];
-            if (!((b >= b0.x && b < b0.y) || (b >= b1.x && b < b1.y))) continue;
-            const float gy = axis_weight(L.g + dd.gy_off, dd.ny, e, b);
-            if (a < dd.nx) acc = fmaf(v.sign * gy, u[(long long)y * u_cols + a], acc);
+        for (int y0 = 0; y0 < w.N; y0 += 32, ++turn) {
+            if ((turn & 31) != warp) continue;
+            float gy = 0.0f;
+            if (y0 + lane < w.N) {
+                const AxisEnt e = axis_entry(v.ay + (long long)(y0 + lane) * v.bp, v.n, v.periodic, v.inv_n);
+                const int2 b0 = L.band[dd.tband_y + (e.idx & 0xffff) / kDmTile], b1 = L.band[dd.tband_y + (e.idx >> 16) / kDmTile];
+                if ((b >= b0.x && b < b0.y) || (b >= b1.x && b < b1.y)) gy = v.sign * axis_weight(L.g + dd.gy_off, dd.ny, e, b);
+            }
+            if (!__ballot_sync(0xffffffffu, gy != 0.0f)) continue;
+#pragma unroll 8
+            for (int q = 0; q < 32; ++q) {
+                const float g = __shfl_sync(0xffffffffu, gy, q);
+                if (g != 0.0f && a < dd.nx) acc = fmaf(g, u[(long long)(y0 + q) * u_cols + a], acc);
+            }
         }
     }
     s_sum[warp][lane] = acc;
     __syncthreads();
     if (warp == 0 && a < dd.nx) {
         float s = 0.0f;
-        for (int q = 0; q < 8; ++q) s += s_sum[q][lane];
+        for (int q = 0; q < 32; ++q) s += s_sum[q][lane];
         const int cmd = L.act_map[dd.map_off + (long long)b * dd.nx + a];
         if (cmd >= 0) L.gc[(long long)vec * L.n_cmd + cmd] = s;
     }
@@ -478,12 +543,14 @@ __global__ void __launch_bounds__(128) phase_adjoint_kernel(ProjLaunch L, float*
 
 cudaError_t launch_dm_rows(const ProjLaunch& L, int n_px, int sm_count, cudaStream_t s) {
     if (!L.n_valid || !L.n_dms) return cudaSuccess;
-    const size_t bytes = sizeof(float) * (2 * n_px * n_px + 3 * n_px * kAdjMaxBand);   // at most 57344
-    cudaError_t e = cudaFuncSetAttribute(dm_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    const int nbw = std::max(1, std::min(L.max_band, kAdjMaxBand));
+    const size_t bytes = sizeof(float) * (2 * n_px * n_px + L.n_dms * 3 * n_px * nbw);   // at most 204800
+    const auto kernel = L.rotated ? dm_rows_kernel<true> : dm_rows_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
-    // parts of a DM's commands: two blocks per SM where the subapertures alone do not give them
-    const int parts = std::max(1, std::min(16, 2 * sm_count / std::max(1, L.n_valid * L.n_dms)));
-    dm_rows_kernel<<<dim3((unsigned)L.n_valid, (unsigned)L.n_dms, (unsigned)parts), kAdjThreads, bytes, s>>>(L);
+    // parts of the commands: two blocks per SM where the subapertures alone do not give them
+    const int parts = std::max(1, std::min(16, 2 * sm_count / L.n_valid));
+    kernel<<<dim3((unsigned)L.n_valid, 1u, (unsigned)parts), kAdjThreads, bytes, s>>>(L, nbw);
     return cudaGetLastError();
 }
 
@@ -496,9 +563,10 @@ cudaError_t launch_dm_range(const ProjLaunch& L, cudaStream_t s) {
 cudaError_t launch_dm_project(const ProjLaunch& L, int n_wfs, int max_n, int max_nx, int max_ny, const float* g_phase,
                               long long phase_stride, float* U, cudaStream_t s) {
     if (!L.n_dms || !n_wfs) return cudaSuccess;
-    dm_project_x<<<dim3((unsigned)((max_n + 7) / 8), (unsigned)(n_wfs * L.n_dms), (unsigned)L.n_vec), 256, 0, s>>>(
+    dm_project_x<<<dim3((unsigned)((max_n + 7) / 8), (unsigned)(n_wfs * L.n_dms), (unsigned)(L.n_vec * ((max_nx + 31) / 32))),
+                   256, 0, s>>>(
         L, g_phase, phase_stride, U, max_n, max_nx);
-    dm_project_y<<<dim3((unsigned)((max_nx + 31) / 32), (unsigned)max_ny, (unsigned)(L.n_dms * L.n_vec)), 256, 0, s>>>(
+    dm_project_y<<<dim3((unsigned)((max_nx + 31) / 32), (unsigned)max_ny, (unsigned)(L.n_dms * L.n_vec)), 1024, 0, s>>>(
         L, n_wfs, U, max_n, max_nx);
     return cudaGetLastError();
 }

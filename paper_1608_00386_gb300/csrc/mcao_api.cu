@@ -141,8 +141,9 @@ struct mcao_sim {
     float* d_dm_g = nullptr;
     int dm_nb = 1;                        // largest actuator band of a 64 x 64 DM block (either axis)
     int2* d_dm_band = nullptr;
+    std::vector<int2> dm_band_host;
     int* d_dm_map = nullptr;
-    int* d_cmd_act = nullptr;             // [n_cmd] actuator of each command
+    int* d_cmd_act = nullptr;             // [n_cmd] actuator of each command, then each DM's row starts
     float* d_dm_surf = nullptr;
     int dm_tile_start[kMaxDms + 1] = {0};
     int n_cmd = 0;
@@ -1255,6 +1256,7 @@ mcao_status mcao_set_misregistration(mcao_sim* S, int dm, double shift_x, double
     CK(cudaMemcpyAsync(S->d_dm_band, band.data(), sizeof(int2) * band.size(), cudaMemcpyHostToDevice, S->s0));
     CK(cudaMemcpyAsync(S->d_dm_desc, S->dm_desc.data(), sizeof(DmDesc) * S->n_dms, cudaMemcpyHostToDevice, S->s0));
     CK(cudaStreamSynchronize(S->s0));
+    S->dm_band_host = band;
     return MCAO_OK;
 }
 
@@ -1314,6 +1316,16 @@ mcao_status mcao_load_dms(mcao_sim* S, int n_dms, const mcao_dm* dms) {
         S->dm_desc.push_back(D);
     }
     for (int m = n_dms; m <= kMaxDms; ++m) S->dm_tile_start[m] = tiles;
+    // commands before each DM row, after the actuators of the commands
+    for (int m = 0; m < n_dms; ++m) {
+        const mcao_dm& d = dms[m];
+        S->dm_desc[m].row_off = (int)cmd_act.size();
+        int before = 0;
+        for (int a = 0; a <= d.nx * d.ny; ++a) {
+            if (a % d.nx == 0) cmd_act.push_back(before);
+            if (a < d.nx * d.ny && d.valid[a]) ++before;
+        }
+    }
     S->n_cmd = ncmd;
     S->dm_misreg.assign(n_dms, {0.0, 0.0, 0.0, 1.0});
     { mcao_status r_ = build_dm_tables(S, g, band); if (r_ != MCAO_OK) return r_; }
@@ -1340,6 +1352,7 @@ mcao_status mcao_load_dms(mcao_sim* S, int n_dms, const mcao_dm* dms) {
         CK(dalloc(p, (size_t)S->n_real * std::max(ncmd, 1)));
         CK(cudaMemsetAsync(*p, 0, sizeof(float) * (size_t)S->n_real * std::max(ncmd, 1), S->s0));
     }
+    S->dm_band_host = band;
     mcao_status r = rebuild_views(S);
     if (r != MCAO_OK) return r;
     S->dms_loaded = true;
@@ -1803,7 +1816,38 @@ static ProjLaunch make_proj_launch(mcao_sim* S, const SubapDev* subaps, int n) {
     J.n_slopes = S->n_slopes;
     J.n_cmd = S->n_cmd;
     J.err = S->d_adj_err;
+    for (const auto& d : S->dm_desc) J.rotated |= d.general;
     return J;
+}
+
+// Upper bound of the actuators per axis that a footprint of a run's subapertures meets: on a separable
+// DM the bands of as many adjacent tiles as it can touch, on a rotated one the reach around its
+// diagonal.  Above what the rows kernel holds its own check refuses.
+static int footprint_band(const mcao_sim* S, const WfsRun& r) {
+    int most = 1;
+    for (const auto& W : S->wfs) {
+        if (W.p.n_px != r.n_px) continue;
+        for (int m = 0; m < S->n_dms; ++m) {
+            const DmDesc& D = S->dm_desc[m];
+            const double f = W.p.type == MCAO_WFS_LGS ? 1.0 - S->dms[m].alt_m / W.p.height : 1.0;
+            const double side = (double)W.p.n_px * W.dx * f / S->dms[m].surf_dx + 3.0;   // surface samples
+            if (D.general) {
+                most = std::max(most, (int)std::ceil(1.5 * side * S->dms[m].surf_dx * D.inv_mag / S->dms[m].pitch_m + 2.0 * D.rc) + 2);
+                continue;
+            }
+            const int span = std::min(D.tiles_x, (int)(side / kDmTile) + 2);
+            for (long long tb : {D.tband_x, D.tband_y})
+                for (int t = 0; t + span <= D.tiles_x; ++t) {
+                    int lo = 1 << 30, hi = 0;
+                    for (int q = t; q < t + span; ++q) {
+                        const int2 b = S->dm_band_host[tb + q];
+                        if (b.y > b.x) { lo = std::min(lo, b.x); hi = std::max(hi, b.y); }
+                    }
+                    most = std::max(most, hi - lo);
+                }
+        }
+    }
+    return most;
 }
 
 // waits for the queued calibration work; a band overflow becomes MCAO_E_UNSUPPORTED
@@ -1827,6 +1871,7 @@ static mcao_status run_matrix(mcao_sim* S, float* D, long long ld) {
     if (e == cudaSuccess && S->n_dms == 0) e = cudaMemsetAsync(D, 0, sizeof(float) * (size_t)S->n_slopes * ld, S->s0);
     for (const auto& r : S->runs) {
         ProjLaunch J = make_proj_launch(S, r.d_subaps, r.n_subaps);
+        J.max_band = footprint_band(S, r);
         J.D = D;
         J.ld = ld;
         if (e == cudaSuccess) e = launch_dm_rows(J, r.n_px, S->sm_count, S->s0);
@@ -1842,7 +1887,6 @@ static mcao_status run_vjp(mcao_sim* S, const float* gvec, int n_vec, float* gc,
     { mcao_status r_ = sync_all(S); if (r_ != MCAO_OK) return r_; }
     long long phase_total = 0;
     int max_n = 1, max_nx = 1, max_ny = 1, n_all = 0;
-    bool rotated = false;
     for (const auto& W : S->wfs) {
         phase_total += (long long)W.N * W.N;
         max_n = std::max(max_n, W.N);
@@ -1851,7 +1895,6 @@ static mcao_status run_vjp(mcao_sim* S, const float* gvec, int n_vec, float* gc,
     for (const auto& d : S->dm_desc) {
         max_nx = std::max(max_nx, d.nx);
         max_ny = std::max(max_ny, d.ny);
-        rotated = rotated || d.general;
     }
     const int group = std::min(n_vec, kGroup), n_wfs = (int)S->wfs.size();
     // workspace of a group: the pupil gradients (unless the caller takes them), then U
@@ -1894,7 +1937,8 @@ static mcao_status run_vjp(mcao_sim* S, const float* gvec, int n_vec, float* gc,
                 ProjLaunch K = J;
                 K.subaps = r.d_subaps;
                 K.n_valid = r.n_subaps;
-                if (e == cudaSuccess && rotated) e = launch_dm_rows(K, r.n_px, S->sm_count, S->s0);
+                K.max_band = footprint_band(S, r);
+                if (e == cudaSuccess && J.rotated) e = launch_dm_rows(K, r.n_px, S->sm_count, S->s0);
             }
         }
     }

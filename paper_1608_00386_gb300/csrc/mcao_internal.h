@@ -126,6 +126,7 @@ struct DmDesc {
     float inv2s2;        // 1 / (2 sigma^2) of the influence function (DM coordinates)
     float rc;            // window radius in actuator pitches (weights below 1e-10 left out)
     int cmd0, n_cmd;     // this DM's block of the command vector
+    int row_off;         // ProjLaunch::cmd_act: commands before each of the ny rows, and n_cmd
 };
 constexpr int kDmTile = 32;
 constexpr int kDmMaxBand = 64;   // actuators per tile and axis (checked on the host)
@@ -306,7 +307,8 @@ struct ProjLaunch {
     const float* g;
     const int2* band;
     const int* act_map;
-    const int* cmd_act;      // [n_cmd] actuator of each command: column | row << 16
+    const int* cmd_act;      // [n_cmd] actuator of each command: column | row << 16; then per DM at
+                             // DmDesc::row_off the commands before each row
     const SubapDev* subaps;  // valid subapertures (of one or several sensors)
     int n_valid;
     const float* sens;       // d slope / d phase (WfsDev::sens0)
@@ -317,6 +319,8 @@ struct ProjLaunch {
     float* gc;               // [n_vec][n_cmd] accumulated (or null)
     int n_cmd;
     int* err;                // set when a footprint meets more actuators than a block holds
+    int rotated;             // some DM is rotated (DmDesc::general)
+    int max_band;            // no footprint of these subapertures meets more actuators per axis
 };
 // noise-free slopes of L.subaps (sensors of n_px samples per subaperture) without forming an image,
 // and their derivatives with respect to the phase (realization `real`) into sens
