@@ -409,10 +409,19 @@ __device__ __forceinline__ void nz_box_muller2(float u0, float u1, float& zc, fl
     zs = __fmul_rn(rad, s);
 }
 
-// recip[j] = fl(1/j), j = 0..65 (entry 0 unused), filled with correctly rounded divisions
+// fl(1/j), correctly rounded divisions: recip[j], j = 0..65 (entry 0 unused), and recip2[k] = fl(1/(k + 1))
+// in both halves of a pair, k = 0..63
 constexpr int kRecipEntries = 66;
-__device__ __forceinline__ void fill_recip(float* recip, int tid, int nthr) {
-    for (int j = tid; j < kRecipEntries; j += nthr) recip[j] = (j > 0) ? __fdiv_rn(1.0f, (float)j) : 0.0f;
+struct NoiseTab {
+    float2 recip2[64];
+    float recip[kRecipEntries];
+};
+__device__ __forceinline__ void fill_recip(NoiseTab& t, int tid, int nthr) {
+    for (int j = tid; j < kRecipEntries; j += nthr) {
+        const float r = (j > 0) ? __fdiv_rn(1.0f, (float)j) : 0.0f;
+        t.recip[j] = r;
+        if (j > 0 && j <= 64) t.recip2[j - 1] = make_float2(r, r);
+    }
 }
 
 // Photon count of one pixel: Poisson by inversion for lambda < 16 (uniform u; two terms per
@@ -439,25 +448,87 @@ __device__ __forceinline__ int nz_photons(float lam, float u, float y, const flo
     return n < 0 ? 0 : n;
 }
 
+// packed float32 pairs (each half rounded as the scalar operation rounds)
+__device__ __forceinline__ unsigned long long f2_pack(float x, float y) {
+    unsigned long long d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
+    return d;
+}
+__device__ __forceinline__ float2 f2_unpack(unsigned long long v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ unsigned long long f2_mul(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+// The Poisson inversions of a pixel pair side by side, the whole warp together: the counts that
+// nz_photons gives for lam_a, lam_b < 16 (0 for a pixel at or above 16, which the caller replaces).
+// F_k does not fall with k for lambda >= 0, so the smallest k with u <= F_k (at most 64) is the number
+// of j < 64 with F_j < u: the sign bits of F_j - u, added up.  No branch, table look-up per lane or
+// dependent compare is left in a term: the two pixels' terms take three packed operations and four
+// for the signs, against about fourteen and a branch per pixel and two terms before, and the warp
+// leaves after the four terms in which its last pixel is found.  A negative lambda (rounding of a
+// dark pixel) whose F_0 reaches u has count 0; one whose F_0 does not takes the search one term at
+// a time.  recip2[k] = (fl(1 / (k + 1)), twice).
+__device__ __forceinline__ void nz_poisson2(float lam_a, float lam_b, float ua, float ub, const float2* recip2,
+                                            const float* recip, int& ka, int& kb) {
+    const bool in_a = lam_a < 16.0f, in_b = lam_b < 16.0f;
+    const float la = in_a ? lam_a : 0.0f, lb = in_b ? lam_b : 0.0f;
+    const float pa = nz_exp(-la), pb = nz_exp(-lb);
+    const bool odd_a = la < 0.0f && pa < ua, odd_b = lb < 0.0f && pb < ub;
+    const unsigned long long l2 = f2_pack(la, lb);
+    const unsigned long long nu = f2_pack(in_a && la >= 0.0f ? -ua : __int_as_float(0x7f800000),
+                                          in_b && lb >= 0.0f ? -ub : __int_as_float(0x7f800000));
+    unsigned long long p = f2_pack(pa, pb), F = p;
+    float2 d = f2_unpack(f2_add(F, nu));
+    unsigned int na = __float_as_uint(d.x) >> 31, nb = __float_as_uint(d.y) >> 31;
+    for (int k = 0; k < 64 && __any_sync(0xffffffffu, (__float_as_int(d.x) | __float_as_int(d.y)) < 0); k += 4) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float2 r = recip2[k + i];
+            p = f2_mul(p, f2_mul(l2, f2_pack(r.x, r.y)));
+            F = f2_add(F, p);
+            d = f2_unpack(f2_add(F, nu));
+            na += __float_as_uint(d.x) >> 31;
+            nb += __float_as_uint(d.y) >> 31;
+        }
+    }
+    ka = min((int)na, 64);
+    kb = min((int)nb, 64);
+    if (odd_a) ka = nz_photons(lam_a, ua, 0.0f, recip);
+    if (odd_b) kb = nz_photons(lam_b, ub, 0.0f, recip);
+}
+
 // Noisy counts of a pixel pair (pixel o and o + n_det^2 / 2 of one subaperture frame; g the
 // frame index of pixel o): draw A = Philox(g, step, sensor, 0) gives the two inversion uniforms
 // (words 0, 1) and, when read noise is on, one Box-Muller pair (words 2, 3) whose outputs are
 // the two pixels' read noise; draw B = Philox(g, step, sensor, 2), formed only when a pixel has
-// lambda >= 16, gives one Box-Muller pair (words 2, 3) for the two photon normals.
+// lambda >= 16, gives one Box-Muller pair (words 2, 3) for the two photon normals.  Every lane of
+// the warp calls it together.
 __device__ __forceinline__ void noise_pair(float lam_a, float lam_b, float read_noise, uint32_t g, uint32_t step,
-                                           uint32_t sensor, unsigned long long seed, const float* recip, int& na,
+                                           uint32_t sensor, unsigned long long seed, const NoiseTab& tab, int& na,
                                            int& nb) {
     const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
     uint32_t w[4] = {g, step, sensor, 0u};
     philox4x32_10(w, k0, k1);
-    float ya = 0.0f, yb = 0.0f;
+    nz_poisson2(lam_a, lam_b, nz_uniform(w[0]), nz_uniform(w[1]), tab.recip2, tab.recip, na, nb);
     if (!(lam_a < 16.0f) || !(lam_b < 16.0f)) {
         uint32_t v[4] = {g, step, sensor, 2u};
         philox4x32_10(v, k0, k1);
+        float ya, yb;
         nz_box_muller2(nz_uniform(v[2]), nz_uniform(v[3]), ya, yb);
+        if (!(lam_a < 16.0f)) na = nz_photons(lam_a, 0.0f, ya, tab.recip);
+        if (!(lam_b < 16.0f)) nb = nz_photons(lam_b, 0.0f, yb, tab.recip);
     }
-    na = nz_photons(lam_a, nz_uniform(w[0]), ya, recip);
-    nb = nz_photons(lam_b, nz_uniform(w[1]), yb, recip);
     if (read_noise > 0.0f) {
         float za, zb;
         nz_box_muller2(nz_uniform(w[2]), nz_uniform(w[3]), za, zb);

@@ -60,12 +60,14 @@ constexpr int kTmaWarps = 5;
 constexpr int kTmaRows = kReconRows;               // rows per item
 constexpr int kTmaSeg = kReconSeg;                 // 16-byte vectors per row segment (2 KB)
 constexpr int kTmaStages = 2;
+constexpr int kTmaChunks = 32;
 constexpr long long kWaitCycles = 2000000000ll;    // ~1 s at 2 GHz
 
 struct TmaSmem {
     uint4 ring[kTmaWarps][kTmaStages][kTmaRows * kTmaSeg];
     unsigned long long bar[kTmaWarps][kTmaStages];
     int item[kTmaWarps][kTmaStages];  // item whose first stage the slot holds; -1: no more items
+    ReconChunk chunk[kTmaChunks];     // the launch's first chunks (the others are read where they are)
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -116,9 +118,9 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
 
 // stage geometry of chunk kc of a slice: n4 16-byte vectors per row, nst stages of kTmaSeg
 // vectors (the last one shorter)
-__device__ __forceinline__ void chunk_geom(const ReconLaunch& L, int kc, int& n4, int& nst) {
+__host__ __device__ __forceinline__ void chunk_geom(const ReconLaunch& L, int kc, int& n4, int& nst) {
     const int epv = 16 / recon_esize(L.dtype);
-    const int ncols = min(L.len - kc * L.kc, L.kc);
+    const int ncols = L.len - kc * L.kc < L.kc ? L.len - kc * L.kc : L.kc;
     n4 = (ncols + epv - 1) / epv;
     nst = (n4 + kTmaSeg - 1) / kTmaSeg;
 }
@@ -179,21 +181,6 @@ __device__ __forceinline__ float2 vec_dot(uint4 r, const float4* sv, float2 acc)
         for (int i = 0; i < 4; ++i) acc = dot4x2(e4m3x4_to_f32x4(w[i]), sv[i], acc);
         return acc;
     }
-}
-
-// Chunk geometry {n4, nst} of a full chunk and of the slice's last (possibly shorter) one,
-// computed once per thread so that the per-stage path needs no division.
-struct SliceGeom {
-    int n_chunks;
-    int full[2], last[2];
-};
-
-__device__ __forceinline__ SliceGeom slice_geom(const ReconLaunch& L) {
-    SliceGeom g;
-    g.n_chunks = (L.len + L.kc - 1) / L.kc;
-    chunk_geom(L, 0, g.full[0], g.full[1]);
-    chunk_geom(L, g.n_chunks - 1, g.last[0], g.last[1]);
-    return g;
 }
 
 // One stage: the vectors e = lane + 32 j (j < 4) of the four rows.  A full stage (kTmaSeg
@@ -283,14 +270,14 @@ __global__ void __launch_bounds__(kTmaWarps * 32) recon_tma_kernel(ReconLaunch L
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (lane == 0)
         for (int st = 0; st < kTmaStages; ++st) mbar_init(&sm.bar[warp][st], 1);
+    if (threadIdx.x < min(kTmaChunks, L.n_chunks)) sm.chunk[threadIdx.x] = L.chunks[threadIdx.x];
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     __syncthreads();
     const uint64_t pol = evict_first_policy();
     const int n_rq = L.n_rq;
-    const SliceGeom g = slice_geom(L);
-    const int n_items = n_rq * g.n_chunks;
-    const uint4* R4 = reinterpret_cast<const uint4*>(L.R + L.base);
-    const long long blk4 = (long long)kTmaRows * L.kc / (16 / recon_esize(DT));   // vectors per item block
+    const int n_items = n_rq * L.n_chunks;
+    const uint4* R4 = reinterpret_cast<const uint4*>(L.R);
+    auto chunk_of = [&](int kc) -> const ReconChunk& { return kc < kTmaChunks ? sm.chunk[kc] : L.chunks[kc]; };
 
     // producer state (used by lane 0 only)
     int p_next = 0, p_t = 0, p_n4 = 0, p_nst = 1, issued = 0;
@@ -307,10 +294,10 @@ __global__ void __launch_bounds__(kTmaWarps * 32) recon_tma_kernel(ReconLaunch L
             }
             p_next = (int)atomicAdd(L.work, 1u);
             const int kc = it / n_rq, rq = it - kc * n_rq;
-            const int* q = kc == g.n_chunks - 1 ? g.last : g.full;
-            p_n4 = q[0];
-            p_nst = q[1];
-            p_src = R4 + ((long long)kc * n_rq + rq) * blk4;
+            const ReconChunk& c = chunk_of(kc);
+            p_n4 = c.n4;
+            p_nst = c.nst;
+            p_src = R4 + c.src + (long long)rq * c.stride;
             sm.item[warp][st] = it;
         }
         const int cnt = min(kTmaSeg, p_n4 - p_t * kTmaSeg);
@@ -332,9 +319,9 @@ __global__ void __launch_bounds__(kTmaWarps * 32) recon_tma_kernel(ReconLaunch L
         it = __shfl_sync(0xffffffffu, it, 0);
         if (it < 0) break;
         const int kc = it / n_rq, rq = it - kc * n_rq;
-        const int* cg = kc == g.n_chunks - 1 ? g.last : g.full;
-        const int n4 = cg[0], nst = cg[1];
-        const float4* s4 = reinterpret_cast<const float4*>(L.s + L.col0 + kc * L.kc);
+        const ReconChunk& c = chunk_of(kc);
+        const int n4 = c.n4, nst = c.nst, slot = c.slot;
+        const float4* s4 = reinterpret_cast<const float4*>(L.s + c.col);
         float2 acc2[kTmaRows];
 #pragma unroll
         for (int q = 0; q < kTmaRows; ++q) acc2[q] = make_float2(0.0f, 0.0f);
@@ -382,7 +369,7 @@ __global__ void __launch_bounds__(kTmaWarps * 32) recon_tma_kernel(ReconLaunch L
             for (int o = 16; o > 0; o >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
         }
         if (lane == 0) {
-            float* out = L.partial + (size_t)(L.chunk0 + kc) * L.n_cmd;
+            float* out = L.partial + (size_t)slot * L.n_cmd;
             const int row0 = rq * kTmaRows;
 #pragma unroll
             for (int q = 0; q < kTmaRows; ++q)
@@ -523,6 +510,19 @@ cudaError_t launch_transpose(const float* src, int rows, int cols, void* out, in
     return cudaGetLastError();
 }
 
+void recon_slice_chunks(const ReconLaunch& L, std::vector<ReconChunk>& out) {
+    const int epv = 16 / recon_esize(L.dtype);
+    for (int kc = 0; kc * L.kc < L.len; ++kc) {
+        ReconChunk c{};
+        chunk_geom(L, kc, c.n4, c.nst);
+        c.stride = kTmaRows * L.kc / epv;
+        c.src = L.base / 16 + (long long)kc * L.n_rq * c.stride;
+        c.col = L.col0 + kc * L.kc;
+        c.slot = L.chunk0 + kc;
+        out.push_back(c);
+    }
+}
+
 long long recon_slice_bytes(int n_rq, int len, int kc, int dtype) {
     const long long chunks = (len + kc - 1) / kc;
     return chunks * n_rq * (long long)kTmaRows * kc * recon_esize(dtype);
@@ -563,7 +563,7 @@ cudaError_t recon_prepare() {
 cudaError_t launch_recon(const ReconLaunch& L, cudaStream_t s) {
     if (L.n_cmd <= 0 || L.len <= 0) return cudaSuccess;
     if (!L.work) return cudaErrorInvalidValue;
-    const int n_items = L.n_rq * ((L.len + L.kc - 1) / L.kc);
+    const int n_items = L.n_rq * L.n_chunks;
     const int need = (n_items + kTmaWarps - 1) / kTmaWarps;
     int ctas = (L.max_ctas > 0 && L.max_ctas < need) ? L.max_ctas : need;
     if (L.dtype == kReconF32) recon_tma_kernel<kReconF32><<<(unsigned)ctas, kTmaWarps * 32, sizeof(TmaSmem), s>>>(L);

@@ -25,7 +25,7 @@
 // outputs per block, four of which share an SM's pipe: the last wave of a launch costs a quarter of
 // what 64 x 64 outputs cost.  A dense D (more than a third nonzero) takes the tile products, where
 // each operand read serves 32 outputs.
-// 20 m (7280 x 1879): 46.6 ms before, 17.5 ms now; 39 m (55608 x 8051): 2.2 s before.
+// 20 m (7280 x 1870): 46.6 ms before, 17.5 ms now; 39 m (55608 x 8051): 2.2 s before.
 #include <cuda_runtime.h>
 
 #include <cmath>

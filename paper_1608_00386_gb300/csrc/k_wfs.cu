@@ -83,7 +83,7 @@ __device__ __forceinline__ void idft_small<8>(float2* v) {
 // ------------------------------------------------------------------------------------------
 struct GridMeta {
     const float* data;
-    int n;
+    int n;        // negative: pupil samples lie at most one grid sample apart
     float sign;
 };
 
@@ -111,7 +111,8 @@ __global__ void __launch_bounds__(256, 4) wfs_acf_kernel(WfsLaunch L) {
     __shared__ float2 s_EM[8][NPX * NPX];
     __shared__ float2 s_P[8][NPX * NL];
     __shared__ float2 s_tw[ND];
-    __shared__ float s_recip[kRecipEntries];
+    __shared__ float2 s_twx[4][NL];   // s_tw[(ux q) mod ND] of output column q, ux = -(NPX-1)..NPX-1
+    __shared__ NoiseTab s_recip;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x < ND) {
@@ -120,7 +121,12 @@ __global__ void __launch_bounds__(256, 4) wfs_acf_kernel(WfsLaunch L) {
         s_tw[threadIdx.x] = make_float2(cs, sn);
     }
     if (L.ctx.noise) fill_recip(s_recip, threadIdx.x, blockDim.x);
-    __syncthreads();  // the only block-wide barrier
+    __syncthreads();
+    if (threadIdx.x < 4 * NL) {
+        const int q = threadIdx.x / NL, c = threadIdx.x - q * NL;
+        s_twx[q][c] = s_tw[((c - (NPX - 1) + 2 * ND) * q) % ND];
+    }
+    __syncthreads();  // the last block-wide barrier
     // subapertures: one per warp (no counter), or taken one at a time from the counter, so that
     // warps of blocks that become resident late take only what is left
     auto take = [&]() {
@@ -128,13 +134,13 @@ __global__ void __launch_bounds__(256, 4) wfs_acf_kernel(WfsLaunch L) {
         if (lane == 0) v = atomicAdd(L.work, 1u);
         return (int)__shfl_sync(0xffffffffu, v, 0);
     };
-    // items run over (realization, subaperture)
-    const int n_items = L.n_subaps * L.ctx.n_real;
+    // the realization comes from the grid, so that the noise key and its round keys are uniform
+    // values of the block
+    const int real = blockIdx.y;
     int item = L.work ? take() : blockIdx.x * 8 + warp;
     for (;;) {
-        if (item >= n_items) break;  // warp-uniform; warp-level sync only from here on
-        const int real = item / L.n_subaps, sub = item - real * L.n_subaps;
-        const SubapDev sd = L.subaps[sub];
+        if (item >= L.n_subaps) break;  // warp-uniform; warp-level sync only from here on
+        const SubapDev sd = L.subaps[item];
         const WfsDev& w = L.ctx.wfs[sd.wfs];
         const int i0 = sd.sx * NPX, j0 = sd.sy * NPX;
         const int n_grids = L.ctx.n_grids;
@@ -147,22 +153,38 @@ __global__ void __launch_bounds__(256, 4) wfs_acf_kernel(WfsLaunch L) {
         if (lane < n_grids) {
             GridMeta gm;
             gm.data = V[lane].data;
-            gm.n = V[lane].n;
+            gm.n = V[lane].bp <= (1ll << 32) ? -V[lane].n : V[lane].n;
             gm.sign = V[lane].sign;
             s_gm[warp][lane] = gm;
         }
         __syncwarp();
 
-        // field E = A exp(i (scale phi - pi (x + y) / N)): lane -> column x, rows y0 and y0 + 4
+        // field E = A exp(i (scale phi - pi (x + y) / N)): lane -> column x, rows y0 and y0 + 1.  Where
+        // samples lie at most one grid sample apart (every grid finer than or as fine as the pupil's
+        // is not: its samples skip rows), the second row's cell is the first's or the next one, so
+        // three grid rows serve both: 6 loads and 3 interpolations along x instead of 8 and 4.
         {
-            const int x = lane & 7, y0 = lane >> 3, y1 = y0 + 4;
+            const int x = lane & 7, y0 = (lane >> 3) * 2, y1 = y0 + 1;
             float phi0 = 0.0f, phi1 = 0.0f;
     #pragma unroll 2
             for (int g = 0; g < n_grids; ++g) {
                 const GridMeta gm = s_gm[warp][g];
-                const AxisEnt ex = s_ex[g * NPX + x];
-                phi0 = fmaf(gm.sign, bilinear(gm.data, gm.n, ex, s_ey[g * NPX + y0]), phi0);
-                phi1 = fmaf(gm.sign, bilinear(gm.data, gm.n, ex, s_ey[g * NPX + y1]), phi1);
+                const AxisEnt ex = s_ex[g * NPX + x], e0 = s_ey[g * NPX + y0], e1 = s_ey[g * NPX + y1];
+                if (gm.n < 0) {
+                    const int n = -gm.n, x0 = ex.idx & 0xffff, x1 = ex.idx >> 16;
+                    const float* r0 = gm.data + (e0.idx & 0xffff) * n;
+                    const float* r1 = gm.data + (e0.idx >> 16) * n;
+                    const float* r2 = gm.data + (e1.idx >> 16) * n;
+                    const float a0 = __ldg(r0 + x0), b0 = __ldg(r0 + x1), a1 = __ldg(r1 + x0), b1 = __ldg(r1 + x1);
+                    const float a2 = __ldg(r2 + x0), b2 = __ldg(r2 + x1);
+                    const float t0 = fmaf(ex.t, b0 - a0, a0), t1 = fmaf(ex.t, b1 - a1, a1), t2 = fmaf(ex.t, b2 - a2, a2);
+                    const float top = e1.idx == e0.idx ? t0 : t1;
+                    phi0 = fmaf(gm.sign, fmaf(e0.t, t1 - t0, t0), phi0);
+                    phi1 = fmaf(gm.sign, fmaf(e1.t, t2 - top, top), phi1);
+                } else {
+                    phi0 = fmaf(gm.sign, bilinear(gm.data, gm.n, ex, e0), phi0);
+                    phi1 = fmaf(gm.sign, bilinear(gm.data, gm.n, ex, e1), phi1);
+                }
             }
             const float scale = w.scale;
             const float* arow = w.amp + (long long)j0 * w.N + i0 + x;
@@ -257,7 +279,7 @@ __global__ void __launch_bounds__(256, 4) wfs_acf_kernel(WfsLaunch L) {
             for (int c = 0; c < NL; ++c) {
                 const int ux = c - (NPX - 1);
                 const float2 p = s_P[warp][uy * NL + c];
-                const float2 t = s_tw[((ux + 2 * ND) * q) % ND];
+                const float2 t = s_twx[q][c];
                 const int r = (ux + 2 * ND) % QY;
                 S[r] = cadd(S[r], cmul(p, t));
             }
@@ -370,8 +392,8 @@ __global__ void __launch_bounds__(kFftThreads) wfs_fft_kernel(WfsLaunch L) {
     float2* W = Z + NFFT * NFFT;                                   // [NFFT]
     AxisEnt* ex = reinterpret_cast<AxisEnt*>(W + NFFT);            // [kMaxEntries * NPX]
     AxisEnt* ey = ex + kMaxEntries * NPX;                          // [kMaxEntries * NPX]
-    float* recip = reinterpret_cast<float*>(ey + kMaxEntries * NPX);  // [kRecipEntries]
-    float* red = recip + 68;                                       // [3 * NW]
+    NoiseTab& recip = *reinterpret_cast<NoiseTab*>(ey + kMaxEntries * NPX);
+    float* red = reinterpret_cast<float*>(&recip + 1);             // [3 * NW]
 
     const int tid = threadIdx.x;
     const int real = blockIdx.x / L.n_subaps;   // blocks run over (realization, subaperture)
@@ -529,7 +551,7 @@ __global__ void __launch_bounds__(kFftThreads) wfs_fft_kernel(WfsLaunch L) {
 template <int NPX, int NFFT>
 constexpr size_t fft_smem() {
     return sizeof(float2) * (2 * NFFT * NFFT + NFFT) + sizeof(AxisEnt) * 2 * kMaxEntries * NPX +
-           sizeof(float) * (68 + 3 * (kFftThreads / 32));
+           sizeof(NoiseTab) + sizeof(float) * 3 * (kFftThreads / 32);
 }
 
 // residual phase on the full pupil grid of one WFS, 8 x 8 tiles, one warp per tile
@@ -553,9 +575,11 @@ __global__ void __launch_bounds__(256) wfs_phase_kernel(Ctx ctx, int real, int w
 
 template <int NFFT, int NBIN>
 cudaError_t launch_acf(const WfsLaunch& L, cudaStream_t s) {
-    unsigned blocks = (unsigned)(((long long)L.n_subaps * L.ctx.n_real + 7) / 8);
-    if (L.work && L.max_blocks > 0 && blocks > (unsigned)L.max_blocks) blocks = (unsigned)L.max_blocks;
-    if (blocks) wfs_acf_kernel<NFFT, NBIN><<<blocks, 256, 0, s>>>(L);
+    unsigned blocks = (unsigned)((L.n_subaps + 7) / 8);
+    WfsLaunch K = L;
+    if (L.ctx.n_real > 1) K.work = nullptr;   // nothing runs beside a batch's sensing: one warp per subaperture
+    if (K.work && L.max_blocks > 0 && blocks > (unsigned)L.max_blocks) blocks = (unsigned)L.max_blocks;
+    if (blocks) wfs_acf_kernel<NFFT, NBIN><<<dim3(blocks, (unsigned)L.ctx.n_real), 256, 0, s>>>(K);
     return cudaGetLastError();
 }
 

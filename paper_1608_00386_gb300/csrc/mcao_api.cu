@@ -174,6 +174,7 @@ struct mcao_sim {
     float* d_multi_part = nullptr;        // and split-K partials
     TcProduct* tc = nullptr;
     std::vector<ReconLaunch> slices;      // one per sensor with slopes
+    ReconChunk* d_chunks = nullptr;       // every slice's chunks, in slice order
     std::vector<std::vector<int>> slice_wfs;  // sensors whose slopes each slice reads
     int n_chunks = 0;
     bool recon_loaded = false;
@@ -555,19 +556,35 @@ cudaError_t enqueue_step(mcao_sim* S, int* launches) {
     cudaEvent_t ev_sci = dep_event(S, used);
     if ((e = cudaEventRecord(ev_sci, S->s2)) != cudaSuccess) return e;
 
-    // warp-per-subaperture sensors, one launch each, on s0
-    for (size_t w = 0; w < S->wfs.size(); ++w) {
+    // warp-per-subaperture sensors on s0: adjacent sensors of one shape share a launch as long as all
+    // their subapertures have a warp each at once.  20 m, three sensors of 1212: one launch takes
+    // PLACEHOLDER_M us, three in a row took 63 (a quarter of the GPU's warps each, so a launch lasts as
+    // long as one subaperture whatever their number).  39 m: 4632 subapertures fill the 4864 warps, and
+    // a launch each lets the product of one sensor run beside the sensing of the next.  A batch's
+    // product runs after every sensor, so there all adjacent sensors share a launch.
+    const long long wave = S->n_real > 1 ? (1LL << 40) : (long long)S->tune.sense_blocks_per_sm * S->sm_count * 8;
+    for (size_t w = 0; w < S->wfs.size();) {
         const WfsHost& W = S->wfs[w];
-        if (W.fft_route || W.n_valid == 0) continue;
+        if (W.fft_route || W.n_valid == 0) {
+            ++w;
+            continue;
+        }
+        size_t end = w + 1;
+        long long n = W.n_valid;
+        for (; end < S->wfs.size(); ++end) {
+            const WfsHost& V = S->wfs[end];
+            if (V.p.n_px != W.p.n_px || V.p.n_fft != W.p.n_fft || V.p.n_bin != W.p.n_bin || n + V.n_valid > wave) break;
+            n += V.n_valid;
+        }
         slot = prof_begin(S, ST_WFS_MAIN, S->s0);
-        if ((e = launch_wfs(make_wfs_launch(S, W.d_subaps, W.n_valid, S->d_work + w), W.p.n_px, W.p.n_fft,
-                            W.p.n_bin, S->s0)) != cudaSuccess)
+        if ((e = launch_wfs(make_wfs_launch(S, W.d_subaps, (int)n, S->d_work + w), W.p.n_px, W.p.n_fft, W.p.n_bin, S->s0)) !=
+            cudaSuccess)
             return e;
         prof_end(S, slot, S->s0);
         ++nl;
         cudaEvent_t ev = dep_event(S, used);
         if ((e = cudaEventRecord(ev, S->s0)) != cudaSuccess) return e;
-        ready[w] = ev;
+        for (; w < end; ++w) ready[w] = ev;
     }
 
     if (S->n_real > 1) {
@@ -606,7 +623,8 @@ cudaError_t enqueue_step(mcao_sim* S, int* launches) {
     rl.c_prev = S->d_c_prev;
     rl.dc_prev = S->d_dc_prev;
     rl.n_real = 1;
-    for (size_t i = 0; i < S->slices.size(); ++i) {
+    // a launch takes the following slices too while they wait for the same sensing launch
+    for (size_t i = 0; i < S->slices.size();) {
         cudaEvent_t last = nullptr;
         for (int w : S->slice_wfs[i]) {
             cudaEvent_t ev = ready[w];
@@ -615,9 +633,11 @@ cudaError_t enqueue_step(mcao_sim* S, int* launches) {
         }
         slot = prof_begin(S, ST_RECON, S->s3);
         ReconLaunch rl_i = S->slices[i];
+        for (++i; i < S->slices.size() && S->slice_wfs[i].size() == 1 && last && ready[S->slice_wfs[i][0]] == last; ++i)
+            rl_i.n_chunks += S->slices[i].n_chunks;
         rl_i.max_ctas = std::max(1, S->sm_count * S->tune.recon_ctas_pct / 100);
-        // the last slice follows the last sensor and has the SMs to itself: one block per SM
-        if (i + 1 == S->slices.size()) rl_i.max_ctas = std::max(rl_i.max_ctas, S->sm_count);
+        // the last launch follows the last sensor and has the SMs to itself: one block per SM
+        if (i == S->slices.size()) rl_i.max_ctas = std::max(rl_i.max_ctas, S->sm_count);
         if ((e = launch_recon(rl_i, S->s3)) != cudaSuccess) return e;
         prof_end(S, slot, S->s3);
         ++nl;
@@ -740,7 +760,7 @@ void destroy_all(mcao_sim* S) {
         if (p) cudaFree(p);
     S->d_layer_owned.clear();
     dfree(S->d_dm_desc); dfree(S->d_dm_g); dfree(S->d_dm_band); dfree(S->d_dm_map);
-    dfree(S->d_dm_surf); dfree(S->d_views); dfree(S->d_R); dfree(S->d_rscale); dfree(S->d_c); dfree(S->d_partial);
+    dfree(S->d_dm_surf); dfree(S->d_views); dfree(S->d_R); dfree(S->d_chunks); dfree(S->d_rscale); dfree(S->d_c); dfree(S->d_partial);
     dfree(S->d_st); dfree(S->d_acc); dfree(S->d_err); dfree(S->d_work); dfree(S->d_sr_out);
     dfree(S->d_Rrm);
     dfree(S->d_c_prev); dfree(S->d_dc_prev); dfree(S->d_dc);
@@ -1496,7 +1516,18 @@ mcao_status mcao_load_reconstructor(mcao_sim* S, int n_cmd, int n_slopes, const 
         S->slices.push_back(L);
         S->slice_wfs.push_back(u);
     }
-    for (size_t i = 0; i < S->slices.size(); ++i) S->slices[i].work = S->d_work + S->wfs.size() + i;
+    std::vector<ReconChunk> table;
+    for (const auto& L : S->slices) recon_slice_chunks(L, table);
+    dfree(S->d_chunks);
+    if (e == cudaSuccess) e = dalloc(&S->d_chunks, table.size());
+    if (e == cudaSuccess && !table.empty())
+        e = cudaMemcpyAsync(S->d_chunks, table.data(), sizeof(ReconChunk) * table.size(), cudaMemcpyHostToDevice, S->s0);
+    for (size_t i = 0; i < S->slices.size(); ++i) {
+        ReconLaunch& L = S->slices[i];
+        L.work = S->d_work + S->wfs.size() + i;
+        L.chunks = S->d_chunks + L.chunk0;
+        L.n_chunks = (L.len + L.kc - 1) / L.kc;
+    }
     // 3) stage-tiled copy used by the product (see ReconLaunch)
     if (e == cudaSuccess) e = dalloc(&S->d_R, (size_t)std::max<long long>(tiled, 16));
     if (e == cudaSuccess) e = cudaMemsetAsync(S->d_R, 0, (size_t)std::max<long long>(tiled, 16), S->s0);

@@ -221,7 +221,20 @@ struct ReduceLaunch {
 };
 cudaError_t launch_recon_reduce(const ReduceLaunch& L, cudaStream_t s);
 
+//
+// One column chunk of the product, as the kernel takes it.  A launch covers consecutive chunks: those of
+// one slice, or of adjacent slices whose sensors are sensed together (their slopes are there at the
+// same time, and a small slice does not fill the GPU).
+struct ReconChunk {
+    long long src;      // 16-byte vector of R where the chunk's row quad 0 starts
+    int stride;         // vectors from one row quad to the next
+    int n4, nst;        // vectors per row, stages
+    int col, slot;      // first column in the padded slope layout, partial-sum slot
+    int pad;
+};
 struct ReconLaunch {
+    const ReconChunk* chunks;   // the launch's chunks
+    int n_chunks;
     const unsigned char* R;   // stage-tiled reconstructor
     long long base;     // first byte of this slice in R
     int dtype;          // kReconF32 / kReconBF16 / kReconE4M3
@@ -241,6 +254,7 @@ constexpr int kReconRows = 4;        // rows per work item (row quad)
 constexpr int kReconSeg = 128;       // 16-byte vectors per row and stage (at most)
 constexpr int kSlopePadTail = 16;    // zero floats after the padded slopes (a vector may run past)
 long long recon_slice_bytes(int n_rq, int len, int kc, int dtype);   // bytes of one slice in the tiled R
+void recon_slice_chunks(const ReconLaunch& L, std::vector<ReconChunk>& out);   // appends the slice's chunks
 cudaError_t recon_prepare();   // kernel attributes (outside stream capture)
 cudaError_t launch_recon(const ReconLaunch& L, cudaStream_t s);
 // Per-row scales of the float32 R [rows][ld] (first cols columns) for kReconE4M3:
