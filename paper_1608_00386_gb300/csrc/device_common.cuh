@@ -76,6 +76,21 @@ __device__ __forceinline__ float bilinear(const float* data, int n, AxisEnt ex, 
     return fmaf(ey.t, bot - top, top);
 }
 
+// bilinear samples of two vertically adjacent positions (column entry ex, row entries e0 and e1) at most
+// one grid sample apart: the second's cell is the first's or the one below, so three grid rows serve
+// both, with the same interpolations as two calls of bilinear
+__device__ __forceinline__ float2 bilinear_rows(const float* data, int n, AxisEnt ex, AxisEnt e0, AxisEnt e1) {
+    const int x0 = ex.idx & 0xffff, x1 = ex.idx >> 16;
+    const float* r0 = data + (e0.idx & 0xffff) * n;
+    const float* r1 = data + (e0.idx >> 16) * n;
+    const float* r2 = data + (e1.idx >> 16) * n;
+    const float a0 = __ldg(r0 + x0), b0 = __ldg(r0 + x1), a1 = __ldg(r1 + x0), b1 = __ldg(r1 + x1);
+    const float a2 = __ldg(r2 + x0), b2 = __ldg(r2 + x1);
+    const float t0 = fmaf(ex.t, b0 - a0, a0), t1 = fmaf(ex.t, b1 - a1, a1), t2 = fmaf(ex.t, b2 - a2, a2);
+    const float top = e1.idx == e0.idx ? t0 : t1;
+    return make_float2(fmaf(e0.t, t1 - t0, t0), fmaf(e1.t, t2 - top, top));
+}
+
 // residual phase (layers - DMs) at tile sample (x, y)
 __device__ __forceinline__ float tile_phase(const GridView* V, int n_grids, const AxisEnt* ex,
                                             const AxisEnt* ey, int T, int x, int y) {

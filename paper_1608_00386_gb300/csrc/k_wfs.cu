@@ -83,7 +83,7 @@ __device__ __forceinline__ void idft_small<8>(float2* v) {
 // ------------------------------------------------------------------------------------------
 struct GridMeta {
     const float* data;
-    int n;        // negative: pupil samples lie at most one grid sample apart
+    int n;
     float sign;
 };
 
@@ -153,37 +153,33 @@ __global__ void __launch_bounds__(256, 4) wfs_acf_kernel(WfsLaunch L) {
         if (lane < n_grids) {
             GridMeta gm;
             gm.data = V[lane].data;
-            gm.n = V[lane].bp <= (1ll << 32) ? -V[lane].n : V[lane].n;
+            gm.n = V[lane].n;
             gm.sign = V[lane].sign;
             s_gm[warp][lane] = gm;
         }
+        // pupil samples at most one grid sample apart in every grid
+        const bool near = __all_sync(0xffffffffu, lane >= n_grids || V[lane].bp <= (1ll << 32));
         __syncwarp();
 
-        // field E = A exp(i (scale phi - pi (x + y) / N)): lane -> column x, rows y0 and y0 + 1.  Where
-        // samples lie at most one grid sample apart (every grid finer than or as fine as the pupil's
-        // is not: its samples skip rows), the second row's cell is the first's or the next one, so
-        // three grid rows serve both: 6 loads and 3 interpolations along x instead of 8 and 4.
+        // field E = A exp(i (scale phi - pi (x + y) / N)): lane -> column x, rows y0 and y0 + 1, with
+        // three grid rows for both where they lie close enough (6 loads instead of 8)
         {
             const int x = lane & 7, y0 = (lane >> 3) * 2, y1 = y0 + 1;
             float phi0 = 0.0f, phi1 = 0.0f;
+            if (near) {
     #pragma unroll 2
-            for (int g = 0; g < n_grids; ++g) {
-                const GridMeta gm = s_gm[warp][g];
-                const AxisEnt ex = s_ex[g * NPX + x], e0 = s_ey[g * NPX + y0], e1 = s_ey[g * NPX + y1];
-                if (gm.n < 0) {
-                    const int n = -gm.n, x0 = ex.idx & 0xffff, x1 = ex.idx >> 16;
-                    const float* r0 = gm.data + (e0.idx & 0xffff) * n;
-                    const float* r1 = gm.data + (e0.idx >> 16) * n;
-                    const float* r2 = gm.data + (e1.idx >> 16) * n;
-                    const float a0 = __ldg(r0 + x0), b0 = __ldg(r0 + x1), a1 = __ldg(r1 + x0), b1 = __ldg(r1 + x1);
-                    const float a2 = __ldg(r2 + x0), b2 = __ldg(r2 + x1);
-                    const float t0 = fmaf(ex.t, b0 - a0, a0), t1 = fmaf(ex.t, b1 - a1, a1), t2 = fmaf(ex.t, b2 - a2, a2);
-                    const float top = e1.idx == e0.idx ? t0 : t1;
-                    phi0 = fmaf(gm.sign, fmaf(e0.t, t1 - t0, t0), phi0);
-                    phi1 = fmaf(gm.sign, fmaf(e1.t, t2 - top, top), phi1);
-                } else {
-                    phi0 = fmaf(gm.sign, bilinear(gm.data, gm.n, ex, e0), phi0);
-                    phi1 = fmaf(gm.sign, bilinear(gm.data, gm.n, ex, e1), phi1);
+                for (int g = 0; g < n_grids; ++g) {
+                    const GridMeta gm = s_gm[warp][g];
+                    const float2 p = bilinear_rows(gm.data, gm.n, s_ex[g * NPX + x], s_ey[g * NPX + y0], s_ey[g * NPX + y1]);
+                    phi0 = fmaf(gm.sign, p.x, phi0);
+                    phi1 = fmaf(gm.sign, p.y, phi1);
+                }
+            } else {
+                for (int g = 0; g < n_grids; ++g) {
+                    const GridMeta gm = s_gm[warp][g];
+                    const AxisEnt ex = s_ex[g * NPX + x];
+                    phi0 = fmaf(gm.sign, bilinear(gm.data, gm.n, ex, s_ey[g * NPX + y0]), phi0);
+                    phi1 = fmaf(gm.sign, bilinear(gm.data, gm.n, ex, s_ey[g * NPX + y1]), phi1);
                 }
             }
             const float scale = w.scale;
@@ -381,6 +377,49 @@ __global__ void __launch_bounds__(256, 4) wfs_acf_kernel(WfsLaunch L) {
 // ------------------------------------------------------------------------------------------
 constexpr int kFftThreads = 1024;
 
+// One radix-R Stockham stage (sub-length NS) of the transforms of an N x N array: of the first `batch`
+// rows (COL = false; consecutive threads take consecutive butterflies of a row) or of every column
+// (consecutive threads take consecutive columns, so that a warp reads and writes whole rows of shared
+// memory; with the butterflies of a column side by side a warp met one bank).  Index arithmetic is by
+// constants.  A block of this kernel has 4 subapertures' worth of work on the whole GPU in the 39 m
+// and 20 m systems, so its time is the latency of its 6 (elongated: 18) stages.
+template <int N, int NS, int R, bool COL>
+__device__ __forceinline__ void fft_stage(const float2* src, float2* dst, int batch, const float2* W, int tid) {
+    constexpr int NR = N / R, TW = N / (NS * R), ES = COL ? N : 1;
+#pragma unroll 2
+    for (int idx = tid; idx < batch * NR; idx += kFftThreads) {
+        const int f = COL ? idx % N : idx / NR, j = COL ? idx / N : idx % NR;
+        const float2* s = src + (COL ? f : f * N);
+        float2* d = dst + (COL ? f : f * N);
+        const int k = j % NS;
+        float2 v[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = s[(j + r * NR) * ES];
+        if constexpr (NS > 1) {
+#pragma unroll
+            for (int r = 1; r < R; ++r) v[r] = cmul(v[r], W[r * k * TW]);
+        }
+        small_dft<R>(v);
+        const int base = (j / NS) * NS * R + k;
+#pragma unroll
+        for (int r = 0; r < R; ++r) d[(base + r * NS) * ES] = v[r];
+    }
+}
+
+// the transforms of the first `batch` rows (or of all columns); returns the buffer holding the result (a
+// block-wide barrier follows every stage)
+template <int N, bool COL, int NS = 1>
+__device__ __forceinline__ float2* fft_pass(float2* a, float2* b, int batch, const float2* W, int tid) {
+    if constexpr (NS >= N) {
+        return a;
+    } else {
+        constexpr int R = ct_radix(N / NS);
+        fft_stage<N, NS, R, COL>(a, b, batch, W, tid);
+        __syncthreads();
+        return fft_pass<N, COL, NS * R>(b, a, batch, W, tid);
+    }
+}
+
 template <int NPX, int NFFT, int NBIN>
 __global__ void __launch_bounds__(kFftThreads) wfs_fft_kernel(WfsLaunch L) {
     constexpr int ND = NFFT / NBIN;
@@ -427,16 +466,9 @@ __global__ void __launch_bounds__(kFftThreads) wfs_fft_kernel(WfsLaunch L) {
         X[y * NFFT + x] = make_float2(a * cs, a * sn);
     }
     __syncthreads();
-    int rad[8];
-    int nr = 0;
-    for (int n = NFFT; n > 1;) {
-        int r = (n % 4 == 0) ? 4 : 2;
-        rad[nr++] = r;
-        n /= r;
-    }
     // rows holding the field (others are zero), then every column
-    float2* R1 = stockham_fft(X, Z, NFFT, rad, nr, NPX, NFFT, 1, W, tid, NT);
-    float2* R2 = stockham_fft(R1, R1 == X ? Z : X, NFFT, rad, nr, NFFT, 1, NFFT, W, tid, NT);
+    float2* R1 = fft_pass<NFFT, false>(X, Z, NPX, W, tid);
+    float2* R2 = fft_pass<NFFT, true>(R1, R1 == X ? Z : X, NFFT, W, tid);
 
     // sodium elongation (block-uniform branch): I <- Re IFFT2(FFT2(I) OTF), the inverse taken as
     // conj(FFT2(conj .)) and its 1 / N^2 left to the flux normalisation
@@ -447,8 +479,8 @@ __global__ void __launch_bounds__(kFftThreads) wfs_fft_kernel(WfsLaunch L) {
         float2* Bf = (R2 == X) ? Z : X;
         for (int q = tid; q < NFFT * NFFT; q += NT) A[q] = make_float2(A[q].x * A[q].x + A[q].y * A[q].y, 0.0f);
         __syncthreads();
-        float2* S1 = stockham_fft(A, Bf, NFFT, rad, nr, NFFT, NFFT, 1, W, tid, NT);
-        S1 = stockham_fft(S1, S1 == A ? Bf : A, NFFT, rad, nr, NFFT, 1, NFFT, W, tid, NT);
+        float2* S1 = fft_pass<NFFT, false>(A, Bf, NFFT, W, tid);
+        S1 = fft_pass<NFFT, true>(S1, S1 == A ? Bf : A, NFFT, W, tid);
         for (int q = tid; q < NFFT * NFFT; q += NT) {
             const int kx = q % NFFT, ky = q / NFFT;
             const float ux = (float)(kx < NFFT / 2 ? kx : kx - NFFT), uy = (float)(ky < NFFT / 2 ? ky : ky - NFFT);
@@ -457,8 +489,8 @@ __global__ void __launch_bounds__(kFftThreads) wfs_fft_kernel(WfsLaunch L) {
             S1[q] = make_float2(S1[q].x * o, -S1[q].y * o);
         }
         __syncthreads();
-        float2* S2 = stockham_fft(S1, S1 == A ? Bf : A, NFFT, rad, nr, NFFT, NFFT, 1, W, tid, NT);
-        img = stockham_fft(S2, S2 == A ? Bf : A, NFFT, rad, nr, NFFT, 1, NFFT, W, tid, NT);
+        float2* S2 = fft_pass<NFFT, false>(S1, S1 == A ? Bf : A, NFFT, W, tid);
+        img = fft_pass<NFFT, true>(S2, S2 == A ? Bf : A, NFFT, W, tid);
     }
 
     // |.|^2 (or the elongated image), shift by NFFT/2, bin NBIN x NBIN
