@@ -480,7 +480,8 @@ mcao_status mcao_tikhonov_reconstructor(const float* D, int n_slopes, int n_cmd,
  *   MCAO_TUNE_RECON_CTAS_PCT       reconstructor slices: blocks per SM x 100, [25, 400] (85); the
  *                                  step's last slice, which runs after the last sensor, takes at
  *                                  least one block per SM
- *   MCAO_TUNE_SCIENCE_AFTER_AUX    science waits for the block-per-subaperture sensors, 0 or 1 (1)
+ *   MCAO_TUNE_SCIENCE_AFTER_AUX    where the step has several warp-per-subaperture launches, science waits
+ *                                  for the block-per-subaperture sensors, 0 or 1 (1)
  *   MCAO_TUNE_TC_CHUNK             tensor-core batched product: k-blocks per TMEM accumulator,
  *                                  [1, 64] (8)
  *   MCAO_TUNE_MULTI_BLOCKS_PER_SM  batched float32 product: blocks per SM, [1, 2] (2)

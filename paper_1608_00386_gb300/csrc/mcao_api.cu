@@ -94,6 +94,7 @@ struct mcao_sim {
     cudaStream_t s0 = nullptr, s1 = nullptr, s2 = nullptr, s3 = nullptr;
     cudaStream_t user = nullptr;
     bool user_set = false;
+    bool s0_pending = true;               // see begin_async
     std::vector<cudaEvent_t> ev_pool;     // dependency events used while capturing
     cudaEvent_t ev_user = nullptr, ev_done = nullptr;
     // per-step readout (mcao_read_async): each read takes one slot of a device ring on s0 (a
@@ -103,6 +104,7 @@ struct mcao_sim {
     float* d_ring_c = nullptr;            // [kReadRing][ring_ncmd]
     double* d_ring_s = nullptr;           // [kReadRing][2 ring_nsci]
     int ring_ncmd = -1, ring_nsci = -1, ring_pos = 0;
+    int ring_last = -1;                   // last slot copied from, until a direct readout is ordered behind it
     std::vector<cudaEvent_t> ring_ready, ring_free;   // per slot: snapshot written / copied out
     std::vector<char> ring_busy;
 
@@ -182,7 +184,10 @@ struct mcao_sim {
     StepState* d_st = nullptr;
     SciAcc* d_acc = nullptr;
     double* d_sr_out = nullptr;           // staging of mcao_read_async's Strehl ratios
-    int* d_err = nullptr;                 // device-side error code (bounded waits)
+    double* d_psf_out = nullptr;          // PSF image in output order (allocated by the first image read)
+    size_t psf_out_n = 0;
+    int* h_err = nullptr;                 // error code of the bounded device waits, in mapped host memory: the
+    int* d_err = nullptr;                 // host reads it after a wait without a copy (d_err: its device address)
     unsigned int* d_work = nullptr;       // work counters: [n_wfs] sensing launches, [n_wfs + 1] slices
 
     // graph
@@ -509,6 +514,38 @@ cudaError_t enqueue_batched_product(mcao_sim* S, int n, float alpha, float beta,
     return cudaSuccess;
 }
 
+// Sensing launches of the warp-per-subaperture sensors: adjacent sensors of one shape share a launch as
+// long as all their subapertures have a warp each at once.  20 m, three sensors of 1212: one launch
+// takes 27 us, three in a row took 63 (a quarter of the GPU's warps each, so a launch lasts as long as
+// one subaperture whatever their number).  39 m: 4632 subapertures fill the 4864 warps, and a launch
+// each lets the product of one sensor run beside the sensing of the next.  A batch's product runs
+// after every sensor, so there all adjacent sensors share a launch.
+struct SenseGroup {
+    size_t first, end;   // sensors [first, end)
+    int n_subaps;
+};
+std::vector<SenseGroup> sensing_groups(const mcao_sim* S) {
+    const long long wave = S->n_real > 1 ? (1LL << 40) : (long long)S->tune.sense_blocks_per_sm * S->sm_count * 8;
+    std::vector<SenseGroup> out;
+    for (size_t w = 0; w < S->wfs.size();) {
+        const WfsHost& W = S->wfs[w];
+        if (W.fft_route || W.n_valid == 0) {
+            ++w;
+            continue;
+        }
+        size_t end = w + 1;
+        long long n = W.n_valid;
+        for (; end < S->wfs.size(); ++end) {
+            const WfsHost& V = S->wfs[end];
+            if (V.p.n_px != W.p.n_px || V.p.n_fft != W.p.n_fft || V.p.n_bin != W.p.n_bin || n + V.n_valid > wave) break;
+            n += V.n_valid;
+        }
+        out.push_back({w, end, (int)n});
+        w = end;
+    }
+    return out;
+}
+
 cudaError_t enqueue_step(mcao_sim* S, int* launches) {
     cudaError_t e;
     int nl = 0;
@@ -535,14 +572,15 @@ cudaError_t enqueue_step(mcao_sim* S, int* launches) {
         for (int w : g.wfs) ready[w] = ev;
     }
 
-    // science on s2 (low priority): after the block-per-subaperture sensors, so that it fills
-    // the SMs the first warp-per-subaperture launch leaves rather than racing it for them
-    {
+    // science on s2 (low priority): after the block-per-subaperture sensors, so that it fills the SMs that
+    // the first of several warp-per-subaperture launches leaves rather than racing it for them (39 m:
+    // 399 against 407 us a step).  A loop with one such launch ends about when the science does: there
+    // the science starts at once (20 m: 52.9 against 57.8 us).
+    if (S->tune.science_after_aux && sensing_groups(S).size() > 1) {
         cudaEvent_t after = nullptr;
         for (cudaEvent_t ev : ready)
             if (ev) after = ev;
-        if (S->tune.science_after_aux && after && (e = cudaStreamWaitEvent(S->s2, after, 0)) != cudaSuccess)
-            return e;
+        if (after && (e = cudaStreamWaitEvent(S->s2, after, 0)) != cudaSuccess) return e;
     }
     for (size_t q = 0; q < S->sci.size(); ++q) {
         SciLaunch L = make_sci_launch(S, (int)q);
@@ -556,35 +594,18 @@ cudaError_t enqueue_step(mcao_sim* S, int* launches) {
     cudaEvent_t ev_sci = dep_event(S, used);
     if ((e = cudaEventRecord(ev_sci, S->s2)) != cudaSuccess) return e;
 
-    // warp-per-subaperture sensors on s0: adjacent sensors of one shape share a launch as long as all
-    // their subapertures have a warp each at once.  20 m, three sensors of 1212: one launch takes
-    // PLACEHOLDER_M us, three in a row took 63 (a quarter of the GPU's warps each, so a launch lasts as
-    // long as one subaperture whatever their number).  39 m: 4632 subapertures fill the 4864 warps, and
-    // a launch each lets the product of one sensor run beside the sensing of the next.  A batch's
-    // product runs after every sensor, so there all adjacent sensors share a launch.
-    const long long wave = S->n_real > 1 ? (1LL << 40) : (long long)S->tune.sense_blocks_per_sm * S->sm_count * 8;
-    for (size_t w = 0; w < S->wfs.size();) {
-        const WfsHost& W = S->wfs[w];
-        if (W.fft_route || W.n_valid == 0) {
-            ++w;
-            continue;
-        }
-        size_t end = w + 1;
-        long long n = W.n_valid;
-        for (; end < S->wfs.size(); ++end) {
-            const WfsHost& V = S->wfs[end];
-            if (V.p.n_px != W.p.n_px || V.p.n_fft != W.p.n_fft || V.p.n_bin != W.p.n_bin || n + V.n_valid > wave) break;
-            n += V.n_valid;
-        }
+    // warp-per-subaperture sensors on s0
+    for (const SenseGroup& g : sensing_groups(S)) {
+        const WfsHost& W = S->wfs[g.first];
         slot = prof_begin(S, ST_WFS_MAIN, S->s0);
-        if ((e = launch_wfs(make_wfs_launch(S, W.d_subaps, (int)n, S->d_work + w), W.p.n_px, W.p.n_fft, W.p.n_bin, S->s0)) !=
-            cudaSuccess)
+        if ((e = launch_wfs(make_wfs_launch(S, W.d_subaps, g.n_subaps, S->d_work + g.first), W.p.n_px, W.p.n_fft, W.p.n_bin,
+                            S->s0)) != cudaSuccess)
             return e;
         prof_end(S, slot, S->s0);
         ++nl;
         cudaEvent_t ev = dep_event(S, used);
         if ((e = cudaEventRecord(ev, S->s0)) != cudaSuccess) return e;
-        for (; w < end; ++w) ready[w] = ev;
+        for (size_t w = g.first; w < g.end; ++w) ready[w] = ev;
     }
 
     if (S->n_real > 1) {
@@ -713,6 +734,31 @@ mcao_status build_graph(mcao_sim* S) {
     return MCAO_OK;
 }
 
+// Asynchronous calls (steps, readouts) queue their work on the caller's stream when one is set: what
+// follows there needs no wait between streams, and s0 is ordered behind it by an event that nothing on
+// the caller's stream waits for.  Otherwise they queue it on s0.  s0_pending: s0 may hold work that the
+// caller's stream is not ordered behind yet.
+mcao_status begin_async(mcao_sim* S, cudaStream_t* q) {
+    *q = S->user_set ? S->user : S->s0;
+    if (S->user_set && S->s0_pending) {
+        CK(cudaEventRecord(S->ev_user, S->s0));
+        CK(cudaStreamWaitEvent(S->user, S->ev_user, 0));
+        S->s0_pending = false;
+    }
+    return MCAO_OK;
+}
+
+mcao_status end_async(mcao_sim* S) {
+    if (!S->user_set) {
+        S->s0_pending = true;
+        return MCAO_OK;
+    }
+    CK(cudaEventRecord(S->ev_done, S->user));
+    CK(cudaStreamWaitEvent(S->s0, S->ev_done, 0));
+    return MCAO_OK;
+}
+
+// the same order for calls that queue on s0
 mcao_status order_after_user(mcao_sim* S) {
     if (!S->user_set) return MCAO_OK;
     CK(cudaEventRecord(S->ev_user, S->user));
@@ -721,20 +767,24 @@ mcao_status order_after_user(mcao_sim* S) {
 }
 
 mcao_status signal_user(mcao_sim* S) {
+    S->s0_pending = true;
     if (!S->user_set) return MCAO_OK;
     CK(cudaEventRecord(S->ev_done, S->s0));
     CK(cudaStreamWaitEvent(S->user, S->ev_done, 0));
     return MCAO_OK;
 }
 
+// Waits for all queued work.  Every step's and call's branches join s0 (s1 to s3 only carry work while a
+// step is captured into its graph), so s0 and the readout stream are all there is to wait for.
 mcao_status sync_all(mcao_sim* S) {
-    for (cudaStream_t st : {S->s0, S->s1, S->s2, S->s3}) CK(cudaStreamSynchronize(st));
+    CK(cudaStreamSynchronize(S->s0));
+    S->s0_pending = false;
     if (S->s_read) CK(cudaStreamSynchronize(S->s_read));
-    if (S->d_err) {
-        int e = 0;
-        CK(cudaMemcpy(&e, S->d_err, sizeof(int), cudaMemcpyDeviceToHost));
+    if (S->h_err) {
+        volatile int* flag = S->h_err;   // written by the device before the wait above returned
+        const int e = *flag;
         if (e != 0) {
-            CK(cudaMemsetAsync(S->d_err, 0, sizeof(int), S->s0));
+            *flag = 0;
             return fail(S, MCAO_E_TIMEOUT, "a bounded device wait gave up (code %d): results of the last steps are invalid",
                         e);
         }
@@ -761,7 +811,9 @@ void destroy_all(mcao_sim* S) {
     S->d_layer_owned.clear();
     dfree(S->d_dm_desc); dfree(S->d_dm_g); dfree(S->d_dm_band); dfree(S->d_dm_map);
     dfree(S->d_dm_surf); dfree(S->d_views); dfree(S->d_R); dfree(S->d_chunks); dfree(S->d_rscale); dfree(S->d_c); dfree(S->d_partial);
-    dfree(S->d_st); dfree(S->d_acc); dfree(S->d_err); dfree(S->d_work); dfree(S->d_sr_out);
+    dfree(S->d_st); dfree(S->d_acc); dfree(S->d_work); dfree(S->d_psf_out);
+    if (S->h_err) cudaFreeHost(S->h_err);
+    dfree(S->d_sr_out);
     dfree(S->d_Rrm);
     dfree(S->d_c_prev); dfree(S->d_dc_prev); dfree(S->d_dc);
     tc_destroy(S->tc);
@@ -830,6 +882,18 @@ mcao_status validate_config(const mcao_config* c) {
     return MCAO_OK;
 }
 
+// device address of a page-locked host buffer (false: any other memory, or one not aligned to its type)
+template <class T>
+static bool mapped(T* host, T*& dev) {
+    cudaPointerAttributes a{};
+    if (cudaPointerGetAttributes(&a, host) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    dev = static_cast<T*>(a.devicePointer);
+    return a.type == cudaMemoryTypeHost && dev != nullptr && reinterpret_cast<uintptr_t>(dev) % sizeof(T) == 0;
+}
+
 mcao_status d2h(mcao_sim* S, void* dst, const void* src, size_t bytes) {
     CK(cudaSetDevice(S->device));
     mcao_status r = sync_all(S);
@@ -891,8 +955,9 @@ mcao_status mcao_sim_create(const mcao_config* cfg, mcao_sim** out) {
     CKC(wfs_prepare());
     CKC(recon_prepare());
     CKC(multi_prepare());
-    CKC(dalloc(&S->d_err, 1));
-    CKC(cudaMemsetAsync(S->d_err, 0, sizeof(int), S->s0));
+    CKC(cudaHostAlloc((void**)&S->h_err, sizeof(int), cudaHostAllocMapped));
+    *S->h_err = 0;
+    CKC(cudaHostGetDevicePointer((void**)&S->d_err, S->h_err, 0));
     CKC(dalloc(&S->d_work, (size_t)(2 * cfg->n_wfs + 1)));
     CKC(cudaMemsetAsync(S->d_work, 0, sizeof(unsigned int) * (2 * cfg->n_wfs + 1), S->s0));
 
@@ -1099,6 +1164,7 @@ mcao_status mcao_set_stream(mcao_sim* S, void* stream) {
     if (!S) return MCAO_E_INVALID_ARG;
     S->user = (cudaStream_t)stream;
     S->user_set = true;
+    S->s0_pending = true;
     return MCAO_OK;
 }
 
@@ -1566,11 +1632,12 @@ mcao_status mcao_step(mcao_sim* S, int n_steps) {
         mcao_status r = build_graph(S);
         if (r != MCAO_OK) return r;
     }
-    mcao_status r = order_after_user(S);
+    cudaStream_t q = nullptr;
+    mcao_status r = begin_async(S, &q);
     if (r != MCAO_OK) return r;
     int i = 0;
     if (S->graph_k_steps > 1)
-        for (; i + S->graph_k_steps <= n_steps; i += S->graph_k_steps) CK(cudaGraphLaunch(S->exec_k, S->s0));
+        for (; i + S->graph_k_steps <= n_steps; i += S->graph_k_steps) CK(cudaGraphLaunch(S->exec_k, q));
     for (; i < n_steps; ++i) {
         if (S->profiling) {
             S->prof_step_begin.push_back(S->prof_records.size());
@@ -1590,9 +1657,9 @@ mcao_status mcao_step(mcao_sim* S, int n_steps) {
                 S->prof_records.push_back({p.stage, {ea, eb}});
             }
         }
-        CK(cudaGraphLaunch(S->exec, S->s0));
+        CK(cudaGraphLaunch(S->exec, q));
     }
-    return signal_user(S);
+    return end_async(S);
 }
 
 mcao_status mcao_step_group(mcao_sim* const* sims, int n_sims, int n_steps) {
@@ -2213,13 +2280,16 @@ mcao_status mcao_get_psf(mcao_sim* S, int sci, double* out, size_t n, double* sr
     if (sr_long) *sr_long = acc.n_sr ? acc.sr_sum / (double)acc.n_sr : 0.0;
     if (sr_last) *sr_last = acc.sr_last;
     if (out) {
-        std::vector<double> t(M * M);
-        r = d2h(S, t.data(), C.d_psf_t + (size_t)S->cur * M * M, sizeof(double) * M * M);
-        if (r != MCAO_OK) return r;
-        double norm = acc.n_psf ? 1.0 / ((double)acc.n_psf * C.sum_amp * C.sum_amp) : 0.0;
-        for (size_t j = 0; j < M; ++j)
-            for (size_t i = 0; i < M; ++i)
-                out[j * M + i] = t[((i + M / 2) % M) * M + (j + M / 2) % M] * norm;
+        const double norm = acc.n_psf ? 1.0 / ((double)acc.n_psf * C.sum_amp * C.sum_amp) : 0.0;
+        if (S->psf_out_n < M * M) {
+            dfree(S->d_psf_out);
+            S->psf_out_n = 0;
+            CK(dalloc(&S->d_psf_out, M * M));
+            S->psf_out_n = M * M;
+        }
+        CK(launch_psf_out(C.d_psf_t + (size_t)S->cur * M * M, C.M, norm, S->d_psf_out, S->s0));
+        CK(cudaStreamSynchronize(S->s0));
+        CK(cudaMemcpy(out, S->d_psf_out, sizeof(double) * M * M, cudaMemcpyDeviceToHost));
     }
     return MCAO_OK;
 }
@@ -2239,6 +2309,22 @@ mcao_status mcao_read_async(mcao_sim* S, float* commands, double* strehl) {
     if (commands && !S->dms_loaded) return fail(S, MCAO_E_STATE, "DMs not loaded");
     CK(cudaSetDevice(S->device));
     const int n_cmd = S->dms_loaded ? S->n_cmd : 0, n_sci = (int)S->sci.size();
+    const int nc = (commands && n_cmd > 0) ? n_cmd : 0, ns = strehl ? n_sci : 0;
+    cudaStream_t q = nullptr;
+    mcao_status r = begin_async(S, &q);
+    if (r != MCAO_OK) return r;
+    // page-locked buffers: the readout kernel writes them itself, in stream order.  (Through the ring the
+    // values took two copies on a third stream and two waits between streams more: 8 m step and
+    // readout 52 us, 26 us now, with the work on the caller's stream.)
+    float* host_c = nullptr;
+    double* host_s = nullptr;
+    if ((!nc || mapped(commands, host_c)) && (!ns || mapped(strehl, host_s))) {
+        if (S->ring_last >= 0) CK(cudaStreamWaitEvent(q, S->ring_free[S->ring_last], 0));   // earlier copies land first
+        S->ring_last = -1;
+        CK(launch_readout(S->d_c + (size_t)S->cur * std::max(n_cmd, 1), nc, S->d_acc + (size_t)S->cur * std::max(n_sci, 1), ns,
+                          host_c, host_s, q));
+        return end_async(S);
+    }
     if (S->ring_ncmd != n_cmd || S->ring_nsci != n_sci) {
         // (re)size the ring after every earlier read has completed
         if (S->s_read) CK(cudaStreamSynchronize(S->s_read));
@@ -2257,25 +2343,24 @@ mcao_status mcao_read_async(mcao_sim* S, float* commands, double* strehl) {
         S->ring_ncmd = n_cmd;
         S->ring_nsci = n_sci;
         S->ring_pos = 0;
+        S->ring_last = -1;
     }
-    mcao_status r = order_after_user(S);
-    if (r != MCAO_OK) return r;
     const int slot = S->ring_pos;
     S->ring_pos = (S->ring_pos + 1) % kReadRing;
     float* rc = S->d_ring_c + (size_t)slot * std::max(n_cmd, 1);
     double* rs = S->d_ring_s + (size_t)slot * 2 * std::max(n_sci, 1);
     // the slot's previous copy to the host is done before the snapshot overwrites it
-    if (S->ring_busy[slot]) CK(cudaStreamWaitEvent(S->s0, S->ring_free[slot], 0));
-    const int nc = (commands && n_cmd > 0) ? n_cmd : 0, ns = strehl ? n_sci : 0;
+    if (S->ring_busy[slot]) CK(cudaStreamWaitEvent(q, S->ring_free[slot], 0));
     CK(launch_readout(S->d_c + (size_t)S->cur * std::max(n_cmd, 1), nc, S->d_acc + (size_t)S->cur * std::max(n_sci, 1),
-                      ns, rc, rs, S->s0));
-    CK(cudaEventRecord(S->ring_ready[slot], S->s0));
+                      ns, rc, rs, q));
+    CK(cudaEventRecord(S->ring_ready[slot], q));
     CK(cudaStreamWaitEvent(S->s_read, S->ring_ready[slot], 0));
     if (nc) CK(cudaMemcpyAsync(commands, rc, sizeof(float) * nc, cudaMemcpyDeviceToHost, S->s_read));
     if (ns) CK(cudaMemcpyAsync(strehl, rs, sizeof(double) * 2 * ns, cudaMemcpyDeviceToHost, S->s_read));
     CK(cudaEventRecord(S->ring_free[slot], S->s_read));
     S->ring_busy[slot] = 1;
-    r = signal_user(S);
+    S->ring_last = slot;
+    r = end_async(S);
     if (r != MCAO_OK) return r;
     // work queued on the caller's stream afterwards also sees the host copies
     if (S->user_set) CK(cudaStreamWaitEvent(S->user, S->ring_free[slot], 0));

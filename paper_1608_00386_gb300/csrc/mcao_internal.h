@@ -16,7 +16,7 @@ constexpr int kMaxEntries = 16;   // layers + DMs sampled along one direction
 struct Tuning {
     int sense_blocks_per_sm = 4;    // warp-per-subaperture sensing: grid cap, blocks per SM
     int recon_ctas_pct = 85;        // reconstructor slices: blocks per SM x 100
-    int science_after_aux = 1;      // science waits for the block-per-subaperture sensors
+    int science_after_aux = 1;      // with several sensing launches, science waits for the block-per-subaperture sensors
     int tc_chunk = 8;               // tensor-core product: k-blocks per TMEM accumulator
     int multi_blocks_per_sm = 2;    // batched float32 product: blocks per SM
     int steps_per_graph = 1;        // steps captured in one graph launch (stage profiler off)
@@ -363,6 +363,9 @@ cudaError_t launch_strehl_out(const SciAcc* acc, int n_sci, double* out, cudaStr
 // science direction q (n_cmd or n_sci may be 0)
 cudaError_t launch_readout(const float* c, int n_cmd, const SciAcc* acc, int n_sci, float* ring_c, double* ring_s,
                            cudaStream_t s);
+
+// PSF accumulator (transposed, unshifted) into image order, times norm
+cudaError_t launch_psf_out(const double* psf_t, int M, double norm, double* out, cudaStream_t s);
 
 // twiddles of a science FFT of size M in the layout its kernels read (stage-major for the sizes
 // with a compile-time transform, exp(-2 pi i m / M) otherwise)
