@@ -8,9 +8,9 @@
 // the screen is Re sum_k c_k exp(+2 pi i k x / n) (an unnormalized inverse DFT), computed as
 // the real part of the forward DFT of conj(c).  (z_c, z_s) is the Box-Muller pair of the
 // detector-noise sampler drawn from Philox4x32-10 with counter (index, 0, 0, 1), key = seed.
-// Two passes of row FFTs in shared memory, each storing its result transposed: the first
-// generates its rows of coefficients in place (no coefficient array in HBM), the second keeps
-// the real part.
+// The powers of two from 256 on take half-spectrum passes (screen_pass below); other sizes two
+// passes of row FFTs in shared memory, each storing its result transposed: the first generates its
+// rows of coefficients in place (no coefficient array in HBM), the second keeps the real part.
 #include "device_common.cuh"
 #include "mcao_internal.h"
 
@@ -36,30 +36,6 @@ __global__ void screen_twiddle_kernel(int n, float2* W) {
     }
 }
 
-// Twiddle table of the compile-time transform laid out stage by stage, so that a warp's
-// butterflies (consecutive k) read consecutive entries: for the stage of sub-length ns and
-// radix R, entry off + (r - 1) ns + k = exp(-2 pi i r k / (ns R)), r = 1 .. R-1, k < ns (the
-// same float values as the single table exp(-2 pi i m / N) at m = r k N / (ns R)).
-template <int N>
-__global__ void screen_stage_twiddles(float2* T) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    int off = 0, ns = 1;
-    while (ns < N) {
-        const int R = ct_radix(N / ns);
-        const int cnt = ns * (R - 1);
-        if (e < off + cnt) {
-            const int q = e - off, r = q / ns + 1, k = q - (r - 1) * ns;
-            const int m = (r * k * (N / (ns * R))) % N;
-            double sn, cs;
-            sincospi(-2.0 * (double)m / (double)N, &sn, &cs);
-            T[e] = make_float2((float)cs, (float)sn);
-            return;
-        }
-        off += cnt;
-        ns *= R;
-    }
-}
-
 struct ScreenPass {
     int n, rows;
     // first pass: coefficients generated in place (amp0 = sqrt(0.023 r0^-5/3) / (n pixel), frequencies
@@ -76,26 +52,42 @@ struct ScreenPass {
     int n_radices;
 };
 
-// conj(c_k) of coefficient k = ky n + kx: a_k (z_c - i z_s), a_k = amp0 (kx'^2 + ky'^2 + l2)^(-11/12)
-// (the spectrum in cell units), Box-Muller pair of Philox words 0, 1 at counter (k, 0, 0, 1)
-__device__ __forceinline__ float2 screen_coeff(int n, int kx, int ky, float amp0, float l2, uint32_t key0,
-                                               uint32_t key1) {
-    const uint32_t k = (uint32_t)ky * (uint32_t)n + (uint32_t)kx;
-    uint32_t w[4] = {k, 0u, 0u, 1u};
+// (z_c, z_s) of coefficient k = ky n + kx: Box-Muller pair of Philox words 0, 1 at counter (k, 0, 0, 1)
+__device__ __forceinline__ float2 screen_normals(int n, int kx, int ky, uint32_t key0, uint32_t key1) {
+    uint32_t w[4] = {(uint32_t)ky * (uint32_t)n + (uint32_t)kx, 0u, 0u, 1u};
     philox4x32_10(w, key0, key1);
-    float zc, zs;
-    nz_box_muller2(nz_uniform(w[0]), nz_uniform(w[1]), zc, zs);
-    const float sx = (float)(kx <= (n - 1) / 2 ? kx : kx - n);
-    const float sy = (float)(ky <= (n - 1) / 2 ? ky : ky - n);
-    const float a = (kx == 0 && ky == 0) ? 0.0f : amp0 * exp2f(-11.0f / 12.0f * log2f(sx * sx + sy * sy + l2));
-    return make_float2(zc * a, -zs * a);
+    float2 z;
+    nz_box_muller2(nz_uniform(w[0]), nz_uniform(w[1]), z.x, z.y);
+    return z;
 }
 
-// NCT > 0: the transform length is NCT, known at compile time (constant index arithmetic)
-template <bool GEN, int NCT>
+// a_k = amp0 x^(-11/12), x = kx'^2 + ky'^2 + l2 (the spectrum in cell units), 0 at DC; a_-k = a_k.  With
+// x = 2^e m the power of two leaves the logarithm, whose rounding at the size of log2(x) would otherwise
+// be most of the screen's error: 2^(-11 e / 12) = 2^i 2^(k / 12), the rest an exponent within (-1, 1).
+__device__ __forceinline__ float screen_amp(int n, int kx, int ky, float amp0, float l2) {
+    const float sx = (float)(kx <= (n - 1) / 2 ? kx : kx - n);
+    const float sy = (float)(ky <= (n - 1) / 2 ? ky : ky - n);
+    const float x = sx * sx + sy * sy + l2;
+    if ((kx == 0 && ky == 0) || !(x < 3.0e38f)) return 0.0f;
+    const uint32_t b = __float_as_uint(x);   // x >= 1 away from DC
+    const int q = 11 * (127 - (int)(b >> 23)) + 12 * 128, i = q / 12, k = q - 12 * i;
+    const float m = __uint_as_float((b & 0x007fffffu) | 0x3f800000u);
+    const float f = exp2f(fmaf(-11.0f / 12.0f, log2f(m), (float)k * (1.0f / 12.0f)));
+    return amp0 * f * __uint_as_float((uint32_t)(i - 1) << 23);   // 2^(i - 128)
+}
+
+// conj(c_k) = a_k (z_c - i z_s)
+__device__ __forceinline__ float2 screen_coeff(int n, int kx, int ky, float amp0, float l2, uint32_t key0,
+                                               uint32_t key1) {
+    const float2 z = screen_normals(n, kx, ky, key0, key1);
+    const float a = screen_amp(n, kx, ky, amp0, l2);
+    return make_float2(z.x * a, -z.y * a);
+}
+
+template <bool GEN>
 __global__ void __launch_bounds__(kScreenThreads) screen_fft_pass(ScreenPass P) {
     extern __shared__ float4 smem_raw[];
-    const int n = NCT > 0 ? NCT : P.n, rows = NCT > 0 ? screen_rows(NCT) : P.rows;
+    const int n = P.n, rows = P.rows;
     float2* A = reinterpret_cast<float2*>(smem_raw);
     float2* B = A + rows * n;
     float2* W = B + rows * n;
@@ -112,9 +104,7 @@ __global__ void __launch_bounds__(kScreenThreads) screen_fft_pass(ScreenPass P) 
         A[q] = v;
     }
     __syncthreads();
-    const float2* R;
-    if constexpr (NCT > 0) R = fft_tab<NCT>(A, B, rows, W, tid, nthr);
-    else R = stockham_fft(A, B, n, P.radices, P.n_radices, rows, n, 1, W, tid, nthr);
+    const float2* R = stockham_fft(A, B, n, P.radices, P.n_radices, rows, n, 1, W, tid, nthr);
     for (int q = tid; q < rows * n; q += nthr) {
         const int c = q / rows, r = q - c * rows;
         if (row0 + r >= n) continue;
@@ -124,28 +114,241 @@ __global__ void __launch_bounds__(kScreenThreads) screen_fft_pass(ScreenPass P) 
     }
 }
 
+// ------------------------------------------------------------------------------------------
+// powers of two: half-spectrum passes with register transforms
+// ------------------------------------------------------------------------------------------
+// The screen is real, so it is the transform of the Hermitian half D_k = conj(c_k + conj(c_-k)) / 2:
+//   pass 1: rows ky = 0 .. n/2 of D, generated in registers, transformed along kx, G[ky][x];
+//   pass 2: per pair of columns x, the transform along ky of G[.][x] + i G[.][x + 1] (rows above n/2 from
+//   the Hermitian symmetry), whose real and imaginary parts are the two columns of the screen.
+// Half the transforms and half the intermediate bytes of transforming c and keeping the real part.
+// A transform of N points takes N / 16 threads with 16 points each in registers: radix 16, radix 16,
+// radix N / 256, with one exchange through shared memory between (rows padded by one entry in 16, so
+// that the first exchange's stride of 16 meets every bank); the first stage's inputs are generated or
+// read straight into the registers and the last stage's outputs stored from them.  Twiddles are
+// formed by the block.  The passes are bound by the instructions of the two Philox draws and
+// Box-Muller pairs per coefficient (pass 1) and by shared memory and the L2 gathers (pass 2).
+// 2048 x 2048: 38 + 19 us; six radix-4 exchanges of the full spectrum and a
+// twiddle kernel took 55 + 40 + 7 us.
+__device__ __forceinline__ float2 rot4(float2 a) { return make_float2(a.y, -a.x); }   // -i a
+
+// forward 4-point transform of v[0], v[s], v[2 s], v[3 s], in place
+template <int S>
+__device__ __forceinline__ void dft4(float2* v) {
+    const float2 a = cadd(v[0], v[2 * S]), b = csub(v[0], v[2 * S]);
+    const float2 c = cadd(v[S], v[3 * S]), d = rot4(csub(v[S], v[3 * S]));
+    v[0] = cadd(a, c);
+    v[S] = cadd(b, d);
+    v[2 * S] = csub(a, c);
+    v[3 * S] = csub(b, d);
+}
+
+// forward R-point transform of v[0], v[S], .. v[(R - 1) S], in place and in natural order
+template <int R, int S>
+__device__ __forceinline__ void dft_reg(float2* v) {
+    if constexpr (R == 2) {
+        const float2 a = v[0];
+        v[0] = cadd(a, v[S]);
+        v[S] = csub(a, v[S]);
+    } else if constexpr (R == 4) {
+        dft4<S>(v);
+    } else if constexpr (R == 8) {
+        // 2 x 4: transforms of the even and odd points, then butterflies
+        dft4<2 * S>(v);
+        dft4<2 * S>(v + S);
+        const float h = 0.707106781186547524f;
+        float2 o[4] = {v[S], v[3 * S], v[5 * S], v[7 * S]}, e[4] = {v[0], v[2 * S], v[4 * S], v[6 * S]};
+        o[1] = make_float2(h * (o[1].x + o[1].y), h * (o[1].y - o[1].x));
+        o[2] = rot4(o[2]);
+        o[3] = make_float2(h * (o[3].y - o[3].x), -h * (o[3].x + o[3].y));
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            v[b * S] = cadd(e[b], o[b]);
+            v[(b + 4) * S] = csub(e[b], o[b]);
+        }
+    } else if constexpr (R == 16) {
+        // 4 x 4: out[b + 4 c] = sum_a w16^(a b) w4^(a c) X_a[b], X_a the transform of points a, a + 4, ..
+        const float c1 = 0.923879532511286756f, s1 = 0.382683432365089772f, h = 0.707106781186547524f;
+#pragma unroll
+        for (int a = 0; a < 4; ++a) dft4<4 * S>(v + a * S);
+        const float2 w[4][4] = {{{1, 0}, {1, 0}, {1, 0}, {1, 0}},
+                                {{1, 0}, {c1, -s1}, {h, -h}, {s1, -c1}},
+                                {{1, 0}, {h, -h}, {0, -1}, {-h, -h}},
+                                {{1, 0}, {s1, -c1}, {-h, -h}, {-c1, s1}}};
+#pragma unroll
+        for (int a = 1; a < 4; ++a)
+#pragma unroll
+            for (int b = 1; b < 4; ++b) v[(a + 4 * b) * S] = cmul(v[(a + 4 * b) * S], w[a][b]);
+#pragma unroll
+        for (int b = 0; b < 4; ++b) dft4<S>(v + 4 * b * S);   // over a; output c at 4 b + c
+        float2 t[16];
+#pragma unroll
+        for (int q = 0; q < 16; ++q) t[q] = v[q * S];
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) v[(b + 4 * c) * S] = t[4 * b + c];
+    }
+}
+
+// NF transforms per block
+template <int N, int NF>
+struct HalfFft {
+    static constexpr int T = N / 16;                       // threads per transform
+    static constexpr int R3 = N / 256;                     // last stage's radix
+    static constexpr int F = NF;
+    static constexpr int kThreads = T * F;
+    static constexpr int kRow = N + N / 16;                // padded row in shared memory
+    static constexpr int kTw = 15 * 16 + (R3 - 1) * 256;   // twiddles of stages 2 and 3
+    static constexpr size_t smem = sizeof(float2) * ((size_t)F * kRow + kTw);
+};
+__device__ __forceinline__ int fft_pad(int i) { return i + (i >> 4); }
+
+template <int N>
+__device__ __forceinline__ void half_twiddles(float2* tw, int tid, int nthr) {
+    for (int e = tid; e < HalfFft<N, 1>::kTw; e += nthr) {
+        // stage 2: entry (r - 1) 16 + k, angle r k / 256; stage 3: (r - 1) 256 + k, angle r k / N
+        const int q = e < 240 ? e : e - 240, ns = e < 240 ? 16 : 256;
+        const int r = q / ns + 1, k = q % ns;
+        float sn, cs;
+        sincospif(-2.0f * (float)(r * k) / (e < 240 ? 256.0f : (float)N), &sn, &cs);
+        tw[e] = make_float2(cs, sn);
+    }
+}
+
+// Transform of the 16 points v[m] = in[t + m T] of this thread; on return v[q + r (16 / R3)] is output
+// t + q T + 256 r (q < 16 / R3, r < R3).  row: the transform's shared memory.  Every thread of the block
+// calls it.
+template <int N>
+__device__ __forceinline__ void half_fft(float2 (&v)[16], float2* row, const float2* tw, int t) {
+    using H = HalfFft<N, 1>;
+    constexpr int Q = 16 / H::R3;
+    dft_reg<16, 1>(v);
+#pragma unroll
+    for (int r = 0; r < 16; ++r) row[fft_pad(16 * t + r)] = v[r];
+    __syncthreads();   // also covers the twiddles
+#pragma unroll
+    for (int m = 0; m < 16; ++m) v[m] = row[fft_pad(t + m * H::T)];
+    const int k = t & 15;
+#pragma unroll
+    for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], tw[(r - 1) * 16 + k]);
+    dft_reg<16, 1>(v);
+    if constexpr (H::R3 > 1) {
+        __syncthreads();
+        const int base = (t >> 4) * 256 + k;
+#pragma unroll
+        for (int r = 0; r < 16; ++r) row[fft_pad(base + 16 * r)] = v[r];
+        __syncthreads();
+#pragma unroll
+        for (int m = 0; m < 16; ++m) v[m] = row[fft_pad(t + m * H::T)];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+#pragma unroll
+            for (int r = 1; r < H::R3; ++r) v[q + r * Q] = cmul(v[q + r * Q], tw[240 + (r - 1) * 256 + t + q * H::T]);
+            dft_reg<H::R3, Q>(v + q);
+        }
+    } else {
+        // 256 points: stage 2 is the last; its output r of butterfly t is t + 16 r = t + T r
+    }
+}
+
+template <int N, int NF>
+__global__ void __launch_bounds__(HalfFft<N, NF>::kThreads) screen_half_rows(ScreenPass P) {
+    using H = HalfFft<N, NF>;
+    extern __shared__ float4 smem_raw[];
+    float2* tw = reinterpret_cast<float2*>(smem_raw);
+    const int f = threadIdx.x / H::T, t = threadIdx.x % H::T;
+    float2* row = tw + H::kTw + f * H::kRow;
+    const int ky = min((int)blockIdx.x * H::F + f, N / 2);   // a block's spare transforms repeat the last row
+    half_twiddles<N>(tw, threadIdx.x, H::kThreads);
+    float2 v[16];
+    const int my = (N - ky) % N;
+#pragma unroll 2
+    for (int m = 0; m < 16; ++m) {
+        const int kx = t + m * H::T, mx = (N - kx) % N;
+        const float2 z = screen_normals(N, kx, ky, P.key0, P.key1), y = screen_normals(N, mx, my, P.key0, P.key1);
+        const float a = 0.5f * screen_amp(N, kx, ky, P.amp0, P.l2);
+        row[fft_pad(kx)] = make_float2(a * (z.x + y.x), a * (y.y - z.y));   // conj(c_k + conj(c_-k)) / 2
+    }
+    // the thread's own entries back into registers (kept out of them while they are drawn)
+#pragma unroll
+    for (int m = 0; m < 16; ++m) v[m] = row[fft_pad(t + m * H::T)];
+    __syncthreads();
+    half_fft<N>(v, row, tw, t);
+    float2* out = P.dst_c + (size_t)ky * N;
+    constexpr int Q = H::R3 > 1 ? 16 / H::R3 : 1;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        const int o = H::R3 > 1 ? t + (i % Q) * H::T + 256 * (i / Q) : t + 16 * i;
+        out[o] = v[i];
+    }
+}
+
+template <int N, int NF>
+__global__ void __launch_bounds__(HalfFft<N, NF>::kThreads) screen_half_cols(ScreenPass P) {
+    using H = HalfFft<N, NF>;
+    extern __shared__ float4 smem_raw[];
+    float2* tw = reinterpret_cast<float2*>(smem_raw);
+    // neighbouring threads take neighbouring column pairs
+    const int f = threadIdx.x % H::F, t = threadIdx.x / H::F;
+    float2* row = tw + H::kTw + f * H::kRow;
+    const int x = 2 * (blockIdx.x * H::F + f);
+    half_twiddles<N>(tw, threadIdx.x, H::kThreads);
+    float2 v[16];
+#pragma unroll
+    for (int m = 0; m < 16; ++m) {
+        const int ky = t + m * H::T;
+        const bool up = ky > N / 2;
+        const float4 g = *reinterpret_cast<const float4*>(P.src + (size_t)(up ? N - ky : ky) * N + x);
+        v[m] = up ? make_float2(g.x + g.w, g.z - g.y) : make_float2(g.x - g.w, g.y + g.z);
+    }
+    half_fft<N>(v, row, tw, t);
+    constexpr int Q = H::R3 > 1 ? 16 / H::R3 : 1;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        const int o = H::R3 > 1 ? t + (i % Q) * H::T + 256 * (i / Q) : t + 16 * i;
+        *reinterpret_cast<float2*>(P.dst_r + (size_t)o * N + x) = v[i];
+    }
+}
+
 }  // namespace
 
 size_t screen_fft_smem(int n) { return sizeof(float2) * (2 * (size_t)screen_rows(n) * n + n); }
 
 namespace {
 
-template <int NCT>
-cudaError_t screen_passes(ScreenPass P, unsigned blocks, cudaStream_t s) {
+cudaError_t screen_passes(ScreenPass P, cudaStream_t s) {
     const size_t bytes = screen_fft_smem(P.n);
-    cudaError_t e = cudaFuncSetAttribute(screen_fft_pass<true, NCT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)bytes);
+    cudaError_t e = cudaFuncSetAttribute(screen_fft_pass<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(screen_fft_pass<false, NCT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        e = cudaFuncSetAttribute(screen_fft_pass<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
+    const unsigned blocks = (unsigned)((P.n + P.rows - 1) / P.rows);
     float2* work = P.dst_c;
     float* out = P.dst_r;
     P.dst_r = nullptr;
-    screen_fft_pass<true, NCT><<<blocks, kScreenThreads, bytes, s>>>(P);
+    screen_fft_pass<true><<<blocks, kScreenThreads, bytes, s>>>(P);
     P.src = work;
     P.dst_c = nullptr;
     P.dst_r = out;
-    screen_fft_pass<false, NCT><<<blocks, kScreenThreads, bytes, s>>>(P);
+    screen_fft_pass<false><<<blocks, kScreenThreads, bytes, s>>>(P);
+    return cudaGetLastError();
+}
+
+template <int N>
+cudaError_t half_passes(ScreenPass P, cudaStream_t s) {
+    // rows: two transforms per block (four at 256), so that small screens spread over the SMs; columns:
+    // four, so that a block stores whole 32-byte sectors, where their shared memory leaves two blocks per SM
+    using A = HalfFft<N, N == 256 ? 4 : 2>;
+    using B = HalfFft<N, N == 4096 ? 2 : 4>;
+    const auto rows = screen_half_rows<N, A::F>;
+    const auto cols = screen_half_cols<N, B::F>;
+    cudaError_t e = cudaFuncSetAttribute(rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)A::smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(cols, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B::smem);
+    if (e != cudaSuccess) return e;
+    rows<<<(N / 2 + 1 + A::F - 1) / A::F, A::kThreads, A::smem, s>>>(P);
+    P.src = P.dst_c;
+    cols<<<N / 2 / B::F, B::kThreads, B::smem, s>>>(P);
     return cudaGetLastError();
 }
 
@@ -153,15 +356,6 @@ cudaError_t screen_passes(ScreenPass P, unsigned blocks, cudaStream_t s) {
 
 cudaError_t launch_screen(int n, double pixel, double r0, double L0, unsigned long long seed, const int* radices,
                           int n_radices, float2* work, float2* W, float* out, cudaStream_t s) {
-    // twiddles: stage-major for the compile-time sizes, the plain table otherwise
-    switch (n) {
-        case 256: screen_stage_twiddles<256><<<1, 256, 0, s>>>(W); break;
-        case 512: screen_stage_twiddles<512><<<2, 256, 0, s>>>(W); break;
-        case 1024: screen_stage_twiddles<1024><<<4, 256, 0, s>>>(W); break;
-        case 2048: screen_stage_twiddles<2048><<<8, 256, 0, s>>>(W); break;
-        case 4096: screen_stage_twiddles<4096><<<16, 256, 0, s>>>(W); break;
-        default: screen_twiddle_kernel<<<(n + 255) / 256, 256, 0, s>>>(n, W);
-    }
     ScreenPass P{};
     P.n = n;
     P.rows = screen_rows(n);
@@ -175,15 +369,16 @@ cudaError_t launch_screen(int n, double pixel, double r0, double L0, unsigned lo
     for (int i = 0; i < n_radices && i < 16; ++i) P.radices[i] = radices[i];
     P.dst_c = work;
     P.dst_r = out;
-    const unsigned blocks = (unsigned)((n + P.rows - 1) / P.rows);
-    switch (n) {   // the power-of-two sizes get compile-time transforms
-        case 256: return screen_passes<256>(P, blocks, s);
-        case 512: return screen_passes<512>(P, blocks, s);
-        case 1024: return screen_passes<1024>(P, blocks, s);
-        case 2048: return screen_passes<2048>(P, blocks, s);
-        case 4096: return screen_passes<4096>(P, blocks, s);
-        default: return screen_passes<0>(P, blocks, s);
+    // the half-spectrum passes store pairs of columns, so they need an 8-byte aligned screen
+    if (reinterpret_cast<uintptr_t>(out) % 8 == 0) switch (n) {
+        case 256: return half_passes<256>(P, s);
+        case 512: return half_passes<512>(P, s);
+        case 1024: return half_passes<1024>(P, s);
+        case 2048: return half_passes<2048>(P, s);
+        case 4096: return half_passes<4096>(P, s);
     }
+    screen_twiddle_kernel<<<(n + 255) / 256, 256, 0, s>>>(n, W);
+    return screen_passes(P, s);
 }
 
 }  // namespace mcao
