@@ -26,6 +26,7 @@
 // turns; rings above 96 KB keep the science kernels off the SM and slow the step.  Every mbarrier wait is bounded
 // (about one second of clock); on expiry the warp records kErrReconTimeout, waits (bounded)
 // for its copies in flight and exits.
+#include "bulk_copy.cuh"
 #include "mcao_internal.h"
 
 namespace mcao {
@@ -61,7 +62,6 @@ constexpr int kTmaRows = kReconRows;               // rows per item
 constexpr int kTmaSeg = kReconSeg;                 // 16-byte vectors per row segment (2 KB)
 constexpr int kTmaStages = 2;
 constexpr int kTmaChunks = 32;
-constexpr long long kWaitCycles = 2000000000ll;    // ~1 s at 2 GHz
 
 struct TmaSmem {
     uint4 ring[kTmaWarps][kTmaStages][kTmaRows * kTmaSeg];
@@ -69,52 +69,6 @@ struct TmaSmem {
     int item[kTmaWarps][kTmaStages];  // item whose first stage the slot holds; -1: no more items
     ReconChunk chunk[kTmaChunks];     // the launch's first chunks (the others are read where they are)
 };
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(unsigned long long* bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive_expect_tx(unsigned long long* bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-                 : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(unsigned long long* bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// wait for the given phase parity, giving up after kWaitCycles
-__device__ __forceinline__ bool mbar_wait_bounded(unsigned long long* bar, uint32_t parity) {
-    if (mbar_try_wait(bar, parity)) return true;
-    const long long t0 = clock64();
-    while (!mbar_try_wait(bar, parity))
-        if (clock64() - t0 > kWaitCycles) return false;
-    return true;
-}
-
-__device__ __forceinline__ uint64_t evict_first_policy() {
-    uint64_t pol;
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-    return pol;
-}
-
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, unsigned long long* bar,
-                                         uint64_t pol) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
-        ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)), "l"(pol)
-        : "memory");
-}
 
 // stage geometry of chunk kc of a slice: n4 16-byte vectors per row, nst stages of kTmaSeg
 // vectors (the last one shorter)
@@ -475,40 +429,7 @@ __global__ void recon_reduce_kernel(ReduceLaunch L) {
     reduce_row(L, t >> 3, (int)(t & 7), n_rows);
 }
 
-// transpose of a row-major float32 [rows][cols] into [cols][ld_out] (float32 or bfloat16),
-// 32 x 32 tiles through shared memory
-template <bool BF16>
-__global__ void transpose_kernel(const float* __restrict__ src, int rows, int cols, void* out, int ld_out) {
-    __shared__ float tile[32][33];
-    const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int r = r0 + i, c = c0 + threadIdx.x;
-        tile[i][threadIdx.x] = (r < rows && c < cols) ? src[(long long)r * cols + c] : 0.0f;
-    }
-    __syncthreads();
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int c = c0 + i, r = r0 + threadIdx.x;
-        if (c < cols && r < ld_out) {
-            const float v = tile[threadIdx.x][i];
-            if (BF16) {
-                uint32_t h = f32x2_to_bf16x2(v, 0.0f) & 0xffffu;
-                reinterpret_cast<uint16_t*>(out)[(long long)c * ld_out + r] = (uint16_t)h;
-            } else {
-                reinterpret_cast<float*>(out)[(long long)c * ld_out + r] = v;
-            }
-        }
-    }
-}
-
 }  // namespace
-
-cudaError_t launch_transpose(const float* src, int rows, int cols, void* out, int ld_out, int bf16, cudaStream_t st) {
-    if (rows <= 0 || cols <= 0) return cudaSuccess;
-    dim3 grid((unsigned)((cols + 31) / 32), (unsigned)((ld_out + 31) / 32)), block(32, 8);
-    if (bf16) transpose_kernel<true><<<grid, block, 0, st>>>(src, rows, cols, out, ld_out);
-    else transpose_kernel<false><<<grid, block, 0, st>>>(src, rows, cols, out, ld_out);
-    return cudaGetLastError();
-}
 
 void recon_slice_chunks(const ReconLaunch& L, std::vector<ReconChunk>& out) {
     const int epv = 16 / recon_esize(L.dtype);

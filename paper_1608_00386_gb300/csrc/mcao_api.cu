@@ -168,7 +168,7 @@ struct mcao_sim {
     float* d_c_prev = nullptr;            // [n_real][n_cmd]
     float* d_dc_prev = nullptr;           // [n_real][n_cmd]
     float* d_dc = nullptr;                // [n_real][n_cmd] batched update (controller on)
-    // batched product (n_real > 1).  float32 R: column-major [ld][rows_pad] copy streamed by the
+    // batched product (n_real > 1).  float32 R: a copy in blocks of 128 rows streamed by the
     // CUDA-core product in groups of kMultiRhs realizations; bfloat16 R: the tensor-core product
     // (its own bfloat16 copy, split slopes and partials)
     float* d_Rrm = nullptr;
@@ -497,8 +497,7 @@ cudaError_t enqueue_batched_product(mcao_sim* S, int n, float alpha, float beta,
     }
     MultiLaunch M{};
     M.R = S->d_Rrm;
-    M.bf16 = 0;
-    M.rows_pad = S->rows_pad;
+    M.err = S->d_err;
     M.n_cmd = S->n_cmd;
     M.K = S->ld;
     M.s_t = S->d_multi_st;
@@ -1490,7 +1489,7 @@ mcao_status mcao_load_reconstructor(mcao_sim* S, int n_cmd, int n_slopes, const 
                                   sizeof(float) * len, n_cmd, kind, S->s0);
     }
     if (S->n_real > 1) {
-        // batched product: float32 R column-major for the CUDA-core product, or the tensor-core
+        // batched product: float32 R in row blocks for the CUDA-core product, or the tensor-core
         // product's bfloat16 copy
         dfree(S->d_Rrm);
         dfree(S->d_multi_st);
@@ -1499,10 +1498,9 @@ mcao_status mcao_load_reconstructor(mcao_sim* S, int n_cmd, int n_slopes, const 
         tc_destroy(S->tc);
         S->tc = nullptr;
         if (dtype == MCAO_DTYPE_F32) {
-            // column-major [ld][rows_pad] (streamed column by column), scratch for kMultiRhs
-            // realizations per pass
-            if (e == cudaSuccess) e = dalloc(&S->d_Rrm, elems);
-            if (e == cudaSuccess) e = launch_transpose(tmp, S->rows_pad, S->ld, S->d_Rrm, S->rows_pad, 0, S->s0);
+            // blocks of 128 rows, scratch for kMultiRhs realizations per pass
+            if (e == cudaSuccess) e = dalloc(&S->d_Rrm, multi_tiled_floats(n_cmd, S->ld));
+            if (e == cudaSuccess) e = launch_multi_tile(tmp, S->rows_pad, n_cmd, S->ld, S->d_Rrm, S->s0);
             if (e == cudaSuccess) e = dalloc(&S->d_multi_st, (size_t)S->ld * kMultiRhs);
             if (e == cudaSuccess)
                 e = dalloc(&S->d_multi_part, (size_t)multi_chunks(S->ld) * kMultiRhs * std::max(n_cmd, 1));
@@ -1869,14 +1867,8 @@ mcao_status mcao_reconstruct_batch(mcao_sim* S, const float* slopes, int n_rhs, 
     CK(cudaSetDevice(S->device));
     CK(cudaDeviceSynchronize());   // inputs produced on any stream are complete
     { mcao_status r_ = sync_all(S); if (r_ != MCAO_OK) return r_; }
-    // the user layout [n_rhs][n_slopes] scattered into the padded layout of the product
-    const int ps = pad_stride(S);
-    CK(cudaMemsetAsync(S->d_slopes_pad, 0, sizeof(float) * (size_t)n_rhs * ps, S->s0));
-    for (const WfsHost& W : S->wfs)
-        if (W.n_valid > 0)
-            CK(cudaMemcpy2DAsync(S->d_slopes_pad + W.rcol0, sizeof(float) * ps, slopes + W.slope0,
-                                 sizeof(float) * S->n_slopes, sizeof(float) * 2 * W.n_valid, n_rhs,
-                                 cudaMemcpyDeviceToDevice, S->s0));
+    // the user layout [n_rhs][n_slopes] into the padded layout of the product (its padding stays zero)
+    CK(launch_pad_slopes(slopes, S->n_slopes, n_rhs, S->d_wfs, (int)S->wfs.size(), S->d_slopes_pad, pad_stride(S), S->s0));
     int nl = 0;
     CK(enqueue_batched_product(S, n_rhs, 1.0f, 0.0f, out, &nl));
     return sync_all(S);

@@ -268,10 +268,6 @@ cudaError_t launch_quantize_rows(const float* src, int rows, int cols, int ld, i
                                  const float* scale, cudaStream_t s);
 constexpr int kErrReconTimeout = 1;
 
-// row-major float32 [rows][cols] -> [cols][ld_out] (float32, or bfloat16 codes when bf16 != 0);
-// rows >= ld_out are not read, rows in [rows, ld_out) are written as zeros
-cudaError_t launch_transpose(const float* src, int rows, int cols, void* out, int ld_out, int bf16, cudaStream_t st);
-
 // ---------------------------------------------------------------------------------------------
 // science
 // ---------------------------------------------------------------------------------------------
@@ -375,18 +371,23 @@ std::vector<float2> sci_twiddles(int M);
 // second (self-check of the timeout path)
 cudaError_t launch_wait_probe(int* err, cudaStream_t s);
 
-// batched product for up to kMultiRhs realizations sharing R (column-major [K][rows_pad]):
-// one pass over R, split-K partials, fixed-order reduction into out[r][i] = alpha D + beta out
+// batched product for up to kMultiRhs realizations sharing a float32 R, held in blocks of 128 rows
+// ([row block][K][128], launch_multi_tile): one pass over R, split-K partials, fixed-order reduction into
+// out[r][i] = alpha D + beta out
 constexpr int kMultiRhs = 16;
 struct MultiLaunch {
-    const void* R;           // float32 or bfloat16, column-major [K][rows_pad]
-    int bf16;
-    long long rows_pad;      // multiple of 4
+    const float* R;
     int n_cmd, K;
     float* s_t;              // [K][kMultiRhs] scratch (transposed slopes)
     float* partial;          // [multi_chunks(K)][kMultiRhs][n_cmd] scratch
+    int* err;                // set to a nonzero code if a bounded wait gives up
 };
-int multi_chunks(int K);
+__host__ __device__ int multi_chunks(int K);
+// slopes [n_rhs][n_slopes] into the padded column layout [n_rhs][pad_stride] (padding columns untouched)
+cudaError_t launch_pad_slopes(const float* slopes, int n_slopes, int n_rhs, const WfsDev* wfs, int n_wfs, float* pad,
+                              int pad_stride, cudaStream_t s);
+size_t multi_tiled_floats(int n_cmd, int K);
+cudaError_t launch_multi_tile(const float* src, int rows, int n_cmd, int ld, float* out, cudaStream_t s);
 cudaError_t multi_prepare();   // kernel attributes (outside stream capture)
 cudaError_t launch_recon_multi(const MultiLaunch& L, int n_real, int pad_stride, const float* slopes_pad, float alpha,
                                float beta, float* out, int sm_count, int blocks_per_sm, cudaStream_t s);
