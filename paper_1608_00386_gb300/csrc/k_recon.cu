@@ -487,6 +487,13 @@ cudaError_t launch_recon(const ReconLaunch& L, cudaStream_t s) {
     const int n_items = L.n_rq * L.n_chunks;
     const int need = (n_items + kTmaWarps - 1) / kTmaWarps;
     int ctas = (L.max_ctas > 0 && L.max_ctas < need) ? L.max_ctas : need;
+    // items are few per warp: up to a sixteenth more blocks (never more than SMs) where that saves a round
+    // (39 m: 6048 items a slice; 129 blocks take 10 rounds and 404 us a step, 135 take 9 and 394)
+    const int rounds = (n_items + ctas * kTmaWarps - 1) / (ctas * kTmaWarps);
+    if (rounds > 1) {
+        const int more = (n_items + (rounds - 1) * kTmaWarps - 1) / ((rounds - 1) * kTmaWarps);
+        if (more <= ctas + ctas / 16 && more <= L.sm_count) ctas = more;
+    }
     if (L.dtype == kReconF32) recon_tma_kernel<kReconF32><<<(unsigned)ctas, kTmaWarps * 32, sizeof(TmaSmem), s>>>(L);
     else if (L.dtype == kReconBF16) recon_tma_kernel<kReconBF16><<<(unsigned)ctas, kTmaWarps * 32, sizeof(TmaSmem), s>>>(L);
     else if (L.dtype == kReconE4M3) recon_tma_kernel<kReconE4M3><<<(unsigned)ctas, kTmaWarps * 32, sizeof(TmaSmem), s>>>(L);
