@@ -106,9 +106,14 @@ __global__ void __launch_bounds__(256, 6) sci_field_kernel(SciLaunch L0) {
     if (lane == 0) L.sr_part[tile] = make_float4(sr, si, s1, s2);
 }
 
-// Strehl of this step from the field partial sums, and the Marechal residual variance
-// (piston removed, amplitude-weighted, science band) from the phase sums; fixed order, double
-__device__ void finalize_strehl(const SciLaunch& L, double* red, int tid, int nthr) {
+// Strehl of this step from the field partial sums, and the Marechal residual variance (piston removed,
+// amplitude-weighted, science band) from the phase sums; fixed order, double.  One block per
+// realization, launched beside the FFT passes: as an extra block of the row pass it was that pass's
+// longest (8 m: 8.9 us, the column pass of the same size 4.7), and the column pass waited for it.
+__global__ void __launch_bounds__(256) sci_strehl_kernel(SciLaunch L0) {
+    const SciLaunch L = sci_for_real(L0, blockIdx.y);
+    __shared__ double red[8][4];
+    const int tid = threadIdx.x, nthr = blockDim.x;
     double v[4] = {0.0, 0.0, 0.0, 0.0};
     // the thread's partials q = tid, tid + nthr, ... in that order, loaded eight at a time (the
     // loads of a batch in flight together)
@@ -129,24 +134,32 @@ __device__ void finalize_strehl(const SciLaunch& L, double* red, int tid, int nt
             v[3] += p[i].w;
         }
     }
-    for (int i = 0; i < 4; ++i) red[i * nthr + tid] = v[i];
+    const SciAcc old = *L.acc;   // read while the sums are formed
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+    if ((tid & 31) == 0)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) red[tid >> 5][i] = v[i];
     __syncthreads();
-    for (int o = nthr / 2; o > 0; o >>= 1) {
-        if (tid < o)
-            for (int i = 0; i < 4; ++i) red[i * nthr + tid] += red[i * nthr + tid + o];
-        __syncthreads();
+    if (tid < 4) {
+        double t = 0.0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) t += red[w][tid];
+        red[0][tid] = t;
     }
+    __syncwarp();
     if (tid == 0) {
-        const double s = (red[0] * red[0] + red[nthr] * red[nthr]) / (L.sum_amp * L.sum_amp);
-        L.acc->sr_sum += s;
+        const double s = (red[0][0] * red[0][0] + red[0][1] * red[0][1]) / (L.sum_amp * L.sum_amp);
+        L.acc->sr_sum = old.sr_sum + s;
         L.acc->sr_last = s;
-        L.acc->n_sr += 1;
-        const double mean = red[2 * nthr] / L.sum_amp;
-        const double var = red[3 * nthr] / L.sum_amp - mean * mean;
-        L.acc->var_sum += var;
+        L.acc->n_sr = old.n_sr + 1;
+        const double mean = red[0][2] / L.sum_amp;
+        const double var = red[0][3] / L.sum_amp - mean * mean;
+        L.acc->var_sum = old.var_sum + var;
         L.acc->var_last = var;
     }
-    __syncthreads();
 }
 
 __device__ __forceinline__ bool psf_step(const SciLaunch& L) {
@@ -159,14 +172,7 @@ __global__ void __launch_bounds__(256) sci_rows_kernel(SciLaunch L0) {
     float2* A = reinterpret_cast<float2*>(smem_raw);
     float2* B = A + kRowsPerBlock * L.M;
     float2* W = B + kRowsPerBlock * L.M;
-    double* red = reinterpret_cast<double*>(W + L.M);
     const int tid = threadIdx.x, nthr = blockDim.x;
-
-    // the grid's last block only reduces the Strehl partials; it runs beside the FFT blocks
-    if (blockIdx.x == gridDim.x - 1) {
-        finalize_strehl(L, red, tid, nthr);
-        return;
-    }
     if (!psf_step(L)) return;
 
     const int row0 = blockIdx.x * kRowsPerBlock;
@@ -225,14 +231,7 @@ __global__ void __launch_bounds__(256) sci_rows_ct(SciLaunch L0) {
     float2* A = reinterpret_cast<float2*>(smem_raw);
     float2* B = A + kCtRows * M;
     float2* W = B + kCtRows * M;
-    double* red = reinterpret_cast<double*>(W + M);
     const int tid = threadIdx.x, nthr = blockDim.x;
-    // the grid's last block only reduces the Strehl partials (on the FP64 pipe of one SM, about
-    // as long as an FFT block's work); it runs beside the FFT blocks
-    if (blockIdx.x == gridDim.x - 1) {
-        finalize_strehl(L, red, tid, nthr);
-        return;
-    }
     if (!psf_step(L)) return;
     static_assert((kCtRows * M) % kCtThreads == 0, "whole passes per thread");
     constexpr int PER = kCtRows * M / kCtThreads, PW = (M + kCtThreads - 1) / kCtThreads;
@@ -307,7 +306,7 @@ __global__ void __launch_bounds__(256) sci_cols_ct(SciLaunch L0) {
 
 template <int M>
 size_t ct_smem() {
-    return sizeof(float2) * (2 * kCtRows * (size_t)M + M) + sizeof(double) * 4 * 256;
+    return sizeof(float2) * (2 * kCtRows * (size_t)M + M);
 }
 
 template <int M>
@@ -321,7 +320,7 @@ cudaError_t ct_prepare() {
 
 template <int M>
 cudaError_t ct_rows(const SciLaunch& L, cudaStream_t s) {
-    sci_rows_ct<M><<<dim3((unsigned)((L.N + kCtRows - 1) / kCtRows + 1), (unsigned)L.ctx.n_real), 256, ct_smem<M>(), s>>>(L);
+    sci_rows_ct<M><<<dim3((unsigned)((L.N + kCtRows - 1) / kCtRows), (unsigned)L.ctx.n_real), 256, ct_smem<M>(), s>>>(L);
     return cudaGetLastError();
 }
 
@@ -335,7 +334,7 @@ cudaError_t ct_cols(const SciLaunch& L, cudaStream_t s) {
 #define MCAO_SCI_CT_SIZES(X) X(128) X(256) X(512) X(640) X(1024) X(1280) X(2048)
 
 size_t fft_smem_bytes(int M) {
-    return sizeof(float2) * (2 * kRowsPerBlock * (size_t)M + M) + sizeof(double) * 4 * 256;
+    return sizeof(float2) * (2 * kRowsPerBlock * (size_t)M + M);
 }
 
 cudaError_t set_smem(const void* fn, size_t bytes) {
@@ -347,6 +346,11 @@ cudaError_t set_smem(const void* fn, size_t bytes) {
 cudaError_t launch_sci_field(const SciLaunch& L, cudaStream_t s) {
     int tiles = (L.N / 8) * (L.N / 8);
     sci_field_kernel<<<dim3((unsigned)((tiles + 7) / 8), (unsigned)L.ctx.n_real), 256, 0, s>>>(L);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sci_strehl(const SciLaunch& L, cudaStream_t s) {
+    sci_strehl_kernel<<<dim3(1u, (unsigned)L.ctx.n_real), 256, 0, s>>>(L);
     return cudaGetLastError();
 }
 
@@ -402,7 +406,7 @@ cudaError_t launch_sci_rows(const SciLaunch& L, cudaStream_t s) {
     MCAO_SCI_CT_SIZES(MCAO_CT_ROWS)
 #undef MCAO_CT_ROWS
     size_t sm = fft_smem_bytes(L.M);
-    sci_rows_kernel<<<dim3((unsigned)((L.N + kRowsPerBlock - 1) / kRowsPerBlock + 1), (unsigned)L.ctx.n_real), 256, sm, s>>>(L);
+    sci_rows_kernel<<<dim3((unsigned)((L.N + kRowsPerBlock - 1) / kRowsPerBlock), (unsigned)L.ctx.n_real), 256, sm, s>>>(L);
     return cudaGetLastError();
 }
 

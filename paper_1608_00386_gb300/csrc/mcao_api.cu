@@ -585,10 +585,14 @@ cudaError_t enqueue_step(mcao_sim* S, int* launches) {
         SciLaunch L = make_sci_launch(S, (int)q);
         slot = prof_begin(S, ST_SCIENCE, S->s2);
         if ((e = launch_sci_field(L, S->s2)) != cudaSuccess) return e;
+        cudaEvent_t ev_field = dep_event(S, used);
+        if ((e = cudaEventRecord(ev_field, S->s2)) != cudaSuccess) return e;
+        if ((e = cudaStreamWaitEvent(S->s1, ev_field, 0)) != cudaSuccess) return e;
+        if ((e = launch_sci_strehl(L, S->s1)) != cudaSuccess) return e;
         if ((e = launch_sci_rows(L, S->s2)) != cudaSuccess) return e;
         if ((e = launch_sci_cols(L, S->s2)) != cudaSuccess) return e;
         prof_end(S, slot, S->s2);
-        nl += 3;
+        nl += 4;
     }
     cudaEvent_t ev_sci = dep_event(S, used);
     if ((e = cudaEventRecord(ev_sci, S->s2)) != cudaSuccess) return e;
@@ -610,9 +614,11 @@ cudaError_t enqueue_step(mcao_sim* S, int* launches) {
     if (S->n_real > 1) {
         // batched: after every sensor of every realization, C += g R S for all realizations at
         // once (one pass over R), then the step counter
-        cudaEvent_t ev_s1b = dep_event(S, used);
-        if ((e = cudaEventRecord(ev_s1b, S->s1)) != cudaSuccess) return e;
-        if ((e = cudaStreamWaitEvent(S->s0, ev_s1b, 0)) != cudaSuccess) return e;
+        cudaEvent_t last = nullptr;
+        for (cudaEvent_t ev : ready) {
+            if (ev && ev != last && (e = cudaStreamWaitEvent(S->s0, ev, 0)) != cudaSuccess) return e;
+            last = ev;
+        }
         slot = prof_begin(S, ST_RECON, S->s0);
         // integrator: C += g R S in place; controller: D = R S, then the filter
         const float alpha = S->use_ctl ? 1.0f : (float)S->cfg.gain, beta = S->use_ctl ? 0.0f : 1.0f;
@@ -629,9 +635,11 @@ cudaError_t enqueue_step(mcao_sim* S, int* launches) {
         if ((e = launch_recon_reduce(fin, S->s0)) != cudaSuccess) return e;
         nl += 2;
         if ((e = cudaStreamWaitEvent(S->s0, ev_sci, 0)) != cudaSuccess) return e;
-        cudaEvent_t ev_s3 = dep_event(S, used);   // s3 forked: join it back untouched
-        if ((e = cudaEventRecord(ev_s3, S->s3)) != cudaSuccess) return e;
-        if ((e = cudaStreamWaitEvent(S->s0, ev_s3, 0)) != cudaSuccess) return e;
+        for (cudaStream_t st : {S->s1, S->s3}) {   // the other forked streams join too
+            cudaEvent_t ev = dep_event(S, used);
+            if ((e = cudaEventRecord(ev, st)) != cudaSuccess) return e;
+            if ((e = cudaStreamWaitEvent(S->s0, ev, 0)) != cudaSuccess) return e;
+        }
         if (launches) *launches = nl;
         return cudaSuccess;
     }
@@ -774,8 +782,8 @@ mcao_status signal_user(mcao_sim* S) {
     return MCAO_OK;
 }
 
-// Waits for all queued work.  Every step's and call's branches join s0 (s1 to s3 only carry work while a
-// step is captured into its graph), so s0 and the readout stream are all there is to wait for.
+// Waits for all queued work.  The branches of every step and call join s0, so s0 and the readout stream
+// are all there is to wait for.
 mcao_status sync_all(mcao_sim* S) {
     CK(cudaStreamSynchronize(S->s0));
     S->s0_pending = false;
@@ -880,6 +888,26 @@ mcao_status validate_config(const mcao_config* c) {
             return fail(S, MCAO_E_UNSUPPORTED, "science %d: FFT size %d must factor into 2,3,5 and be <= 4096", q, M);
     }
     return MCAO_OK;
+}
+
+// One launch per run of sensors, behind s0's work so far and before its later work.  The first run stays
+// on s0, the others go to s1 beside it: a run of low-order sensors is a few blocks, whose latency (13 us
+// at 20 m) would otherwise add to the laser stars'.
+template <class F>
+cudaError_t for_each_run(mcao_sim* S, F&& launch) {
+    cudaError_t e = cudaSuccess;
+    const bool fork = S->runs.size() > 1;
+    if (fork) {
+        e = cudaEventRecord(S->ev_done, S->s0);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(S->s1, S->ev_done, 0);
+    }
+    for (size_t i = 0; i < S->runs.size() && e == cudaSuccess; ++i)
+        if (S->runs[i].n_subaps > 0) e = launch(S->runs[i], i == 0 ? S->s0 : S->s1);
+    if (fork) {
+        if (e == cudaSuccess) e = cudaEventRecord(S->ev_done, S->s1);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(S->s0, S->ev_done, 0);
+    }
+    return e;
 }
 
 // device address of a page-locked host buffer (false: any other memory, or one not aligned to its type)
@@ -1828,11 +1856,10 @@ static cudaError_t enqueue_sensing(mcao_sim* S, int noise) {
     if (e != cudaSuccess) return e;
     // nobody keeps the images of a noise-free measurement: slopes straight from the field's lags.  The
     // loop stays on the image route, noise or not: its Strehl ratios are doubles of the commands.
-    if (!noise && !S->cfg.keep_frames) {
-        for (const auto& r : S->runs)
-            if ((e = launch_wfs_lag(make_wfs_launch(S, r.d_subaps, r.n_subaps), r.n_px, S->s0)) != cudaSuccess) return e;
-        return cudaSuccess;
-    }
+    if (!noise && !S->cfg.keep_frames)
+        return for_each_run(S, [&](const WfsRun& r, cudaStream_t st) {
+            return launch_wfs_lag(make_wfs_launch(S, r.d_subaps, r.n_subaps), r.n_px, st);
+        });
     auto run = [&](const SubapDev* sub, int n, unsigned int* work, int npx, int nfft, int nbin) {
         WfsLaunch L = make_wfs_launch(S, sub, n, work);
         L.ctx.noise = noise;
@@ -1885,8 +1912,10 @@ static cudaError_t enqueue_sens(mcao_sim* S) {
         if (e == cudaSuccess) e = cudaMemsetAsync(S->d_adj_err, 0, sizeof(int), S->s0);
     }
     if (e == cudaSuccess) e = launch_dm_surfaces(make_dm_launch(S), S->s0);
-    for (const auto& r : S->runs)
-        if (e == cudaSuccess) e = launch_sens(make_wfs_launch(S, r.d_subaps, r.n_subaps), r.n_px, S->cur, S->d_sens, S->s0);
+    if (e == cudaSuccess)
+        e = for_each_run(S, [&](const WfsRun& r, cudaStream_t st) {
+            return launch_sens(make_wfs_launch(S, r.d_subaps, r.n_subaps), r.n_px, S->cur, S->d_sens, st);
+        });
     return e;
 }
 
@@ -1960,13 +1989,14 @@ static mcao_status run_matrix(mcao_sim* S, float* D, long long ld) {
     { mcao_status r_ = sync_all(S); if (r_ != MCAO_OK) return r_; }
     cudaError_t e = enqueue_sens(S);
     if (e == cudaSuccess && S->n_dms == 0) e = cudaMemsetAsync(D, 0, sizeof(float) * (size_t)S->n_slopes * ld, S->s0);
-    for (const auto& r : S->runs) {
-        ProjLaunch J = make_proj_launch(S, r.d_subaps, r.n_subaps);
-        J.max_band = footprint_band(S, r);
-        J.D = D;
-        J.ld = ld;
-        if (e == cudaSuccess) e = launch_dm_rows(J, r.n_px, S->sm_count, S->s0);
-    }
+    if (e == cudaSuccess)
+        e = for_each_run(S, [&](const WfsRun& r, cudaStream_t st) {
+            ProjLaunch J = make_proj_launch(S, r.d_subaps, r.n_subaps);
+            J.max_band = footprint_band(S, r);
+            J.D = D;
+            J.ld = ld;
+            return launch_dm_rows(J, r.n_px, S->sm_count, st);
+        });
     return finish_adjoint(S, e);
 }
 
