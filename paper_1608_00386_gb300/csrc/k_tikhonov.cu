@@ -25,7 +25,7 @@
 // outputs per block, four of which share an SM's pipe: the last wave of a launch costs a quarter of
 // what 64 x 64 outputs cost.  A dense D (more than a third nonzero) takes the tile products, where
 // each operand read serves 32 outputs.
-// 20 m (7280 x 1870): 46.6 ms before, 17.5 ms now; 39 m (55608 x 8051): 2.2 s before.
+// 20 m (7280 x 1870): 46.6 ms before, 15.9 ms now; 39 m (55608 x 8051): 2.2 s before.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -322,36 +322,34 @@ __global__ void tik_regularize_kernel(double* __restrict__ G, long long ldg, int
 // ------------------------------------------------------------------------------------------
 // 4. Cholesky factor and its inverse
 // ------------------------------------------------------------------------------------------
-// 1 / sqrt(d): the float reciprocal square root of the significand and one third-order
-// Newton-Halley step y (1 + e/2 + 3 e^2 / 8), e = 1 - d y^2 (|e| < 2^-21, so the step leaves less
-// than 2^-60), the even power of two of d put back exactly
-__device__ __forceinline__ double inv_sqrt(double d) {
-    int ex;
-    double m = frexp(d, &ex);        // m in [1/2, 1)
-    if (ex & 1) {
-        m *= 0.5;
-        ex += 1;
-    }
-    const double y = (double)rsqrtf((float)m), e = fma(-m * y, y, 1.0);
-    return ldexp(fma(y * e, fma(0.375, e, 0.5), y), -ex / 2);
+// 1 / d: float reciprocal of the significand (2^-23) and two Newton steps y + y (1 - m y), the exponent
+// put back in the high word; zeros, subnormals and infinities take the division
+__device__ __forceinline__ double reciprocal(double d) {
+    const int hi = __double2hiint(d), ex = (hi >> 20) & 0x7ff;
+    if (ex == 0 || ex >= 2045) return 1.0 / d;
+    const double m = __hiloint2double((hi & 0xfffff) | 0x3ff00000, __double2loint(d));   // [1, 2)
+    double y = (double)(1.0f / (float)m);
+    y = fma(y, fma(-m, y, 1.0), y);
+    y = fma(y, fma(-m, y, 1.0), y);
+    return __hiloint2double(__double2hiint(y) + ((1023 - ex) << 20), __double2loint(y));
 }
 
 // 4a. Linv = L^(-1) of the diagonal block S = L L^T, in one block: the lower triangle of a 64 x 64
-// array W, 8 or 9 entries (m, c) per thread in registers, starts as S and ends as L^(-1).  Before step
-// j the columns c >= j of the rows m >= j hold the trailing matrix S, the columns c < j the rows of
-// X = L^(-1) so far.  Step j takes r = 1 / sqrt(S_jj), L_mj = r S_mj, u_c = r X_jc (c < j), r (c = j),
-// L_cj (c > j), then W_mc -= L_mj u_c on every row below (W_mj counts as 0 there: column j of X
-// begins), and row j of X is u.  So factor and inverse cost one pass of 64^3 / 3 multiply-adds with
-// two barriers a step.  Entries are dealt row by row, so finished rows leave whole warps idle.
-// Bound by the latency of the double operations in the chain from one pivot to the next (its 87 k
-// multiply-adds alone are 22 us of one SM's pipe).  Before, factor
-// and inverse one after the other in shared memory took 228 us a block, 6.9 of 46.6 ms at 20 m;
-// 114 us now.  A pivot <= 0 (or NaN) sets *err and is replaced by 1 so that the remaining
-// steps stay finite.
+// array W, 8 or 9 entries (m, c) per thread in registers, starts as S and ends as the inverse of the
+// unit factor of S = U D U^T.  Before step j the columns c >= j of the rows m >= j hold the trailing
+// matrix S, the columns c < j the rows of X = U^(-1) so far.  Step j takes v_m = S_mj / S_jj and u_c =
+// X_jc (c < j), 1 (c = j), S_cj (c > j), then W_mc -= v_m u_c on every row below (W_mj counts as 0
+// there: column j of X begins).  At the end row m is scaled by 1 / sqrt(D_m).  So factor and inverse cost
+// one pass of 64^3 / 3 multiply-adds with two barriers a step, and no square root is in the chain from
+// one pivot to the next.  Entries are dealt row by row, so finished rows leave whole warps idle.
+// Bound by the latency of the double operations of that chain (the 87 k multiply-adds alone are 22 us
+// of one SM's pipe).  Factor and inverse one after the other in shared memory took 228 us a block, 6.9
+// of 46.6 ms at 20 m; in one pass with L and its square roots 114 us; 75 us now.  A pivot <= 0
+// (or NaN) sets *err and is replaced by 1 so that the remaining steps stay finite.
 __global__ void __launch_bounds__(256) tik_potrf_kernel(const double* __restrict__ A, long long lda, int k,
                                                         double* __restrict__ Linv, int* __restrict__ err) {
     constexpr int kEnt = kT * (kT + 1) / 2, kPer = (kEnt + 255) / 256;
-    __shared__ double s_v[kT], s_u[kT], s_d;
+    __shared__ double s_col[2][kT], s_u[2][kT], s_v[2][kT], s_diag[kT];
     const int tid = threadIdx.x;
     const long long o = (long long)k * kT;
     double w[kPer];
@@ -363,99 +361,104 @@ __global__ void __launch_bounds__(256) tik_potrf_kernel(const double* __restrict
         if (p < kEnt) tri_index(p, m, c);
         mc[i] = m << 8 | c;
         w[i] = p < kEnt ? A[(o + m) * lda + o + c] : 0.0;
-        if (p == 0) s_d = w[i];
     }
     for (int j = 0; j < kT; ++j) {
-        // column j of the rows below and row j, unscaled
+        double *col = s_col[j & 1], *u = s_u[j & 1], *v = s_v[j & 1];   // the other pair may still be read
+        // column j from the diagonal down, and row j of X
 #pragma unroll
         for (int i = 0; i < kPer; ++i) {
             const int m = mc[i] >> 8, c = mc[i] & 255;
-            if (m < kT && c == j && m > j) s_v[m] = w[i];
-            if (m == j && c < j) s_u[c] = w[i];
+            if (m < kT && c == j) col[m] = w[i];
+            if (m == j && c < j) u[c] = w[i];
         }
         __syncthreads();
         if (tid < kT) {
-            double d = s_d;
+            double d = col[j];
             if (!(d > 0.0)) {
                 if (tid == 0) atomicExch(err, 1);
                 d = 1.0;
             }
-            const double r = inv_sqrt(d);
-            if (tid > j) s_u[tid] = s_v[tid] = s_v[tid] * r;
-            else s_u[tid] = tid < j ? s_u[tid] * r : r;
+            if (tid == j) {
+                s_diag[j] = d;
+                u[j] = 1.0;
+            } else if (tid > j) {
+                u[tid] = col[tid];
+                v[tid] = col[tid] * reciprocal(d);
+            }
         }
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < kPer; ++i) {
             const int m = mc[i] >> 8, c = mc[i] & 255;
-            if (m == j) w[i] = s_u[c];
-            else if (m > j && m < kT) {
-                w[i] = fma(-s_v[m], s_u[c], c == j ? 0.0 : w[i]);
-                if (m == j + 1 && c == j + 1) s_d = w[i];
-            }
+            if (m > j && m < kT) w[i] = fma(-v[m], u[c], c == j ? 0.0 : w[i]);
+            else if (m == j && c == j) w[i] = 1.0;
         }
-        __syncthreads();   // s_v and s_u are read before the next step writes them
     }
+    __syncthreads();
+    if (tid < kT) s_v[0][tid] = 1.0 / sqrt(s_diag[tid]);
     double* Lk = Linv + (long long)k * kT * kT;
     for (int q = tid; q < kT * kT; q += 256)
         if (q % kT > q / kT) Lk[q] = 0.0;
+    __syncthreads();
 #pragma unroll
     for (int i = 0; i < kPer; ++i) {
         const int m = mc[i] >> 8, c = mc[i] & 255;
-        if (m < kT) Lk[m * kT + c] = w[i];
+        if (m < kT) Lk[m * kT + c] = w[i] * s_v[0][m];
     }
 }
 
 // 4b. block column k of L below the diagonal, A[i][k] <- A[i][k] Linv_kk^T, and block row k of X,
-// X[k][j] <- Linv_kk X[k][j] for j < k, X[k][k] = Linv_kk, both in place.  One block per strip of 32
-// rows (A) or columns (X): the strip is read whole before it is written; Linv is lower triangular, so
-// its first 32 rows need half the depth.
+// X[k][j] <- Linv_kk X[k][j] for j < k, X[k][k] = Linv_kk, both in place.  One block per strip of 16
+// rows (A) or columns (X), read whole before it is written; Linv is lower triangular, so its first 32
+// rows need half the depth.  (Strips of 32: 41 us a launch at 20 m, 60 blocks on 152 SMs; 26
+// us with 120.)
+constexpr int kStrip = 16;
 __global__ void __launch_bounds__(kThreads) tik_panel_kernel(double* __restrict__ A, double* __restrict__ X, long long ld, int k,
                                                              int nt, const double* __restrict__ Linv) {
-    __shared__ Chunk ch;
-    const int below = nt - k - 1;
+    __shared__ double s_l[kT][kT + 1];         // Linv
+    __shared__ double s_p[kT][kStrip + 1];     // the strip, [depth][row or column]
+    constexpr int kPerTile = kT / kStrip;
+    const int n_a = kPerTile * (nt - k - 1), t = threadIdx.x;
+    const bool is_a = (int)blockIdx.x < n_a;
     const double* Lk = Linv + (long long)k * kT * kT;
-    double c[2][2][4] = {};   // [half of Linv's rows]
-    if ((int)blockIdx.x < 2 * below) {
-        double* P = A + ((long long)(k + 1) * kT + blockIdx.x * kS) * ld + (long long)k * kT;   // 32 x 64 strip
-        for (int k0 = 0; k0 < kT; k0 += kS) {
-            load_trans(ch.a, P, ld, 0, k0, kS, kT);   // a[m][r] = P[r][k0 + m]
-            for (int h = k0 / kS; h < 2; ++h) {
-                load_trans(ch.b, Lk, kT, h * kS, k0, kT, kT);   // b[m][q] = Linv[32 h + q][k0 + m]
-                __syncthreads();
-                chunk_fma(ch, c[h]);
-                __syncthreads();
-            }
-        }
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int i = 0; i < 2; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) P[out_row(i) * ld + h * kS + out_col(j)] = c[h][i][j];
+    const int q0 = is_a ? 0 : ((int)blockIdx.x - n_a) * kStrip;   // first column of a strip of X
+    double* P = is_a ? A + ((long long)(k + 1) * kT + blockIdx.x * kStrip) * ld + (long long)k * kT : X + (long long)k * kT * ld + q0;
+    if (!is_a && q0 >= k * kT) {
+        for (int q = t; q < kT * kStrip; q += kThreads)
+            P[q / kStrip * ld + q % kStrip] = Lk[q / kStrip * kT + q0 - k * kT + q % kStrip];
         return;
     }
-    const int q0 = (blockIdx.x - 2 * below) * kS;   // first column of the strip of X
-    double* P = X + (long long)k * kT * ld + q0;     // 64 x 32 strip
-    if (q0 >= k * kT) {
-        for (int q = threadIdx.x; q < kT * kS; q += kThreads) P[q / kS * ld + q % kS] = Lk[q / kS * kT + q0 - k * kT + q % kS];
-        return;
+    for (int q = t; q < kT * kT; q += kThreads) s_l[q / kT][q % kT] = Lk[q];
+    for (int q = t; q < kT * kStrip; q += kThreads) {
+        if (is_a) s_p[q % kT][q / kT] = P[q / kT * ld + q % kT];
+        else s_p[q / kStrip][q % kStrip] = P[q / kStrip * ld + q % kStrip];
     }
-    for (int k0 = 0; k0 < kT; k0 += kS) {
-        load_direct(ch.b, P, ld, k0, 0, kT, kS);   // b[m][q] = P[k0 + m][q]
-        for (int h = k0 / kS; h < 2; ++h) {
-            load_trans(ch.a, Lk, kT, h * kS, k0, kT, kT);   // a[m][r] = Linv[32 h + r][k0 + m]
-            __syncthreads();
-            chunk_fma(ch, c[h]);
-            __syncthreads();
-        }
+    __syncthreads();
+    // this thread: strip entry e, Linv rows g, g + 8, ..
+    const int e = t % kStrip, g = t / kStrip;
+    double c[8] = {};
+#pragma unroll 4
+    for (int m = 0; m < kT / 2; ++m) {
+        const double p = s_p[m][e];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) c[i] = fma(p, s_l[g + 8 * i][m], c[i]);
     }
+#pragma unroll 4
+    for (int m = kT / 2; m < kT; ++m) {
+        const double p = s_p[m][e];
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
+        for (int i = 4; i < 8; ++i) c[i] = fma(p, s_l[g + 8 * i][m], c[i]);
+    }
+    if (is_a) {
+        __syncthreads();
 #pragma unroll
-        for (int i = 0; i < 2; ++i)
+        for (int i = 0; i < 8; ++i) s_p[g + 8 * i][e] = c[i];
+        __syncthreads();
+        for (int q = t; q < kT * kStrip; q += kThreads) P[q / kT * ld + q % kT] = s_p[q % kT][q / kT];
+    } else {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) P[(h * kS + out_row(i)) * ld + out_col(j)] = c[h][i][j];
+        for (int i = 0; i < 8; ++i) P[(g + 8 * i) * ld + e] = c[i];
+    }
 }
 
 // 4c. with L[.][k] and X[k][.] final: A[i][j] -= L[i][k] L[j][k]^T for the lower tiles i >= j > k, and
@@ -679,7 +682,7 @@ extern "C" mcao_status mcao_tikhonov_reconstructor(const float* D, int n_slopes,
         for (int k = 0; k < nt; ++k) {
             const long long below = nt - k - 1, rest = 2 * below;
             tik_potrf_kernel<<<1, 256, 0, st>>>(G, npad, k, Linv, d_err);
-            tik_panel_kernel<<<(unsigned)(2 * below + 2 * (k + 1)), kThreads, 0, st>>>(G, X, npad, k, nt, Linv);
+            tik_panel_kernel<<<(unsigned)(kT / kStrip * nt), kThreads, 0, st>>>(G, X, npad, k, nt, Linv);
             if (below > 0)
                 tik_update_kernel<<<(unsigned)(rest * (rest + 1) / 2 + rest * 2 * (k + 1)), kThreads, 0, st>>>(G, X, npad, k, nt);
         }
