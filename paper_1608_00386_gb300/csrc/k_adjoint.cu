@@ -214,13 +214,14 @@ __global__ void misreg_sum_kernel(const double* __restrict__ rec, int n_rows, do
     }
 }
 
-// n floats from p set to zero by the block: whole 16-byte vectors between the unaligned ends
-__device__ __forceinline__ void zero_run(float* p, int n, int tid, int nthr) {
+// n floats from p set to zero by the warp: whole 16-byte vectors between the unaligned ends
+__device__ __forceinline__ void zero_run(float* p, int n, int lane) {
     const int head = min(n, (int)((16 - (reinterpret_cast<uintptr_t>(p) & 15)) & 15) / 4), vecs = (n - head) / 4;
     float4* v = reinterpret_cast<float4*>(p + head);
-    for (int q = tid; q < vecs; q += nthr) __stcs(v + q, make_float4(0.0f, 0.0f, 0.0f, 0.0f));
+#pragma unroll 4
+    for (int q = lane; q < vecs; q += 32) __stcs(v + q, make_float4(0.0f, 0.0f, 0.0f, 0.0f));
     const int rest = n - 4 * vecs;   // at most 3 before and 3 after
-    if (tid < rest) __stcs(p + (tid < head ? tid : tid + 4 * vecs), 0.0f);
+    if (lane < rest) __stcs(p + (lane < head ? lane : lane + 4 * vecs), 0.0f);
 }
 
 // Interaction-matrix rows of both slopes of one subaperture (block x) over a part of the commands
@@ -230,7 +231,9 @@ __device__ __forceinline__ void zero_run(float* p, int n, int tid, int nthr) {
 // rows of the band (each command checked against the band's columns) and a run of zeros.  One block
 // does every DM, so that the three barriers of the setup are paid once per 2 n_cmd stored floats and
 // hide behind the other blocks' stores; a sensor of a few subapertures is cut into enough parts to
-// fill the GPU.  39 m (55608 x 8051, 1.79 GB), six laser stars: 484 us; with a block per DM and
+// fill the GPU.  39 m (55608 x 8051, 1.79 GB), six laser stars: 470 us (484 with the zeros as four runs per DM by the whole block and the weights
+// formed again for every sample row; 580 with whole rows cleared first and the band written over them);
+// with a block per DM and
 // a check of every command 789 us; before that the matrix was cleared and one block per slope
 // scattered its band: 6 x 160 us and 3 x 131 us (natural stars) on top of the clearing.
 // With gvec set (rotated DMs only) the rows are not stored: sum over both slopes of g row is added
@@ -238,12 +241,12 @@ __device__ __forceinline__ void zero_run(float* p, int n, int tid, int nthr) {
 struct RowsDm {                // one DM's view from the block's subaperture
     AxisEnt ex[kMaxNpx], ey[kMaxNpx];
     int rng[4];                // actuators [a0, a1) x [b0, b1)
-    int c0, c1;                // commands of rows [b0, b1)
+    int c0, c1;                // commands of rows [b0, b1) in the block's part
 };
 
 // nbw: most actuators per axis on a footprint, at most kAdjMaxBand (shared-memory row length)
 template <bool ROTATED>
-__global__ void __launch_bounds__(kAdjThreads, ROTATED ? 2 : 8) dm_rows_kernel(ProjLaunch L, int nbw) {
+__global__ void __launch_bounds__(kAdjThreads, ROTATED ? 2 : 6) dm_rows_kernel(ProjLaunch L, int nbw) {
     extern __shared__ float rows_sm[];
     __shared__ RowsDm s_dm[kMaxDms];
     const int tid = threadIdx.x, nthr = blockDim.x;
@@ -251,25 +254,31 @@ __global__ void __launch_bounds__(kAdjThreads, ROTATED ? 2 : 8) dm_rows_kernel(P
     const WfsDev& w = L.ctx.wfs[sd.wfs];
     const int npx = w.n_px, i0 = sd.sx * npx, j0 = sd.sy * npx;
     const GridView* V = L.ctx.views + L.real * L.ctx.view_stride + (long long)sd.wfs * L.ctx.n_grids + L.n_layers;
+    const int lane = tid & 31, warp = tid >> 5, n_warps = nthr >> 5;
+    const bool staged = npx <= 16;                         // column weights kept (they fit)
     float* s_L = rows_sm;                                  // [2][npx][npx]
     float* s_T = s_L + 2 * npx * npx;                      // [n_dms][2][npx][nbw]
-    float* s_gy = s_T + L.n_dms * 2 * npx * nbw;   // [n_dms][nbw][npx]
+    float* s_gy = s_T + L.n_dms * 2 * npx * nbw;           // [n_dms][nbw][npx]
+    float* s_gx = s_gy + L.n_dms * npx * nbw;              // [n_dms][npx][nbw], staged only
     const float *lx = sens_row(L.sens, w, 0, sd.rank), *ly = sens_row(L.sens, w, 1, sd.rank);
     for (int q = tid; q < npx * npx; q += nthr) {
         s_L[q] = lx[q];
         s_L[npx * npx + q] = ly[q];
     }
-    for (int q = tid; q < L.n_dms * 2 * npx; q += nthr) {
-        const int m = q / (2 * npx), r = q - m * 2 * npx;
-        const GridView& v = V[m];
-        if (r < npx) s_dm[m].ex[r] = axis_entry(v.ax + (long long)(i0 + r) * v.bp, v.n, v.periodic, v.inv_n);
-        else s_dm[m].ey[r - npx] = axis_entry(v.ay + (long long)(j0 + r - npx) * v.bp, v.n, v.periodic, v.inv_n);
+    for (int m = warp; m < 2 * L.n_dms; m += n_warps) {    // one warp per DM and axis
+        const GridView& v = V[m >> 1];
+        if (lane < npx) {
+            if (m & 1) s_dm[m >> 1].ey[lane] = axis_entry(v.ay + (long long)(j0 + lane) * v.bp, v.n, v.periodic, v.inv_n);
+            else s_dm[m >> 1].ex[lane] = axis_entry(v.ax + (long long)(i0 + lane) * v.bp, v.n, v.periodic, v.inv_n);
+        }
     }
     __syncthreads();
-    if ((tid & 31) == 0 && tid / 32 < L.n_dms) {
+    const int len = (L.n_cmd + gridDim.z - 1) / gridDim.z, first = min((int)blockIdx.z * len, L.n_cmd);
+    const int last = min(L.n_cmd, first + len);
+    if (lane == 0 && warp < L.n_dms) {
         // the axis entries ascend (a DM grid does not wrap): the footprint is the first and last
-        RowsDm& d = s_dm[tid / 32];
-        const DmDesc& dd = L.desc[tid / 32];
+        RowsDm& d = s_dm[warp];
+        const DmDesc& dd = L.desc[warp];
         int rng[4];
         actuator_range(dd, L.band, d.ex[0].idx & 0xffff, d.ex[npx - 1].idx >> 16, d.ey[0].idx & 0xffff,
                        d.ey[npx - 1].idx >> 16, rng);
@@ -280,44 +289,73 @@ __global__ void __launch_bounds__(kAdjThreads, ROTATED ? 2 : 8) dm_rows_kernel(P
         }
         if (L.gvec && !dd.general) rng[3] = rng[2];
         for (int q = 0; q < 4; ++q) d.rng[q] = rng[q];
-        const int* row0 = L.cmd_act + dd.row_off;          // first command of each DM row, and the total
-        d.c0 = row0[min(rng[2], dd.ny)];
-        d.c1 = row0[min(rng[3], dd.ny)];
-    }
-    __syncthreads();
-    const int len = (L.n_cmd + gridDim.z - 1) / gridDim.z, first = blockIdx.z * len;
-    const int last = min(L.n_cmd, first + len);
-    for (int m = 0; m < L.n_dms; ++m) {
-        const DmDesc& dd = L.desc[m];
-        const RowsDm& d = s_dm[m];
-        const int a0 = d.rng[0], na = d.rng[1] - a0, b0 = d.rng[2], nbd = d.rng[3] - b0;
-        if (ROTATED && dd.general) continue;
-        if (dd.cmd0 >= last || dd.cmd0 + dd.n_cmd <= first) continue;   // not in this part
-        // T[axis][y][a] = sum_x L[axis][y][x] gx_a(x)
-        const float *Gx = L.g + dd.gx_off + a0, *Gy = L.g + dd.gy_off + b0;
-        float* T = s_T + m * 2 * npx * nbw;
-        float* gy = s_gy + m * npx * nbw;
-        for (int idx = tid; idx < na * npx; idx += nthr) {
-            const int y = idx / na, a = idx - y * na;
-            float ax = 0.0f, ay = 0.0f;
-#pragma unroll 4
-            for (int x = 0; x < npx; ++x) {
-                const float g = axis_weight(Gx, dd.nx, d.ex[x], a);
-                ax = fmaf(s_L[y * npx + x], g, ax);
-                ay = fmaf(s_L[(npx + y) * npx + x], g, ay);
-            }
-            T[y * nbw + a] = ax;
-            T[(npx + y) * nbw + a] = ay;
-        }
-        for (int idx = tid; idx < nbd * npx; idx += nthr) {
-            const int y = idx / nbd, b = idx - y * nbd;
-            gy[b * npx + y] = axis_weight(Gy, dd.ny, d.ey[y], b);
-        }
+        const int* row0 = L.cmd_act + dd.row_off;          // commands before each DM row, and the total
+        // this part's share of the DM's commands, split at the band's rows
+        const int lo = max(first, dd.cmd0), hi = max(lo, min(last, dd.cmd0 + dd.n_cmd));
+        d.c0 = min(max(dd.cmd0 + row0[min(rng[2], dd.ny)], lo), hi);
+        d.c1 = min(max(dd.cmd0 + row0[min(rng[3], dd.ny)], d.c0), hi);
     }
     __syncthreads();
     const int row_x = w.slope0 + sd.rank, row_y = row_x + w.n_valid;
     float* out_x = L.D ? L.D + (long long)row_x * L.ld : nullptr;
     float* out_y = L.D ? L.D + (long long)row_y * L.ld : nullptr;
+    // the zeros between the DMs' bands, one warp per run and row
+    if (L.D)
+        for (int r = warp; r < 2 * (L.n_dms + 1); r += n_warps) {
+            const int m = r >> 1, from = m ? s_dm[m - 1].c1 : first, to = m < L.n_dms ? s_dm[m].c0 : last;
+            zero_run((r & 1 ? out_y : out_x) + from, to - from, lane);
+        }
+    // weights of the footprint's columns and rows
+    for (int m = 0; m < L.n_dms; ++m) {
+        const DmDesc& dd = L.desc[m];
+        const RowsDm& d = s_dm[m];
+        const int a0 = d.rng[0], na = d.rng[1] - a0, b0 = d.rng[2], nbd = d.rng[3] - b0;
+        if ((ROTATED && dd.general) || d.c0 == d.c1) continue;
+        const float *Gx = L.g + dd.gx_off + a0, *Gy = L.g + dd.gy_off + b0;
+        for (int y = warp; y < npx; y += n_warps) {
+            if (staged)
+                for (int a = lane; a < na; a += 32) s_gx[(m * npx + y) * nbw + a] = axis_weight(Gx, dd.nx, d.ex[y], a);
+            for (int b = lane; b < nbd; b += 32) s_gy[(m * nbw + b) * npx + y] = axis_weight(Gy, dd.ny, d.ey[y], b);
+        }
+    }
+    __syncthreads();
+    // T[axis][y][a] = sum_x L[axis][y][x] gx_a(x)
+    for (int m = 0; m < L.n_dms; ++m) {
+        const DmDesc& dd = L.desc[m];
+        const RowsDm& d = s_dm[m];
+        const int a0 = d.rng[0], na = d.rng[1] - a0;
+        if ((ROTATED && dd.general) || d.c0 == d.c1) continue;
+        const float* Gx = L.g + dd.gx_off + a0;
+        float* T = s_T + m * 2 * npx * nbw;
+        if (staged) {
+            for (int y = warp; y < npx; y += n_warps)
+                for (int a = lane; a < na; a += 32) {
+                    float tx = 0.0f, ty = 0.0f;
+#pragma unroll 8
+                    for (int x = 0; x < npx; ++x) {
+                        const float g = s_gx[(m * npx + x) * nbw + a];
+                        tx = fmaf(s_L[y * npx + x], g, tx);
+                        ty = fmaf(s_L[(npx + y) * npx + x], g, ty);
+                    }
+                    T[y * nbw + a] = tx;
+                    T[(npx + y) * nbw + a] = ty;
+                }
+        } else {
+            for (int idx = tid; idx < na * npx; idx += nthr) {
+                const int y = idx / na, a = idx - y * na;
+                float tx = 0.0f, ty = 0.0f;
+#pragma unroll 4
+                for (int x = 0; x < npx; ++x) {
+                    const float g = axis_weight(Gx, dd.nx, d.ex[x], a);
+                    tx = fmaf(s_L[y * npx + x], g, tx);
+                    ty = fmaf(s_L[(npx + y) * npx + x], g, ty);
+                }
+                T[y * nbw + a] = tx;
+                T[(npx + y) * nbw + a] = ty;
+            }
+        }
+    }
+    __syncthreads();
     for (int m = 0; m < L.n_dms; ++m) {
         const DmDesc& dd = L.desc[m];
         const RowsDm& d = s_dm[m];
@@ -325,15 +363,7 @@ __global__ void __launch_bounds__(kAdjThreads, ROTATED ? 2 : 8) dm_rows_kernel(P
         const float sign = V[m].sign;
         const float* T = s_T + m * 2 * npx * nbw;
         const float* gy = s_gy + m * npx * nbw;
-        // this part's share of the DM's commands, split at the band's rows
-        const int lo = max(first, dd.cmd0), hi = max(lo, min(last, dd.cmd0 + dd.n_cmd));
-        const int c0 = min(max(dd.cmd0 + d.c0, lo), hi), c1 = min(max(dd.cmd0 + d.c1, c0), hi);
-        if (L.D) {
-            zero_run(out_x + lo, c0 - lo, tid, nthr);
-            zero_run(out_y + lo, c0 - lo, tid, nthr);
-            zero_run(out_x + c1, hi - c1, tid, nthr);
-            zero_run(out_y + c1, hi - c1, tid, nthr);
-        }
+        const int c0 = d.c0, c1 = d.c1;
         for (int j = c0 + tid; j < c1; j += nthr) {
             const int ab = __ldg(L.cmd_act + j), a = (ab & 0xffff) - a0, b = (int)((unsigned)ab >> 16) - b0;
             float vx = 0.0f, vy = 0.0f;
@@ -544,7 +574,7 @@ __global__ void __launch_bounds__(128) phase_adjoint_kernel(ProjLaunch L, float*
 cudaError_t launch_dm_rows(const ProjLaunch& L, int n_px, int sm_count, cudaStream_t s) {
     if (!L.n_valid || !L.n_dms) return cudaSuccess;
     const int nbw = std::max(1, std::min(L.max_band, kAdjMaxBand));
-    const size_t bytes = sizeof(float) * (2 * n_px * n_px + L.n_dms * 3 * n_px * nbw);   // at most 204800
+    const size_t bytes = sizeof(float) * (2 * n_px * n_px + L.n_dms * (n_px <= 16 ? 4 : 3) * n_px * nbw);   // at most 204800
     const auto kernel = L.rotated ? dm_rows_kernel<true> : dm_rows_kernel<false>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
