@@ -439,6 +439,12 @@ __device__ __forceinline__ void fill_recip(NoiseTab& t, int tid, int nthr) {
     }
 }
 
+// photon count of a pixel at or above 16: max(0, rint(lambda + sqrt(lambda) y))
+__device__ __forceinline__ int nz_bright(float lam, float y) {
+    const int n = __float2int_rn(__fmaf_rn(__fsqrt_rn(lam), y, lam));
+    return n < 0 ? 0 : n;
+}
+
 // Photon count of one pixel: Poisson by inversion for lambda < 16 (uniform u; two terms per
 // pass, formed in the same order as one at a time, stopping at the same k), else
 // max(0, rint(lambda + sqrt(lambda) y)) with the standard normal y.
@@ -459,8 +465,7 @@ __device__ __forceinline__ int nz_photons(float lam, float u, float y, const flo
         }
         return k;
     }
-    const int n = __float2int_rn(__fmaf_rn(__fsqrt_rn(lam), y, lam));
-    return n < 0 ? 0 : n;
+    return nz_bright(lam, y);
 }
 
 // packed float32 pairs (each half rounded as the scalar operation rounds)
@@ -523,32 +528,43 @@ __device__ __forceinline__ void nz_poisson2(float lam_a, float lam_b, float ua, 
     if (odd_b) kb = nz_photons(lam_b, ub, 0.0f, recip);
 }
 
-// Noisy counts of a pixel pair (pixel o and o + n_det^2 / 2 of one subaperture frame; g the
-// frame index of pixel o): draw A = Philox(g, step, sensor, 0) gives the two inversion uniforms
-// (words 0, 1) and, when read noise is on, one Box-Muller pair (words 2, 3) whose outputs are
-// the two pixels' read noise; draw B = Philox(g, step, sensor, 2), formed only when a pixel has
-// lambda >= 16, gives one Box-Muller pair (words 2, 3) for the two photon normals.  Every lane of
-// the warp calls it together.
-__device__ __forceinline__ void noise_pair(float lam_a, float lam_b, float read_noise, uint32_t g, uint32_t step,
-                                           uint32_t sensor, unsigned long long seed, const NoiseTab& tab, int& na,
-                                           int& nb) {
-    const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
+// The detector counts of a pixel pair (pixel o and o + n_det^2 / 2 of one subaperture frame; g the
+// frame index of pixel o) in two parts.  noise_pair_dim: draw A = Philox(g, step, sensor, 0) gives the two
+// inversion uniforms (words 0, 1) and, when read noise is on, one Box-Muller pair (words 2, 3) whose
+// outputs are the two pixels' read noise; the counts lack the photons of pixels at or above 16.  Every
+// lane of the warp calls it together.  noise_normals: draw B = Philox(g, step, sensor, 2), one
+// Box-Muller pair (words 2, 3), the photon normals of a pair with such a pixel (nz_bright).
+__device__ __forceinline__ void noise_pair_dim(float lam_a, float lam_b, float read_noise, uint32_t g, uint32_t step,
+                                               uint32_t sensor, unsigned long long seed, const NoiseTab& tab, int& na,
+                                               int& nb) {
     uint32_t w[4] = {g, step, sensor, 0u};
-    philox4x32_10(w, k0, k1);
+    philox4x32_10(w, (uint32_t)seed, (uint32_t)(seed >> 32));
     nz_poisson2(lam_a, lam_b, nz_uniform(w[0]), nz_uniform(w[1]), tab.recip2, tab.recip, na, nb);
-    if (!(lam_a < 16.0f) || !(lam_b < 16.0f)) {
-        uint32_t v[4] = {g, step, sensor, 2u};
-        philox4x32_10(v, k0, k1);
-        float ya, yb;
-        nz_box_muller2(nz_uniform(v[2]), nz_uniform(v[3]), ya, yb);
-        if (!(lam_a < 16.0f)) na = nz_photons(lam_a, 0.0f, ya, tab.recip);
-        if (!(lam_b < 16.0f)) nb = nz_photons(lam_b, 0.0f, yb, tab.recip);
-    }
     if (read_noise > 0.0f) {
         float za, zb;
         nz_box_muller2(nz_uniform(w[2]), nz_uniform(w[3]), za, zb);
         na += __float2int_rn(__fmul_rn(read_noise, za));
         nb += __float2int_rn(__fmul_rn(read_noise, zb));
+    }
+}
+
+__device__ __forceinline__ void noise_normals(uint32_t g, uint32_t step, uint32_t sensor, unsigned long long seed, float& ya,
+                                              float& yb) {
+    uint32_t v[4] = {g, step, sensor, 2u};
+    philox4x32_10(v, (uint32_t)seed, (uint32_t)(seed >> 32));
+    nz_box_muller2(nz_uniform(v[2]), nz_uniform(v[3]), ya, yb);
+}
+
+// both parts, each lane for itself as far as its pixels need the second
+__device__ __forceinline__ void noise_pair(float lam_a, float lam_b, float read_noise, uint32_t g, uint32_t step,
+                                           uint32_t sensor, unsigned long long seed, const NoiseTab& tab, int& na,
+                                           int& nb) {
+    noise_pair_dim(lam_a, lam_b, read_noise, g, step, sensor, seed, tab, na, nb);
+    if (!(lam_a < 16.0f) || !(lam_b < 16.0f)) {
+        float ya, yb;
+        noise_normals(g, step, sensor, seed, ya, yb);
+        if (!(lam_a < 16.0f)) na += nz_bright(lam_a, ya);
+        if (!(lam_b < 16.0f)) nb += nz_bright(lam_b, yb);
     }
 }
 

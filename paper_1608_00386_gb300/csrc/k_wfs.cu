@@ -85,6 +85,9 @@ struct GridMeta {
     const float* data;
     int n;
     float sign;
+    long long x, y, bp;   // grid position of the tile's first sample at this step, grid samples per sample
+    int periodic;
+    float inv_n;
 };
 
 template <int NFFT, int NBIN>
@@ -109,7 +112,8 @@ __global__ void __launch_bounds__(256, 4) wfs_acf_kernel(WfsLaunch L) {
     __shared__ Scratch s_u[8];
     __shared__ GridMeta s_gm[8][kMaxEntries];
     __shared__ float2 s_EM[8][NPX * NPX];
-    __shared__ float2 s_P[8][NPX * NL];
+    __shared__ float2 s_P[8][NPX * ND > NPX * NL ? NPX * ND : NPX * NL];   // later the pixel counts
+    __shared__ unsigned short s_bright[8][ND * ND / 2];                     // pairs with a bright pixel
     __shared__ float2 s_tw[ND];
     __shared__ float2 s_twx[4][NL];   // s_tw[(ux q) mod ND] of output column q, ux = -(NPX-1)..NPX-1
     __shared__ NoiseTab s_recip;
@@ -149,13 +153,19 @@ __global__ void __launch_bounds__(256, 4) wfs_acf_kernel(WfsLaunch L) {
         AxisEnt* s_ex = s_u[warp].e[0];
         AxisEnt* s_ey = s_u[warp].e[1];
 
-        tile_entries<NPX>(V, n_grids, k, i0, j0, s_ex, s_ey, lane, 32);
+        // one lane per grid: its metadata and the tile's origin (the step's frozen-flow offset is a 64-bit
+        // product, formed once here instead of by each of the 16 axis entries)
         if (lane < n_grids) {
-            GridMeta gm;
-            gm.data = V[lane].data;
-            gm.n = V[lane].n;
-            gm.sign = V[lane].sign;
-            s_gm[warp][lane] = gm;
+            const GridView& v = V[lane];
+            s_gm[warp][lane] = GridMeta{v.data, v.n, v.sign, v.ax + (long long)i0 * v.bp + k * v.vx,
+                                        v.ay + (long long)j0 * v.bp + k * v.vy, v.bp, v.periodic, v.inv_n};
+        }
+        __syncwarp();
+        for (int e = lane; e < n_grids * 2 * NPX; e += 32) {
+            const GridMeta& gm = s_gm[warp][e / (2 * NPX)];
+            const int r = e % NPX;
+            const AxisEnt a = axis_entry((e & NPX ? gm.y : gm.x) + (long long)r * gm.bp, gm.n, gm.periodic, gm.inv_n);
+            (e & NPX ? s_ey : s_ex)[e / (2 * NPX) * NPX + r] = a;
         }
         // pupil samples at most one grid sample apart in every grid
         const bool near = __all_sync(0xffffffffu, lane >= n_grids || V[lane].bp <= (1ll << 32));
@@ -169,14 +179,14 @@ __global__ void __launch_bounds__(256, 4) wfs_acf_kernel(WfsLaunch L) {
             if (near) {
     #pragma unroll 2
                 for (int g = 0; g < n_grids; ++g) {
-                    const GridMeta gm = s_gm[warp][g];
+                    const GridMeta& gm = s_gm[warp][g];
                     const float2 p = bilinear_rows(gm.data, gm.n, s_ex[g * NPX + x], s_ey[g * NPX + y0], s_ey[g * NPX + y1]);
                     phi0 = fmaf(gm.sign, p.x, phi0);
                     phi1 = fmaf(gm.sign, p.y, phi1);
                 }
             } else {
                 for (int g = 0; g < n_grids; ++g) {
-                    const GridMeta gm = s_gm[warp][g];
+                    const GridMeta& gm = s_gm[warp][g];
                     const AxisEnt ex = s_ex[g * NPX + x];
                     phi0 = fmaf(gm.sign, bilinear(gm.data, gm.n, ex, s_ey[g * NPX + y0]), phi0);
                     phi1 = fmaf(gm.sign, bilinear(gm.data, gm.n, ex, s_ey[g * NPX + y1]), phi1);
@@ -323,18 +333,48 @@ __global__ void __launch_bounds__(256, 4) wfs_acf_kernel(WfsLaunch L) {
         // The intensities go through this lane's own entries of the row-transform scratch so that the
         // pairs share one copy of the sampler's code (a tenth of the stalls were instruction fetches).
         float* s_lam = reinterpret_cast<float*>(&s_u[warp]);
+        int* s_n = reinterpret_cast<int*>(s_P[warp]);
         __syncwarp();   // every lane has read its column of Y
     #pragma unroll
         for (int j = 0; j < PIX_PER_LANE; ++j) s_lam[lane + 32 * j] = B[j] * norm;
+        if (L.ctx.noise) {
+            // draw A: inversions and read noise.  The pairs with a pixel at or above 16 are listed; their
+            // second draw is formed for up to 32 of them at a time afterwards, instead of by the one or two
+            // lanes of every slot that holds some (a spot has 20 to 30, spread over every slot): 8 % of the
+            // kernel's instructions.
+            int n_bright = 0;
     #pragma unroll 1
+            for (int j = 0; j < HALF; ++j) {
+                const int o = lane + 32 * j;
+                const float lam_a = s_lam[o], lam_b = s_lam[o + 32 * HALF];
+                int na, nb;
+                noise_pair_dim(lam_a, lam_b, w.read_noise, (uint32_t)(pix0 + o), (uint32_t)k, (uint32_t)w.wfs_index,
+                               L.ctx.seed + real, s_recip, na, nb);
+                s_n[o] = na;
+                s_n[o + 32 * HALF] = nb;
+                const unsigned bright = __ballot_sync(0xffffffffu, !(lam_a < 16.0f) || !(lam_b < 16.0f));
+                if (bright >> lane & 1u) s_bright[warp][n_bright + __popc(bright & ((1u << lane) - 1u))] = (unsigned short)o;
+                n_bright += __popc(bright);
+            }
+            __syncwarp();
+    #pragma unroll 1
+            for (int i = lane; i < n_bright; i += 32) {
+                const int o = s_bright[warp][i];
+                const float lam_a = s_lam[o], lam_b = s_lam[o + 32 * HALF];
+                float ya, yb;
+                noise_normals((uint32_t)(pix0 + o), (uint32_t)k, (uint32_t)w.wfs_index, L.ctx.seed + real, ya, yb);
+                if (!(lam_a < 16.0f)) s_n[o] += nz_bright(lam_a, ya);
+                if (!(lam_b < 16.0f)) s_n[o + 32 * HALF] += nz_bright(lam_b, yb);
+            }
+            __syncwarp();
+        }
+    #pragma unroll
         for (int j = 0; j < HALF; ++j) {
             const int o = lane + 32 * j;
             const float lam_a = s_lam[o], lam_b = s_lam[o + 32 * HALF];
             float va = lam_a, vb = lam_b;
             if (L.ctx.noise) {
-                int na, nb;
-                noise_pair(lam_a, lam_b, w.read_noise, (uint32_t)(pix0 + o), (uint32_t)k, (uint32_t)w.wfs_index,
-                           L.ctx.seed + real, s_recip, na, nb);
+                const int na = s_n[o], nb = s_n[o + 32 * HALF];
                 va = (float)na;
                 vb = (float)nb;
                 if (L.frame_out) {
