@@ -665,6 +665,8 @@ cudaError_t enqueue_step(mcao_sim* S, int* launches) {
             rl_i.n_chunks += S->slices[i].n_chunks;
         rl_i.max_ctas = std::max(1, S->sm_count * S->tune.recon_ctas_pct / 100);
         rl_i.sm_count = S->sm_count;
+        rl_i.follows = rl.follows;
+        rl.follows = 1;
         // the last launch follows the last sensor and has the SMs to itself: one block per SM
         if (i == S->slices.size()) rl_i.max_ctas = std::max(rl_i.max_ctas, S->sm_count);
         if ((e = launch_recon(rl_i, S->s3)) != cudaSuccess) return e;
