@@ -25,7 +25,7 @@
 // outputs per block, four of which share an SM's pipe: the last wave of a launch costs a quarter of
 // what 64 x 64 outputs cost.  A dense D (more than a third nonzero) takes the tile products, where
 // each operand read serves 32 outputs.
-// 20 m (7280 x 1870): 46.6 ms before, 15.9 ms now; 39 m (55608 x 8051): 2.2 s before.
+// 20 m (7280 x 1870): 46.6 ms before, 14.1 ms now; 39 m (55608 x 8051): 2.2 s before.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -167,10 +167,12 @@ __global__ void __launch_bounds__(1024) tik_scan_kernel(int* __restrict__ count,
     if (threadIdx.x == 0) count[n] = base;
 }
 
-// columns and values of each row's nonzeros, ascending
+// columns and values of each row's nonzeros, ascending; the values as doubles, since each of them meets
+// thousands of products and a conversion takes the double pipe half as long as a multiply-add (20 m,
+// Gram 885 -> 765 us and product 4400 -> 2700; 2660 is the double pipes' time)
 __global__ void __launch_bounds__(256) tik_row_fill_kernel(const float* __restrict__ D, long long ld, int n_slopes, int n_cmd,
                                                            const int* __restrict__ row, int* __restrict__ col,
-                                                           float* __restrict__ val) {
+                                                           double* __restrict__ val) {
     const int r = blockIdx.x * 8 + threadIdx.x / 32, lane = threadIdx.x & 31;
     if (r >= n_slopes) return;
     int at = row[r];
@@ -181,7 +183,7 @@ __global__ void __launch_bounds__(256) tik_row_fill_kernel(const float* __restri
         if (v != 0.0f) {
             const int p = at + __popc(m & ((1u << lane) - 1u));
             col[p] = c;
-            val[p] = v;
+            val[p] = (double)v;
         }
         at += __popc(m);
     }
@@ -217,7 +219,7 @@ __global__ void __launch_bounds__(32 * kCscWarps) tik_col_fill_kernel(const floa
 // are read while this one is added).
 __global__ void __launch_bounds__(128) tik_gram_sparse_kernel(const int* __restrict__ col_at, const int* __restrict__ col_row,
                                                               const float* __restrict__ col_val, const int* __restrict__ row,
-                                                              const int* __restrict__ col, const float* __restrict__ val,
+                                                              const int* __restrict__ col, const double* __restrict__ val,
                                                               double* __restrict__ G, long long ldg) {
     extern __shared__ double gram_acc[];
     const int a = gridDim.x - 1 - blockIdx.x;   // the longest rows of G first
@@ -226,24 +228,25 @@ __global__ void __launch_bounds__(128) tik_gram_sparse_kernel(const int* __restr
     const int p0 = col_at[a], p1 = col_at[a + 1];
     __syncthreads();
     int q0 = 0, q1 = 0, b = 0;
-    float dsa = 0.0f, v = 0.0f;
+    float dsa = 0.0f;
+    double v = 0.0;
     auto fetch = [&](int p) {
         const int s = col_row[p];
         dsa = col_val[p];
         q0 = row[s];
         q1 = row[s + 1];
         b = q0 + tid < q1 ? col[q0 + tid] : a + 1;
-        v = q0 + tid < q1 ? val[q0 + tid] : 0.0f;
+        v = q0 + tid < q1 ? val[q0 + tid] : 0.0;
     };
     if (p0 < p1) fetch(p0);
     for (int p = p0; p < p1; ++p) {
         const int bb = b, n = q1, first = q0;
-        const double vv = (double)v, d = (double)dsa;
+        const double vv = v, d = (double)dsa;
         if (p + 1 < p1) fetch(p + 1);
         if (bb <= a) gram_acc[bb] = fma(d, vv, gram_acc[bb]);
         for (int q = first + 128 + tid; q < n; q += 128) {
             const int e = col[q];
-            if (e <= a) gram_acc[e] = fma(d, (double)val[q], gram_acc[e]);
+            if (e <= a) gram_acc[e] = fma(d, val[q], gram_acc[e]);
         }
         __syncthreads();
     }
@@ -539,7 +542,7 @@ __global__ void __launch_bounds__(kThreads) tik_xtx_kernel(const double* __restr
 template <typename Out>
 __global__ void __launch_bounds__(256) tik_apply_sparse_kernel(const double* __restrict__ Minv, long long ldm,
                                                                const int* __restrict__ row, const int* __restrict__ col,
-                                                               const float* __restrict__ val, int n_slopes, int n_cmd,
+                                                               const double* __restrict__ val, int n_slopes, int n_cmd,
                                                                Out* __restrict__ R, long long ldr) {
     __shared__ Out s_r[kT][33];
     const int lane = threadIdx.x & 31, w = threadIdx.x / 32;
@@ -553,7 +556,7 @@ __global__ void __launch_bounds__(256) tik_apply_sparse_kernel(const double* __r
 #pragma unroll 4
             for (int p = row[s]; p < p1; ++p) {
                 const double2 m = *reinterpret_cast<const double2*>(M + (long long)__ldg(col + p) * ldm);
-                const double d = (double)__ldg(val + p);
+                const double d = __ldg(val + p);
                 x = fma(m.x, d, x);
                 y = fma(m.y, d, y);
             }
@@ -623,7 +626,8 @@ extern "C" mcao_status mcao_tikhonov_reconstructor(const float* D, int n_slopes,
     cudaStream_t st = (cudaStream_t)stream;
     double *G = nullptr, *X = nullptr, *Linv = nullptr, *d_lam = nullptr;
     int *at = nullptr, *idx = nullptr, *d_err = nullptr;
-    float* val = nullptr;
+    double* val = nullptr;       // of the rows
+    float* col_val = nullptr;
     unsigned char* mask = nullptr;
     cudaError_t e = cudaMalloc(&G, sizeof(double) * npad * npad);
     if (e == cudaSuccess) e = cudaMalloc(&X, sizeof(double) * npad * npad);
@@ -649,11 +653,12 @@ extern "C" mcao_status mcao_tikhonov_reconstructor(const float* D, int n_slopes,
                         n_cmd <= 28000;
     if (e == cudaSuccess && sparse) {
         e = cudaMalloc(&idx, sizeof(int) * 2 * (size_t)(nnz > 0 ? nnz : 1));
-        if (e == cudaSuccess) e = cudaMalloc(&val, sizeof(float) * 2 * (size_t)(nnz > 0 ? nnz : 1));
+        if (e == cudaSuccess) e = cudaMalloc(&val, sizeof(double) * (size_t)(nnz > 0 ? nnz : 1));
+        if (e == cudaSuccess) e = cudaMalloc(&col_val, sizeof(float) * (size_t)(nnz > 0 ? nnz : 1));
     }
     if (e == cudaSuccess && !sparse) e = cudaMalloc(&mask, (size_t)nS * nt);
     auto cleanup = [&]() {
-        for (void* p : {(void*)G, (void*)X, (void*)Linv, (void*)at, (void*)idx, (void*)val, (void*)mask, (void*)d_err}) cudaFree(p);
+        for (void* p : {(void*)G, (void*)X, (void*)Linv, (void*)at, (void*)idx, (void*)val, (void*)col_val, (void*)mask, (void*)d_err}) cudaFree(p);
     };
     if (e != cudaSuccess) {
         cleanup();
@@ -671,8 +676,8 @@ extern "C" mcao_status mcao_tikhonov_reconstructor(const float* D, int n_slopes,
     if (e == cudaSuccess) {
         if (sparse) {
             tik_row_fill_kernel<<<(n_slopes + 7) / 8, 256, 0, st>>>(D, ld, n_slopes, n_cmd, at, idx, val);
-            tik_col_fill_kernel<<<(n_cmd + 31) / 32, 32 * kCscWarps, 0, st>>>(D, ld, n_slopes, n_cmd, col_at, idx + nnz, val + nnz);
-            tik_gram_sparse_kernel<<<n_cmd, 128, gram_smem, st>>>(col_at, idx + nnz, val + nnz, at, idx, val, G, npad);
+            tik_col_fill_kernel<<<(n_cmd + 31) / 32, 32 * kCscWarps, 0, st>>>(D, ld, n_slopes, n_cmd, col_at, idx + nnz, col_val);
+            tik_gram_sparse_kernel<<<n_cmd, 128, gram_smem, st>>>(col_at, idx + nnz, col_val, at, idx, val, G, npad);
         } else {
             tik_mask_kernel<<<dim3(nt, nS), kThreads, 0, st>>>(D, ld, n_slopes, n_cmd, nt, mask);
             tik_gram_kernel<<<(unsigned)((long long)2 * nt * (2 * nt + 1) / 2), kThreads, 0, st>>>(D, ld, n_slopes, n_cmd, nS, nt,
