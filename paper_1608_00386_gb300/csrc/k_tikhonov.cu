@@ -25,7 +25,7 @@
 // outputs per block, four of which share an SM's pipe: the last wave of a launch costs a quarter of
 // what 64 x 64 outputs cost.  A dense D (more than a third nonzero) takes the tile products, where
 // each operand read serves 32 outputs.
-// 20 m (7280 x 1870): 46.6 ms before, 14.1 ms now; 39 m (55608 x 8051): 2.2 s before.
+// 20 m (7280 x 1870): 46.6 ms before, 12.3 ms now; 39 m (55608 x 8051): 2.2 s before.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -349,8 +349,16 @@ __device__ __forceinline__ double reciprocal(double d) {
 // of one SM's pipe).  Factor and inverse one after the other in shared memory took 228 us a block, 6.9
 // of 46.6 ms at 20 m; in one pass with L and its square roots 114 us; 75 us now.  A pivot <= 0
 // (or NaN) sets *err and is replaced by 1 so that the remaining steps stay finite.
+// For k > 0 the block first takes panel k - 1 out of its tile (4c leaves that tile to it), and the
+// update of the other tiles runs at the same time as a programmatic dependent: 114 us on one SM beside
+// the 205 us of an update at 20 m (14.1 -> 12.3 ms a call).  The block asks for more shared memory than it uses, so that no
+// update block shares its SM's double pipe (sharing it, the chain took longer than the update).
+constexpr int kPotrfSmem = 210 * 1024;
+static_assert(kT * (kT + 1) * sizeof(double) <= kPotrfSmem);
 __global__ void __launch_bounds__(256) tik_potrf_kernel(const double* __restrict__ A, long long lda, int k,
                                                         double* __restrict__ Linv, int* __restrict__ err) {
+    extern __shared__ double s_pan[];   // [64][65]: L[k][k - 1]
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     constexpr int kEnt = kT * (kT + 1) / 2, kPer = (kEnt + 255) / 256;
     __shared__ double s_col[2][kT], s_u[2][kT], s_v[2][kT], s_diag[kT];
     const int tid = threadIdx.x;
@@ -364,6 +372,20 @@ __global__ void __launch_bounds__(256) tik_potrf_kernel(const double* __restrict
         if (p < kEnt) tri_index(p, m, c);
         mc[i] = m << 8 | c;
         w[i] = p < kEnt ? A[(o + m) * lda + o + c] : 0.0;
+    }
+    if (k > 0) {
+        for (int q = tid; q < kT * kT; q += 256) s_pan[q / kT * (kT + 1) + q % kT] = A[(o + q / kT) * lda + o - kT + q % kT];
+        __syncthreads();
+        double acc[kPer] = {};
+#pragma unroll 2
+        for (int q = 0; q < kT; ++q)
+#pragma unroll
+            for (int i = 0; i < kPer; ++i) {
+                const int m = min(mc[i] >> 8, kT - 1), c = mc[i] & 255;
+                acc[i] = fma(s_pan[m * (kT + 1) + q], s_pan[c * (kT + 1) + q], acc[i]);
+            }
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) w[i] -= acc[i];
     }
     for (int j = 0; j < kT; ++j) {
         double *col = s_col[j & 1], *u = s_u[j & 1], *v = s_v[j & 1];   // the other pair may still be read
@@ -464,19 +486,21 @@ __global__ void __launch_bounds__(kThreads) tik_panel_kernel(double* __restrict_
     }
 }
 
-// 4c. with L[.][k] and X[k][.] final: A[i][j] -= L[i][k] L[j][k]^T for the lower tiles i >= j > k, and
-// X[m][j] -= L[m][k] X[k][j] for m > k, j <= k, in 32 x 32 blocks of one launch (blocks of the trailing
-// matrix first, in order of rows)
+// 4c. with L[.][k] and X[k][.] final: A[i][j] -= L[i][k] L[j][k]^T for the lower tiles i >= j > k but the
+// first (the next diagonal block's launch takes that one), and X[m][j] -= L[m][k] X[k][j] for m > k,
+// j <= k, in 32 x 32 blocks of one launch (blocks of the trailing matrix first, in order of rows).  It
+// starts beside that launch, whose end the last block waits for: what follows needs both.
 __global__ void __launch_bounds__(kThreads) tik_update_kernel(double* __restrict__ A, double* __restrict__ X, long long ld, int k,
                                                               int nt) {
     __shared__ Chunk ch;
     const int rest = 2 * (nt - k - 1);   // 32-row blocks below
     const long long n_a = (long long)rest * (rest + 1) / 2;
     const long long L0 = (long long)(k + 1) * kT, kc = (long long)k * kT, npad = (long long)nt * kT;
+    const long long b0 = (long long)blockIdx.x + 3;   // three 32 x 32 blocks of the first tile
     double c[2][4] = {};
-    if (blockIdx.x < n_a) {
+    if (b0 < n_a) {
         int i, j;
-        tri_index(blockIdx.x, i, j);
+        tri_index(b0, i, j);
         for (int k0 = 0; k0 < kT; k0 += kS) {
             load_trans(ch.a, A, ld, L0 + i * kS, kc + k0, npad, npad);
             load_trans(ch.b, A, ld, L0 + j * kS, kc + k0, npad, npad);
@@ -491,7 +515,7 @@ __global__ void __launch_bounds__(kThreads) tik_update_kernel(double* __restrict
             for (int b = 0; b < 4; ++b) P[out_row(a) * ld + out_col(b)] -= c[a][b];
         return;
     }
-    const int t = (int)(blockIdx.x - n_a), cols = 2 * (k + 1);
+    const int t = (int)(b0 - n_a), cols = 2 * (k + 1);
     const long long r0 = L0 + (long long)(t / cols) * kS, c0 = (long long)(t % cols) * kS;
     for (int k0 = 0; k0 < kT; k0 += kS) {
         load_trans(ch.a, A, ld, r0, kc + k0, npad, npad);
@@ -505,6 +529,7 @@ __global__ void __launch_bounds__(kThreads) tik_update_kernel(double* __restrict
     for (int a = 0; a < 2; ++a)
 #pragma unroll
         for (int b = 0; b < 4; ++b) P[out_row(a) * ld + out_col(b)] -= c[a][b];
+    if (blockIdx.x == gridDim.x - 1) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // 5. Minv[I][J] = sum_m X[m][I]^T X[m][J] over the 32-row blocks m >= I (X lower triangular) for the
@@ -673,6 +698,7 @@ extern "C" mcao_status mcao_tikhonov_reconstructor(const float* D, int n_slopes,
     if (e == cudaSuccess) e = cudaMemsetAsync(X, 0, sizeof(double) * npad * npad, st);
     if (e == cudaSuccess && sparse)
         e = cudaFuncSetAttribute(tik_gram_sparse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, gram_smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(tik_potrf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPotrfSmem);
     if (e == cudaSuccess) {
         if (sparse) {
             tik_row_fill_kernel<<<(n_slopes + 7) / 8, 256, 0, st>>>(D, ld, n_slopes, n_cmd, at, idx, val);
@@ -684,12 +710,22 @@ extern "C" mcao_status mcao_tikhonov_reconstructor(const float* D, int n_slopes,
                                                                                                  mask, G, npad);
         }
         tik_regularize_kernel<<<1, 1024, 0, st>>>(G, npad, n_cmd, (int)npad, alpha, d_lam);
+        tik_potrf_kernel<<<1, 256, kPotrfSmem, st>>>(G, npad, 0, Linv, d_err);
         for (int k = 0; k < nt; ++k) {
             const long long below = nt - k - 1, rest = 2 * below;
-            tik_potrf_kernel<<<1, 256, 0, st>>>(G, npad, k, Linv, d_err);
             tik_panel_kernel<<<(unsigned)(kT / kStrip * nt), kThreads, 0, st>>>(G, X, npad, k, nt, Linv);
-            if (below > 0)
-                tik_update_kernel<<<(unsigned)(rest * (rest + 1) / 2 + rest * 2 * (k + 1)), kThreads, 0, st>>>(G, X, npad, k, nt);
+            if (below == 0) break;
+            tik_potrf_kernel<<<1, 256, kPotrfSmem, st>>>(G, npad, k + 1, Linv, d_err);
+            cudaLaunchConfig_t cfg{};
+            cfg.gridDim = dim3((unsigned)(rest * (rest + 1) / 2 - 3 + rest * 2 * (k + 1)));
+            cfg.blockDim = dim3(kThreads);
+            cfg.stream = st;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[0].val.programmaticStreamSerializationAllowed = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            cudaLaunchKernelEx(&cfg, tik_update_kernel, G, X, npad, k, nt);
         }
         // M^-1 over the factor
         tik_xtx_kernel<<<(unsigned)((long long)2 * nt * (2 * nt + 1) / 2), kThreads, 0, st>>>(X, npad, 2 * nt, G, npad);
