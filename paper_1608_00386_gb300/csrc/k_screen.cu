@@ -128,8 +128,9 @@ __global__ void __launch_bounds__(kScreenThreads) screen_fft_pass(ScreenPass P) 
 // read straight into the registers and the last stage's outputs stored from them.  Twiddles are
 // formed by the block.  The passes are bound by the instructions of the two Philox draws and
 // Box-Muller pairs per coefficient (pass 1) and by shared memory and the L2 gathers (pass 2).
-// 2048 x 2048: 38 + 19 us; six radix-4 exchanges of the full spectrum and a
-// twiddle kernel took 55 + 40 + 7 us.
+// 2048 x 2048: 37 + 14 us alone, 45 a screen in a row of ten; six radix-4 exchanges of the full
+// spectrum and a twiddle kernel took 55 + 40 + 7.  (Of the 14: 19 with the four transforms' rows
+// starting in the same bank.)
 __device__ __forceinline__ float2 rot4(float2 a) { return make_float2(a.y, -a.x); }   // -i a
 
 // forward 4-point transform of v[0], v[s], v[2 s], v[3 s], in place
@@ -198,7 +199,9 @@ struct HalfFft {
     static constexpr int R3 = N / 256;                     // last stage's radix
     static constexpr int F = NF;
     static constexpr int kThreads = T * F;
-    static constexpr int kRow = N + N / 16;                // padded row in shared memory
+    // padded row in shared memory; where a warp holds points of all F transforms, their rows start in
+    // different banks
+    static constexpr int kRow = N + N / 16 + 16 / F;
     static constexpr int kTw = 15 * 16 + (R3 - 1) * 256;   // twiddles of stages 2 and 3
     static constexpr size_t smem = sizeof(float2) * ((size_t)F * kRow + kTw);
 };
@@ -252,29 +255,39 @@ __device__ __forceinline__ void half_fft(float2 (&v)[16], float2* row, const flo
     }
 }
 
+// 64 registers a thread: the 513 blocks of a 2048 screen are resident at once (73 registers: three per SM, so
+// that a ninth of them ran alone after the others)
 template <int N, int NF>
-__global__ void __launch_bounds__(HalfFft<N, NF>::kThreads) screen_half_rows(ScreenPass P) {
+__global__ void __launch_bounds__(HalfFft<N, NF>::kThreads, 1024 / HalfFft<N, NF>::kThreads) screen_half_rows(ScreenPass P) {
     using H = HalfFft<N, NF>;
     extern __shared__ float4 smem_raw[];
     float2* tw = reinterpret_cast<float2*>(smem_raw);
     const int f = threadIdx.x / H::T, t = threadIdx.x % H::T;
     float2* row = tw + H::kTw + f * H::kRow;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int ky = min((int)blockIdx.x * H::F + f, N / 2);   // a block's spare transforms repeat the last row
     half_twiddles<N>(tw, threadIdx.x, H::kThreads);
     float2 v[16];
     const int my = (N - ky) % N;
+    // conj(c_k + conj(c_-k)) / 2
+    auto draw = [&](int kx, float a) {
+        const float2 z = screen_normals(N, kx, ky, P.key0, P.key1), y = screen_normals(N, (N - kx) % N, my, P.key0, P.key1);
+        row[fft_pad(kx)] = make_float2(a * (z.x + y.x), a * (y.y - z.y));
+    };
+    // kx and N - kx share an amplitude (0 and N / 2 do not, and go together)
 #pragma unroll 2
-    for (int m = 0; m < 16; ++m) {
-        const int kx = t + m * H::T, mx = (N - kx) % N;
-        const float2 z = screen_normals(N, kx, ky, P.key0, P.key1), y = screen_normals(N, mx, my, P.key0, P.key1);
+    for (int m = 0; m < 8; ++m) {
+        const int kx = t + m * H::T;
         const float a = 0.5f * screen_amp(N, kx, ky, P.amp0, P.l2);
-        row[fft_pad(kx)] = make_float2(a * (z.x + y.x), a * (y.y - z.y));   // conj(c_k + conj(c_-k)) / 2
+        draw(kx, a);
+        draw(kx ? N - kx : N / 2, kx ? a : 0.5f * screen_amp(N, N / 2, ky, P.amp0, P.l2));
     }
-    // the thread's own entries back into registers (kept out of them while they are drawn)
+    __syncthreads();
 #pragma unroll
     for (int m = 0; m < 16; ++m) v[m] = row[fft_pad(t + m * H::T)];
     __syncthreads();
     half_fft<N>(v, row, tw, t);
+    asm volatile("griddepcontrol.wait;" ::: "memory");   // nothing above reads or writes global memory
     float2* out = P.dst_c + (size_t)ky * N;
     constexpr int Q = H::R3 > 1 ? 16 / H::R3 : 1;
 #pragma unroll
@@ -292,8 +305,10 @@ __global__ void __launch_bounds__(HalfFft<N, NF>::kThreads) screen_half_cols(Scr
     // neighbouring threads take neighbouring column pairs
     const int f = threadIdx.x % H::F, t = threadIdx.x / H::F;
     float2* row = tw + H::kTw + f * H::kRow;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int x = 2 * (blockIdx.x * H::F + f);
     half_twiddles<N>(tw, threadIdx.x, H::kThreads);
+    asm volatile("griddepcontrol.wait;" ::: "memory");   // the rows
     float2 v[16];
 #pragma unroll
     for (int m = 0; m < 16; ++m) {
@@ -346,10 +361,28 @@ cudaError_t half_passes(ScreenPass P, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)A::smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(cols, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B::smem);
     if (e != cudaSuccess) return e;
-    rows<<<(N / 2 + 1 + A::F - 1) / A::F, A::kThreads, A::smem, s>>>(P);
+    // both passes are programmatic dependents of what is before them on the stream: the columns' blocks
+    // take over the SMs that the rows leave, and the next screen is drawn beside this one's columns.  Each waits
+    // for all of the kernel before it (griddepcontrol.wait) ahead of its first access to global memory.
+    // A captured launch may follow the allocation of its buffers, not a kernel: plain there.
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if ((e = cudaStreamIsCapturing(s, &capture)) != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = capture == cudaStreamCaptureStatusNone ? 1 : 0;
+    cfg.stream = s;
+    cfg.gridDim = dim3((N / 2 + 1 + A::F - 1) / A::F);
+    cfg.blockDim = dim3(A::kThreads);
+    cfg.dynamicSmemBytes = A::smem;
+    if ((e = cudaLaunchKernelEx(&cfg, rows, P)) != cudaSuccess) return e;
     P.src = P.dst_c;
-    cols<<<N / 2 / B::F, B::kThreads, B::smem, s>>>(P);
-    return cudaGetLastError();
+    cfg.gridDim = dim3(N / 2 / B::F);
+    cfg.blockDim = dim3(B::kThreads);
+    cfg.dynamicSmemBytes = B::smem;
+    return cudaLaunchKernelEx(&cfg, cols, P);
 }
 
 }  // namespace
