@@ -61,6 +61,74 @@ __device__ __forceinline__ float2 screen_normals(int n, int kx, int ky, uint32_t
     return z;
 }
 
+// two of them at once, coefficients (kx, ky) and (lx, ly): the same operations in the same order, the
+// polynomials of both on packed pairs (2048: 45 us a screen with each by itself, 43 so)
+__device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
+    unsigned long long d;
+    asm("{\n\t.reg .b64 ra, rb, rc;\n\tmov.b64 ra, {%1, %2};\n\tmov.b64 rb, {%3, %4};\n\t"
+        "mov.b64 rc, {%5, %6};\n\tfma.rn.f32x2 %0, ra, rb, rc;\n\t}"
+        : "=l"(d)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(d));
+    return r;
+}
+__device__ __forceinline__ float2 fmul2(float2 a, float2 b) { return f2_unpack(f2_mul(f2_pack(a.x, a.y), f2_pack(b.x, b.y))); }
+__device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
+
+__device__ __forceinline__ void screen_normals2(int n, int kx, int ky, int lx, int ly, uint32_t key0, uint32_t key1, float2& z,
+                                                float2& y) {
+    uint32_t w[4] = {(uint32_t)ky * (uint32_t)n + (uint32_t)kx, 0u, 0u, 1u};
+    uint32_t v[4] = {(uint32_t)ly * (uint32_t)n + (uint32_t)lx, 0u, 0u, 1u};
+    philox4x32_10(w, key0, key1);
+    philox4x32_10(v, key0, key1);
+    // log of the first uniforms (nz_log)
+    const float u[2] = {nz_uniform(w[0]), nz_uniform(v[0])};
+    float m[2], e[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const uint32_t b = __float_as_uint(u[i]);
+        int x = (int)((b >> 23) & 0xffu) - 127;
+        m[i] = __uint_as_float((b & 0x007fffffu) | 0x3f800000u);
+        if (m[i] > 1.41421356f) {
+            m[i] = __fmul_rn(m[i], 0.5f);
+            x += 1;
+        }
+        e[i] = (float)x;
+    }
+    const float2 s = make_float2(__fmul_rn(__fsub_rn(m[0], 1.0f), __frcp_rn(__fadd_rn(m[0], 1.0f))),
+                                 __fmul_rn(__fsub_rn(m[1], 1.0f), __frcp_rn(__fadd_rn(m[1], 1.0f))));
+    const float2 s2 = fmul2(s, s), ef = make_float2(e[0], e[1]);
+    float2 p = ffma2(both(1.11111112e-01f), s2, both(1.42857149e-01f));
+    p = ffma2(p, s2, both(2.00000003e-01f));
+    p = ffma2(p, s2, both(3.33333343e-01f));
+    p = ffma2(p, s2, both(1.0f));
+    const float2 lm = fmul2(fmul2(both(2.0f), s), p);
+    const float2 lg = fmul2(both(-2.0f), ffma2(ef, both(0.693145752f), ffma2(ef, both(1.42860677e-06f), lm)));
+    const float2 rad = make_float2(__fsqrt_rn(lg.x), __fsqrt_rn(lg.y));
+    // cosine and sine of the second (nz_sincos2pi)
+    const float2 t = make_float2(nz_uniform(w[1]), nz_uniform(v[1]));
+    const float2 t4 = fmul2(both(4.0f), t);
+    const float2 q = make_float2(rintf(t4.x), rintf(t4.y));
+    const float2 g = fmul2(ffma2(both(-0.25f), q, t), both(6.28318548f));   // u - q / 4 is exact either way
+    const float2 g2 = fmul2(g, g);
+    float2 a = ffma2(both(2.75573188e-06f), g2, both(-1.98412701e-04f));
+    a = ffma2(a, g2, both(8.33333377e-03f));
+    a = ffma2(a, g2, both(-1.66666672e-01f));
+    const float2 sp = ffma2(fmul2(a, g2), g, g);
+    a = ffma2(both(2.48015876e-05f), g2, both(-1.38888892e-03f));
+    a = ffma2(a, g2, both(4.16666679e-02f));
+    a = ffma2(a, g2, both(-0.5f));
+    const float2 cp = ffma2(a, g2, both(1.0f));
+    auto turn = [](float r, float qf, float sn, float cs) {
+        const int k = ((int)qf) & 3;
+        const float c = (k & 1) ? sn : cs, b = (k & 1) ? cs : sn;
+        return make_float2(__fmul_rn(r, (k == 1 || k == 2) ? -c : c), __fmul_rn(r, (k >= 2) ? -b : b));
+    };
+    z = turn(rad.x, q.x, sp.x, cp.x);
+    y = turn(rad.y, q.y, sp.y, cp.y);
+}
+
 // a_k = amp0 x^(-11/12), x = kx'^2 + ky'^2 + l2 (the spectrum in cell units), 0 at DC; a_-k = a_k.  With
 // x = 2^e m the power of two leaves the logarithm, whose rounding at the size of log2(x) would otherwise
 // be most of the screen's error: 2^(-11 e / 12) = 2^i 2^(k / 12), the rest an exponent within (-1, 1).
@@ -128,7 +196,7 @@ __global__ void __launch_bounds__(kScreenThreads) screen_fft_pass(ScreenPass P) 
 // read straight into the registers and the last stage's outputs stored from them.  Twiddles are
 // formed by the block.  The passes are bound by the instructions of the two Philox draws and
 // Box-Muller pairs per coefficient (pass 1) and by shared memory and the L2 gathers (pass 2).
-// 2048 x 2048: 37 + 14 us alone, 45 a screen in a row of ten; six radix-4 exchanges of the full
+// 2048 x 2048: 35 + 14 us alone, 43 a screen in a row of ten; six radix-4 exchanges of the full
 // spectrum and a twiddle kernel took 55 + 40 + 7.  (Of the 14: 19 with the four transforms' rows
 // starting in the same bank.)
 __device__ __forceinline__ float2 rot4(float2 a) { return make_float2(a.y, -a.x); }   // -i a
@@ -271,7 +339,8 @@ __global__ void __launch_bounds__(HalfFft<N, NF>::kThreads, 1024 / HalfFft<N, NF
     const int my = (N - ky) % N;
     // conj(c_k + conj(c_-k)) / 2
     auto draw = [&](int kx, float a) {
-        const float2 z = screen_normals(N, kx, ky, P.key0, P.key1), y = screen_normals(N, (N - kx) % N, my, P.key0, P.key1);
+        float2 z, y;
+        screen_normals2(N, kx, ky, (N - kx) % N, my, P.key0, P.key1, z, y);
         row[fft_pad(kx)] = make_float2(a * (z.x + y.x), a * (y.y - z.y));
     };
     // kx and N - kx share an amplitude (0 and N / 2 do not, and go together)
