@@ -32,6 +32,7 @@ __device__ __forceinline__ int2 block_band(const int2* band, long long off, int 
 
 __global__ void __launch_bounds__(kDmThreads, 3) dm_surface_kernel(DmLaunch L) {
     extern __shared__ __align__(16) float dm_sm[];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // see enqueue_step: the sensing launch
     if (blockIdx.x == 0 && blockIdx.y == 0) {
         if (threadIdx.x == 0 && L.st) L.st->k = L.st->k_next;
         for (int i = threadIdx.x; i < L.n_work; i += blockDim.x) L.work[i] = 0u;

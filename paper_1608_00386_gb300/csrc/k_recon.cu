@@ -490,27 +490,6 @@ cudaError_t recon_prepare() {
     return e;
 }
 
-namespace {
-
-// launches kernel(arg); programmatic: it may start once every block of the kernel before it on the stream
-// has let its dependents go or left (griddepcontrol in the kernels says where each waits for that one's end)
-template <class A>
-cudaError_t launch_after(void (*kernel)(A), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool programmatic, const A& arg) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = programmatic ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, arg);
-}
-
-}  // namespace
-
 cudaError_t launch_recon(const ReconLaunch& L, cudaStream_t s) {
     if (L.n_cmd <= 0 || L.len <= 0) return cudaSuccess;
     if (!L.work) return cudaErrorInvalidValue;

@@ -131,6 +131,7 @@ __global__ void __launch_bounds__(256, 4) wfs_acf_kernel(WfsLaunch L) {
         s_twx[q][c] = s_tw[((c - (NPX - 1) + 2 * ND) * q) % ND];
     }
     __syncthreads();  // the last block-wide barrier
+    asm volatile("griddepcontrol.wait;" ::: "memory");   // nothing above reads or writes global memory
     // subapertures: one per warp (no counter), or taken one at a time from the counter, so that
     // warps of blocks that become resident late take only what is left
     auto take = [&]() {
@@ -657,8 +658,8 @@ cudaError_t launch_acf(const WfsLaunch& L, cudaStream_t s) {
     WfsLaunch K = L;
     if (L.ctx.n_real > 1) K.work = nullptr;   // nothing runs beside a batch's sensing: one warp per subaperture
     if (K.work && L.max_blocks > 0 && blocks > (unsigned)L.max_blocks) blocks = (unsigned)L.max_blocks;
-    if (blocks) wfs_acf_kernel<NFFT, NBIN><<<dim3(blocks, (unsigned)L.ctx.n_real), 256, 0, s>>>(K);
-    return cudaGetLastError();
+    if (!blocks) return cudaSuccess;
+    return launch_after(wfs_acf_kernel<NFFT, NBIN>, dim3(blocks, (unsigned)L.ctx.n_real), dim3(256), 0, s, L.follows, K);
 }
 
 template <int NPX, int NFFT, int NBIN>

@@ -175,6 +175,7 @@ struct WfsLaunch {
     // slots that the concurrent reconstructor stream leaves; without one, one warp per subaperture
     unsigned int* work;
     int max_blocks;
+    int follows = 0;         // may start while the surfaces before it on the stream are evaluated
 };
 
 bool wfs_variant_supported(int n_px, int n_fft, int n_bin, bool elongated);
@@ -411,5 +412,22 @@ void tc_destroy(TcProduct* P);
 cudaError_t tc_launch(TcProduct* P, const float* slopes_pad, int pad_stride, int n_real, float alpha, float beta,
                       float* out, int* err, int chunk, cudaStream_t st, int* launches);
 long long tc_bytes(const TcProduct* P);   // bytes of its bfloat16 R
+
+// launches kernel(arg); programmatic: it may start once every block of the kernel before it on the stream
+// has let its dependents go or left (griddepcontrol in the kernels says where each waits for that one's end)
+template <class A>
+cudaError_t launch_after(void (*kernel)(A), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool programmatic, const A& arg) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = programmatic ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, arg);
+}
 
 }  // namespace mcao
