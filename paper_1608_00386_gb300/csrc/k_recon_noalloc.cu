@@ -8,6 +8,7 @@
 // created when the library is loaded on a device and lives until the process exits.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdint>
@@ -20,6 +21,8 @@ namespace {
 
 constexpr long long kScratchFloats = 1ll << 19;   // 524288 partial sums = 2 MiB
 constexpr int kChunk = 4096;                       // slope columns per block (at most)
+constexpr int kMinChunk = 256;                     // not less, where more blocks are wanted
+constexpr int kBlocksPerSm = 16;                   // blocks wanted
 constexpr int kRowsPerWarp = 4;
 constexpr int kRowBlock = 32;
 constexpr int kMaxDevices = 64;
@@ -89,6 +92,7 @@ __global__ void __launch_bounds__(256) noalloc_gemv(const float* __restrict__ R,
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
     }
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (lane == 0) {
         float* p = partial + (size_t)kc * n_cmd;
 #pragma unroll
@@ -97,13 +101,20 @@ __global__ void __launch_bounds__(256) noalloc_gemv(const float* __restrict__ R,
     }
 }
 
+// Eight lanes per row: lane l adds the partial sums l, l + 8, .., then the lanes pairwise, in a fixed
+// order.  It starts beside the product's last blocks and waits for them.
 __global__ void noalloc_reduce(const float* __restrict__ partial, int n_chunks, int n_cmd, float* __restrict__ c,
                                float gain) {
-    int row = blockIdx.x * blockDim.x + threadIdx.x;
-    if (row >= n_cmd) return;
+    const int row = (blockIdx.x * blockDim.x + threadIdx.x) / 8, lane = threadIdx.x & 7;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     float acc = 0.0f;
-    for (int kc = 0; kc < n_chunks; ++kc) acc += partial[(size_t)kc * n_cmd + row];
-    c[row] = fmaf(gain, acc, c[row]);
+    if (row < n_cmd) {
+#pragma unroll 4
+        for (int kc = lane; kc < n_chunks; kc += 8) acc += partial[(size_t)kc * n_cmd + row];
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0 && row < n_cmd) c[row] = fmaf(gain, acc, c[row]);
 }
 
 std::mutex g_mu;
@@ -130,9 +141,13 @@ extern "C" mcao_status mcao_reconstruct_noalloc(const float* R, int n_cmd, int n
     if (((uintptr_t)R) % 16 != 0) return report(err, err_len, MCAO_E_INVALID_ARG, "R must be 16-byte aligned");
     if (!std::isfinite(gain)) return report(err, err_len, MCAO_E_INVALID_ARG, "gain must be finite");
     int n_chunks = (n_slopes + kChunk - 1) / kChunk;
-    int kc_len = (n_slopes + n_chunks - 1) / n_chunks;
-    kc_len = (kc_len + 3) / 4 * 4;
-    n_chunks = (n_slopes + kc_len - 1) / kc_len;
+    int kc_len = 0;
+    auto split = [&]() {
+        kc_len = (n_slopes + n_chunks - 1) / n_chunks;
+        kc_len = (kc_len + 3) / 4 * 4;
+        n_chunks = (n_slopes + kc_len - 1) / kc_len;
+    };
+    split();
     if ((long long)n_chunks * n_cmd > kScratchFloats)
         return report(err, err_len, MCAO_E_SHAPE,
                       "n_cmd x column chunks = %d x %d exceeds the %lld-float scratch of the allocation-free update",
@@ -161,13 +176,35 @@ extern "C" mcao_status mcao_reconstruct_noalloc(const float* R, int n_cmd, int n
         }
         scratch = g_scratch[dev];
     }
+    // shorter chunks where the longest ones leave SMs without blocks, as far as the scratch holds their sums
+    // (us a call with chunks of up to 4096 and a reduction of one thread per row, and now: 300 x 2000 13.3,
+    // 6.2; 1870 x 7280 28.7, 12.5; 1300 x 15000 32.8, 18.4; 41 x 55000 16.4, 8.2; 8051 x 55608 288.1, 284.5
+    // with the same chunks; four to eight blocks per SM or 512 columns: 8.2, 12.4, 20.5, 8.2, 284.5)
+    int sm_count = 0;
+    e = cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return report(err, err_len, MCAO_E_CUDA, "cudaDeviceGetAttribute: %s", cudaGetErrorString(e));
+    const int row_blocks = (n_cmd + kRowBlock - 1) / kRowBlock;
+    const long long want = std::min<long long>({(long long)(kBlocksPerSm * sm_count + row_blocks - 1) / row_blocks,
+                                                (n_slopes + kMinChunk - 1) / kMinChunk, kScratchFloats / n_cmd});
+    if (want > n_chunks) {
+        n_chunks = (int)want;
+        split();
+    }
     cudaStream_t st = (cudaStream_t)stream;
-    dim3 grid((unsigned)((n_cmd + kRowBlock - 1) / kRowBlock), (unsigned)n_chunks);
+    dim3 grid((unsigned)row_blocks, (unsigned)n_chunks);
     noalloc_gemv<<<grid, 256, 0, st>>>(R, n_cmd, n_slopes, ld, s, scratch, kc_len);
     e = cudaGetLastError();
     if (e != cudaSuccess) return report(err, err_len, MCAO_E_CUDA, "product launch: %s", cudaGetErrorString(e));
-    noalloc_reduce<<<(unsigned)((n_cmd + 255) / 256), 256, 0, st>>>(scratch, n_chunks, n_cmd, c, gain);
-    e = cudaGetLastError();
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)((8ll * n_cmd + 255) / 256));
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, noalloc_reduce, (const float*)scratch, n_chunks, n_cmd, c, gain);
     if (e != cudaSuccess) return report(err, err_len, MCAO_E_CUDA, "reduction launch: %s", cudaGetErrorString(e));
     return MCAO_OK;
 }
