@@ -107,11 +107,12 @@ __global__ void __launch_bounds__(256, 6) sci_field_kernel(SciLaunch L0) {
 }
 
 // Strehl of this step from the field partial sums, and the Marechal residual variance (piston removed,
-// amplitude-weighted, science band) from the phase sums; fixed order, double.  One block per
-// realization, launched beside the FFT passes: as an extra block of the row pass it was that pass's
-// longest (8 m: 8.9 us, the column pass of the same size 4.7), and the column pass waited for it.
-__global__ void __launch_bounds__(256) sci_strehl_kernel(SciLaunch L0) {
-    const SciLaunch L = sci_for_real(L0, blockIdx.y);
+// amplitude-weighted, science band) from the phase sums; fixed order, double.  The first block of the
+// column pass forms them, beside the transforms' blocks.  As the last block of the row pass it was that
+// pass's longest and the column pass waited for it (8 m: 20.5 us a step); as a kernel of its own beside
+// the passes a single loop is faster (8 m 18.3, here 20.0) but 63 loops advanced together take 1.86 ms
+// a step instead of 1.34.
+__device__ void strehl_sums(const SciLaunch& L) {
     __shared__ double red[8][4];
     const int tid = threadIdx.x, nthr = blockDim.x;
     double v[4] = {0.0, 0.0, 0.0, 0.0};
@@ -194,13 +195,17 @@ __global__ void __launch_bounds__(256) sci_rows_kernel(SciLaunch L0) {
 
 __global__ void __launch_bounds__(256) sci_cols_kernel(SciLaunch L0) {
     const SciLaunch L = sci_for_real(L0, blockIdx.y);
+    if (blockIdx.x == 0) {
+        strehl_sums(L);
+        return;
+    }
     if (!psf_step(L)) return;
     extern __shared__ float4 smem_raw[];
     float2* A = reinterpret_cast<float2*>(smem_raw);
     float2* B = A + kRowsPerBlock * L.M;
     float2* W = B + kRowsPerBlock * L.M;
     const int tid = threadIdx.x, nthr = blockDim.x;
-    const int c0 = blockIdx.x * kRowsPerBlock;
+    const int c0 = (blockIdx.x - 1) * kRowsPerBlock;
     for (int q = tid; q < L.M; q += nthr) W[q] = L.w[q];
     for (int q = tid; q < kRowsPerBlock * L.M; q += nthr) {
         int r = q / L.M, j = q - r * L.M;
@@ -214,7 +219,7 @@ __global__ void __launch_bounds__(256) sci_cols_kernel(SciLaunch L0) {
         float p = fmaf(v.x, v.x, v.y * v.y);   // frame intensity in float, accumulated in double
         L.psf_t[(long long)(c0 + r) * L.M + j] += (double)p;
     }
-    if (blockIdx.x == 0 && tid == 0) L.acc->n_psf += 1;
+    if (c0 == 0 && tid == 0) L.acc->n_psf += 1;
 }
 
 // Compile-time-size versions of the two FFT passes (2 rows / columns per block, 256 threads);
@@ -263,6 +268,10 @@ __global__ void __launch_bounds__(256) sci_rows_ct(SciLaunch L0) {
 template <int M>
 __global__ void __launch_bounds__(256) sci_cols_ct(SciLaunch L0) {
     const SciLaunch L = sci_for_real(L0, blockIdx.y);
+    if (blockIdx.x == 0) {
+        strehl_sums(L);
+        return;
+    }
     if (!psf_step(L)) return;
     extern __shared__ float4 smem_raw[];
     float2* A = reinterpret_cast<float2*>(smem_raw);
@@ -271,7 +280,7 @@ __global__ void __launch_bounds__(256) sci_cols_ct(SciLaunch L0) {
     const int tid = threadIdx.x, nthr = blockDim.x;
     static_assert((kCtRows * M) % kCtThreads == 0, "whole passes per thread");
     constexpr int PER = kCtRows * M / kCtThreads, PW = (M + kCtThreads - 1) / kCtThreads;
-    const int c0 = blockIdx.x * kCtRows;
+    const int c0 = (blockIdx.x - 1) * kCtRows;
     {
         float2 w[PW], v[PER];
 #pragma unroll
@@ -301,7 +310,7 @@ __global__ void __launch_bounds__(256) sci_cols_ct(SciLaunch L0) {
         const float p = fmaf(v.x, v.x, v.y * v.y);   // frame intensity in float, accumulated in double
         psf[q] = acc[i] + (double)p;
     }
-    if (blockIdx.x == 0 && tid == 0) L.acc->n_psf += 1;
+    if (c0 == 0 && tid == 0) L.acc->n_psf += 1;
 }
 
 template <int M>
@@ -326,7 +335,7 @@ cudaError_t ct_rows(const SciLaunch& L, cudaStream_t s) {
 
 template <int M>
 cudaError_t ct_cols(const SciLaunch& L, cudaStream_t s) {
-    sci_cols_ct<M><<<dim3((unsigned)(M / kCtRows), (unsigned)L.ctx.n_real), 256, ct_smem<M>(), s>>>(L);
+    sci_cols_ct<M><<<dim3((unsigned)(M / kCtRows + 1), (unsigned)L.ctx.n_real), 256, ct_smem<M>(), s>>>(L);
     return cudaGetLastError();
 }
 
@@ -346,11 +355,6 @@ cudaError_t set_smem(const void* fn, size_t bytes) {
 cudaError_t launch_sci_field(const SciLaunch& L, cudaStream_t s) {
     int tiles = (L.N / 8) * (L.N / 8);
     sci_field_kernel<<<dim3((unsigned)((tiles + 7) / 8), (unsigned)L.ctx.n_real), 256, 0, s>>>(L);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_sci_strehl(const SciLaunch& L, cudaStream_t s) {
-    sci_strehl_kernel<<<dim3(1u, (unsigned)L.ctx.n_real), 256, 0, s>>>(L);
     return cudaGetLastError();
 }
 
@@ -416,7 +420,7 @@ cudaError_t launch_sci_cols(const SciLaunch& L, cudaStream_t s) {
     MCAO_SCI_CT_SIZES(MCAO_CT_COLS)
 #undef MCAO_CT_COLS
     size_t sm = fft_smem_bytes(L.M);
-    sci_cols_kernel<<<dim3((unsigned)(L.M / kRowsPerBlock), (unsigned)L.ctx.n_real), 256, sm, s>>>(L);
+    sci_cols_kernel<<<dim3((unsigned)(L.M / kRowsPerBlock + 1), (unsigned)L.ctx.n_real), 256, sm, s>>>(L);
     return cudaGetLastError();
 }
 

@@ -585,14 +585,10 @@ cudaError_t enqueue_step(mcao_sim* S, int* launches) {
         SciLaunch L = make_sci_launch(S, (int)q);
         slot = prof_begin(S, ST_SCIENCE, S->s2);
         if ((e = launch_sci_field(L, S->s2)) != cudaSuccess) return e;
-        cudaEvent_t ev_field = dep_event(S, used);
-        if ((e = cudaEventRecord(ev_field, S->s2)) != cudaSuccess) return e;
-        if ((e = cudaStreamWaitEvent(S->s1, ev_field, 0)) != cudaSuccess) return e;
-        if ((e = launch_sci_strehl(L, S->s1)) != cudaSuccess) return e;
         if ((e = launch_sci_rows(L, S->s2)) != cudaSuccess) return e;
         if ((e = launch_sci_cols(L, S->s2)) != cudaSuccess) return e;
         prof_end(S, slot, S->s2);
-        nl += 4;
+        nl += 3;
     }
     cudaEvent_t ev_sci = dep_event(S, used);
     if ((e = cudaEventRecord(ev_sci, S->s2)) != cudaSuccess) return e;

@@ -300,9 +300,8 @@ struct SciLaunch {
 cudaError_t sci_prepare(int M);   // kernel attributes (outside stream capture)
 size_t sci_smem_bytes(int M);
 cudaError_t launch_sci_field(const SciLaunch& L, cudaStream_t s);
-cudaError_t launch_sci_strehl(const SciLaunch& L, cudaStream_t s);   // after the field, beside the FFT passes
 cudaError_t launch_sci_rows(const SciLaunch& L, cudaStream_t s);
-cudaError_t launch_sci_cols(const SciLaunch& L, cudaStream_t s);
+cudaError_t launch_sci_cols(const SciLaunch& L, cudaStream_t s);   // also the Strehl and phase sums
 
 // ---------------------------------------------------------------------------------------------
 // phase screens (von Karman, FFT method)
