@@ -426,15 +426,6 @@ cudaError_t launch_sci_cols(const SciLaunch& L, cudaStream_t s) {
 
 namespace {
 
-// (long-exposure, instantaneous) Strehl ratio of each science direction from its accumulators
-__global__ void strehl_out_kernel(const SciAcc* acc, int n_sci, double* out) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= n_sci) return;
-    const SciAcc a = acc[q];
-    out[2 * q] = a.n_sr ? a.sr_sum / (double)a.n_sr : 0.0;
-    out[2 * q + 1] = a.sr_last;
-}
-
 // out[j][i] = psf_t[(i + M/2) mod M][(j + M/2) mod M] norm, 32 x 32 tiles through shared memory.  (The host
 // did this over the copied accumulator, one strided read and two remainders per pixel: reading a
 // 1280 x 1280 image took 4.9 ms; under half a millisecond now, most of it the copy.)
@@ -449,8 +440,8 @@ __global__ void __launch_bounds__(256) psf_out_kernel(const double* __restrict__
         if (j0 + y < M && i0 + x < M) out[(size_t)(j0 + y) * M + i0 + x] = tile[x][y] * norm;
 }
 
-// a step's readout into one slot of the device ring (or into page-locked host buffers): the commands copied, the (long, last)
-// Strehl ratios of each science direction formed as strehl_out_kernel does
+// a step's readout into one slot of the device ring (or into page-locked host buffers): the commands copied, the
+// (long-exposure, instantaneous) Strehl ratios of each science direction from its accumulators
 __global__ void readout_kernel(const float* __restrict__ c, int n_cmd, const SciAcc* __restrict__ acc, int n_sci,
                                float* __restrict__ ring_c, double* __restrict__ ring_s) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -474,11 +465,6 @@ cudaError_t launch_readout(const float* c, int n_cmd, const SciAcc* acc, int n_s
                            cudaStream_t s) {
     const int n = std::max(n_cmd, n_sci);
     if (n > 0) readout_kernel<<<(n + 255) / 256, 256, 0, s>>>(c, n_cmd, acc, n_sci, ring_c, ring_s);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_strehl_out(const SciAcc* acc, int n_sci, double* out, cudaStream_t s) {
-    if (n_sci > 0) strehl_out_kernel<<<(n_sci + 63) / 64, 64, 0, s>>>(acc, n_sci, out);
     return cudaGetLastError();
 }
 

@@ -183,7 +183,6 @@ struct mcao_sim {
 
     StepState* d_st = nullptr;
     SciAcc* d_acc = nullptr;
-    double* d_sr_out = nullptr;           // staging of mcao_read_async's Strehl ratios
     double* d_psf_out = nullptr;          // PSF image in output order (allocated by the first image read)
     size_t psf_out_n = 0;
     int* h_err = nullptr;                 // error code of the bounded device waits, in mapped host memory: the
@@ -824,7 +823,6 @@ void destroy_all(mcao_sim* S) {
     dfree(S->d_dm_surf); dfree(S->d_views); dfree(S->d_R); dfree(S->d_chunks); dfree(S->d_rscale); dfree(S->d_c); dfree(S->d_partial);
     dfree(S->d_st); dfree(S->d_acc); dfree(S->d_work); dfree(S->d_psf_out);
     if (S->h_err) cudaFreeHost(S->h_err);
-    dfree(S->d_sr_out);
     dfree(S->d_Rrm);
     dfree(S->d_c_prev); dfree(S->d_dc_prev); dfree(S->d_dc);
     tc_destroy(S->tc);
@@ -1176,7 +1174,6 @@ mcao_status mcao_sim_create(const mcao_config* cfg, mcao_sim** out) {
         CKC(sci_prepare(maxM));
     }
     CKC(dalloc(&S->d_acc, NR * std::max(cfg->n_sci, 1)));
-    CKC(dalloc(&S->d_sr_out, 2 * (size_t)std::max(cfg->n_sci, 1)));
     CKC(cudaMemsetAsync(S->d_acc, 0, sizeof(SciAcc) * NR * std::max(cfg->n_sci, 1), S->s0));
     CKC(dalloc(&S->d_st, 1));
     CKC(cudaMemsetAsync(S->d_st, 0, sizeof(StepState), S->s0));
