@@ -32,7 +32,8 @@
  *     MCAO_E_SHAPE.  mcao_query() returns the element count each getter needs.
  *   - Work is queued on library-owned CUDA streams.  mcao_set_stream() names a caller stream
  *     (for example PyTorch's current stream) that every call orders itself after and that
- *     waits for the call's device work.  Getters synchronise before returning.
+ *     waits for the call's device work; steps and asynchronous readouts are then queued on that
+ *     stream itself.  Getters synchronise before returning.
  */
 #ifndef MCAO_H
 #define MCAO_H
@@ -369,10 +370,10 @@ mcao_status mcao_check_bounded_wait(mcao_sim* sim);
  * return at once: a closed loop can read each step's result without waiting for it.  The values
  * are in place after mcao_sync, or once the stream set by mcao_set_stream passes this point.
  * Host buffers should be pinned (cudaHostAlloc / page-locked) for the copies to overlap the
- * next steps; the caller keeps them alive until then.  The values are first snapshotted on the
- * device (one small kernel after the queued steps, into one of 64 ring slots) and copied to the
- * host from there on a stream of their own, so the next steps do not wait for the copies; a
- * slot is reused once its earlier copy is done.  Errors: MCAO_E_INVALID_ARG (both NULL),
+ * next steps; the caller keeps them alive until then.  Pinned buffers that the device can address are
+ * written by one small kernel after the queued steps.  Other buffers are filled from one of 64 ring
+ * slots on the device, which that kernel writes, by copies on a stream of their own, so the next
+ * steps do not wait for them; a slot is reused once its earlier copy is done.  Errors: MCAO_E_INVALID_ARG (both NULL),
  * MCAO_E_STATE (commands before the DMs are loaded), MCAO_E_CUDA. */
 mcao_status mcao_read_async(mcao_sim* sim, float* commands, double* strehl);
 
@@ -431,8 +432,8 @@ mcao_status mcao_misreg_normal_equations(mcao_sim* sim, int dm, const float* D_m
  *   g_layers    device [n_vec][sum over layers of n_l^2] = (d s / d screen)^T g on every turbulent
  *               layer's screen (the adjoint of the cone-beam projection at this step's frozen-flow
  *               position), layers concatenated in order (or NULL).
- * Outputs are overwritten.  Command and layer gradients are accumulated with atomic adds
- * (summation order not fixed).  Synchronous.  Errors: MCAO_E_INVALID_ARG (null g, n_vec < 1,
+ * Outputs are overwritten.  Layer gradients and the command gradients of rotated DMs are accumulated
+ * with atomic adds (summation order not fixed).  Synchronous.  Errors: MCAO_E_INVALID_ARG (null g, n_vec < 1,
  * every output NULL), MCAO_E_STATE, MCAO_E_UNSUPPORTED, MCAO_E_OOM, MCAO_E_CUDA. */
 mcao_status mcao_slopes_vjp(mcao_sim* sim, const float* g_slopes, int n_vec, float* g_commands, float* g_phase,
                             float* g_layers);
@@ -462,12 +463,12 @@ mcao_status mcao_reconstruct_batch(mcao_sim* sim, const float* slopes, int n_rhs
  *           format mcao_load_reconstructor takes) or float64 (r_fp64 = 1); overwritten.
  *   stream  CUDA stream (cudaStream_t) or NULL for the legacy stream.
  *   lambda  optional host pointer: receives lambda.
- * Every step runs in double precision in the library's kernels on 64 x 64 tiles: the Gram matrix
- * (tiles of D that hold only zeros are skipped: a subaperture sees only nearby actuators), its
- * regularisation, a blocked Cholesky factorisation L L^T, L^(-1), M^(-1) = L^-T L^-1 and
- * -M^(-1) D^T (zero tiles skipped again); float32 output is rounded once, at the store.
- * Temporaries of 2 (64 ceil(n_cmd / 64))^2 doubles are allocated and freed by the call (1.04 GB
- * for n_cmd = 8051).  Synchronous.  Errors: MCAO_E_INVALID_ARG (null pointers, alpha < 0 or not
+ * Every step runs in double precision in the library's kernels: the Gram matrix over the nonzeros of D
+ * (a subaperture sees only nearby actuators; a D with more than a third of nonzeros is taken in
+ * 64 x 64 tiles), its regularisation, a blocked Cholesky factorisation L L^T together with L^(-1),
+ * M^(-1) = L^-T L^-1 and -M^(-1) D^T; float32 output is rounded once, at the store.
+ * Temporaries of 2 (64 ceil(n_cmd / 64))^2 doubles (1.04 GB for n_cmd = 8051) and 20 bytes per nonzero
+ * are allocated and freed by the call.  Synchronous.  Errors: MCAO_E_INVALID_ARG (null pointers, alpha < 0 or not
  * finite, r_fp64 not 0 or 1), MCAO_E_SHAPE, MCAO_E_OOM, MCAO_E_UNSUPPORTED (a Cholesky pivot <= 0:
  * the regularised matrix is not positive definite in double precision; raise alpha), MCAO_E_CUDA.
  * err receives a message on failure (err_len bytes, may be NULL). */
