@@ -16,6 +16,7 @@
 
 #include "device_common.cuh"
 #include "mcao_internal.h"
+#include "row_parts.h"
 
 namespace mcao {
 
@@ -241,7 +242,7 @@ __device__ __forceinline__ void zero_run(float* p, int n, int lane) {
 struct RowsDm {                // one DM's view from the block's subaperture
     AxisEnt ex[kMaxNpx], ey[kMaxNpx];
     int rng[4];                // actuators [a0, a1) x [b0, b1)
-    int c0, c1;                // commands of rows [b0, b1) in the block's part
+    CmdRange cmds;             // commands of rows [b0, b1) in the block's part
 };
 
 // nbw: most actuators per axis on a footprint, at most kAdjMaxBand (shared-memory row length)
@@ -273,8 +274,7 @@ __global__ void __launch_bounds__(kAdjThreads, ROTATED ? 2 : 6) dm_rows_kernel(P
         }
     }
     __syncthreads();
-    const int len = (L.n_cmd + gridDim.z - 1) / gridDim.z, first = min((int)blockIdx.z * len, L.n_cmd);
-    const int last = min(L.n_cmd, first + len);
+    const CmdRange part = command_part(L.n_cmd, (int)gridDim.z, (int)blockIdx.z);
     if (lane == 0 && warp < L.n_dms) {
         // the axis entries ascend (a DM grid does not wrap): the footprint is the first and last
         RowsDm& d = s_dm[warp];
@@ -290,10 +290,7 @@ __global__ void __launch_bounds__(kAdjThreads, ROTATED ? 2 : 6) dm_rows_kernel(P
         if (L.gvec && !dd.general) rng[3] = rng[2];
         for (int q = 0; q < 4; ++q) d.rng[q] = rng[q];
         const int* row0 = L.cmd_act + dd.row_off;          // commands before each DM row, and the total
-        // this part's share of the DM's commands, split at the band's rows
-        const int lo = max(first, dd.cmd0), hi = max(lo, min(last, dd.cmd0 + dd.n_cmd));
-        d.c0 = min(max(dd.cmd0 + row0[min(rng[2], dd.ny)], lo), hi);
-        d.c1 = min(max(dd.cmd0 + row0[min(rng[3], dd.ny)], d.c0), hi);
+        d.cmds = band_in_part(part, dd.cmd0 + row0[min(rng[2], dd.ny)], dd.cmd0 + row0[min(rng[3], dd.ny)]);
     }
     __syncthreads();
     const int row_x = w.slope0 + sd.rank, row_y = row_x + w.n_valid;
@@ -302,15 +299,16 @@ __global__ void __launch_bounds__(kAdjThreads, ROTATED ? 2 : 6) dm_rows_kernel(P
     // the zeros between the DMs' bands, one warp per run and row
     if (L.D)
         for (int r = warp; r < 2 * (L.n_dms + 1); r += n_warps) {
-            const int m = r >> 1, from = m ? s_dm[m - 1].c1 : first, to = m < L.n_dms ? s_dm[m].c0 : last;
-            zero_run((r & 1 ? out_y : out_x) + from, to - from, lane);
+            const int m = r >> 1;
+            const CmdRange z = zeros_between(part, m ? &s_dm[m - 1].cmds : nullptr, m < L.n_dms ? &s_dm[m].cmds : nullptr);
+            zero_run((r & 1 ? out_y : out_x) + z.lo, z.hi - z.lo, lane);
         }
     // weights of the footprint's columns and rows
     for (int m = 0; m < L.n_dms; ++m) {
         const DmDesc& dd = L.desc[m];
         const RowsDm& d = s_dm[m];
         const int a0 = d.rng[0], na = d.rng[1] - a0, b0 = d.rng[2], nbd = d.rng[3] - b0;
-        if ((ROTATED && dd.general) || d.c0 == d.c1) continue;
+        if ((ROTATED && dd.general) || d.cmds.lo == d.cmds.hi) continue;
         const float *Gx = L.g + dd.gx_off + a0, *Gy = L.g + dd.gy_off + b0;
         for (int y = warp; y < npx; y += n_warps) {
             if (staged)
@@ -324,7 +322,7 @@ __global__ void __launch_bounds__(kAdjThreads, ROTATED ? 2 : 6) dm_rows_kernel(P
         const DmDesc& dd = L.desc[m];
         const RowsDm& d = s_dm[m];
         const int a0 = d.rng[0], na = d.rng[1] - a0;
-        if ((ROTATED && dd.general) || d.c0 == d.c1) continue;
+        if ((ROTATED && dd.general) || d.cmds.lo == d.cmds.hi) continue;
         const float* Gx = L.g + dd.gx_off + a0;
         float* T = s_T + m * 2 * npx * nbw;
         if (staged) {
@@ -363,8 +361,7 @@ __global__ void __launch_bounds__(kAdjThreads, ROTATED ? 2 : 6) dm_rows_kernel(P
         const float sign = V[m].sign;
         const float* T = s_T + m * 2 * npx * nbw;
         const float* gy = s_gy + m * npx * nbw;
-        const int c0 = d.c0, c1 = d.c1;
-        for (int j = c0 + tid; j < c1; j += nthr) {
+        for (int j = d.cmds.lo + tid; j < d.cmds.hi; j += nthr) {
             const int ab = __ldg(L.cmd_act + j), a = (ab & 0xffff) - a0, b = (int)((unsigned)ab >> 16) - b0;
             float vx = 0.0f, vy = 0.0f;
             if ((unsigned)a < (unsigned)na && (unsigned)b < (unsigned)nbd) {

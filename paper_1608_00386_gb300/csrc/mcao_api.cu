@@ -1420,7 +1420,6 @@ mcao_status mcao_load_dms(mcao_sim* S, int n_dms, const mcao_dm* dms) {
             } else map.push_back(-1);
         }
         D.cmd0 = ncmd;
-        D.n_cmd = cnt;
         ncmd += cnt;
         S->dm_cmd0[m + 1] = ncmd;
         D.surf_off = surf_total;

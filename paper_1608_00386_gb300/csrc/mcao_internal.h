@@ -125,7 +125,7 @@ struct DmDesc {
     float dx, pitch;     // surface sample pitch, actuator pitch (m)
     float inv2s2;        // 1 / (2 sigma^2) of the influence function (DM coordinates)
     float rc;            // window radius in actuator pitches (weights below 1e-10 left out)
-    int cmd0, n_cmd;     // this DM's block of the command vector
+    int cmd0;            // first command
     int row_off;         // ProjLaunch::cmd_act: commands before each of the ny rows, and n_cmd
 };
 constexpr int kDmTile = 32;
