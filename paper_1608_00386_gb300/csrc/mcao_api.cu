@@ -1642,6 +1642,7 @@ mcao_status mcao_load_reconstructor(mcao_sim* S, int n_cmd, int n_slopes, const 
         CK(cudaMemcpyAsync(S->d_sref, s_ref, sizeof(float) * n_slopes, kind, S->s0));
     else
         CK(cudaMemsetAsync(S->d_sref, 0, sizeof(float) * n_slopes, S->s0));
+    CK(cudaStreamSynchronize(S->s0));   // the next step may run on the caller's stream (begin_async)
     release_graph(S);
     S->recon_loaded = true;
     return MCAO_OK;
