@@ -23,9 +23,9 @@
 // concurrently, hiding their ALU work under the HBM stream.  Inside the step, five warps with
 // two stages each stream faster than three with four (same or less shared memory): the block's
 // warps compete for issue slots with the co-resident sensing warps, and more of them get more
-// turns; rings above 96 KB keep the science kernels off the SM and slow the step.  A slice behind
-// another one is a programmatic dependent launch: its blocks take over the SMs whose warps find no
-// item left while the slice before drains (39 m: 382 -> 375 us a step, 20 m 56.2 -> 50.9; a 20-step
+// turns; rings above 96 KB keep the science kernels off the SM and slow the step.  A slice depends
+// programmatically on the slice before it, and on that one alone (capture_edges.h): its blocks take over
+// the SMs whose warps find no item left while the slice before drains (39 m: 382 -> 375 us a step, 20 m 56.2 -> 50.9; a 20-step
 // 39 m exposure 7500 -> 7440).  Every mbarrier wait is bounded
 // (about one second of clock); on expiry the warp records kErrReconTimeout, waits (bounded)
 // for its copies in flight and exits.
@@ -503,13 +503,12 @@ cudaError_t launch_recon(const ReconLaunch& L, cudaStream_t s) {
         const int more = (n_items + (rounds - 1) * kTmaWarps - 1) / ((rounds - 1) * kTmaWarps);
         if (more <= ctas + ctas / 16 && more <= L.sm_count) ctas = more;
     }
-    // behind another slice: a programmatic dependent of it, so that the slice before drains while this
-    // one fills (figures above)
     const dim3 grid((unsigned)ctas), block(kTmaWarps * 32);
-    if (L.dtype == kReconF32) return launch_after(recon_tma_kernel<kReconF32>, grid, block, sizeof(TmaSmem), s, L.follows, L);
-    if (L.dtype == kReconBF16) return launch_after(recon_tma_kernel<kReconBF16>, grid, block, sizeof(TmaSmem), s, L.follows, L);
-    if (L.dtype == kReconE4M3) return launch_after(recon_tma_kernel<kReconE4M3>, grid, block, sizeof(TmaSmem), s, L.follows, L);
-    return cudaErrorInvalidValue;
+    if (L.dtype == kReconF32) recon_tma_kernel<kReconF32><<<grid, block, sizeof(TmaSmem), s>>>(L);
+    else if (L.dtype == kReconBF16) recon_tma_kernel<kReconBF16><<<grid, block, sizeof(TmaSmem), s>>>(L);
+    else if (L.dtype == kReconE4M3) recon_tma_kernel<kReconE4M3><<<grid, block, sizeof(TmaSmem), s>>>(L);
+    else return cudaErrorInvalidValue;
+    return cudaGetLastError();
 }
 
 cudaError_t launch_recon_scales(const float* src, int rows, int cols, int ld, float* scale, cudaStream_t s) {

@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "../../include/mcao.h"
+#include "capture_edges.h"
 #include "mcao_internal.h"
 
 using namespace mcao;
@@ -652,6 +653,7 @@ cudaError_t enqueue_step(mcao_sim* S, int* launches) {
     rl.dc_prev = S->d_dc_prev;
     rl.n_real = 1;
     // a launch takes the following slices too while they wait for the same sensing launch
+    cudaGraphNode_t slice = nullptr;   // the slice launched before
     for (size_t i = 0; i < S->slices.size();) {
         cudaEvent_t last = nullptr;
         for (int w : S->slice_wfs[i]) {
@@ -665,11 +667,13 @@ cudaError_t enqueue_step(mcao_sim* S, int* launches) {
             rl_i.n_chunks += S->slices[i].n_chunks;
         rl_i.max_ctas = std::max(1, S->sm_count * S->tune.recon_ctas_pct / 100);
         rl_i.sm_count = S->sm_count;
-        rl_i.follows = rl.follows;
         rl.follows = 1;
         // the last launch follows the last sensor and has the SMs to itself: one block per SM
         if (i == S->slices.size()) rl_i.max_ctas = std::max(rl_i.max_ctas, S->sm_count);
+        // it fills while the slice before drains; its slopes it reads at once, so the sensing is complete
+        if ((e = overlap_captured(S->s3, slice)) != cudaSuccess) return e;
         if ((e = launch_recon(rl_i, S->s3)) != cudaSuccess) return e;
+        if ((e = captured_kernel(S->s3, &slice)) != cudaSuccess) return e;
         prof_end(S, slot, S->s3);
         ++nl;
     }

@@ -249,7 +249,6 @@ struct ReconLaunch {
     const float* scale; // per-row scales (kReconE4M3), else null
     float* partial;     // [n_chunks][n_cmd]
     int max_ctas;       // grid size cap (0: enough blocks for every item); may be passed by a sixteenth, up
-    int follows;        // another slice comes before it on the stream: start while that one drains
     int sm_count;       // to the number of SMs, where that saves a round of items
     unsigned int* work; // item counter, zero when the launch starts
     int* err;           // set to a nonzero code if a bounded wait gives up
