@@ -76,6 +76,10 @@ __device__ __forceinline__ float bilinear(const float* data, int n, AxisEnt ex, 
     return fmaf(ey.t, bot - top, top);
 }
 
+// Q32.32 step between adjacent samples that bilinear_rows takes: forward, at most one grid sample (a beam
+// that has crossed its axis, under a DM above its star, samples that DM backwards)
+__device__ __forceinline__ bool rows_overlap(long long bp) { return bp >= 0 && bp <= (1ll << 32); }
+
 // bilinear samples of two vertically adjacent positions (column entry ex, row entries e0 and e1) at most
 // one grid sample apart: the second's cell is the first's or the one below, so three grid rows serve
 // both, with the same interpolations as two calls of bilinear

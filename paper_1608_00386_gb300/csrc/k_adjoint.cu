@@ -35,17 +35,23 @@ __device__ __forceinline__ float axis_weight(const float* G, int na, AxisEnt e, 
     return (1.0f - e.t) * G[(long long)(e.idx & 0xffff) * na + a] + e.t * G[(long long)(e.idx >> 16) * na + a];
 }
 
-// Actuators [a0, a1) x [b0, b1) of a DM that act on surface samples [cx0, cx1] x [cy0, cy1]: for a
+// surface samples [x, y] that a run of adjacent pupil samples meets, from its first and last entries:
+// they ascend, or descend under a DM above the star (a DM grid does not wrap)
+__device__ __forceinline__ int2 footprint(AxisEnt a, AxisEnt b) {
+    return make_int2(min(a.idx & 0xffff, b.idx & 0xffff), max(a.idx >> 16, b.idx >> 16));
+}
+
+// Actuators [a0, a1) x [b0, b1) of a DM that act on surface samples [cx.x, cx.y] x [cy.x, cy.y]: for a
 // separable DM the union of the forward's per-tile bands over the tiles the footprint touches, for a
 // rotated one the actuators within rc pitches of the footprint's corners.
-__device__ void actuator_range(const DmDesc& dd, const int2* band, int cx0, int cx1, int cy0, int cy1, int (&rng)[4]) {
+__device__ void actuator_range(const DmDesc& dd, const int2* band, int2 cx, int2 cy, int (&rng)[4]) {
     int a0 = dd.nx, a1 = 0, b0 = dd.ny, b1 = 0;
     if (dd.general) {
         const float c0 = 0.5f * (float)(dd.surf_n - 1), ca = 0.5f * (float)(dd.nx - 1), cb = 0.5f * (float)(dd.ny - 1);
         float lo_a = 1e30f, hi_a = -1e30f, lo_b = 1e30f, hi_b = -1e30f;
         for (int c = 0; c < 4; ++c) {
-            const float x = ((float)((c & 1) ? cx1 : cx0) - c0) * dd.dx - dd.shx;
-            const float y = ((float)((c & 2) ? cy1 : cy0) - c0) * dd.dx - dd.shy;
+            const float x = ((float)((c & 1) ? cx.y : cx.x) - c0) * dd.dx - dd.shx;
+            const float y = ((float)((c & 2) ? cy.y : cy.x) - c0) * dd.dx - dd.shy;
             const float ua = (dd.cr * x + dd.sr * y) * dd.inv_mag / dd.pitch + ca;
             const float ub = (-dd.sr * x + dd.cr * y) * dd.inv_mag / dd.pitch + cb;
             lo_a = fminf(lo_a, ua); hi_a = fmaxf(hi_a, ua);
@@ -54,11 +60,11 @@ __device__ void actuator_range(const DmDesc& dd, const int2* band, int cx0, int 
         a0 = max(0, (int)ceilf(lo_a - dd.rc)); a1 = min(dd.nx - 1, (int)floorf(hi_a + dd.rc)) + 1;
         b0 = max(0, (int)ceilf(lo_b - dd.rc)); b1 = min(dd.ny - 1, (int)floorf(hi_b + dd.rc)) + 1;
     } else {
-        for (int t = cx0 / kDmTile; t <= cx1 / kDmTile; ++t) {
+        for (int t = cx.x / kDmTile; t <= cx.y / kDmTile; ++t) {
             const int2 bt = band[dd.tband_x + t];
             if (bt.y > bt.x) { a0 = min(a0, bt.x); a1 = max(a1, bt.y); }
         }
-        for (int t = cy0 / kDmTile; t <= cy1 / kDmTile; ++t) {
+        for (int t = cy.x / kDmTile; t <= cy.y / kDmTile; ++t) {
             const int2 bt = band[dd.tband_y + t];
             if (bt.y > bt.x) { b0 = min(b0, bt.x); b1 = max(b1, bt.y); }
         }
@@ -276,12 +282,10 @@ __global__ void __launch_bounds__(kAdjThreads, ROTATED ? 2 : 6) dm_rows_kernel(P
     __syncthreads();
     const CmdRange part = command_part(L.n_cmd, (int)gridDim.z, (int)blockIdx.z);
     if (lane == 0 && warp < L.n_dms) {
-        // the axis entries ascend (a DM grid does not wrap): the footprint is the first and last
         RowsDm& d = s_dm[warp];
         const DmDesc& dd = L.desc[warp];
         int rng[4];
-        actuator_range(dd, L.band, d.ex[0].idx & 0xffff, d.ex[npx - 1].idx >> 16, d.ey[0].idx & 0xffff,
-                       d.ey[npx - 1].idx >> 16, rng);
+        actuator_range(dd, L.band, footprint(d.ex[0], d.ex[npx - 1]), footprint(d.ey[0], d.ey[npx - 1]), rng);
         if (rng[1] - rng[0] > nbw || rng[3] - rng[2] > nbw) {
             atomicExch(L.err, 1);
             rng[1] = rng[0];
@@ -424,11 +428,12 @@ __global__ void dm_range_kernel(ProjLaunch L) {
     const SubapDev sd = L.subaps[i - m * L.n_valid];
     const WfsDev& w = L.ctx.wfs[sd.wfs];
     const GridView& v = L.ctx.views[L.real * L.ctx.view_stride + (long long)sd.wfs * L.ctx.n_grids + L.n_layers + m];
-    auto at = [&](long long a, int i0, int q) { return axis_entry(a + (long long)(i0 + q) * v.bp, v.n, v.periodic, v.inv_n).idx; };
-    const int i0 = sd.sx * w.n_px, j0 = sd.sy * w.n_px;
+    auto at = [&](long long a, int i) {
+        return footprint(axis_entry(a + (long long)i * v.bp, v.n, v.periodic, v.inv_n),
+                         axis_entry(a + (long long)(i + w.n_px - 1) * v.bp, v.n, v.periodic, v.inv_n));
+    };
     int rng[4];
-    actuator_range(L.desc[m], L.band, at(v.ax, i0, 0) & 0xffff, at(v.ax, i0, w.n_px - 1) >> 16, at(v.ay, j0, 0) & 0xffff,
-                   at(v.ay, j0, w.n_px - 1) >> 16, rng);
+    actuator_range(L.desc[m], L.band, at(v.ax, sd.sx * w.n_px), at(v.ay, sd.sy * w.n_px), rng);
     if (rng[1] - rng[0] > kAdjMaxBand || rng[3] - rng[2] > kAdjMaxBand) atomicExch(L.err, 1);
 }
 
@@ -460,8 +465,8 @@ __global__ void __launch_bounds__(256) dm_project_x(ProjLaunch L, const float* _
     const int tiles = (N + 31) / 32;
     for (int t = threadIdx.x; t < tiles; t += 256) {
         int lo = dd.nx, hi = 0;
-        const int t1 = (entry(min(32 * t + 32, N) - 1).idx >> 16) / kDmTile;
-        for (int q = (entry(32 * t).idx & 0xffff) / kDmTile; q <= t1; ++q) {
+        const int2 c = footprint(entry(32 * t), entry(min(32 * t + 32, N) - 1));
+        for (int q = c.x / kDmTile; q <= c.y / kDmTile; ++q) {
             const int2 bt = L.band[dd.tband_x + q];
             if (bt.y > bt.x) { lo = min(lo, bt.x); hi = max(hi, bt.y); }
         }

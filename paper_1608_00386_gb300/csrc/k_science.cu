@@ -52,13 +52,13 @@ __global__ void __launch_bounds__(256, 6) sci_field_kernel(SciLaunch L0) {
     tile_entries<8>(V, n_grids, L.ctx.st->k, i0, j0, s_ex[warp], s_ey[warp], lane, 32);
     __syncwarp();
     // phase of samples (x, 2h) and (x, 2h + 1), h = lane / 8: where samples lie at most one grid sample
-    // apart (bp <= 1, here for every grid) the second row's cell is the first's or the next one, so
+    // apart (rows_overlap, here for every grid) the second row's cell is the first's or the next one, so
     // that three grid rows serve both: 6 loads instead of 8, two grids' loads in flight together.
     // The kernel waits for these gathers: 32.7 us before, 22.8 us now at 640 x 640 samples and 13 grids.
     // (Four grids in flight and 80 registers: 2.4 us less a step at 20 m, but 6 us more at 39 m, where the
     // blocks take the laser stars' places.)
     if (lane < n_grids) s_gm[warp][lane] = SciGrid{V[lane].data, V[lane].n, V[lane].sign};
-    const bool near = __all_sync(0xffffffffu, lane >= n_grids || V[lane].bp <= (1ll << 32));
+    const bool near = __all_sync(0xffffffffu, lane >= n_grids || rows_overlap(V[lane].bp));
     __syncwarp();
     const int x = lane & 7, yy = (lane >> 3) * 2;
     float p0 = 0.0f, p1 = 0.0f;

@@ -168,8 +168,8 @@ __global__ void __launch_bounds__(256, 4) wfs_acf_kernel(WfsLaunch L) {
             const AxisEnt a = axis_entry((e & NPX ? gm.y : gm.x) + (long long)r * gm.bp, gm.n, gm.periodic, gm.inv_n);
             (e & NPX ? s_ey : s_ex)[e / (2 * NPX) * NPX + r] = a;
         }
-        // pupil samples at most one grid sample apart in every grid
-        const bool near = __all_sync(0xffffffffu, lane >= n_grids || V[lane].bp <= (1ll << 32));
+        // pupil samples at most one grid sample apart, forward, in every grid
+        const bool near = __all_sync(0xffffffffu, lane >= n_grids || rows_overlap(V[lane].bp));
         __syncwarp();
 
         // field E = A exp(i (scale phi - pi (x + y) / N)): lane -> column x, rows y0 and y0 + 1, with

@@ -1953,7 +1953,7 @@ static int footprint_band(const mcao_sim* S, const WfsRun& r) {
         if (W.p.n_px != r.n_px) continue;
         for (int m = 0; m < S->n_dms; ++m) {
             const DmDesc& D = S->dm_desc[m];
-            const double f = W.p.type == MCAO_WFS_LGS ? 1.0 - S->dms[m].alt_m / W.p.height : 1.0;
+            const double f = W.p.type == MCAO_WFS_LGS ? std::fabs(1.0 - S->dms[m].alt_m / W.p.height) : 1.0;
             const double side = (double)W.p.n_px * W.dx * f / S->dms[m].surf_dx + 3.0;   // surface samples
             if (D.general) {
                 most = std::max(most, (int)std::ceil(1.5 * side * S->dms[m].surf_dx * D.inv_mag / S->dms[m].pitch_m + 2.0 * D.rc) + 2);
