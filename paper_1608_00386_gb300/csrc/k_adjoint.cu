@@ -409,8 +409,9 @@ __global__ void __launch_bounds__(kAdjThreads, ROTATED ? 2 : 6) dm_rows_kernel(P
                 vy *= sign;
                 if (L.gvec)
                     for (int vv = 0; vv < L.n_vec; ++vv) {
-                        const float* g = L.gvec + (long long)vv * L.n_slopes;
-                        const float add = fmaf(g[row_x], vx, g[row_y] * vy);
+                        const float gx = L.gvec[(long long)vv * L.n_slopes + row_x], gy = L.gvec[(long long)vv * L.n_slopes + row_y];
+                        // a slope that the vector leaves out adds nothing, a NaN derivative neither
+                        const float add = fmaf(gx, gx != 0.0f ? vx : 0.0f, gy * (gy != 0.0f ? vy : 0.0f));
                         if (add != 0.0f) atomicAdd(L.gc + (long long)vv * L.n_cmd + j, add);
                     }
             }
@@ -549,8 +550,9 @@ __global__ void __launch_bounds__(1024) dm_project_y(ProjLaunch L, int n_wfs, co
 // Per subaperture and vector: g_phi = g_v[x slope] L_x + g_v[y slope] L_y on its pupil samples,
 // stored in g_phase[v][sensor's offset + (j0 + y) N + i0 + x] and/or scattered onto the layers (the
 // adjoint of the periodic bilinear sampling at the frozen-flow position of the step) in
-// g_layers[v][...].  The subapertures of every sensor in one launch, block y = vector.
-__global__ void __launch_bounds__(128) phase_adjoint_kernel(ProjLaunch L, float* g_phase, long long phase_stride,
+// g_layers[v][...].  The subapertures of every sensor in one launch, block y = vector.  proj, for the
+// command gradients, is laid out as g_phase and leaves slopes with g = 0 out: their derivatives may be NaN.
+__global__ void __launch_bounds__(128) phase_adjoint_kernel(ProjLaunch L, float* g_phase, float* proj, long long phase_stride,
                                                             float* g_layers, long long layer_stride,
                                                             const long long* layer_off) {
     const SubapDev sd = L.subaps[blockIdx.x];
@@ -567,7 +569,9 @@ __global__ void __launch_bounds__(128) phase_adjoint_kernel(ProjLaunch L, float*
     for (int q = threadIdx.x; q < npx * npx; q += blockDim.x) {
         const int x = q % npx, y = q / npx;
         const float gp = gx * lx[q] + gy * ly[q];
-        if (g_phase) g_phase[off + (long long)(j0 + y) * w.N + i0 + x] = gp;
+        const long long at = off + (long long)(j0 + y) * w.N + i0 + x;
+        if (g_phase) g_phase[at] = gp;
+        if (proj) proj[at] = gx * (gx != 0.0f ? lx[q] : 0.0f) + gy * (gy != 0.0f ? ly[q] : 0.0f);
         if (!g_layers || gp == 0.0f) continue;
         for (int l = 0; l < L.n_layers; ++l) {
             const GridView& v = V[l];
@@ -627,10 +631,10 @@ cudaError_t launch_misreg_sum(const double* rec, int n_rows, double* out, cudaSt
     return cudaGetLastError();
 }
 
-cudaError_t launch_phase_adjoint(const ProjLaunch& L, float* g_phase, long long phase_stride, float* g_layers,
+cudaError_t launch_phase_adjoint(const ProjLaunch& L, float* g_phase, float* proj, long long phase_stride, float* g_layers,
                                  long long layer_stride, const long long* layer_off, cudaStream_t s) {
     if (L.n_valid)
-        phase_adjoint_kernel<<<dim3((unsigned)L.n_valid, (unsigned)L.n_vec), 128, 0, s>>>(L, g_phase, phase_stride, g_layers,
+        phase_adjoint_kernel<<<dim3((unsigned)L.n_valid, (unsigned)L.n_vec), 128, 0, s>>>(L, g_phase, proj, phase_stride, g_layers,
                                                                                          layer_stride, layer_off);
     return cudaGetLastError();
 }

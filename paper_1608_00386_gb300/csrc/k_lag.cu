@@ -149,7 +149,8 @@ __global__ void __launch_bounds__(LagShape<NPX>::G* LagShape<NPX>::NG) wfs_lag_k
         v[2] = fmaf(E[i].x, cy[i].x, fmaf(-E[i].y, cy[i].y, v[2]));
     }
     group_sum3<NPX>(v, s_red, t);
-    const float inv = v[0] > 0.0f ? 1.0f / v[0] : 0.0f;
+    // without light no derivatives; a NaN phase gives NaN
+    const float inv = v[0] != 0.0f ? 1.0f / v[0] : 0.0f;
     if constexpr (SENS) {
         float* rx = sens + w.sens0 + (long long)sd.rank * (NPX * NPX);
         float* ry = rx + (long long)w.n_valid * (NPX * NPX);
@@ -157,8 +158,8 @@ __global__ void __launch_bounds__(LagShape<NPX>::G* LagShape<NPX>::NG) wfs_lag_k
 #pragma unroll
         for (int i = 0; i < S::PPT; ++i) {
             const int q = t + i * S::G;
-            rx[q] = v[0] > 0.0f ? f * fmaf(E[i].x, cx[i].y, E[i].y * cx[i].x) : 0.0f;
-            ry[q] = v[0] > 0.0f ? f * fmaf(E[i].x, cy[i].y, E[i].y * cy[i].x) : 0.0f;
+            rx[q] = v[0] != 0.0f ? f * fmaf(E[i].x, cx[i].y, E[i].y * cx[i].x) : 0.0f;
+            ry[q] = v[0] != 0.0f ? f * fmaf(E[i].x, cy[i].y, E[i].y * cy[i].x) : 0.0f;
         }
     } else if (t == 0) {
         const int ix = w.slope0 + sd.rank, iy = ix + w.n_valid;

@@ -2022,8 +2022,8 @@ static mcao_status run_vjp(mcao_sim* S, const float* gvec, int n_vec, float* gc,
         max_ny = std::max(max_ny, d.ny);
     }
     const int group = std::min(n_vec, kGroup), n_wfs = (int)S->wfs.size();
-    // workspace of a group: the pupil gradients (unless the caller takes them), then U
-    const size_t need_phase = (gc && !g_phase) ? (size_t)group * phase_total : 0;
+    // workspace of a group: the pupil gradients that the projection takes, then U
+    const size_t need_phase = gc ? (size_t)group * phase_total : 0;
     const size_t need = need_phase + (gc ? (size_t)group * n_wfs * S->n_dms * max_n * max_nx : 0);
     cudaError_t e = cudaSuccess;
     if (need > S->vjp_floats) {
@@ -2050,14 +2050,15 @@ static mcao_status run_vjp(mcao_sim* S, const float* gvec, int n_vec, float* gc,
         J.gvec = gvec + (size_t)v0 * S->n_slopes;
         J.n_vec = std::min(group, n_vec - v0);
         J.gc = gc ? gc + (size_t)v0 * S->n_cmd : nullptr;
-        float* gp = g_phase ? g_phase + (size_t)v0 * phase_total : gc ? S->d_vjp : nullptr;
-        if (gp && !g_phase) e = cudaMemsetAsync(gp, 0, sizeof(float) * (size_t)J.n_vec * phase_total, S->s0);
+        float* proj = gc ? S->d_vjp : nullptr;
+        if (proj) e = cudaMemsetAsync(proj, 0, sizeof(float) * (size_t)J.n_vec * phase_total, S->s0);
         if (e == cudaSuccess)
-            e = launch_phase_adjoint(J, gp, phase_total, g_layers ? g_layers + (size_t)v0 * loff[S->n_layers] : nullptr,
-                                     loff[S->n_layers], d_loff, S->s0);
+            e = launch_phase_adjoint(J, g_phase ? g_phase + (size_t)v0 * phase_total : nullptr, proj, phase_total,
+                                     g_layers ? g_layers + (size_t)v0 * loff[S->n_layers] : nullptr, loff[S->n_layers], d_loff,
+                                     S->s0);
         if (e == cudaSuccess && gc && v0 == 0) e = launch_dm_range(J, S->s0);
         if (e == cudaSuccess && gc) {
-            e = launch_dm_project(J, n_wfs, max_n, max_nx, max_ny, gp, phase_total, S->d_vjp + need_phase, S->s0);
+            e = launch_dm_project(J, n_wfs, max_n, max_nx, max_ny, proj, phase_total, S->d_vjp + need_phase, S->s0);
             for (const auto& r : S->runs) {
                 ProjLaunch K = J;
                 K.subaps = r.d_subaps;

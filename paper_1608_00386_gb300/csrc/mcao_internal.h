@@ -353,7 +353,7 @@ cudaError_t launch_dm_project(const ProjLaunch& L, int n_wfs, int max_n, int max
 cudaError_t launch_misreg_gn(const ProjLaunch& L, int m, const float* D_meas, long long ld_meas, int cmd0, double* rec,
                              cudaStream_t s);
 cudaError_t launch_misreg_sum(const double* rec, int n_rows, double* out, cudaStream_t s);
-cudaError_t launch_phase_adjoint(const ProjLaunch& L, float* g_phase, long long phase_stride, float* g_layers,
+cudaError_t launch_phase_adjoint(const ProjLaunch& L, float* g_phase, float* proj, long long phase_stride, float* g_layers,
                                  long long layer_stride, const long long* layer_off, cudaStream_t s);
 
 // one readout slot: ring_c[0..n_cmd) = c, ring_s[2q], ring_s[2q+1] = (long, last) Strehl of
