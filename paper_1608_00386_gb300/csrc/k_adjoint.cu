@@ -593,9 +593,11 @@ __global__ void __launch_bounds__(128) phase_adjoint_kernel(ProjLaunch L, float*
 cudaError_t launch_dm_rows(const ProjLaunch& L, int n_px, int sm_count, cudaStream_t s) {
     if (!L.n_valid || !L.n_dms) return cudaSuccess;
     const int nbw = std::max(1, std::min(L.max_band, kAdjMaxBand));
-    const size_t bytes = sizeof(float) * (2 * n_px * n_px + L.n_dms * (n_px <= 16 ? 4 : 3) * n_px * nbw);   // at most 204800
+    const size_t bytes = sizeof(float) * (2 * n_px * n_px + L.n_dms * (n_px <= 16 ? 4 : 3) * n_px * nbw);
     const auto kernel = L.rotated ? dm_rows_kernel<true> : dm_rows_kernel<false>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    // the limit is the kernel's, for every thread: always the largest, 4 DMs with full bands at 32 samples
+    constexpr int kMost = (int)sizeof(float) * (2 * kMaxNpx * kMaxNpx + kMaxDms * 3 * kMaxNpx * kAdjMaxBand);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
     if (e != cudaSuccess) return e;
     // parts of the commands: two blocks per SM where the subapertures alone do not give them
     const int parts = std::max(1, std::min(16, 2 * sm_count / L.n_valid));

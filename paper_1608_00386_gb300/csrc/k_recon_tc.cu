@@ -605,7 +605,7 @@ cudaError_t tc_create(const float* R_rm, int rows_in, int ld, int n_cmd, int n_r
                              !make_map(&P->tmB, P->S, (long long)P->KB * 3 * P->npad, kTcK, 3 * P->npad)))
         e = cudaErrorNotSupported;
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(recon_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P->smem);
+        e = cudaFuncSetAttribute(recon_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemLimit);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
         tc_destroy(P);

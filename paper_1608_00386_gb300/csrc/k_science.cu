@@ -387,7 +387,9 @@ std::vector<float2> sci_twiddles(int M) {
 }
 
 cudaError_t sci_prepare(int M) {
-    size_t sm = fft_smem_bytes(M);
+    // the limit is the kernel's, not one simulation's: always that of the largest size that fits, so that
+    // simulations of different sizes coexist
+    const size_t sm = std::max(fft_smem_bytes(3200), fft_smem_bytes(M));
     cudaError_t e = set_smem((const void*)sci_rows_kernel, sm);
     if (e != cudaSuccess) return e;
     e = set_smem((const void*)sci_cols_kernel, sm);

@@ -403,9 +403,11 @@ namespace {
 
 cudaError_t screen_passes(ScreenPass P, cudaStream_t s) {
     const size_t bytes = screen_fft_smem(P.n);
-    cudaError_t e = cudaFuncSetAttribute(screen_fft_pass<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(screen_fft_pass<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    // the limit is the kernel's, for every thread: always the target, which no size up to 4096 exceeds
+    constexpr int kMost = (int)kScreenSmemTarget;
+    static_assert(3 * sizeof(float2) * 4096 <= kScreenSmemTarget, "one row per block fits");
+    cudaError_t e = cudaFuncSetAttribute(screen_fft_pass<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(screen_fft_pass<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
     if (e != cudaSuccess) return e;
     const unsigned blocks = (unsigned)((P.n + P.rows - 1) / P.rows);
     float2* work = P.dst_c;

@@ -40,6 +40,7 @@ namespace {
 constexpr int kT = 64;          // tile side
 constexpr int kS = 32;          // output side and k depth of one block's product
 constexpr int kThreads = 128;   // 16 x 8 threads, 2 x 4 outputs each
+constexpr int kGramMaxCmd = 28000;   // commands whose row of G fits in shared memory
 
 // One chunk of a product: a[k][r], b[k][c] for k < kS (rows padded by one double).
 struct Chunk {
@@ -675,7 +676,7 @@ extern "C" mcao_status mcao_tikhonov_reconstructor(const float* D, int n_slopes,
     // and as long as a row of G fits in shared memory; above, the tile products read less
     const int gram_smem = n_cmd * (int)sizeof(double);
     const bool sparse = (long long)n_slopes * n_cmd < (1LL << 31) && (long long)nnz * 3 <= (long long)n_slopes * n_cmd &&
-                        n_cmd <= 28000;
+                        n_cmd <= kGramMaxCmd;
     if (e == cudaSuccess && sparse) {
         e = cudaMalloc(&idx, sizeof(int) * 2 * (size_t)(nnz > 0 ? nnz : 1));
         if (e == cudaSuccess) e = cudaMalloc(&val, sizeof(double) * (size_t)(nnz > 0 ? nnz : 1));
@@ -696,8 +697,9 @@ extern "C" mcao_status mcao_tikhonov_reconstructor(const float* D, int n_slopes,
     e = cudaMemsetAsync(d_err, 0, sizeof(int), st);
     if (e == cudaSuccess) e = cudaMemsetAsync(G, 0, sizeof(double) * npad * npad, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(X, 0, sizeof(double) * npad * npad, st);
-    if (e == cudaSuccess && sparse)
-        e = cudaFuncSetAttribute(tik_gram_sparse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, gram_smem);
+    // the limit is the kernel's, for calls of every size from every thread
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(tik_gram_sparse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGramMaxCmd * (int)sizeof(double));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(tik_potrf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPotrfSmem);
     if (e == cudaSuccess) {
         if (sparse) {
