@@ -464,8 +464,8 @@ mcao_status mcao_reconstruct_batch(mcao_sim* sim, const float* slopes, int n_rhs
  *   stream  CUDA stream (cudaStream_t) or NULL for the legacy stream.
  *   lambda  optional host pointer: receives lambda.
  * Every step runs in double precision in the library's kernels: the Gram matrix over the nonzeros of D
- * (a subaperture sees only nearby actuators; a D with more than a third of nonzeros is taken in
- * 64 x 64 tiles), its regularisation, a blocked Cholesky factorisation L L^T together with L^(-1),
+ * (a subaperture sees only nearby actuators; a D with more than a third of nonzeros, or whose nonzeros
+ * the device has no room for, is taken in 64 x 64 tiles), its regularisation, a blocked Cholesky factorisation L L^T together with L^(-1),
  * M^(-1) = L^-T L^-1 and -M^(-1) D^T; float32 output is rounded once, at the store.
  * Temporaries of 2 (64 ceil(n_cmd / 64))^2 doubles (1.04 GB for n_cmd = 8051) and 20 bytes per nonzero
  * are allocated and freed by the call.  Synchronous.  Errors: MCAO_E_INVALID_ARG (null pointers, alpha < 0 or not

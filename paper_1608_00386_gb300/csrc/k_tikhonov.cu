@@ -672,15 +672,24 @@ extern "C" mcao_status mcao_tikhonov_reconstructor(const float* D, int n_slopes,
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(&nnz, at + n_slopes, sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    // compressed products up to a third of nonzeros (more than 2^31 of them wrap to a negative count)
-    // and as long as a row of G fits in shared memory; above, the tile products read less
+    // compressed products up to a third of nonzeros (more than 2^31 of them wrap to a negative count),
+    // as long as a row of G fits in shared memory and the device has room for the nonzeros; else tile products
     const int gram_smem = n_cmd * (int)sizeof(double);
-    const bool sparse = (long long)n_slopes * n_cmd < (1LL << 31) && (long long)nnz * 3 <= (long long)n_slopes * n_cmd &&
-                        n_cmd <= kGramMaxCmd;
+    bool sparse = (long long)n_slopes * n_cmd < (1LL << 31) && (long long)nnz * 3 <= (long long)n_slopes * n_cmd &&
+                  n_cmd <= kGramMaxCmd;
     if (e == cudaSuccess && sparse) {
         e = cudaMalloc(&idx, sizeof(int) * 2 * (size_t)(nnz > 0 ? nnz : 1));
         if (e == cudaSuccess) e = cudaMalloc(&val, sizeof(double) * (size_t)(nnz > 0 ? nnz : 1));
         if (e == cudaSuccess) e = cudaMalloc(&col_val, sizeof(float) * (size_t)(nnz > 0 ? nnz : 1));
+        if (e == cudaErrorMemoryAllocation) {   // no room beside the factors: the tiles need none
+            cudaGetLastError();
+            for (void* p : {(void*)idx, (void*)val, (void*)col_val}) cudaFree(p);
+            idx = nullptr;
+            val = nullptr;
+            col_val = nullptr;
+            sparse = false;
+            e = cudaSuccess;
+        }
     }
     if (e == cudaSuccess && !sparse) e = cudaMalloc(&mask, (size_t)nS * nt);
     auto cleanup = [&]() {
