@@ -2312,7 +2312,17 @@ mcao_status mcao_get_psf(mcao_sim* S, int sci, double* out, size_t n, double* sr
         if (S->psf_out_n < M * M) {
             dfree(S->d_psf_out);
             S->psf_out_n = 0;
-            CK(dalloc(&S->d_psf_out, M * M));
+            const cudaError_t e = dalloc(&S->d_psf_out, M * M);
+            if (e == cudaErrorMemoryAllocation) {   // no room for a second image: ordered on the host
+                cudaGetLastError();
+                S->d_psf_out = nullptr;
+                std::vector<double> t(M * M);
+                CK(cudaMemcpy(t.data(), C.d_psf_t + (size_t)S->cur * M * M, sizeof(double) * M * M, cudaMemcpyDeviceToHost));
+                for (size_t j = 0; j < M; ++j)
+                    for (size_t i = 0; i < M; ++i) out[j * M + i] = t[((i + M / 2) % M) * M + (j + M / 2) % M] * norm;
+                return MCAO_OK;
+            }
+            CK(e);
             S->psf_out_n = M * M;
         }
         CK(launch_psf_out(C.d_psf_t + (size_t)S->cur * M * M, C.M, norm, S->d_psf_out, S->s0));

@@ -3,9 +3,12 @@ the plain one alone: the same results as with room to spare."""
 import contextlib
 import ctypes as C
 
+import numpy as np
 import pytest
 
-from paper_1608_00386_gb300 import build, mcao
+from paper_1608_00386_gb300 import build, inputs, mcao
+
+from _helpers import mcao_small
 
 pytestmark = pytest.mark.gpu
 
@@ -60,3 +63,23 @@ def test_control_matrix_without_room_for_the_compressed_matrix():
     assert lam2.value == pytest.approx(lam, rel=1e-12)
     # sums of the same terms in another order: the tolerance of both routes against the oracle
     assert float((out - want).abs().max()) <= 1e-10 * float(want.abs().max())
+
+
+def test_psf_image_without_room_for_a_second_one():
+    def stepped():
+        cfg = mcao_small()
+        cfg["science"][0].update(n_px=512, pad=4)   # 2048 x 2048 doubles, 33 MB
+        s = mcao.Sim(cfg)
+        s.load_atmosphere(inputs.make_screens(cfg))
+        s.load_dms()
+        s.load_reconstructor(inputs.random_reconstructor(s.query(mcao.Q_COMMANDS), s.query(mcao.Q_SLOPES), 1e-3, 4))
+        s.step(2)
+        return s
+
+    want = stepped().psf(0)
+    s = stepped()
+    s.sync()
+    with _only(16 << 20):
+        got = s.psf(0)
+    assert np.array_equal(got[0], want[0]) and got[1:] == want[1:]
+    assert np.array_equal(s.psf(0)[0], want[0])   # and with room again
