@@ -2021,18 +2021,26 @@ static mcao_status run_vjp(mcao_sim* S, const float* gvec, int n_vec, float* gc,
         max_nx = std::max(max_nx, d.nx);
         max_ny = std::max(max_ny, d.ny);
     }
-    const int group = std::min(n_vec, kGroup), n_wfs = (int)S->wfs.size();
-    // workspace of a group: the pupil gradients that the projection takes, then U
-    const size_t need_phase = gc ? (size_t)group * phase_total : 0;
-    const size_t need = need_phase + (gc ? (size_t)group * n_wfs * S->n_dms * max_n * max_nx : 0);
-    cudaError_t e = cudaSuccess;
-    if (need > S->vjp_floats) {
+    const int n_wfs = (int)S->wfs.size();
+    cudaError_t e = enqueue_sens(S);
+    // workspace of a group, as many vectors as there is room for: the pupil gradients that the projection
+    // takes, then U
+    int group = std::min(n_vec, kGroup);
+    size_t need_phase = 0;
+    for (; e == cudaSuccess; group = (group + 1) / 2) {
+        need_phase = gc ? (size_t)group * phase_total : 0;
+        const size_t need = need_phase + (gc ? (size_t)group * n_wfs * S->n_dms * max_n * max_nx : 0);
+        if (need <= S->vjp_floats) break;
         dfree(S->d_vjp);
         S->vjp_floats = 0;
-        e = dalloc(&S->d_vjp, need);
-        if (e == cudaSuccess) S->vjp_floats = need;
+        if ((e = dalloc(&S->d_vjp, need)) == cudaSuccess) {
+            S->vjp_floats = need;
+            break;
+        }
+        S->d_vjp = nullptr;
+        if (e != cudaErrorMemoryAllocation || group == 1) break;
+        e = cudaGetLastError() == cudaErrorMemoryAllocation ? cudaSuccess : e;
     }
-    if (e == cudaSuccess) e = enqueue_sens(S);
     if (e == cudaSuccess && gc) e = cudaMemsetAsync(gc, 0, sizeof(float) * (size_t)n_vec * S->n_cmd, S->s0);
     if (e == cudaSuccess && g_phase) e = cudaMemsetAsync(g_phase, 0, sizeof(float) * (size_t)n_vec * phase_total, S->s0);
     // layers concatenated: offsets and total length

@@ -83,3 +83,23 @@ def test_psf_image_without_room_for_a_second_one():
         got = s.psf(0)
     assert np.array_equal(got[0], want[0]) and got[1:] == want[1:]
     assert np.array_equal(s.psf(0)[0], want[0])   # and with room again
+
+
+def test_command_gradients_without_room_for_a_whole_group():
+    import torch
+
+    def loaded():
+        cfg = inputs.mcao_20m()
+        s = mcao.Sim(cfg)
+        s.load_atmosphere(inputs.make_screens(cfg))
+        s.load_dms()
+        s.set_commands(np.random.default_rng(1).normal(0.0, 0.3, s.query(mcao.Q_COMMANDS)).astype(np.float32))
+        return s
+
+    a, b = loaded(), loaded()
+    v = torch.randn((8, a.query(mcao.Q_SLOPES)), device="cuda", generator=torch.Generator(device="cuda").manual_seed(1))
+    want = a.slopes_vjp(v)[0]
+    out = torch.empty_like(want)
+    with _only(12 << 20):   # the derivatives take 2 MB, eight vectors 13 MB more
+        b._ck(mcao.lib().mcao_slopes_vjp(b.h, v.data_ptr(), 8, out.data_ptr(), None, None))
+    assert torch.equal(out, want)   # no sum crosses vectors
