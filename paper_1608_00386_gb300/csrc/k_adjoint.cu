@@ -41,12 +41,6 @@ __device__ __forceinline__ int2 footprint(AxisEnt a, AxisEnt b) {
     return make_int2(min(a.idx & 0xffff, b.idx & 0xffff), max(a.idx >> 16, b.idx >> 16));
 }
 
-// actuator a acts on the two surface samples of entry e: it is in the band of their tiles
-__device__ __forceinline__ bool reaches(const int2* band, AxisEnt e, int a) {
-    const int2 b0 = band[(e.idx & 0xffff) / kDmTile], b1 = band[(e.idx >> 16) / kDmTile];
-    return (a >= b0.x && a < b0.y) || (a >= b1.x && a < b1.y);
-}
-
 // Actuators [a0, a1) x [b0, b1) of a DM that act on surface samples [cx.x, cx.y] x [cy.x, cy.y]: for a
 // separable DM the union of the forward's per-tile bands over the tiles the footprint touches, for a
 // rotated one the actuators within rc pitches of the footprint's corners.
@@ -488,19 +482,15 @@ __global__ void __launch_bounds__(256) dm_project_x(ProjLaunch L, const float* _
         __syncthreads();
         for (int q = threadIdx.x; q < 32 * 32; q += 256) {
             const int x = x0 + (q >> 5), a = a0 + (q & 31);
-            float wt = 0.0f;
-            if (x < N && a >= bt.x && a < bt.y) {
-                const AxisEnt e = entry(x);
-                if (reaches(L.band + dd.tband_x, e, a)) wt = axis_weight(L.g + dd.gx_off, dd.nx, e, a);
-            }
-            s_w[q >> 5][q & 31] = wt;
+            const float wt = (x < N && a >= bt.x && a < bt.y) ? axis_weight(L.g + dd.gx_off, dd.nx, entry(x), a) : 0.0f;
+            s_w[q >> 5][q & 31] = wt < 1e-10f ? 0.0f : wt;   // the band is wider than this sample's own reach
         }
         s_g[warp][lane] = (y < N && x0 + lane < N) ? g_phase[off + (long long)y * N + x0 + lane] : 0.0f;
         __syncthreads();
 #pragma unroll 8
         for (int x = 0; x < 32; ++x) {
             const float wt = s_w[x][lane];
-            acc = wt != 0.0f ? fmaf(s_g[warp][x], wt, acc) : acc;   // a NaN reaches the actuators with a weight alone
+            if (wt != 0.0f) acc = fmaf(s_g[warp][x], wt, acc);   // a NaN reaches the actuators with a weight alone
         }
     }
     if (y < N && a0 + lane < dd.nx) U[(((long long)vec * gridDim.y + blockIdx.y) * u_rows + y) * u_cols + a0 + lane] = acc;
@@ -527,7 +517,8 @@ __global__ void __launch_bounds__(1024) dm_project_y(ProjLaunch L, int n_wfs, co
             float gy = 0.0f;
             if (y0 + lane < w.N) {
                 const AxisEnt e = axis_entry(v.ay + (long long)(y0 + lane) * v.bp, v.n, v.periodic, v.inv_n);
-                if (reaches(L.band + dd.tband_y, e, b)) gy = v.sign * axis_weight(L.g + dd.gy_off, dd.ny, e, b);
+                const int2 b0 = L.band[dd.tband_y + (e.idx & 0xffff) / kDmTile], b1 = L.band[dd.tband_y + (e.idx >> 16) / kDmTile];
+                if ((b >= b0.x && b < b0.y) || (b >= b1.x && b < b1.y)) gy = v.sign * axis_weight(L.g + dd.gy_off, dd.ny, e, b);
             }
             if (!__ballot_sync(0xffffffffu, gy != 0.0f)) continue;
 #pragma unroll 8
