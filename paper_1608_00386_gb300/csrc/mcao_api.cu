@@ -21,6 +21,7 @@
 
 #include "../../include/mcao.h"
 #include "capture_edges.h"
+#include "fork_launches.h"
 #include "mcao_internal.h"
 
 using namespace mcao;
@@ -895,24 +896,13 @@ mcao_status validate_config(const mcao_config* c) {
     return MCAO_OK;
 }
 
-// One launch per run of sensors, behind s0's work so far and before its later work.  The first run stays
-// on s0, the others go to s1 beside it: a run of low-order sensors is a few blocks, whose latency (13 us
-// at 20 m) would otherwise add to the laser stars'.
+// One launch per run of sensors (fork_launches): a run of low-order sensors is a few blocks, whose latency
+// (13 us at 20 m) would otherwise add to the laser stars'.
 template <class F>
 cudaError_t for_each_run(mcao_sim* S, F&& launch) {
-    cudaError_t e = cudaSuccess;
-    const bool fork = S->runs.size() > 1;
-    if (fork) {
-        e = cudaEventRecord(S->ev_done, S->s0);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(S->s1, S->ev_done, 0);
-    }
-    for (size_t i = 0; i < S->runs.size() && e == cudaSuccess; ++i)
-        if (S->runs[i].n_subaps > 0) e = launch(S->runs[i], i == 0 ? S->s0 : S->s1);
-    if (fork) {
-        if (e == cudaSuccess) e = cudaEventRecord(S->ev_done, S->s1);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(S->s0, S->ev_done, 0);
-    }
-    return e;
+    return fork_launches(S->s0, S->s1, S->ev_done, (int)S->runs.size(), [&](int i, cudaStream_t st) {
+        return S->runs[i].n_subaps > 0 ? launch(S->runs[i], st) : cudaSuccess;
+    });
 }
 
 // device address of a page-locked host buffer (false: any other memory, or one not aligned to its type)
@@ -1977,7 +1967,8 @@ static int footprint_band(const mcao_sim* S, const WfsRun& r) {
 // waits for the queued calibration work; a band overflow becomes MCAO_E_UNSUPPORTED
 static mcao_status finish_adjoint(mcao_sim* S, cudaError_t e) {
     int h_err = 0;
-    if (e == cudaSuccess) e = cudaStreamSynchronize(S->s0);
+    const cudaError_t done = cudaStreamSynchronize(S->s0);   // after a failure too: the outputs are the caller's again
+    if (e == cudaSuccess) e = done;
     if (e == cudaSuccess) e = cudaMemcpy(&h_err, S->d_adj_err, sizeof(int), cudaMemcpyDeviceToHost);
     CK(e);
     if (h_err) {
