@@ -2175,6 +2175,8 @@ mcao_status mcao_autotune(mcao_sim* S, int steps_per_trial, int* values, int n, 
     for (auto& kn : knobs) {
         const int k = kn.first;
         int best = cur[k];
+        S->tune = tuning_from(cur);
+        if (k == 2 && sensing_groups(S).size() <= 1) kn.second = {best};   // without effect there
         rep += std::string("; ") + names[k] + ":";
         for (int c : kn.second) {
             if (r != MCAO_OK) break;
