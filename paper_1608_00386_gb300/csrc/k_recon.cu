@@ -36,8 +36,6 @@ namespace mcao {
 
 namespace {
 
-constexpr int kKC = kReconChunk;
-
 // packed FP32 multiply-add (two lanes of a 64-bit register pair per instruction):
 // (c.x, c.y) + (a.x b.x, a.y b.y), each rounded once
 __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {

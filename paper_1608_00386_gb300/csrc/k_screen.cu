@@ -458,6 +458,11 @@ cudaError_t half_passes(ScreenPass P, cudaStream_t s) {
 
 }  // namespace
 
+// powers of two from 256 to 4096; the passes store pairs of columns, so they need an 8-byte aligned screen
+bool screen_is_half(int n, const float* out) {
+    return n >= 256 && n <= 4096 && (n & (n - 1)) == 0 && reinterpret_cast<uintptr_t>(out) % 8 == 0;
+}
+
 cudaError_t launch_screen(int n, double pixel, double r0, double L0, unsigned long long seed, const int* radices,
                           int n_radices, float2* work, float2* W, float* out, cudaStream_t s) {
     ScreenPass P{};
@@ -473,8 +478,7 @@ cudaError_t launch_screen(int n, double pixel, double r0, double L0, unsigned lo
     for (int i = 0; i < n_radices && i < 16; ++i) P.radices[i] = radices[i];
     P.dst_c = work;
     P.dst_r = out;
-    // the half-spectrum passes store pairs of columns, so they need an 8-byte aligned screen
-    if (reinterpret_cast<uintptr_t>(out) % 8 == 0) switch (n) {
+    if (screen_is_half(n, out)) switch (n) {
         case 256: return half_passes<256>(P, s);
         case 512: return half_passes<512>(P, s);
         case 1024: return half_passes<1024>(P, s);

@@ -1045,10 +1045,6 @@ mcao_status mcao_sim_create(const mcao_config* cfg, mcao_sim** out) {
             double sgn = (((u % 2) + 2) % 2) ? -1.0 : 1.0;
             D.h[u + npx - 1] = make_float2((float)(sgn * re), (float)(sgn * im));
         }
-        for (int k = 0; k < H.n_det && k < kMaxNd; ++k) {
-            double a = 2.0 * M_PI * (double)k / (double)H.n_det;
-            D.tw[k] = make_float2((float)std::cos(a), (float)std::sin(a));
-        }
         // lag weights of the centre of gravity: h(u) sum_m (m - c) exp(2 pi i u m / n_det) / (n_bin n_det)
         for (int u = -(npx - 1); u <= npx - 1 && npx <= kMaxNpx; ++u) {
             double hr = 0, hi = 0, dr = 0, di = 0;
@@ -2666,7 +2662,7 @@ mcao_status mcao_generate_screen(int n, double pixel_m, double r0_m, double L0_m
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     float2 *b = nullptr, *w = nullptr;
     e = cudaMallocAsync((void**)&b, sizeof(float2) * (size_t)n * n, st);
-    if (e == cudaSuccess) e = cudaMallocAsync((void**)&w, sizeof(float2) * n, st);
+    if (e == cudaSuccess && !screen_is_half(n, out)) e = cudaMallocAsync((void**)&w, sizeof(float2) * n, st);
     if (e == cudaSuccess) e = launch_screen(n, pixel_m, r0_m, L0_m, seed, rad.data(), (int)rad.size(), b, w, out, st);
     for (float2* p : {b, w})
         if (p) cudaFreeAsync(p, st);

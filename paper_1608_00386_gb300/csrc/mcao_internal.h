@@ -23,7 +23,6 @@ struct Tuning {
 };
 constexpr int kTuningKnobs = 6;
 constexpr int kMaxNpx = 32;       // pupil samples per subaperture side
-constexpr int kMaxNd = 32;        // detector pixels per subaperture side
 constexpr int kMaxDms = 4;
 constexpr int kMaxGridN = 65535;  // grid side (indices are packed in 16 bits)
 
@@ -55,7 +54,6 @@ struct WfsDev {
     float n_photons, read_noise;
     const float* amp;    // [N][N] pupil amplitude
     float2 h[2 * kMaxNpx - 1];  // (-1)^u sum_{t<n_bin} exp(2 pi i u t / n_fft), u = -(n_px-1)..n_px-1
-    float2 tw[kMaxNd];          // exp(2 pi i k / n_det)
     float2 kap[2 * kMaxNpx - 1];   // lag weights of the centre of gravity without elongation (k_lag.cu), u = -(n_px-1)..n_px-1
     long long sens0;            // first float of this sensor's block of slope derivatives: [2 n_valid][n_px^2]
 };
@@ -306,6 +304,7 @@ cudaError_t launch_sci_cols(const SciLaunch& L, cudaStream_t s);   // also the S
 // phase screens (von Karman, FFT method)
 // ---------------------------------------------------------------------------------------------
 size_t screen_fft_smem(int n);
+bool screen_is_half(int n, const float* out);   // by the half-spectrum passes, which need no table W
 cudaError_t launch_screen(int n, double pixel, double r0, double L0, unsigned long long seed, const int* radices,
                           int n_radices, float2* work, float2* W, float* out, cudaStream_t s);
 
