@@ -480,7 +480,8 @@ mcao_status mcao_tikhonov_reconstructor(const float* D, int n_slopes, int n_cmd,
  *   MCAO_TUNE_SENSE_BLOCKS_PER_SM  warp-per-subaperture sensing launches: blocks per SM, [1, 8] (4)
  *   MCAO_TUNE_RECON_CTAS_PCT       reconstructor slices: blocks per SM x 100, [25, 400] (85); the
  *                                  step's last slice, which runs after the last sensor, takes at
- *                                  least one block per SM
+ *                                  least one block per SM; up to a sixteenth more blocks (never
+ *                                  more than SMs) where that saves a round of work items
  *   MCAO_TUNE_SCIENCE_AFTER_AUX    where the step has several warp-per-subaperture launches, science waits
  *                                  for the block-per-subaperture sensors, 0 or 1 (1)
  *   MCAO_TUNE_TC_CHUNK             tensor-core batched product: k-blocks per TMEM accumulator,
@@ -510,10 +511,11 @@ mcao_status mcao_set_tuning(mcao_sim* sim, const int* values, int n);
 
 /* Autotuner: for each launch shape that applies to this configuration (the sensing grid when it
  * has warp-per-subaperture sensors, the slices' grid without batching, the science ordering when
- * it has block-per-subaperture sensors, the batched products' shapes with batching, the steps per
- * graph among 1, 2, 4 and 8), in that order,
+ * it has block-per-subaperture sensors and several warp-per-subaperture launches, the batched
+ * products' shapes with batching, the steps per graph among 1, 2, 4 and 8), in that order,
  * time steps_per_trial steps (after 2 warm-up steps) for every candidate value with the others
- * held at their best so far, and keep the fastest (coordinate descent, CUDA events on the device).
+ * held at their best so far, and keep the fastest (coordinate descent, CUDA events on the device); a
+ * value is left only for one that is faster by half a per cent.
  * The trials advance the simulation; its state is saved first and restored at the end (as
  * mcao_get_state / mcao_set_state), so the caller's run continues as if no trial had run.  The
  * chosen shapes stay set; values (n >= MCAO_N_TUNE, may be NULL) receives them and report (may be

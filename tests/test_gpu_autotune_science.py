@@ -1,5 +1,6 @@
-"""The autotuner and the science's start: with one sensing launch the knob has no effect, so it is not tried
-and stays as it was; with several both values are."""
+"""What the autotuner tries and keeps.  The science's start: with one sensing launch the knob has no effect, so
+it is not tried and stays as it was; with several both values are.  Any knob: a value is left only for one
+that is faster by half a per cent of the best time so far."""
 import re
 
 import pytest
@@ -34,3 +35,29 @@ def test_tried_where_it_has_an_effect(launches, set_to):
     tried = re.findall(r"(\d)=", re.search(r"science_after_aux:(.*?) ->", report).group(1))
     assert tried == ([str(set_to)] if launches == 1 else ["0", "1"])
     assert launches == 2 or chosen["science_after_aux"] == set_to
+
+
+def test_a_value_is_left_only_for_a_faster_one():
+    import torch
+    cfg = inputs.eelt_mcao(noise=True, n_layers=2)   # steps of 0.4 ms: the times' last digit is 0.03 % of them
+    g = mcao.Sim(cfg)
+    g.generate_atmosphere()
+    g.load_dms()
+    g.load_reconstructor(torch.zeros((g.query(mcao.Q_COMMANDS), g.query(mcao.Q_SLOPES)), device="cuda"))
+    now = g.tuning()
+    chosen, report = g.autotune(steps_per_trial=20)
+    best = float(re.search(r"start ([\d.]+) ms", report).group(1))
+    checked = 0
+    for name, trials, kept in re.findall(r"; (\w+):((?: \d+=[\d.]+)+) -> (\d+)", report):
+        value, clear = now[name], True
+        for v, ms in re.findall(r"(\d+)=([\d.]+)", trials):
+            limit = best * (1.0 if int(v) == value else 0.995)
+            clear = clear and abs(float(ms) - limit) > 1.1e-4   # within the last digit either way is right
+            if float(ms) < limit:
+                value, best = int(v), float(ms)
+        if not clear:
+            break
+        assert value == int(kept) == chosen[name], report
+        checked += 1
+    if not checked:
+        pytest.skip("trials at the limit")
