@@ -308,7 +308,8 @@ mcao_status mcao_quantize_rows(const float* R, int rows, int cols, int ld, int d
 
 /* Sodium layer evolution ("The closed loop": the sodium layer temporal evolution): from the
  * next step on, laser sensor `wfs` sees the layer at `height` m (its cone projection) with
- * thickness `na_fwhm` m (its elongation).  Call between steps to follow a profile in time.
+ * thickness `na_fwhm` m (its elongation).  Call between steps to follow a profile in time.  The layer
+ * may come below a DM that was loaded under a higher one.
  * Errors: MCAO_E_INVALID_ARG (not a laser sensor, height not above every layer, negative
  * thickness), MCAO_E_UNSUPPORTED (elongation on a sensor without an elongated-spot kernel). */
 mcao_status mcao_set_sodium(mcao_sim* sim, int wfs, double height, double na_fwhm);
@@ -432,7 +433,8 @@ mcao_status mcao_misreg_normal_equations(mcao_sim* sim, int dm, const float* D_m
  *   g_layers    device [n_vec][sum over layers of n_l^2] = (d s / d screen)^T g on every turbulent
  *               layer's screen (the adjoint of the cone-beam projection at this step's frozen-flow
  *               position), layers concatenated in order (or NULL).
- * Outputs are overwritten.  Layer gradients and the command gradients of rotated DMs are accumulated
+ * Outputs are overwritten.  A slope with g = 0 adds nothing to the command gradients, also where its
+ * derivatives are NaN.  Layer gradients and the command gradients of rotated DMs are accumulated
  * with atomic adds (summation order not fixed).  Synchronous.  Errors: MCAO_E_INVALID_ARG (null g, n_vec < 1,
  * every output NULL), MCAO_E_STATE, MCAO_E_UNSUPPORTED, MCAO_E_OOM, MCAO_E_CUDA. */
 mcao_status mcao_slopes_vjp(mcao_sim* sim, const float* g_slopes, int n_vec, float* g_commands, float* g_phase,

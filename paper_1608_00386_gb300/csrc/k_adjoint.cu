@@ -238,11 +238,10 @@ __device__ __forceinline__ void zero_run(float* p, int n, int lane) {
 // rows of the band (each command checked against the band's columns) and a run of zeros.  One block
 // does every DM, so that the three barriers of the setup are paid once per 2 n_cmd stored floats and
 // hide behind the other blocks' stores; a sensor of a few subapertures is cut into enough parts to
-// fill the GPU.  39 m (55608 x 8051, 1.79 GB), six laser stars: 470 us (484 with the zeros as four runs per DM by the whole block and the weights
-// formed again for every sample row; 580 with whole rows cleared first and the band written over them);
-// with a block per DM and
-// a check of every command 789 us; before that the matrix was cleared and one block per slope
-// scattered its band: 6 x 160 us and 3 x 131 us (natural stars) on top of the clearing.
+// fill the GPU, and no part writes another's commands (row_parts.h).  39 m (55608 x 8051, 1.79 GB), six
+// laser stars: 470 us, bound by the instructions that form the weights and by the writes; clearing the
+// matrix and scattering one slope's band per block took 6 x 160 us and 3 x 131 us more (natural
+// stars), clearing whole rows first 580, a block per DM that checks every command 789.
 // With gvec set (rotated DMs only) the rows are not stored: sum over both slopes of g row is added
 // to the command gradients of every vector.
 struct RowsDm {                // one DM's view from the block's subaperture

@@ -176,10 +176,11 @@ extern "C" mcao_status mcao_reconstruct_noalloc(const float* R, int n_cmd, int n
         }
         scratch = g_scratch[dev];
     }
-    // shorter chunks where the longest ones leave SMs without blocks, as far as the scratch holds their sums
-    // (us a call with chunks of up to 4096 and a reduction of one thread per row, and now: 300 x 2000 13.3,
-    // 6.2; 1870 x 7280 28.7, 12.5; 1300 x 15000 32.8, 18.4; 41 x 55000 16.4, 8.2; 8051 x 55608 288.1, 284.5
-    // with the same chunks; four to eight blocks per SM or 512 columns: 8.2, 12.4, 20.5, 8.2, 284.5)
+    // Shorter chunks where the longest ones leave SMs without blocks, as far as the scratch holds their sums:
+    // 16 blocks per SM hide the loads' latency at every size (us a call with chunks of 4096 columns and one
+    // thread per row in the reduction, and so: 300 x 2000 13.3, 6.2; 1870 x 7280 28.7, 12.5; 1300 x 15000
+    // 32.8, 18.4; 41 x 55000 16.4, 8.2; four to eight blocks or 512 columns 8.2, 12.4, 20.5, 8.2).  8051 x
+    // 55608 keeps its 14 chunks: 288.1, 284.5 with the reduction's eight lanes per row.
     int sm_count = 0;
     e = cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return report(err, err_len, MCAO_E_CUDA, "cudaDeviceGetAttribute: %s", cudaGetErrorString(e));

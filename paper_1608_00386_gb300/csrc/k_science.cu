@@ -5,7 +5,7 @@
 //   long-exposure PSF += |FFT2(E zero-padded to M x M)|^2 accumulated in double.
 // The 2-D FFT runs as two passes of batched radix-4/5/2 Stockham FFTs in shared memory: rows of
 // the field (zero-padded) written transposed, then rows of the transposed array; the PSF
-// accumulator is therefore held transposed and unshifted, [kx][ky] (the host reorders it).
+// accumulator is therefore held transposed and unshifted, [kx][ky] (psf_out_kernel reorders it).
 #include <algorithm>
 #include <cmath>
 #include <vector>

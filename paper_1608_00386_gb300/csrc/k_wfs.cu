@@ -103,7 +103,8 @@ __global__ void __launch_bounds__(256, 4) wfs_acf_kernel(WfsLaunch L) {
     // per warp: axis entries (dead after the field, then reused for the second lag row of each
     // pass and for the row transform),
     // grid metadata, the field (reused for M_uy), the lag products; per block: twiddles and
-    // reciprocals.  About 30 KB per block, so three blocks fit beside a reconstructor block.
+    // reciprocals.  38 KB and 256 threads of 64 registers per block: two fit beside a reconstructor block
+    // (its 160 threads of 128 registers leave room for no third).
     union Scratch {
         AxisEnt e[2][kMaxEntries * NPX];
         float2 y[NPX * ND];

@@ -247,7 +247,8 @@ struct ReconLaunch {
     const float* scale; // per-row scales (kReconE4M3), else null
     float* partial;     // [n_chunks][n_cmd]
     int max_ctas;       // grid size cap (0: enough blocks for every item); may be passed by a sixteenth, up
-    int sm_count;       // to the number of SMs, where that saves a round of items
+                        // to the number of SMs, where that saves a round of items
+    int sm_count;
     unsigned int* work; // item counter, zero when the launch starts
     int* err;           // set to a nonzero code if a bounded wait gives up
 };
